@@ -359,14 +359,12 @@ int collide_chain(const bz_modes *m, int precision, int flags, const void *f, vo
     return rc;
 }
 
-// Transport residual L [cell][nv] of f over the mesh: CWENO gradients into
-// scratch (`ext` if given: transport_scratch_bytes), then the fluxes.
+// Transport residual L [cell][nv] of f over the mesh: one pass for order 1,
+// else the face fluxes or values into scratch (`ext` if given:
+// transport_scratch_bytes), then their sums.
 size_t transport_scratch_bytes(const bz_mesh *mesh, const bz_grid *g, int precision) {
-    if (mesh->order == 1) return 0;
-    // values per (cell, velocity): 5 coefficients, 3 face values (FP32 triangles without walls) or 2 gradients
-    const bool faces = precision == BZ_FP32 && mesh->max_faces <= 3 && mesh->n_walls == 0;
-    const size_t per = mesh->order == 3 ? (size_t)kFvCoef3 : faces ? 3 : 2;
-    return per * mesh->n_cells * g->v.nv * (precision == BZ_FP64 ? sizeof(double) : sizeof(float));
+    return (size_t)fv_scratch_rows(mesh, precision != BZ_FP64) * g->v.nv *
+           (precision == BZ_FP64 ? sizeof(double) : sizeof(float));
 }
 
 int transport_chain(const bz_mesh *mesh, const bz_grid *g, int precision, const void *f, void *L, cudaStream_t st,
@@ -374,61 +372,34 @@ int transport_chain(const bz_mesh *mesh, const bz_grid *g, int precision, const 
     const GridView &v = g->v;
     if (!fv_walls_supported(mesh, v))
         return fail(BZ_ENOTSUP, "transport: walls need N divisible by 4 and at most 32^2 velocities");
-    Scratch s;
-    if (mesh->order == 3) {
-        if (!ext) BZ_TRY(s.alloc(transport_scratch_bytes(mesh, g, precision), st), "transport: scratch");
-        void *C = ext ? ext : s.p;
-        if (precision == BZ_FP64) {
-            BZ_LAUNCH("fv_coef3_f64", st,
-                      launch_fv_coef3_f64(mesh, v, static_cast<const double *>(f), static_cast<double *>(C), st),
-                      "transport: reconstruction");
-            BZ_LAUNCH("fv_flux3_f64", st,
-                      launch_fv_flux3_f64(mesh, v, static_cast<const double *>(f), static_cast<const double *>(C),
-                                          static_cast<double *>(L), st),
-                      "transport: fluxes");
-        } else {
-            BZ_LAUNCH("fv_coef3_f32", st,
-                      launch_fv_coef3_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(C), st),
-                      "transport: reconstruction");
-            BZ_LAUNCH("fv_flux3_f32", st,
-                      launch_fv_flux3_f32(mesh, v, static_cast<const float *>(f), static_cast<const float *>(C),
-                                          static_cast<float *>(L), st),
-                      "transport: fluxes");
-        }
+    const bool d = precision == BZ_FP64;
+    if (mesh->order == 1) {
+        BZ_LAUNCH(d ? "fv_first_f64" : "fv_first_f32", st,
+                  d ? launch_fv_first_f64(mesh, v, static_cast<const double *>(f), static_cast<double *>(L), st)
+                    : launch_fv_first_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(L), st),
+                  "transport: fluxes");
         return BZ_OK;
     }
-    void *G = nullptr;
-    if (mesh->order == 2) {
-        if (!ext) BZ_TRY(s.alloc(transport_scratch_bytes(mesh, g, precision), st), "transport: scratch");
-        G = ext ? ext : s.p;
-        if (precision == BZ_FP32 && fv_face_mode(mesh, v, f, L, G)) {
-            BZ_LAUNCH("fv_gradient_f32", st,
-                      launch_fv_faces_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(G), st),
-                      "transport: reconstruction");
-            BZ_LAUNCH("fv_flux_f32", st,
-                      launch_fv_flux_faces_f32(mesh, v, static_cast<const float *>(G), static_cast<float *>(L), st),
-                      "transport: fluxes");
-            return BZ_OK;
-        }
-        if (precision == BZ_FP64)
-            BZ_LAUNCH("fv_gradient_f64", st,
-                      launch_fv_gradient_f64(mesh, v, static_cast<const double *>(f), static_cast<double *>(G), st),
-                      "transport: reconstruction");
-        else
-            BZ_LAUNCH("fv_gradient_f32", st,
-                      launch_fv_gradient_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(G), st),
-                      "transport: reconstruction");
+    Scratch s;
+    if (!ext) BZ_TRY(s.alloc(transport_scratch_bytes(mesh, g, precision), st), "transport: scratch");
+    void *FX = ext ? ext : s.p;
+    if (!d && fv_value_mode(mesh, v, f, L)) {
+        BZ_LAUNCH("fv_values_f32", st,
+                  launch_fv_values_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(FX), st),
+                  "transport: reconstruction");
+        BZ_LAUNCH("fv_flux_values_f32", st,
+                  launch_fv_flux_values_f32(mesh, v, static_cast<const float *>(FX), static_cast<float *>(L), st),
+                  "transport: fluxes");
+        return BZ_OK;
     }
-    if (precision == BZ_FP64)
-        BZ_LAUNCH("fv_flux_f64", st,
-                  launch_fv_flux_f64(mesh, v, static_cast<const double *>(f), static_cast<const double *>(G),
-                                     static_cast<double *>(L), st),
-                  "transport: fluxes");
-    else
-        BZ_LAUNCH("fv_flux_f32", st,
-                  launch_fv_flux_f32(mesh, v, static_cast<const float *>(f), static_cast<const float *>(G),
-                                     static_cast<float *>(L), st),
-                  "transport: fluxes");
+    BZ_LAUNCH(d ? "fv_faces_f64" : "fv_faces_f32", st,
+              d ? launch_fv_faces_f64(mesh, v, static_cast<const double *>(f), static_cast<double *>(FX), st)
+                : launch_fv_faces_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(FX), st),
+              "transport: face fluxes");
+    BZ_LAUNCH(d ? "fv_sum_f64" : "fv_sum_f32", st,
+              d ? launch_fv_sum_f64(mesh, v, static_cast<const double *>(FX), static_cast<double *>(L), st)
+                : launch_fv_sum_f32(mesh, v, static_cast<const float *>(FX), static_cast<float *>(L), st),
+              "transport: sums");
     return BZ_OK;
 }
 
@@ -441,13 +412,26 @@ int check_input(int precision, const void *f, int64_t count, cudaStream_t st) {
     return BZ_OK;
 }
 
+// Whether a later stage's explicit part weighs stage l (its G and its transport
+// residual), and whether one's implicit part weighs P_l.
+bool explicit_used(const Tableau &t, int l) {
+    for (int q = l + 1; q < t.s; ++q)
+        if (t.At[q][l] != 0.0) return true;
+    return false;
+}
+bool implicit_used(const Tableau &t, int l) {
+    for (int q = l + 1; q < t.s; ++q)
+        if (t.A[q][l] != 0.0) return true;
+    return false;
+}
+
 // One IMEX stage: F_l, P_l by the stage kernel, then G_l = Q(F_l) - P_l.
-// in_step: called by step_sequence (library scratch): stage 0's F (= f^n
-// exactly when A_00 = 0) is not written and the collision reads f^n, and the
-// last stage's G, which no stage reads, is not zeroed.
+// in_step: called by step_sequence on library scratch: what no later stage
+// reads is neither computed nor written, nor are stage 0's F (= f^n exactly
+// when A_00 = 0; *F_src receives where F_l is) and the zero G of the BGK model.
 int run_stage(const bz_modes *m, const Tableau &t, int l, int model, double dt, double eps, const void *f_n,
               void *F_l, void *G, void *P, const void *L_res, int64_t n, int precision, int flags,
-              cudaStream_t st, void *ext = nullptr, bool in_step = false) {
+              cudaStream_t st, void *ext = nullptr, bool in_step = false, const void **F_src = nullptr) {
     const GridView &v = m->g->v;
     StageCoef c;
     memset(&c, 0, sizeof c);
@@ -462,30 +446,31 @@ int run_stage(const bz_modes *m, const Tableau &t, int l, int model, double dt, 
     c.eps = eps;
     c.nuf = (model == BZ_BOLTZMANN) ? m->penalty : 1.0;
     const bool f0 = in_step && l == 0 && c.all == 0.0;     // F_0 = f^n
+    const bool needG = model == BZ_BOLTZMANN && explicit_used(t, l);
     c.store_F = f0 ? 0 : 1;
+    // FP32 stages read zero-weighted terms too (k_imex.cu)
+    c.store_P = !in_step || needG || (precision == BZ_FP64 ? implicit_used(t, l) : l + 1 < t.s);
+    c.use_G = !in_step || model == BZ_BOLTZMANN;
+    if (F_src) *F_src = f0 ? f_n : F_l;
     const int64_t stride = n * v.nv;
     const size_t es = (precision == BZ_FP64) ? sizeof(double) : sizeof(float);
-    cudaError_t e;
-    {
-    ProfScope ps(precision == BZ_FP64 ? "imex_stage_f64" : "imex_stage_f32", st);
-    if (precision == BZ_FP64)
-        e = launch_imex_stage_f64(v, c, static_cast<const double *>(f_n), static_cast<double *>(F_l),
-                                  static_cast<const double *>(G), static_cast<double *>(P),
-                                  static_cast<const double *>(L_res), stride, n, st);
-    else
-        e = launch_imex_stage_f32(v, c, static_cast<const float *>(f_n), static_cast<float *>(F_l),
-                                  static_cast<const float *>(G), static_cast<float *>(P),
-                                  static_cast<const float *>(L_res), stride, n, st);
+    cudaError_t e = cudaSuccess;
+    if (c.store_F || c.store_P) {
+        ProfScope ps(precision == BZ_FP64 ? "imex_stage_f64" : "imex_stage_f32", st);
+        if (precision == BZ_FP64)
+            e = launch_imex_stage_f64(v, c, static_cast<const double *>(f_n), static_cast<double *>(F_l),
+                                      static_cast<const double *>(G), static_cast<double *>(P),
+                                      static_cast<const double *>(L_res), stride, n, st);
+        else
+            e = launch_imex_stage_f32(v, c, static_cast<const float *>(f_n), static_cast<float *>(F_l),
+                                      static_cast<const float *>(G), static_cast<float *>(P),
+                                      static_cast<const float *>(L_res), stride, n, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "imex stage");
-    bool needG = false;
-    for (int q = l + 1; q < t.s; ++q)
-        if (t.At[q][l] != 0.0) needG = true;
     char *Gl = static_cast<char *>(G) + (size_t)l * stride * es;
     const char *Pl = static_cast<const char *>(P) + (size_t)l * stride * es;
-    if (model == BZ_BOLTZMANN && needG)
-        return collide_chain(m, precision, flags, f0 ? f_n : F_l, Gl, Pl, n, st, ext);
-    if (in_step && l == t.s - 1) return BZ_OK;
+    if (needG) return collide_chain(m, precision, flags, f0 ? f_n : F_l, Gl, Pl, n, st, ext);
+    if (in_step && (model == BZ_BGK || l + 1 == t.s || precision == BZ_FP64)) return BZ_OK;
     e = launch_fill_zero(Gl, (int64_t)(stride * es), st);
     if (e != cudaSuccess) return cuda_fail(e, "imex stage: zero G");
     return BZ_OK;
@@ -557,7 +542,7 @@ int step_sequence(const bz_modes *m, const Tableau &t, int model, double dt, dou
 // residual L_l = <L(F_l^w)>_x of the stage value enters the explicit part of
 // every later stage (eq. GIMEX_n; the correction Delta Q vanishes for a
 // reconstruction that keeps the cell averages).  Scratch: step scratch, then
-// [stages][cell][nv] residuals, then the reconstruction's gradients.
+// [stages][cell][nv] residuals, then the face fluxes.
 int step_sequence_fv(const bz_modes *m, const bz_mesh *mesh, const Tableau &t, int model, double dt, double eps,
                      const void *f_n, void *f_out, int64_t n, int precision, int flags, cudaStream_t st,
                      void *scratch, size_t step_bytes) {
@@ -571,10 +556,11 @@ int step_sequence_fv(const bz_modes *m, const bz_mesh *mesh, const Tableau &t, i
     char *tsc = Lbuf + (size_t)t.s * stride * es;
     for (int l = 0; l < t.s; ++l) {
         void *F_l = (l == t.s - 1) ? f_out : static_cast<void *>(Fbuf);
-        int rc = run_stage(m, t, l, model, dt, eps, f_n, F_l, G, P, Lbuf, n, precision, flags, st, coll);
+        const void *F_src = nullptr;
+        int rc = run_stage(m, t, l, model, dt, eps, f_n, F_l, G, P, Lbuf, n, precision, flags, st, coll, true, &F_src);
         if (rc) return rc;
-        if (l < t.s - 1) {
-            rc = transport_chain(mesh, m->g, precision, F_l, Lbuf + (size_t)l * stride * es, st, tsc);
+        if (precision == BZ_FP64 ? explicit_used(t, l) : l + 1 < t.s) {
+            rc = transport_chain(mesh, m->g, precision, F_src, Lbuf + (size_t)l * stride * es, st, tsc);
             if (rc) return rc;
         }
     }

@@ -114,24 +114,27 @@ constexpr int kFvCentral3 = 11;     // degree 2: the cell and its 11 nearest cel
 constexpr int kFvCoef3 = 5;         // degree 2: coefficients of xi, eta, xi^2, xi eta, eta^2
 constexpr int kFvRegularTri = 0x100;  // flag in ncen: a triangle whose stencil starts with its 3 face neighbours
 
+// Tables of the transport step, one row per position p of the processing order
+// (cell order[p]).  Order 2 reconstructs a gradient (B = 2 coefficients from
+// K = kFvCentral stencil cells), order 3 the 5 coefficients of the zero-mean
+// scaled Taylor basis phi = (xi, eta, xi^2 - mu20, xi eta - mu11, eta^2 -
+// mu02), xi = (x - x_b)/h, from K = kFvCentral3 cells.  The FP64 tables have
+// factors folded in that save FP64 operations: order 2 is scaled to xi, eta
+// too, and Rc is divided by lambda_0 where the cell has sectors.
 template <typename T> struct FvTables {
-    const T *inv_area;      // [cell]
-    const T *h2;            // [cell] h_i^2
-    const T *fn;            // [cell][face][2]  |e| n_e
-    const T *off_i;         // [cell][face][2]  x_face - x_b,i
-    const T *off_j;         // [cell][face][2]  x_face - x_b,j (neighbour side)
-    const T *Rc;            // [cell][2][kFvCentral] least-squares gradient rows
-    const T *Rs;            // [cell][face][4]  sector inverses (row-major 2 x 2); degree 2: in the
-                            //                   scaled coordinates (x - x_b) / h
+    const T *Rs;            // [p][face][4]  sector inverses (row-major 2 x 2)
+    const T *quad;          // [p][4]  FP32: (mu20, mu11, mu02, h^2); FP64: the degree-2 smoothness form's
+                            //         coefficients (4 mu20 + 4, mu20 + mu02 + 1, 4 mu02 + 4, 4 mu11)
+    const T *fn;            // [p][face][2]  |e| n_e outward (exactly opposite on the two sides of a face)
+    const T *phi;           // [p][face][B]  means of the basis over the face
+    const T *phig;          // [p][face][2][B]  order 3: the basis at the face's two Gauss points
+    const T *Rc;            // [p][B][K]  least-squares rows
+    const T *inv_area;      // [p]
 };
-// Degree-2 reconstruction (order 3): zero-mean scaled Taylor basis
-// phi = (xi, eta, xi^2 - mu20, xi eta - mu11, eta^2 - mu02), xi = (x - x_b)/h.
-template <typename T> struct FvTables3 {
-    const T *mu;            // [cell][3]  cell means of xi^2, xi eta, eta^2
-    const T *Rc;            // [cell][5][kFvCentral3] least-squares coefficient rows
-    const T *phi_i;         // [cell][face][2 Gauss points][5] basis of the cell at the face's Gauss points
-    const T *phi_j;         // [cell][face][2][5] the neighbour's basis at the same points
-};
+// A thin cell (perimeter times largest radius over area above this; 4 for an
+// equilateral triangle) cancels its face fluxes to L by that much.
+constexpr double kFvThin = 50.0;
+constexpr int kFvThinFlag = 0x10;     // in meta: a thin cell
 }  // namespace bz
 
 struct bz_mesh {
@@ -139,40 +142,41 @@ struct bz_mesh {
     int order;              // 1: piecewise constant, 2: CWENO of degree 1, 3: CWENO of degree 2
     int64_t n_cells, n_faces_interior, n_faces_boundary;
     int max_faces;
-    int *d_nface;           // [cell] faces
-    int *d_nb;              // [cell][face] neighbour, -1 boundary
-    // triangle meshes (max_faces <= 3): per position p of the processing order
-    // three int4 {i, ncen[i], nsec[i], qbits}, {cen[i][0..3]}, {cen[i][4], nb[i][0..2]}
-    // with i = order[p] and qbits holding, in 2 bits per face, the index of
-    // the same face in the neighbour; one level of loads gives a block all its
-    // indices
+    // index tables by position of the processing order (cells sorted along a
+    // Morton curve of their barycentres), values are cell indices
+    int *d_order;           // [p] cell
+    int *d_meta;            // [p] faces | kFvThinFlag | not-owner bits << 8 | boundary bits << 16 | two-sided
+                            // bits << 24 (bit q: face q); the owner of a face is its first cell in the
+                            // processing order; a two-sided face bounds a thin cell
+    int *d_nb;              // [p][face] neighbour, -1 boundary
+    int *d_fid;             // [p][face] face index, numbered in the processing order of the owners
+    int *d_two;             // [p][face] index of a two-sided face
+    int64_t n_two;
+    int *d_ncen;            // [p] central stencil size (<= K), | kFvRegularTri for a triangle whose stencil
+                            // starts with its face neighbours, sector s on faces s, s+1
+    int *d_cen;             // [p][K]
+    int *d_nsec;            // [p] sectors
+    int *d_sec;             // [p][face][2] sector cells
+    // triangle meshes of order 2: per position p three int4 {i, ncen, 0, qbits}, {cen[0..3]},
+    // {cen[4], nb[0..2]} with i = order[p] and qbits holding, in 2 bits per face, the index of the
+    // same face in the neighbour; one level of loads gives a block all its indices
     int4 *d_tripos;
-    int *d_ncen;            // [cell] central stencil size (<= kFvCentral), | kFvRegularTri for a triangle
-                            // whose stencil starts with its face neighbours, sector s on faces s, s+1
-    int *d_cen;             // [cell][kFvCentral]
-    int *d_nsec;            // [cell] sectors
-    int *d_sec;             // [cell][face][2] sector cells
-    int *d_order;           // [cell] processing order: cells sorted along a Morton curve of their barycentres
-    // walls with full accommodation (fv_mesh_set_walls): per face the wall
-    // index (-1: none), per wall (theta_w, u_w1, u_w2) in FP64 and FP32
+    // walls with full accommodation (fv_mesh_set_walls): per position and face
+    // the wall index (-1: none), per wall the face's slot p * kFvMaxFaces + q
+    // and (theta_w, u_w1, u_w2) in FP64 and FP32
     int *d_wall;
+    int64_t *d_wallslot;
     double *d_wall64;
     float *d_wall32;
     int64_t n_walls;
-    // host copies for the wall look-up: counter-clockwise vertex lists (CSR)
-    // and the neighbour of every face
+    // host copies for the wall look-up: counter-clockwise vertex lists (CSR),
+    // the neighbour of every face and the position of every cell
     int64_t *h_ptr, *h_vtx;
-    int *h_nb;
+    int *h_nb, *h_pos;
     void *d_real64;         // one block holding the FvTables<double> arrays
     void *d_real32;         // one block holding the FvTables<float> arrays
     bz::FvTables<double> t64;
     bz::FvTables<float> t32;
-    // order 3 only
-    int *d_ncen3;           // [cell] central stencil size (<= kFvCentral3)
-    int *d_cen3;            // [cell][kFvCentral3]
-    void *d_real3_64, *d_real3_32;
-    bz::FvTables3<double> u64;
-    bz::FvTables3<float> u32;
 };
 
 namespace bz {
@@ -283,6 +287,8 @@ struct StageCoef {
     double dt, eps;
     double nuf;                // penalty rate nu = nuf * rho
     int store_F;               // 0: F_l equals f^n exactly (stage 0 of a step) and is not written
+    int store_P;               // 0: no later stage reads P_l
+    int use_G;                 // 0: every G is zero (a whole step of the BGK model) and none is read
 };
 cudaError_t launch_imex_stage_f64(const GridView &g, const StageCoef &c, const double *fn,
                                   double *F, const double *G, double *P, const double *Lres,
@@ -295,35 +301,26 @@ cudaError_t launch_check_input_f32(const float *f, int64_t count, int *err, cuda
 cudaError_t launch_fill_zero(void *p, int64_t bytes, cudaStream_t st);
 
 // ---- transport residual (k_transport.cu) ----------------------------------
-// G [cell][2][nv] CWENO gradients (order 2 only), then
-// L [cell][nv] = (1/|P_i|) sum_e |e| F_Rusanov(f_L, f_R; v . n_e).
-cudaError_t launch_fv_gradient_f64(const bz_mesh *mesh, const GridView &g, const double *f, double *G,
-                                   cudaStream_t st);
-cudaError_t launch_fv_gradient_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *G,
-                                   cudaStream_t st);
-cudaError_t launch_fv_flux_f64(const bz_mesh *mesh, const GridView &g, const double *f, const double *G, double *L,
-                               cudaStream_t st);
+// Order 1: L from f in one pass.  Orders 2 and 3: the reconstruction pass
+// writes the upwind flux of every face, FX [face][nv], each velocity by the
+// cell it leaves; then L [cell][nv] = the signed sum of a cell's face rows
+// over |P_i|.  FP32, order 2 on triangles without walls (N divisible by 4,
+// 16-byte aligned rows: fv_value_mode): the reconstruction writes each cell's
+// values at its three faces, FV [cell][3][nv], and the flux pass reads those
+// of the cell and its neighbours.  Scratch: fv_scratch_rows() rows of nv.
+bool fv_value_mode(const bz_mesh *mesh, const GridView &g, const void *f, const void *L);
+int64_t fv_scratch_rows(const bz_mesh *mesh, bool f32);
+cudaError_t launch_fv_values_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FV, cudaStream_t st);
+cudaError_t launch_fv_flux_values_f32(const bz_mesh *mesh, const GridView &g, const float *FV, float *L,
+                                      cudaStream_t st);
 // walls need one CTA to hold all velocities of a cell
 bool fv_walls_supported(const bz_mesh *mesh, const GridView &g);
-// FP32 triangle meshes without walls (N divisible by 4, 16-byte aligned rows):
-// the reconstruction writes each cell's values at its three face midpoints,
-// FV [cell][3][nv], and the flux pass reads those of the cell and of its
-// neighbours (indices from the position records d_tripos).
-bool fv_face_mode(const bz_mesh *mesh, const GridView &g, const void *f, const void *L, const void *FV);
-cudaError_t launch_fv_faces_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FV, cudaStream_t st);
-cudaError_t launch_fv_flux_faces_f32(const bz_mesh *mesh, const GridView &g, const float *FV, float *L,
-                                     cudaStream_t st);
-// order 3: coefficients C [cell][5][nv] of the degree-2 CWENO polynomial, then
-// the fluxes at two Gauss points per face
-cudaError_t launch_fv_coef3_f64(const bz_mesh *mesh, const GridView &g, const double *f, double *C,
-                                cudaStream_t st);
-cudaError_t launch_fv_coef3_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *C, cudaStream_t st);
-cudaError_t launch_fv_flux3_f64(const bz_mesh *mesh, const GridView &g, const double *f, const double *C,
-                                double *L, cudaStream_t st);
-cudaError_t launch_fv_flux3_f32(const bz_mesh *mesh, const GridView &g, const float *f, const float *C, float *L,
-                                cudaStream_t st);
-cudaError_t launch_fv_flux_f32(const bz_mesh *mesh, const GridView &g, const float *f, const float *G, float *L,
-                               cudaStream_t st);
+cudaError_t launch_fv_first_f64(const bz_mesh *mesh, const GridView &g, const double *f, double *L, cudaStream_t st);
+cudaError_t launch_fv_first_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *L, cudaStream_t st);
+cudaError_t launch_fv_faces_f64(const bz_mesh *mesh, const GridView &g, const double *f, double *FX, cudaStream_t st);
+cudaError_t launch_fv_faces_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FX, cudaStream_t st);
+cudaError_t launch_fv_sum_f64(const bz_mesh *mesh, const GridView &g, const double *FX, double *L, cudaStream_t st);
+cudaError_t launch_fv_sum_f32(const bz_mesh *mesh, const GridView &g, const float *FX, float *L, cudaStream_t st);
 
 // Device error word of the current device (allocated on first use; api.cu).
 int *device_error_word();

@@ -43,25 +43,10 @@ namespace {
 
 struct HostMesh {
     int64_t n = 0;
+    int B = 0, K = 0;                  // coefficients and stencil cells of the order (0: order 1)
     std::vector<int> nface, nb, nbq, ncen, cen, nsec, sec, order;
-    std::vector<double> inv_area, h2, fn, off_i, off_j, Rc, Rs;
-    // order 3
-    std::vector<int> ncen3, cen3;
-    std::vector<double> mu, Rc3, phi_i, phi_j;
+    std::vector<double> inv_area, h2, fn, Rc, Rs, phi, phig, mu;
 };
-
-constexpr int64_t kReal3PerCell = 3 + kFvCoef3 * kFvCentral3 + 2 * kFvMaxFaces * 2 * kFvCoef3;
-
-template <typename T>
-FvTables3<T> carve3(void *base, int64_t n) {
-    T *p = static_cast<T *>(base);
-    FvTables3<T> t;
-    t.mu = p; p += n * 3;
-    t.Rc = p; p += n * kFvCoef3 * kFvCentral3;
-    t.phi_i = p; p += n * kFvMaxFaces * 2 * kFvCoef3;
-    t.phi_j = p;
-    return t;
-}
 
 // Means over a polygon (vertices px, py in order, translated by (sx, sy)) of
 // xi, eta, xi^2, xi eta, eta^2 with xi = (x - x0)/hh, eta = (y - y0)/hh: the
@@ -121,35 +106,60 @@ bool solve5(double M[5][5], double *B, int nc, double tol) {
 }
 
 template <typename T>
-FvTables<T> carve(void *base, int64_t n) {
+FvTables<T> carve(void *base, const HostMesh &h) {
+    const int64_t n = h.n;
     T *p = static_cast<T *>(base);
     FvTables<T> t;
-    t.inv_area = p; p += n;
-    t.h2 = p; p += n;
+    t.Rs = p; p += n * (h.B ? kFvMaxFaces * 4 : 0);
+    t.quad = p; p += n * (h.B ? 4 : 0);
     t.fn = p; p += n * kFvMaxFaces * 2;
-    t.off_i = p; p += n * kFvMaxFaces * 2;
-    t.off_j = p; p += n * kFvMaxFaces * 2;
-    t.Rc = p; p += n * 2 * kFvCentral;
-    t.Rs = p;
+    t.phi = p; p += n * kFvMaxFaces * h.B;
+    t.phig = p; p += n * kFvMaxFaces * (h.B == kFvCoef3 ? 2 * h.B : 0);
+    t.Rc = p; p += n * h.B * h.K;
+    t.inv_area = p;
     return t;
 }
-constexpr int64_t kRealPerCell = 1 + 1 + 3 * kFvMaxFaces * 2 + 2 * kFvCentral + kFvMaxFaces * 4;
 
-void fill_real(const HostMesh &h, std::vector<double> &out) {
-    const int64_t n = h.n;
-    out.assign((size_t)(n * kRealPerCell), 0.0);
-    double *p = out.data();
-    auto put = [&p](const std::vector<double> &v) {
-        memcpy(p, v.data(), sizeof(double) * v.size());
-        p += v.size();
+// Rows of `width` entries, one per cell, in processing order.
+template <typename X>
+std::vector<X> by_position(const std::vector<X> &v, const std::vector<int> &order, int width) {
+    std::vector<X> out(v.size());
+    if (width)
+        for (size_t p = 0; p < order.size(); ++p)
+            std::copy_n(v.begin() + (size_t)order[p] * width, width, out.begin() + p * width);
+    return out;
+}
+
+// The real tables in carve()'s order; folded: with the FP64 tables' factors.
+std::vector<double> fill_real(const HostMesh &h, bool folded) {
+    std::vector<double> out;
+    auto put = [&](const std::vector<double> &v, int width, auto factor) {
+        std::vector<double> q = by_position(v, h.order, width);
+        if (folded)
+            for (size_t e = 0; e < q.size(); ++e) q[e] *= factor(h.order[e / width]);
+        out.insert(out.end(), q.begin(), q.end());
     };
-    put(h.inv_area);
-    put(h.h2);
-    put(h.fn);
-    put(h.off_i);
-    put(h.off_j);
-    put(h.Rc);
-    put(h.Rs);
+    const bool scale = h.B == 2;                 // order 3's tables are in units of h already
+    auto one = [](int) { return 1.0; };
+    auto hc = [&](int i) { return scale ? sqrt(h.h2[i]) : 1.0; };
+    auto ih = [&](int i) { return scale ? 1.0 / sqrt(h.h2[i]) : 1.0; };
+    put(h.Rs, h.B ? kFvMaxFaces * 4 : 0, hc);
+    if (h.B) {
+        std::vector<double> quad((size_t)h.n * 4, 0.0);
+        for (int64_t i = 0; i < h.n; ++i) {
+            const double m20 = h.mu[3 * i], m11 = h.mu[3 * i + 1], m02 = h.mu[3 * i + 2];
+            const double f[4] = {4.0 * m20 + 4.0, m20 + m02 + 1.0, 4.0 * m02 + 4.0, 4.0 * m11};
+            const double r[4] = {m20, m11, m02, h.h2[i]};
+            std::copy_n(folded ? f : r, 4, &quad[4 * i]);
+        }
+        put(quad, 4, one);
+    }
+    put(h.fn, kFvMaxFaces * 2, one);
+    put(h.phi, kFvMaxFaces * h.B, ih);
+    put(h.phig, h.B == kFvCoef3 ? kFvMaxFaces * 2 * h.B : 0, one);
+    put(h.Rc, h.B * h.K, [&](int i) { return hc(i) * (h.nsec[i] > 0 ? 4.0 / 3.0 : 1.0); });
+    put(h.inv_area, 1, one);
+    return out;
 }
 
 template <typename X> cudaError_t upload(X **d, const std::vector<X> &v) {
@@ -162,8 +172,10 @@ template <typename X> cudaError_t upload(X **d, const std::vector<X> &v) {
 
 void fv_mesh_destroy(bz_mesh *m) {
     if (!m) return;
-    dev_free(m->d_nface);
+    dev_free(m->d_meta);
     dev_free(m->d_nb);
+    dev_free(m->d_fid);
+    dev_free(m->d_two);
     dev_free(m->d_tripos);
     dev_free(m->d_ncen);
     dev_free(m->d_cen);
@@ -171,17 +183,15 @@ void fv_mesh_destroy(bz_mesh *m) {
     dev_free(m->d_sec);
     dev_free(m->d_order);
     dev_free(m->d_wall);
+    dev_free(m->d_wallslot);
     dev_free(m->d_wall64);
     dev_free(m->d_wall32);
     free(m->h_ptr);
     free(m->h_vtx);
     free(m->h_nb);
+    free(m->h_pos);
     dev_free(m->d_real64);
     dev_free(m->d_real32);
-    dev_free(m->d_ncen3);
-    dev_free(m->d_cen3);
-    dev_free(m->d_real3_64);
-    dev_free(m->d_real3_32);
     free(m);
 }
 
@@ -282,8 +292,6 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
     h.nb.assign(n * kFvMaxFaces, -1);
     h.nbq.assign(n * kFvMaxFaces, -1);
     h.fn.assign(n * kFvMaxFaces * 2, 0.0);
-    h.off_i.assign(n * kFvMaxFaces * 2, 0.0);
-    h.off_j.assign(n * kFvMaxFaces * 2, 0.0);
     std::vector<double> fsx(n * kFvMaxFaces, 0.0), fsy(n * kFvMaxFaces, 0.0);   // neighbour shifts
     int64_t interior = 0, boundary = 0;
     int maxf = 0;
@@ -295,12 +303,9 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         for (int q = 0; q < k; ++q) {
             const int64_t a = c[q], b = c[(q + 1) % k];
             const double dx = xy[2 * b] - xy[2 * a], dy = xy[2 * b + 1] - xy[2 * a + 1];
-            const double mx = 0.5 * (xy[2 * a] + xy[2 * b]), my = 0.5 * (xy[2 * a + 1] + xy[2 * b + 1]);
             const size_t s = (size_t)i * kFvMaxFaces + q;
             h.fn[2 * s] = dy;                 // |e| n_e = (dy, -dx)
             h.fn[2 * s + 1] = -dx;
-            h.off_i[2 * s] = mx - bx[i];
-            h.off_i[2 * s + 1] = my - by[i];
             auto it = owner.find(key(vclass[b], vclass[a]));
             if (it != owner.end()) {
                 const int64_t j = it->second.first, wb = it->second.second;   // j's copy of b
@@ -311,37 +316,34 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                 h.nb[s] = (int)j;
                 for (size_t t = 0; t < cells[j].size(); ++t)     // j's face starting at its copy of b
                     if (cells[j][t] == wb) h.nbq[s] = (int)t;
-                h.off_j[2 * s] = mx - fsx[s] - bx[j];
-                h.off_j[2 * s + 1] = my - fsy[s] - by[j];
                 ++interior;
             } else {
                 ++boundary;
             }
         }
     }
-    h.ncen.assign(n, 0);
-    h.cen.assign(n * kFvCentral, 0);
-    h.Rc.assign(n * 2 * kFvCentral, 0.0);
-    h.nsec.assign(n, 0);
-    h.sec.assign(n * kFvMaxFaces * 2, 0);
-    h.Rs.assign(n * kFvMaxFaces * 4, 0.0);
+    if (order >= 2) {
+        h.B = order == 3 ? kFvCoef3 : 2;
+        h.K = order == 3 ? kFvCentral3 : kFvCentral;
+    }
+    const int K = h.K, B = h.B;
+    h.ncen.assign(B ? n : 0, 0);
+    h.cen.assign(n * K, 0);
+    h.Rc.assign(n * B * K, 0.0);
+    h.nsec.assign(B ? n : 0, 0);
+    h.sec.assign(B ? n * kFvMaxFaces * 2 : 0, 0);
+    h.Rs.assign(B ? n * kFvMaxFaces * 4 : 0, 0.0);
+    h.phi.assign(n * kFvMaxFaces * B, 0.0);
+    h.phig.assign(order == 3 ? n * kFvMaxFaces * 2 * B : 0, 0.0);
+    h.mu.assign(B ? n * 3 : 0, 0.0);                    // order 3: cell means of xi^2, xi eta, eta^2
     if (order == 3) {
-        h.ncen3.assign(n, 0);
-        h.cen3.assign(n * kFvCentral3, 0);
-        h.mu.assign(n * 3, 0.0);
-        h.Rc3.assign(n * kFvCoef3 * kFvCentral3, 0.0);
-        h.phi_i.assign(n * kFvMaxFaces * 2 * kFvCoef3, 0.0);
-        h.phi_j.assign(n * kFvMaxFaces * 2 * kFvCoef3, 0.0);
         for (int64_t i = 0; i < n; ++i) {
             double q[5];
             quad_means(cells[i], xy, 0.0, 0.0, bx[i], by[i], sqrt(h.h2[i]), q);
-            h.mu[3 * i] = q[2];
-            h.mu[3 * i + 1] = q[3];
-            h.mu[3 * i + 2] = q[4];
+            for (int l = 0; l < 3; ++l) h.mu[3 * i + l] = q[2 + l];
         }
     }
     if (order >= 2) {
-        const int ncen_max = order == 3 ? kFvCentral3 : kFvCentral;
         // vertex class -> (cell, vertex)
         std::vector<int64_t> vptr(n_vertices + 1, 0);
         std::vector<std::pair<int64_t, int64_t>> vcell;
@@ -402,47 +404,49 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                 double A[kFvCentral3][5];
                 for (int q = 0; q < nc; ++q) {
                     const Img &c = dist[q].m;
-                    h.cen3[i * kFvCentral3 + q] = (int)c.j;
+                    h.cen[i * K + q] = (int)c.j;
                     quad_means(cells[c.j], xy, c.kx * Lx, c.ky * Ly, bx[i], by[i], hi, A[q]);
                     A[q][2] -= h.mu[3 * i];
                     A[q][3] -= h.mu[3 * i + 1];
                     A[q][4] -= h.mu[3 * i + 2];
                 }
-                h.ncen3[i] = nc;
-                double M[5][5], B[5 * kFvCentral3];
+                h.ncen[i] = nc;
+                double M[5][5], S[5 * kFvCentral3];
                 for (int r = 0; r < 5; ++r) {
                     for (int col = 0; col < 5; ++col) {
                         double sum = 0.0;
                         for (int q = 0; q < nc; ++q) sum += A[q][r] * A[q][col];
                         M[r][col] = sum;
                     }
-                    for (int q = 0; q < nc; ++q) B[r * nc + q] = A[q][r];
+                    for (int q = 0; q < nc; ++q) S[r * nc + q] = A[q][r];
                 }
-                if (nc < 5 || !solve5(M, B, nc, 1e-12))
+                if (nc < 5 || !solve5(M, S, nc, 1e-12))
                     return fail(BZ_EINVAL, "build_fv_mesh: order 3 needs a cell neighbourhood that determines a "
                                            "quadratic (mesh too small or degenerate)");
                 for (int r = 0; r < 5; ++r)
-                    for (int q = 0; q < nc; ++q) h.Rc3[((size_t)i * kFvCoef3 + r) * kFvCentral3 + q] = B[r * nc + q];
+                    for (int q = 0; q < nc; ++q) h.Rc[((size_t)i * kFvCoef3 + r) * K + q] = S[r * nc + q];
             }
-            const int nc = (int)std::min<size_t>(kFvCentral, dist.size());
-            double ata[3] = {0, 0, 0};
-            double axs[kFvCentral], ays[kFvCentral];
-            for (int q = 0; q < nc; ++q) {
-                const Img &c = dist[q].m;
-                h.cen[i * kFvCentral + q] = (int)c.j;
-                axs[q] = bx[c.j] + c.kx * Lx - bx[i];
-                ays[q] = by[c.j] + c.ky * Ly - by[i];
-                ata[0] += axs[q] * axs[q];
-                ata[1] += axs[q] * ays[q];
-                ata[2] += ays[q] * ays[q];
-            }
-            h.ncen[i] = nc;
-            const double det = ata[0] * ata[2] - ata[1] * ata[1];
-            if (nc >= 2 && det > 1e-300) {
-                const double i00 = ata[2] / det, i01 = -ata[1] / det, i11 = ata[0] / det;
+            if (order == 2) {
+                const int nc = (int)std::min<size_t>(kFvCentral, dist.size());
+                double ata[3] = {0, 0, 0};
+                double axs[kFvCentral], ays[kFvCentral];
                 for (int q = 0; q < nc; ++q) {
-                    h.Rc[(i * 2 + 0) * kFvCentral + q] = i00 * axs[q] + i01 * ays[q];
-                    h.Rc[(i * 2 + 1) * kFvCentral + q] = i01 * axs[q] + i11 * ays[q];
+                    const Img &c = dist[q].m;
+                    h.cen[i * K + q] = (int)c.j;
+                    axs[q] = bx[c.j] + c.kx * Lx - bx[i];
+                    ays[q] = by[c.j] + c.ky * Ly - by[i];
+                    ata[0] += axs[q] * axs[q];
+                    ata[1] += axs[q] * ays[q];
+                    ata[2] += ays[q] * ays[q];
+                }
+                h.ncen[i] = nc;
+                const double det = ata[0] * ata[2] - ata[1] * ata[1];
+                if (nc >= 2 && det > 1e-300) {
+                    const double i00 = ata[2] / det, i01 = -ata[1] / det, i11 = ata[0] / det;
+                    for (int q = 0; q < nc; ++q) {
+                        h.Rc[(i * 2 + 0) * K + q] = i00 * axs[q] + i01 * ays[q];
+                        h.Rc[(i * 2 + 1) * K + q] = i01 * axs[q] + i11 * ays[q];
+                    }
                 }
             }
             // sectors: consecutive faces with neighbours on both
@@ -471,77 +475,67 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
             }
             h.nsec[i] = ns;
             // A triangle with three sectors whose face neighbours all lie in
-            // its central stencil (nearly every interior cell of a triangle
-            // mesh): the stencil is reordered to start with the face
+            // its full central stencil (nearly every interior cell of a
+            // triangle mesh): the stencil is reordered to start with the face
             // neighbours in face order and the cell is flagged, so that the
             // FP32 reconstruction loads every neighbour row once for the
             // central and the sector gradients (sector s joins faces s and
-            // s + 1 mod 3).  The same for the degree-2 stencil.
-            auto face_first = [&](int *cn, double *R, int nrow, int width, int ncs, int &flagged) {
-                if (k != 3 || ns != 3) return;
+            // s + 1 mod 3).
+            auto face_first = [&](int *cn, double *R) {
+                if (k != 3 || ns != 3 || h.ncen[i] != K) return;
                 int perm[kFvCentral3];
                 bool used[kFvCentral3] = {};
                 for (int q = 0; q < 3; ++q) {
                     const int j = h.nb[(size_t)i * kFvMaxFaces + q];
                     int hit = -1;
-                    for (int t = 0; t < ncs && hit < 0; ++t)
+                    for (int t = 0; t < K && hit < 0; ++t)
                         if (!used[t] && cn[t] == j) hit = t;
                     if (hit < 0) return;
                     used[hit] = true;
                     perm[q] = hit;
                 }
-                for (int t = 0, p = 3; t < ncs; ++t)
+                for (int t = 0, p = 3; t < K; ++t)
                     if (!used[t]) perm[p++] = t;
                 int c0[kFvCentral3];
-                std::vector<double> r0((size_t)nrow * ncs);
-                for (int t = 0; t < ncs; ++t) {
-                    c0[t] = cn[t];
-                    for (int r = 0; r < nrow; ++r) r0[(size_t)r * ncs + t] = R[(size_t)r * width + t];
-                }
-                for (int t = 0; t < ncs; ++t) {
+                double r0[kFvCoef3 * kFvCentral3];
+                std::copy_n(cn, K, c0);
+                std::copy_n(R, B * K, r0);
+                for (int t = 0; t < K; ++t) {
                     cn[t] = c0[perm[t]];
-                    for (int r = 0; r < nrow; ++r) R[(size_t)r * width + t] = r0[(size_t)r * ncs + perm[t]];
+                    for (int r = 0; r < B; ++r) R[r * K + t] = r0[r * K + perm[t]];
                 }
-                flagged |= kFvRegularTri;
+                h.ncen[i] |= kFvRegularTri;
             };
-            if (nc == kFvCentral) {
-                int fl = 0;
-                face_first(&h.cen[i * kFvCentral], &h.Rc[i * 2 * kFvCentral], 2, kFvCentral, nc, fl);
-                h.ncen[i] = nc | fl;
-            }
-            if (order == 3 && h.ncen3[i] == kFvCentral3) {
-                int fl = 0;
-                face_first(&h.cen3[i * kFvCentral3], &h.Rc3[(size_t)i * kFvCoef3 * kFvCentral3], kFvCoef3,
-                           kFvCentral3, kFvCentral3, fl);
-                h.ncen3[i] = kFvCentral3 | fl;
-            }
+            face_first(&h.cen[i * K], &h.Rc[(size_t)i * B * K]);
         }
-    }
-    if (order == 3) {
-        // the basis of the cell and of its neighbour at the face's two
-        // Gauss-Legendre points x_a + t (x_b - x_a), t = 1/2 -+ 1/(2 sqrt 3)
+        // means of the basis over every face: the midpoint for degree 1, the
+        // two Gauss-Legendre points x_a + t (x_b - x_a), t = 1/2 -+ 1/(2 sqrt 3),
+        // for degree 2 (the normal velocity is constant along a face, so the
+        // flux needs the mean of the reconstruction only)
         const double tg[2] = {0.5 - 0.5 / sqrt(3.0), 0.5 + 0.5 / sqrt(3.0)};
-        auto basis = [&](int64_t c, double x, double y, double *out) {
-            const double hc = sqrt(h.h2[c]);
-            const double xi = (x - bx[c]) / hc, eta = (y - by[c]) / hc;
-            out[0] = xi;
-            out[1] = eta;
-            out[2] = xi * xi - h.mu[3 * c];
-            out[3] = xi * eta - h.mu[3 * c + 1];
-            out[4] = eta * eta - h.mu[3 * c + 2];
-        };
         for (int64_t i = 0; i < n; ++i) {
             const auto &c = cells[i];
             const int k = (int)c.size();
+            const double hc = sqrt(h.h2[i]);
             for (int q = 0; q < k; ++q) {
                 const int64_t a = c[q], b = c[(q + 1) % k];
                 const size_t sidx = (size_t)i * kFvMaxFaces + q;
+                double *out = &h.phi[sidx * B];
+                if (order == 2) {
+                    out[0] = 0.5 * (xy[2 * a] + xy[2 * b]) - bx[i];
+                    out[1] = 0.5 * (xy[2 * a + 1] + xy[2 * b + 1]) - by[i];
+                    continue;
+                }
                 for (int g = 0; g < 2; ++g) {
-                    const double x = xy[2 * a] + tg[g] * (xy[2 * b] - xy[2 * a]);
-                    const double y = xy[2 * a + 1] + tg[g] * (xy[2 * b + 1] - xy[2 * a + 1]);
-                    basis(i, x, y, &h.phi_i[(sidx * 2 + g) * kFvCoef3]);
-                    const int j = h.nb[sidx];
-                    if (j >= 0) basis(j, x - fsx[sidx], y - fsy[sidx], &h.phi_j[(sidx * 2 + g) * kFvCoef3]);
+                    const double xi = (xy[2 * a] + tg[g] * (xy[2 * b] - xy[2 * a]) - bx[i]) / hc;
+                    const double eta = (xy[2 * a + 1] + tg[g] * (xy[2 * b + 1] - xy[2 * a + 1]) - by[i]) / hc;
+                    double *pg = &h.phig[(sidx * 2 + g) * B];
+                    pg[0] = xi;
+                    pg[1] = eta;
+                    pg[2] = xi * xi - h.mu[3 * i];
+                    pg[3] = xi * eta - h.mu[3 * i + 1];
+                    pg[4] = eta * eta - h.mu[3 * i + 2];
+                    for (int l = 0; l < B; ++l) out[l] += 0.5 * pg[l];
                 }
             }
         }
@@ -576,6 +570,43 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         h.order.resize(n);
         for (int64_t i = 0; i < n; ++i) h.order[i] = key[i].second;
     }
+    // faces in the processing order of their owners (the first cell of the two
+    // in that order); the other side's normal is the owner's, negated, so both
+    // sides form the same normal velocities up to the sign
+    std::vector<int> meta((size_t)n, 0), fid((size_t)n * kFvMaxFaces, 0), two((size_t)n * kFvMaxFaces, 0);
+    int64_t n_two = 0;
+    {
+        for (int64_t i = 0; i < n; ++i) {
+            double per = 0.0;
+            for (int q = 0; q < h.nface[i]; ++q)
+                per += hypot(h.fn[2 * (i * kFvMaxFaces + q)], h.fn[2 * (i * kFvMaxFaces + q) + 1]);
+            meta[i] = h.nface[i] | (per * sqrt(h.h2[i]) > kFvThin * area[i] ? kFvThinFlag : 0);
+        }
+        std::vector<char> done((size_t)n, 0);
+        int next = 0;
+        for (int64_t p = 0; p < n; ++p) {
+            const int64_t i = h.order[p];
+            for (int q = 0; q < h.nface[i]; ++q) {
+                const size_t s = (size_t)i * kFvMaxFaces + q;
+                const int j = h.nb[s];
+                const bool thin = ((meta[i] | (j < 0 ? 0 : meta[j])) & kFvThinFlag) != 0;
+                if (thin) meta[i] |= (int)(1u << (24 + q));
+                const size_t o = j < 0 ? s : (size_t)j * kFvMaxFaces + h.nbq[s];
+                if (j < 0) meta[i] |= 1 << (16 + q);
+                if (j >= 0 && (done[j] || (j == i && h.nbq[s] < q))) {
+                    meta[i] |= 1 << (8 + q);
+                    fid[s] = fid[o];
+                    two[s] = two[o];
+                    h.fn[2 * s] = -h.fn[2 * o];
+                    h.fn[2 * s + 1] = -h.fn[2 * o + 1];
+                } else {
+                    fid[s] = next++;
+                    if (thin) two[s] = (int)n_two++;
+                }
+            }
+            done[i] = 1;
+        }
+    }
     bz_mesh *m = (bz_mesh *)calloc(1, sizeof(bz_mesh));
     if (!m) return fail(BZ_ENOMEM, "build_fv_mesh: host allocation");
     cudaGetDevice(&m->device);
@@ -584,31 +615,35 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
     m->n_faces_interior = interior / 2;
     m->n_faces_boundary = boundary;
     m->max_faces = maxf;
-    std::vector<double> real;
-    fill_real(h, real);
-    std::vector<float> real32(real.size());
-    for (size_t q = 0; q < real.size(); ++q) real32[q] = (float)real[q];
-    cudaError_t e = upload(&m->d_nface, h.nface);
-    if (e == cudaSuccess) e = upload(&m->d_nb, h.nb);
-    if (e == cudaSuccess) e = upload(&m->d_ncen, h.ncen);
-    if (e == cudaSuccess) e = upload(&m->d_cen, h.cen);
-    if (e == cudaSuccess) e = upload(&m->d_nsec, h.nsec);
-    if (e == cudaSuccess) e = upload(&m->d_sec, h.sec);
-    if (e == cudaSuccess) e = upload(&m->d_order, h.order);
-    if (e == cudaSuccess && maxf <= 3) {
-        std::vector<int4> tp((size_t)n * 3);
-        for (int64_t p = 0; p < n; ++p) {
-            const int i = h.order[p];
-            const int *nb = &h.nb[(size_t)i * kFvMaxFaces], *nq = &h.nbq[(size_t)i * kFvMaxFaces];
-            const int *c = &h.cen[(size_t)i * kFvCentral];
-            int qbits = 0;
-            for (int q = 0; q < 3; ++q)
-                if (nb[q] >= 0) qbits |= (nq[q] & 3) << (2 * q);
-            tp[3 * p] = make_int4(i, h.ncen[i], h.nsec[i], qbits);
-            tp[3 * p + 1] = make_int4(c[0], c[1], c[2], c[3]);
-            tp[3 * p + 2] = make_int4(c[4], nb[0], nb[1], nb[2]);
+    const std::vector<double> real = fill_real(h, true), plain = fill_real(h, false);
+    const std::vector<float> real32(plain.begin(), plain.end());
+    const std::vector<int> meta_p = by_position(meta, h.order, 1), fid_p = by_position(fid, h.order, kFvMaxFaces);
+    cudaError_t e = upload(&m->d_order, h.order);
+    if (e == cudaSuccess) e = upload(&m->d_meta, meta_p);
+    if (e == cudaSuccess) e = upload(&m->d_nb, by_position(h.nb, h.order, kFvMaxFaces));
+    if (e == cudaSuccess) e = upload(&m->d_fid, fid_p);
+    if (e == cudaSuccess) e = upload(&m->d_two, by_position(two, h.order, kFvMaxFaces));
+    m->n_two = n_two;
+    if (order >= 2) {
+        const std::vector<int> ncen_p = by_position(h.ncen, h.order, 1), cen_p = by_position(h.cen, h.order, K);
+        if (e == cudaSuccess) e = upload(&m->d_ncen, ncen_p);
+        if (e == cudaSuccess) e = upload(&m->d_cen, cen_p);
+        if (e == cudaSuccess) e = upload(&m->d_nsec, by_position(h.nsec, h.order, 1));
+        if (e == cudaSuccess) e = upload(&m->d_sec, by_position(h.sec, h.order, kFvMaxFaces * 2));
+        if (e == cudaSuccess && order == 2 && maxf <= 3) {
+            std::vector<int4> tp((size_t)n * 3);
+            for (int64_t p = 0; p < n; ++p) {
+                const int i = h.order[p], *c = &cen_p[p * K];
+                const int *nb = &h.nb[(size_t)i * kFvMaxFaces], *nq = &h.nbq[(size_t)i * kFvMaxFaces];
+                int qbits = 0;
+                for (int q = 0; q < 3; ++q)
+                    if (nb[q] >= 0) qbits |= (nq[q] & 3) << (2 * q);
+                tp[3 * p] = make_int4(i, ncen_p[p], 0, qbits);
+                tp[3 * p + 1] = make_int4(c[0], c[1], c[2], c[3]);
+                tp[3 * p + 2] = make_int4(c[4], nb[0], nb[1], nb[2]);
+            }
+            e = upload(&m->d_tripos, tp);
         }
-        e = upload(&m->d_tripos, tp);
     }
     double *r64 = nullptr;
     float *r32 = nullptr;
@@ -620,37 +655,14 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         fv_mesh_destroy(m);
         return cuda_fail(e, "build_fv_mesh: device tables");
     }
-    m->t64 = carve<double>(m->d_real64, n);
-    m->t32 = carve<float>(m->d_real32, n);
-    if (order == 3) {
-        std::vector<double> r3((size_t)(n * kReal3PerCell));
-        double *p3 = r3.data();
-        for (const std::vector<double> *v : {&h.mu, &h.Rc3, &h.phi_i, &h.phi_j}) {
-            memcpy(p3, v->data(), sizeof(double) * v->size());
-            p3 += v->size();
-        }
-        std::vector<float> r3f(r3.size());
-        for (size_t q = 0; q < r3.size(); ++q) r3f[q] = (float)r3[q];
-        double *d3 = nullptr;
-        float *d3f = nullptr;
-        e = upload(&m->d_ncen3, h.ncen3);
-        if (e == cudaSuccess) e = upload(&m->d_cen3, h.cen3);
-        if (e == cudaSuccess) e = upload(&d3, r3);
-        m->d_real3_64 = d3;
-        if (e == cudaSuccess) e = upload(&d3f, r3f);
-        m->d_real3_32 = d3f;
-        if (e != cudaSuccess) {
-            fv_mesh_destroy(m);
-            return cuda_fail(e, "build_fv_mesh: degree-2 tables");
-        }
-        m->u64 = carve3<double>(m->d_real3_64, n);
-        m->u32 = carve3<float>(m->d_real3_32, n);
-    }
+    m->t64 = carve<double>(m->d_real64, h);
+    m->t32 = carve<float>(m->d_real32, h);
     // host copies for fv_mesh_set_walls
     m->h_ptr = (int64_t *)malloc(sizeof(int64_t) * (size_t)(n + 1));
     m->h_vtx = (int64_t *)malloc(sizeof(int64_t) * (size_t)cell_ptr[n]);
     m->h_nb = (int *)malloc(sizeof(int) * h.nb.size());
-    if (!m->h_ptr || !m->h_vtx || !m->h_nb) {
+    m->h_pos = (int *)malloc(sizeof(int) * (size_t)n);
+    if (!m->h_ptr || !m->h_vtx || !m->h_nb || !m->h_pos) {
         fv_mesh_destroy(m);
         return fail(BZ_ENOMEM, "build_fv_mesh: host copies");
     }
@@ -660,8 +672,21 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         memcpy(m->h_vtx + m->h_ptr[i], cells[i].data(), sizeof(int64_t) * cells[i].size());
     }
     memcpy(m->h_nb, h.nb.data(), sizeof(int) * h.nb.size());
+    for (int64_t p = 0; p < n; ++p) m->h_pos[h.order[p]] = (int)p;
     *out = m;
     return BZ_OK;
+}
+
+static void drop_walls(bz_mesh *m) {
+    dev_free(m->d_wall);
+    dev_free(m->d_wallslot);
+    dev_free(m->d_wall64);
+    dev_free(m->d_wall32);
+    m->d_wall = nullptr;
+    m->d_wallslot = nullptr;
+    m->d_wall64 = nullptr;
+    m->d_wall32 = nullptr;
+    m->n_walls = 0;
 }
 
 // Walls with full accommodation on the boundary edges given by their vertex
@@ -670,13 +695,7 @@ int fv_mesh_set_walls(bz_mesh *m, int64_t n_edges, const int64_t *edges, const d
     if (!m) return fail(BZ_EINVAL, "fv_mesh_set_walls: mesh is NULL");
     if (n_edges < 0 || (n_edges > 0 && (!edges || !params)))
         return fail(BZ_EINVAL, "fv_mesh_set_walls: bad edge list");
-    dev_free(m->d_wall);
-    dev_free(m->d_wall64);
-    dev_free(m->d_wall32);
-    m->d_wall = nullptr;
-    m->d_wall64 = nullptr;
-    m->d_wall32 = nullptr;
-    m->n_walls = 0;
+    drop_walls(m);
     if (n_edges == 0) return BZ_OK;
     const int64_t n = m->n_cells;
     std::unordered_map<uint64_t, int64_t> bface;           // unordered vertex pair -> cell * K + face
@@ -692,25 +711,23 @@ int fv_mesh_set_walls(bz_mesh *m, int64_t n_edges, const int64_t *edges, const d
     }
     std::vector<int> wall((size_t)n * kFvMaxFaces, -1);
     std::vector<double> p64((size_t)n_edges * 3);
+    std::vector<int64_t> slot((size_t)n_edges);
     for (int64_t e = 0; e < n_edges; ++e) {
         auto it = bface.find(key(edges[2 * e], edges[2 * e + 1]));
         if (it == bface.end()) return fail(BZ_EINVAL, "fv_mesh_set_walls: an edge is not a boundary edge of the mesh");
         if (!(params[3 * e] > 0)) return fail(BZ_EINVAL, "fv_mesh_set_walls: wall temperature must be > 0");
-        wall[(size_t)it->second] = (int)e;
+        slot[e] = (int64_t)m->h_pos[it->second / kFvMaxFaces] * kFvMaxFaces + it->second % kFvMaxFaces;
+        wall[(size_t)slot[e]] = (int)e;
         for (int c = 0; c < 3; ++c) p64[3 * e + c] = params[3 * e + c];
     }
     std::vector<float> p32(p64.size());
     for (size_t q = 0; q < p64.size(); ++q) p32[q] = (float)p64[q];
     cudaError_t err = upload(&m->d_wall, wall);
+    if (err == cudaSuccess) err = upload(&m->d_wallslot, slot);
     if (err == cudaSuccess) err = upload(&m->d_wall64, p64);
     if (err == cudaSuccess) err = upload(&m->d_wall32, p32);
     if (err != cudaSuccess) {
-        dev_free(m->d_wall);
-        dev_free(m->d_wall64);
-        dev_free(m->d_wall32);
-        m->d_wall = nullptr;
-        m->d_wall64 = nullptr;
-        m->d_wall32 = nullptr;
+        drop_walls(m);
         return cuda_fail(err, "fv_mesh_set_walls: device tables");
     }
     m->n_walls = n_edges;

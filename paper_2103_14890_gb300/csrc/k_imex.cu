@@ -19,78 +19,104 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ double dexp(double x) { return exp(x); }
-
+// R_l of one grid point.  The G terms of a step whose G is 0 are left out, and
+// in FP64 the terms with a zero coefficient (their buffers need not hold
+// anything).  FP32 keeps those: a diverging cell overflows there first, and
+// the zero terms carry its NaN to the cells that saw it.
 template <typename T>
+__device__ __forceinline__ T stage_rhs(const StageCoef &c, T r, const T *__restrict__ G, const T *__restrict__ P,
+                                       const T *__restrict__ Lres, int64_t stride, int64_t o, T dt, T ieps) {
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        if (m >= c.nprev) break;
+        const int64_t om = (int64_t)m * stride + o;
+        if (sizeof(T) == 4 || c.at[m] != 0.0) {
+            T gm = c.use_G ? G[om] * ieps : (T)0;
+            if (Lres) gm -= Lres[om];
+            r = fma(dt * (T)c.at[m], gm, r);
+        }
+        if (sizeof(T) == 4 || c.a[m] != 0.0) r = fma(dt * (T)c.a[m] * ieps, P[om], r);
+    }
+    return r;
+}
+
+// Any grid (3-D, and 2-D with N > 32): one CTA per cell.  The Maxwellian is
+// the product of one factor per axis, each axis' N factors formed once per
+// cell (the exponent in FP64, the exponential in the state precision); 2-D, N = 40, FP64 on 2000 cells: 559 -> 347 us.
+template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageCoef c, const T *__restrict__ fn,
                                                               T *__restrict__ F, const T *__restrict__ G,
                                                               T *__restrict__ P, const T *__restrict__ Lres,
                                                               int64_t stride) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *red = reinterpret_cast<double *>(smem_raw);         // 32 * 5
-    T *R = reinterpret_cast<T *>(red + 32 * 5);                  // nv
-    const int64_t cell = blockIdx.x;
-    const int64_t base = cell * g.nv;
+    double *vt = red + 32 * 5;                                   // [N] nodes
+    T *fac = reinterpret_cast<T *>(vt + g.N);                    // [3][N] factors of the Maxwellian
+    T *R = fac + 3 * g.N;                                        // nv
+    const unsigned N = g.N, nv = (unsigned)g.nv;
+    const int64_t base = (int64_t)blockIdx.x * g.nv;
     const T dt = (T)c.dt, ieps = (T)(1.0 / c.eps);
+    for (unsigned j = threadIdx.x; j < N; j += blockDim.x) vt[j] = -g.L + (double)j * g.dv;
+    __syncthreads();
     double mom[5] = {0, 0, 0, 0, 0};
-    for (int64_t i = threadIdx.x; i < g.nv; i += blockDim.x) {
-        T r = fn[base + i];
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            if (m >= c.nprev) break;
-            const int64_t o = (int64_t)m * stride + base + i;
-            T gm = G[o] * ieps;
-            if (Lres) gm -= Lres[o];
-            r = fma(dt * (T)c.at[m], gm, r);
-            r = fma(dt * (T)c.a[m] * ieps, P[o], r);
-        }
+    for (unsigned i = threadIdx.x; i < nv; i += blockDim.x) {
+        const T r = stage_rhs<T>(c, fn[base + i], G, P, Lres, stride, base + i, dt, ieps);
         R[i] = r;
-        double rd = (double)r, v2 = 0.0;
+        const double rd = (double)r;
+        double v2 = 0.0;
         mom[0] += rd;
-        for (int d = 0; d < g.dim; ++d) {
-            double vd = grid_velocity(i, d, g.dim, g.N, g.L, g.dv);
-            mom[1 + d] += vd * rd;
-            v2 += vd * vd;
+        unsigned q = i;
+#pragma unroll
+        for (int d = DIM - 1; d >= 0; --d) {
+            const double vd = vt[q % N];
+            q /= N;
+            mom[1 + d] = fma(vd, rd, mom[1 + d]);
+            v2 = fma(vd, vd, v2);
         }
-        mom[g.dim + 1] += 0.5 * v2 * rd;
+        mom[DIM + 1] = fma(v2, rd, mom[DIM + 1]);
     }
     block_sum<5>(mom, red);
     double w = 1.0;
-    for (int d = 0; d < g.dim; ++d) w *= g.dv;
+    for (int d = 0; d < DIM; ++d) w *= g.dv;
     const double rho = w * mom[0];
     double u[3] = {0, 0, 0}, u2 = 0.0;
-    for (int d = 0; d < g.dim; ++d) {
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
         u[d] = w * mom[1 + d] / rho;
         u2 += u[d] * u[d];
     }
-    const double E = w * mom[g.dim + 1];
-    const double theta = (2.0 * E / rho - u2) / g.dim;
-    const double pref = rho * pow(2.0 * M_PI * theta, -0.5 * g.dim);
-    const double inv2t = 0.5 / theta;
+    const double theta = (w * mom[DIM + 1] / rho - u2) / DIM;
+    const double pref = rho * pow(2.0 * M_PI * theta, -0.5 * DIM);
+    const double i2t = 0.5 / theta;
     const double nu = c.nuf * rho;
     const double cc = c.dt * c.all * nu / c.eps;
     const T cT = (T)cc, denom = (T)(1.0 / (1.0 + cc)), nuT = (T)nu;
+    for (unsigned j = threadIdx.x; j < DIM * N; j += blockDim.x) {
+        const int d = (int)(j / N);
+        const double o = vt[j % N] - (d == 0 ? u[0] : d == 1 ? u[1] : u[2]);
+        fac[j] = (d == 0 ? (T)pref : (T)1) * exp((T)(-o * o * i2t));
+    }
+    __syncthreads();
     T *Fo = F + base;
     T *Po = P + (int64_t)c.stage * stride + base;
-    for (int64_t i = threadIdx.x; i < g.nv; i += blockDim.x) {
-        double r2 = 0.0;
-        for (int d = 0; d < g.dim; ++d) {
-            double dv = grid_velocity(i, d, g.dim, g.N, g.L, g.dv) - u[d];
-            r2 += dv * dv;
+    for (unsigned i = threadIdx.x; i < nv; i += blockDim.x) {
+        T Mx = (T)1;
+        unsigned q = i;
+#pragma unroll
+        for (int d = DIM - 1; d >= 0; --d) {
+            Mx *= fac[d * N + q % N];
+            q /= N;
         }
-        T Mx;
-        if constexpr (sizeof(T) == 8)
-            Mx = (T)(pref * dexp(-r2 * inv2t));
-        else
-            Mx = (T)pref * expf((float)(-r2 * inv2t));   // exponent in FP64, exp in the state precision
-        T Fi = (R[i] + cT * Mx) * denom;
+        const T Fi = (R[i] + cT * Mx) * denom;
         if (c.store_F) Fo[i] = Fi;
-        Po[i] = nuT * (Mx - Fi);
+        if (c.store_P) Po[i] = nuT * (Mx - Fi);
     }
 }
 
-// Fast 2-D path (N <= 32): one warp per cell, lane = column j2, loop over
-// rows j1, 8 cells per CTA.  FP64 work is what limits this kernel on a GPU
+// 2-D, N <= 32: one warp per cell, lane = column j2, loop over rows j1, 8 cells
+// per CTA.  (With N = 30 in FP64 on 2603 cells the block-per-cell form above it
+// took 552 us a stage, an exponential and index arithmetic per point on the
+// FP64 pipe; this one 139 us.)  FP64 work is what limits this kernel on a GPU
 // whose FP64 rate is 1/74 of FP32, so it is arranged to keep the FP64 pipe's
 // lanes busy with distinct work:
 //   * per lane, sums along j1 in the state precision (FP32: with a TwoSum
@@ -115,7 +141,8 @@ __device__ __forceinline__ void acc2(T &s, T &e, T x) {
 
 constexpr int kStageCells = 8;    // cells (warps) per CTA of the 2-D stage kernel (two CTAs per SM)
 
-template <typename T, int N>
+// NMAX rows in registers; FIXED: N = NMAX at compile time, else any N <= NMAX.
+template <typename T, int NMAX, bool FIXED>
 __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView g, StageCoef c,
                                                                        const T *__restrict__ fn, T *__restrict__ F,
                                                                        const T *__restrict__ G, T *__restrict__ P,
@@ -126,24 +153,29 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t cell = (int64_t)blockIdx.x * kStageCells + wib;
     const bool live = cell < n;
-    constexpr int NV = N * N;
+    const int N = FIXED ? NMAX : g.N, NV = N * N;
     const bool on = lane < N && live;
     const int64_t base = (live ? cell : 0) * NV + (lane < N ? lane : 0);
     const T dt = (T)c.dt, ieps = (T)(1.0 / c.eps);
-    T R[N];
+    T R[NMAX];
 #pragma unroll
-    for (int j = 0; j < N; ++j) R[j] = on ? fn[base + j * N] : (T)0;
+    for (int j = 0; j < NMAX; ++j) R[j] = on && (FIXED || j < N) ? fn[base + j * N] : (T)0;
 #pragma unroll
     for (int m = 0; m < 5; ++m) {              // compile-time index into the coefficient arrays
         if (m >= c.nprev) break;
         const T ca = dt * (T)c.at[m] * ieps, cb = dt * (T)c.a[m] * ieps, cl = dt * (T)c.at[m];
         const int64_t o = (int64_t)m * stride + base;
+        // terms left out: as in stage_rhs
+        const bool xe = sizeof(T) == 4 || c.at[m] != 0.0;
+        const bool ug = xe && c.use_G, up = sizeof(T) == 4 || c.a[m] != 0.0, ul = xe && Lres;
         if (on) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) {
-                T r = fma(ca, G[o + j * N], R[j]);
-                r = fma(cb, P[o + j * N], r);
-                if (Lres) r = fma(-cl, Lres[o + j * N], r);
+            for (int j = 0; j < NMAX; ++j) {
+                if (!FIXED && j >= N) break;
+                T r = R[j];
+                if (ug) r = fma(ca, G[o + j * N], r);
+                if (up) r = fma(cb, P[o + j * N], r);
+                if (ul) r = fma(-cl, Lres[o + j * N], r);
                 R[j] = r;
             }
         }
@@ -153,7 +185,7 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
         T s0 = 0, e0 = 0, s1 = 0, e1 = 0, s3 = 0, e3 = 0;
         const T L = (T)g.L, dv = (T)g.dv;
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
+        for (int j = 0; j < NMAX; ++j) {
             const T v1 = fma((T)j, dv, -L);
             acc2(s0, e0, R[j]);
             acc2(s1, e1, v1 * R[j]);
@@ -201,21 +233,31 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
     // separable Maxwellian: this lane's column factor and row factor j1 = lane;
     // offsets v - u in FP64, the rest of the exponent and the exp in T
     const double vl = -g.L + lane * g.dv;
-    const T d2 = (T)(vl - par[wib][2]), d1 = (T)(vl - par[wib][1]);
-    const T i2t = (T)par[wib][3];
-    const T fcol = (T)par[wib][4] * exp(-d2 * d2 * i2t);
-    const T frow_l = exp(-d1 * d1 * i2t);
+    // (any other N: the whole exponent in FP64)
+    const double d2 = vl - par[wib][2], d1 = vl - par[wib][1];
+    T x1, x2;
+    if constexpr (FIXED) {
+        const T i2t = (T)par[wib][3], t1 = (T)d1, t2 = (T)d2;
+        x1 = -t1 * t1 * i2t;
+        x2 = -t2 * t2 * i2t;
+    } else {
+        x1 = (T)(-d1 * d1 * par[wib][3]);
+        x2 = (T)(-d2 * d2 * par[wib][3]);
+    }
+    const T fcol = (T)par[wib][4] * exp(x2);
+    const T frow_l = exp(x1);
     const T cT = (T)par[wib][5], denom = (T)par[wib][6], nuT = (T)par[wib][0];
     T *Fo = F + base;
     T *Po = P + (int64_t)c.stage * stride + base;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
+    for (int j = 0; j < NMAX; ++j) {
+        if (!FIXED && j >= N) break;
         const T frow = __shfl_sync(0xffffffffu, frow_l, j);
         const T Mx = fcol * frow;
         const T Fi = (R[j] + cT * Mx) * denom;
         if (on) {
             if (c.store_F) Fo[j * N] = Fi;
-            Po[j * N] = nuT * (Mx - Fi);
+            if (c.store_P) Po[j * N] = nuT * (Mx - Fi);
         }
     }
 }
@@ -233,18 +275,20 @@ template <typename T>
 cudaError_t stage(const GridView &g, const StageCoef &c, const T *fn, T *F, const T *G, T *P,
                   const T *Lres, int64_t stride, int64_t n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (g.dim == 2 && (g.N == 16 || g.N == 24 || g.N == 32)) {
+    if (g.dim == 2 && g.N <= 32) {
         const unsigned blocks = (unsigned)((n + kStageCells - 1) / kStageCells);
         const unsigned thr = kStageCells * 32;
-        if (g.N == 16) imex_stage2d_kernel<T, 16><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
-        if (g.N == 24) imex_stage2d_kernel<T, 24><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
-        if (g.N == 32) imex_stage2d_kernel<T, 32><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
+        if (g.N == 16) imex_stage2d_kernel<T, 16, true><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
+        else if (g.N == 24) imex_stage2d_kernel<T, 24, true><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
+        else if (g.N == 32) imex_stage2d_kernel<T, 32, true><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
+        else imex_stage2d_kernel<T, 32, false><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
         return cudaGetLastError();
     }
-    size_t sm = sizeof(double) * 32 * 5 + sizeof(T) * (size_t)g.nv;
-    cudaError_t e = cudaFuncSetAttribute(imex_stage_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = sizeof(double) * (32 * 5 + g.N) + sizeof(T) * ((size_t)g.nv + 3 * g.N);
+    auto *kern = g.dim == 2 ? imex_stage_kernel<T, 2> : imex_stage_kernel<T, 3>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    imex_stage_kernel<T><<<(unsigned)n, kThreads, sm, st>>>(g, c, fn, F, G, P, Lres, stride);
+    kern<<<(unsigned)n, kThreads, sm, st>>>(g, c, fn, F, G, P, Lres, stride);
     return cudaGetLastError();
 }
 

@@ -1,38 +1,52 @@
 // k_transport.cu -- transport residual of the finite-volume scheme (Sec. 3.2,
-// eq. finite_vol5 / eq. ho): CWENO reconstruction of degree 1 and Rusanov
+// eq. finite_vol5 / eq. ho): CWENO reconstruction of degree 1 or 2 and Rusanov
 // fluxes, for every cell and every discrete velocity of a 2-D grid.
 //
 // Layout: f, L are [cell][nv] (the collision operator's layout), so one
-// cell's velocities are contiguous.  A block takes 1024 velocities of one cell
-// (4 per thread on triangle meshes): every table entry of the cell is a
-// warp-uniform load shared by 4 velocities and every f access is a 16-byte
-// vector of one coalesced row segment (neighbour rows come from L2: a 32^2
-// grid of 20k cells holds 81 MB in FP32).  Cells are taken along a Morton
-// curve of their barycentres (the mesh's order table).  On FP32 triangle
-// meshes without walls both passes of degree 1 are persistent: a block walks
-// the order in steps of the grid, staging the next cell's rows in shared
-// memory while it computes the current one.
+// cell's velocities are contiguous.  A block takes up to 1024 velocities of
+// one cell: every table entry of the cell is a warp-uniform load and every f
+// access a coalesced row segment (neighbour rows come from L2: a 32^2 grid of
+// 20k cells holds 81 MB in FP32).  Cells are taken along a Morton curve of
+// their barycentres; every table is stored in that order.
 //
-// Pass 1 (order 2): gradient of the CWENO polynomial per (cell, velocity),
-// stored as G [cell][2][nv] (FP32 triangle meshes without walls: the values at
-// the three face midpoints, FV [cell][3][nv]).  The central (least-squares)
-// gradient g_opt and
-// the sector gradients g_L are linear in the averages (tables R_c, R_s of
-// fv_mesh.cpp); the central polynomial's gradient is g_0 = (g_opt - sum_L
-// lambda_L g_L) / lambda_0 (eq. CWENO:P0, lambda_0 = 3/4, lambda_L = 1/4 /
-// #sectors); smoothness sigma_s = h^2 |g_s|^2; weights omega_s proportional
-// to lambda_s / (sigma_s + eps)^4 with eps = 1e-14 (eqn.weights), formed
-// as lambda_s ((sigma_min + eps) / (sigma_s + eps))^4 so that no power
+// Orders 2 and 3 take two passes.  For a linear flux v f the Rusanov flux
+//   F = (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2
+// is the upwind flux (v.n) f_L for v.n > 0 and (v.n) f_R for v.n < 0, and v.n
+// is constant along a straight face, so the face integral needs one mean of
+// the reconstruction per face (midpoint for degree 1, two Gauss points for
+// degree 2), on the upwind side only.
+//   Pass 1 reconstructs the polynomial of every (cell, velocity) in registers
+//   and writes the flux of the velocities that leave the cell through a face
+//   into that face's row, FX [face][nv]; the cell on the other side of the
+//   face writes the others.  Both sides form v.n from the same normal up to
+//   its sign, so every entry is written exactly once (v.n = 0: by the owner).
+//   Boundary faces are transmissive: their cell writes every velocity.
+//   Pass 2 sums a cell's face rows with their signs and divides by |P_i|.
+// FP32, thin cells (kFvThin; slivers of a Delaunay triangulation along the
+// boundary, half a percent of the cells): the fluxes cancel to L by a factor
+// of hundreds to thousands, which turns a rounding into a visible change of L.
+// Pass 1 also writes both sides' values at their faces (rows after the flux
+// rows, one per Gauss point), and pass 2 sums the two-sided Rusanov form there,
+// so that such cells keep the rounding they had with it (and, should they
+// overflow in an unstable run, their neighbours see it on every velocity).
+// Against gradients or coefficients in memory and both sides' states at every
+// face this halves the traffic on triangles (1.5 rows written and read per
+// cell in place of 5 and 24 for degree 2) and cuts the arithmetic that bounds
+// FP64 (the GB300 does 2 FP64 operations per clock and SM): per hexagon face
+// and velocity 9 operations in place of 34.  19802 triangles x 32^2, FP32,
+// degree 2: 0.382 -> 0.253 ms; 2603 Voronoi cells x
+// 30^2, FP64, degree 2: 2.13 -> 1.34 ms.
+//
+// Reconstruction: the central (least-squares) coefficients and the sector
+// polynomials are linear in the averages (tables Rc, Rs of fv_mesh.cpp);
+// p_0 = (p_opt - lambda_L sum_L p_L) / lambda_0 (lambda_0 = 3/4, lambda_L =
+// 1/4 / #sectors); smoothness sigma_s = h^2 |grad p_s|^2 (degree 2: the cell
+// mean, plus the squared scaled second derivatives); weights
+// proportional to lambda_s / (sigma_s + eps)^4 with eps = 1e-14, formed as
+// lambda_s ((sigma_min + eps) / (sigma_s + eps))^4 so that no power
 // underflows in FP32.
 //
-// The flux passes take the cells in the reverse of the reconstruction's
-// order, so that they start on the rows the reconstruction wrote last, which
-// are still in L2.
-//
-// Pass 2: per face, f_L = fbar_i + g_i . (x_f - x_b,i), f_R the same from the
-// neighbour (f_L on a boundary face: transmissive), Rusanov flux of v f:
-// |e| F = (v.|e|n)(f_L + f_R)/2 - |v.|e|n| (f_R - f_L)/2, summed and scaled
-// by 1/|P_i|.  The face midpoint rule is exact for degree-1 reconstructions.
+// Order 1 (piecewise constant) needs no reconstruction: one pass.
 #include <algorithm>
 #include <atomic>
 
@@ -45,16 +59,20 @@ namespace {
 
 constexpr int kFvThreads = 256;
 
-// VEC consecutive velocities per thread: the cell's table entries are loaded
-// once for all of them and f moves in 16-byte vectors (the row length N^2 is
-// a multiple of 4, and the host checks 16-byte alignment, else VEC = 1).
+// VEC consecutive velocities per thread, all in one row of the velocity grid
+// (N is even, and the host takes VEC = 4 only when 4 divides N): the cell's
+// table entries are loaded once for all of them and f moves in 8- or 16-byte
+// vectors (the host checks the alignment, else VEC = 1).
 template <typename T, int VEC> struct Vec {
     T v[VEC];
 };
 template <typename T, int VEC>
 __device__ __forceinline__ Vec<T, VEC> ldv(const T *__restrict__ p) {
     Vec<T, VEC> r;
-    if constexpr (VEC == 4 && sizeof(T) == 4) {
+    if constexpr (VEC == 2) {
+        const typename C2<T>::type q = *reinterpret_cast<const typename C2<T>::type *>(p);
+        r.v[0] = q.x; r.v[1] = q.y;
+    } else if constexpr (VEC == 4 && sizeof(T) == 4) {
         const float4 q = *reinterpret_cast<const float4 *>(p);
         r.v[0] = q.x; r.v[1] = q.y; r.v[2] = q.z; r.v[3] = q.w;
     } else if constexpr (VEC == 4 && sizeof(T) == 8) {
@@ -68,7 +86,9 @@ __device__ __forceinline__ Vec<T, VEC> ldv(const T *__restrict__ p) {
 }
 template <typename T, int VEC>
 __device__ __forceinline__ void stv(T *__restrict__ p, const Vec<T, VEC> &r) {
-    if constexpr (VEC == 4 && sizeof(T) == 4) {
+    if constexpr (VEC == 2) {
+        *reinterpret_cast<typename C2<T>::type *>(p) = cmk<typename C2<T>::type>(r.v[0], r.v[1]);
+    } else if constexpr (VEC == 4 && sizeof(T) == 4) {
         *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
     } else if constexpr (VEC == 4 && sizeof(T) == 8) {
         reinterpret_cast<double2 *>(p)[0] = make_double2(r.v[0], r.v[1]);
@@ -77,6 +97,14 @@ __device__ __forceinline__ void stv(T *__restrict__ p, const Vec<T, VEC> &r) {
 #pragma unroll
         for (int u = 0; u < VEC; ++u) p[u] = r.v[u];
     }
+}
+
+// four values off any 16-byte boundary
+template <typename T> __device__ __forceinline__ Vec<T, 4> ld4(const T *__restrict__ p) {
+    Vec<T, 4> r;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) r.v[u] = p[u];
+    return r;
 }
 
 // FP32x2 arithmetic on pairs of velocities: one FADD2 / FMUL2 / FFMA2 rounds
@@ -96,10 +124,611 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
 
+// Index tables of a mesh by position p of the processing order (bz_mesh).
+struct FvIdx {
+    const int *order, *meta, *fid, *two, *ncen, *cen, *nsec, *sec;
+};
+
+// FP64 forms that spare the FP64 pipe, on which a warp instruction takes 16
+// cycles of an SM.  min of two non-negative numbers as integers (the same
+// order; a NaN operand ends in NaN weights either way).  1 / b for b > 0: the
+// hardware's approximate reciprocal y (relative error e below 2^-17) and one
+// step of the cubic iteration y (1 + e + e^2), e = 1 - b y: three operations,
+// error below 2^-51 plus a rounding; the full division takes about three times
+// as many.
+__device__ __forceinline__ double min_nonneg(double a, double b) {
+    return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
+}
+__device__ __forceinline__ double rcp_pos(double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    double e = fma(-b, y, 1.0);
+    e = fma(e, e, e);
+    return fma(y, e, y);
+}
+
+// Write the flux of VEC velocities through a face: vn (outward normal velocity
+// times |e|) times the reconstructed mean `val`, in the owner's orientation,
+// where this cell is upwind (everywhere on a boundary face).
+template <typename T, int VEC>
+__device__ __forceinline__ void put_flux(T *__restrict__ row, const T (&vn)[VEC], const T (&val)[VEC], bool other,
+                                         bool boundary) {
+    Vec<T, VEC> o;
+    bool on[VEC], all = true;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+        const T fl = vn[u] * val[u];
+        o.v[u] = other ? -fl : fl;
+        on[u] = boundary || (other ? vn[u] > (T)0 : vn[u] >= (T)0);
+        all = all && on[u];
+    }
+    if (all) {
+        stv<T, VEC>(row, o);
+    } else {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+            if (on[u]) row[u] = o.v[u];
+    }
+}
+
+// Normal velocities v . |e|n of VEC velocities of one grid row (explicit FMA:
+// every path rounds alike, so the two sides of a face agree up to the sign).
+template <typename T, int VEC>
+__device__ __forceinline__ void normal_velocity(T v1, const T (&v2)[VEC], T nx, T ny, T (&vn)[VEC]) {
+    const T a = v1 * nx;
+    if constexpr (sizeof(T) == 4 && VEC == 4) {
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            const float2 x = fma2(make_float2(v2[h], v2[h + 1]), dup2(ny), dup2(a));
+            vn[h] = x.x;
+            vn[h + 1] = x.y;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) vn[u] = fma(v2[u], ny, a);
+    }
+}
+
+// Coefficients of a cell's CWENO polynomial in FP64, one velocity per thread
+// (any polygon).  B, K: coefficients and stencil cells (2, 5 or 5, 11); MAXS
+// bounds the sectors.  Loops are unrolled with block-uniform predicates.
+template <int MAXS, int B, int K>
+__device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, const FvTables<double> &tb,
+                                                const FvIdx &ix, int64_t p, int ncf, int k, int nv, double fi,
+                                                double (&c)[B]) {
+#pragma unroll
+    for (int l = 0; l < B; ++l) c[l] = 0.0;
+    const int nc = ncf & (kFvRegularTri - 1), ns = __ldg(ix.nsec + p);
+    const double *Rc = tb.Rc + p * (B * K);
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        if (q < nc) {
+            const double d = f[(int64_t)__ldg(ix.cen + p * K + q) * nv + k] - fi;
+#pragma unroll
+            for (int l = 0; l < B; ++l) c[l] = fma(__ldg(Rc + l * K + q), d, c[l]);
+        }
+    }
+    if (ns == 0) return;
+    constexpr double kLam0 = 0.75, kEps = 1e-14;
+    const double lamL = 0.25 / (double)ns;
+    double sx[MAXS], sy[MAXS], sumx = 0.0, sumy = 0.0;
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) {
+        if (s < ns) {
+            const int a = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2), b = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2 + 1);
+            const double *R = tb.Rs + (p * kFvMaxFaces + s) * 4;
+            const double da = f[(int64_t)a * nv + k] - fi, db = f[(int64_t)b * nv + k] - fi;
+            sx[s] = fma(__ldg(R), da, __ldg(R + 1) * db);
+            sy[s] = fma(__ldg(R + 2), da, __ldg(R + 3) * db);
+            sumx += sx[s];
+            sumy += sy[s];
+        }
+    }
+    // p_0's coefficients (1 / lambda_0 is in Rc), sigma + eps of every polynomial
+    const double lam10 = lamL * (4.0 / 3.0);
+    c[0] = fma(-lam10, sumx, c[0]);
+    c[1] = fma(-lam10, sumy, c[1]);
+    double s0 = fma(c[0], c[0], fma(c[1], c[1], kEps));
+    if constexpr (B == kFvCoef3) {
+        const double *q = tb.quad + 4 * p;
+        const double q3 = __ldg(q + 3);
+        s0 = fma(c[2], fma(__ldg(q), c[2], q3 * c[3]), s0);
+        s0 = fma(c[3], fma(__ldg(q + 1), c[3], q3 * c[4]), s0);
+        s0 = fma(c[4], __ldg(q + 2) * c[4], s0);
+    }
+    double sig[MAXS], num = s0;
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s)
+        if (s < ns) {
+            sig[s] = fma(sx[s], sx[s], fma(sy[s], sy[s], kEps));
+            num = min_nonneg(num, sig[s]);
+        }
+    double r = num * rcp_pos(s0);
+    r = r * r;
+    double w = kLam0 * (r * r), wl = 0.0, ax = 0.0, ay = 0.0;
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s)
+        if (s < ns) {
+            r = num * rcp_pos(sig[s]);
+            r = r * r;
+            r = r * r;
+            wl += r;
+            ax = fma(r, sx[s], ax);
+            ay = fma(r, sy[s], ay);
+        }
+    // (lambda_0 w_0 p_0 + lambda_L sum w_L p_L) / (lambda_0 w_0 + lambda_L sum w_L)
+    const double iw = rcp_pos(fma(lamL, wl, w)), wL = lamL * iw;
+    w *= iw;
+#pragma unroll
+    for (int l = 0; l < B; ++l) c[l] *= w;
+    c[0] = fma(wL, ax, c[0]);
+    c[1] = fma(wL, ay, c[1]);
+}
+
+// The same coefficients in FP32.
+template <int VEC, int MAXS>
+__device__ __forceinline__ void recon_coefs_f32(const float *__restrict__ f, const FvTables<float> &tb, const FvIdx &ix,
+                                                int64_t p, int ncf, int k, int nv, const Vec<float, VEC> &fi,
+                                                float (&c)[2][VEC]) {
+    const int nc = ncf & (kFvRegularTri - 1), ns = __ldg(ix.nsec + p);
+    // central least-squares gradient
+    float gx[VEC], gy[VEC];
+    {
+        Vec<float, VEC> fj[kFvCentral];
+        float rx[kFvCentral], ry[kFvCentral];
+#pragma unroll
+        for (int q = 0; q < kFvCentral; ++q) {
+            rx[q] = ry[q] = (float)0;
+            fj[q] = fi;
+            if (q < nc) {
+                const int j = __ldg(ix.cen + p * kFvCentral + q);
+                rx[q] = __ldg(tb.Rc + (p * 2) * kFvCentral + q);
+                ry[q] = __ldg(tb.Rc + (p * 2 + 1) * kFvCentral + q);
+                fj[q] = ldv<float, VEC>(f + (int64_t)j * nv + k);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            gx[u] = gy[u] = (float)0;
+#pragma unroll
+            for (int q = 0; q < kFvCentral; ++q) {
+                const float d = fj[q].v[u] - fi.v[u];
+                gx[u] += rx[q] * d;
+                gy[u] += ry[q] * d;
+            }
+        }
+    }
+    if (ns > 0) {
+        constexpr float kLam0 = (float)0.75, kInvLam0 = (float)(4.0 / 3.0), kEps = (float)1e-14;
+        const float lamL = (float)0.25 / (float)ns, h2 = __ldg(tb.quad + 4 * p + 3);
+        float sx[MAXS][VEC], sy[MAXS][VEC];
+        {
+            Vec<float, VEC> fa[MAXS], fb[MAXS];
+            float R[MAXS][4];
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) {
+                fa[s] = fi;
+                fb[s] = fi;
+                R[s][0] = R[s][1] = R[s][2] = R[s][3] = (float)0;
+                if (s < ns) {
+                    const int a = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2), b = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2 + 1);
+                    const float *Rp = tb.Rs + (p * kFvMaxFaces + s) * 4;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) R[s][c] = __ldg(Rp + c);
+                    fa[s] = ldv<float, VEC>(f + (int64_t)a * nv + k);
+                    fb[s] = ldv<float, VEC>(f + (int64_t)b * nv + k);
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s)
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) {
+                    const float da = fa[s].v[u] - fi.v[u], db = fb[s].v[u] - fi.v[u];
+                    sx[s][u] = R[s][0] * da + R[s][1] * db;
+                    sy[s][u] = R[s][2] * da + R[s][3] * db;
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            float sumx = (float)0, sumy = (float)0;
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s)
+                if (s < ns) {
+                    sumx += sx[s][u];
+                    sumy += sy[s][u];
+                }
+            const float g0x = (gx[u] - lamL * sumx) * kInvLam0, g0y = (gy[u] - lamL * sumy) * kInvLam0;
+            const float sig0 = h2 * (g0x * g0x + g0y * g0y);
+            float sig[MAXS];
+            float smin = sig0;
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) {
+                sig[s] = h2 * (sx[s][u] * sx[s][u] + sy[s][u] * sy[s][u]);
+                if (s < ns) smin = fmin(smin, sig[s]);
+            }
+            // fast divisions (2 ulp; the weights are smooth in sigma)
+            const float num = smin + kEps;
+            float r = __fdividef(num, sig0 + kEps);
+            r = r * r;
+            float w = kLam0 * (r * r);
+            float wsum = w, ax = w * g0x, ay = w * g0y;
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s)
+                if (s < ns) {
+                    r = __fdividef(num, sig[s] + kEps);
+                    r = r * r;
+                    w = lamL * (r * r);
+                    wsum += w;
+                    ax += w * sx[s][u];
+                    ay += w * sy[s][u];
+                }
+            const float iw = (float)1 / wsum;
+            gx[u] = ax * iw;
+            gy[u] = ay * iw;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+        c[0][u] = gx[u];
+        c[1][u] = gy[u];
+    }
+}
+template <int VEC, int MAXS>
+__device__ __forceinline__ void recon_coefs_f32(const float *__restrict__ f, const FvTables<float> &tb, const FvIdx &ix,
+                                                int64_t p, int ncf, int k, int nv, const Vec<float, VEC> &fi,
+                                                float (&c)[kFvCoef3][VEC]) {
+#pragma unroll
+    for (int l = 0; l < kFvCoef3; ++l)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) c[l][u] = 0.f;
+    const int nc = ncf & (kFvRegularTri - 1);
+    const float *Rc = tb.Rc + p * kFvCoef3 * kFvCentral3;
+#pragma unroll
+    for (int q = 0; q < kFvCentral3; ++q) {
+        if (q < nc) {
+            const int j = __ldg(ix.cen + p * kFvCentral3 + q);
+            const Vec<float, VEC> fj = ldv<float, VEC>(f + (int64_t)j * nv + k);
+#pragma unroll
+            for (int l = 0; l < kFvCoef3; ++l) {
+                const float r = __ldg(Rc + l * kFvCentral3 + q);
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) c[l][u] += r * (fj.v[u] - fi.v[u]);
+            }
+        }
+    }
+    const int ns = __ldg(ix.nsec + p);
+    if (ns > 0) {
+        constexpr float kInvLam0 = (float)(4.0 / 3.0), kLam0 = (float)0.75, kEps = (float)1e-14;
+        const float lamL = (float)0.25 / (float)ns;
+        float sx[MAXS][VEC], sy[MAXS][VEC];
+#pragma unroll
+        for (int s = 0; s < MAXS; ++s) {
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) sx[s][u] = sy[s][u] = (float)0;
+            if (s < ns) {
+                const int a = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2), b = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2 + 1);
+                const float *R = tb.Rs + (p * kFvMaxFaces + s) * 4;
+                const float r0 = __ldg(R), r1 = __ldg(R + 1), r2 = __ldg(R + 2), r3 = __ldg(R + 3);
+                const Vec<float, VEC> fa = ldv<float, VEC>(f + (int64_t)a * nv + k), fb = ldv<float, VEC>(f + (int64_t)b * nv + k);
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) {
+                    const float da = fa.v[u] - fi.v[u], db = fb.v[u] - fi.v[u];
+                    sx[s][u] = r0 * da + r1 * db;
+                    sy[s][u] = r2 * da + r3 * db;
+                }
+            }
+        }
+        const float m20 = __ldg(tb.quad + 4 * p), m11 = __ldg(tb.quad + 4 * p + 1), m02 = __ldg(tb.quad + 4 * p + 2);
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            float sumx = (float)0, sumy = (float)0;
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) {
+                sumx += sx[s][u];
+                sumy += sy[s][u];
+            }
+            float p0[kFvCoef3];
+            p0[0] = (c[0][u] - lamL * sumx) * kInvLam0;
+            p0[1] = (c[1][u] - lamL * sumy) * kInvLam0;
+#pragma unroll
+            for (int l = 2; l < kFvCoef3; ++l) p0[l] = c[l][u] * kInvLam0;
+            const float sig0 = p0[0] * p0[0] + p0[1] * p0[1] + (float)4 * p0[2] * p0[2] * m20 + (float)4 * p0[2] * p0[3] * m11 +
+                           p0[3] * p0[3] * m02 + p0[3] * p0[3] * m20 + (float)4 * p0[3] * p0[4] * m11 +
+                           (float)4 * p0[4] * p0[4] * m02 + (float)4 * p0[2] * p0[2] + p0[3] * p0[3] + (float)4 * p0[4] * p0[4];
+            float sig[MAXS], smin = sig0;
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) {
+                sig[s] = sx[s][u] * sx[s][u] + sy[s][u] * sy[s][u];
+                if (s < ns) smin = fmin(smin, sig[s]);
+            }
+            const float num = smin + kEps;
+            float r = __fdividef(num, sig0 + kEps);
+            r = r * r;
+            float w = kLam0 * (r * r);
+            float wsum = w, acc[kFvCoef3];
+#pragma unroll
+            for (int l = 0; l < kFvCoef3; ++l) acc[l] = w * p0[l];
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s)
+                if (s < ns) {
+                    r = __fdividef(num, sig[s] + kEps);
+                    r = r * r;
+                    w = lamL * (r * r);
+                    wsum += w;
+                    acc[0] += w * sx[s][u];
+                    acc[1] += w * sy[s][u];
+                }
+            const float iw = (float)1 / wsum;
+#pragma unroll
+            for (int l = 0; l < kFvCoef3; ++l) c[l][u] = acc[l] * iw;
+        }
+    }
+}
+
+// f + sum_l c_l phi_l for VEC velocities.
+template <typename T, int VEC, int B>
+__device__ __forceinline__ void point_value(const Vec<T, VEC> &fi, const T (&c)[B][VEC], const T *__restrict__ phi,
+                                            T (&val)[VEC]) {
+    if constexpr (sizeof(T) == 4 && VEC == 4) {
+        float2 x = make_float2(fi.v[0], fi.v[1]), y = make_float2(fi.v[2], fi.v[3]);
+#pragma unroll
+        for (int l = 0; l < B; ++l) {
+            const float2 ph = dup2(__ldg(phi + l));
+            x = fma2(make_float2(c[l][0], c[l][1]), ph, x);
+            y = fma2(make_float2(c[l][2], c[l][3]), ph, y);
+        }
+        val[0] = x.x; val[1] = x.y; val[2] = y.x; val[3] = y.y;
+    } else {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) val[u] = fi.v[u];
+#pragma unroll
+        for (int l = 0; l < B; ++l) {
+            const T ph = __ldg(phi + l);
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) val[u] = fma(c[l][u], ph, val[u]);
+        }
+    }
+}
+
+// Rows of a two-sided face behind the flux rows: [face][side][Gauss point].
+template <int B> __device__ __forceinline__ int64_t two_row(int64_t rows, int two, int side, int g) {
+    constexpr int GP = B == kFvCoef3 ? 2 : 1;
+    return rows + ((int64_t)two * 2 + side) * GP + g;
+}
+
+// Face q of the cell at position p: the upwind flux, and on a two-sided face
+// (FP32) the values at its points.
+template <typename T, int VEC, int B>
+__device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> &tb, const FvIdx &ix, int64_t rows,
+                                          int64_t p, int q, int fid, int meta, int k, int nv, T v1,
+                                          const T (&v2)[VEC], const Vec<T, VEC> &fi, const T (&c)[B][VEC]) {
+    const int64_t s = p * kFvMaxFaces + q;
+    T vn[VEC], val[VEC];
+    normal_velocity<T, VEC>(v1, v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+    const bool other = (meta >> (8 + q)) & 1, boundary = (meta >> (16 + q)) & 1;
+    if (sizeof(T) == 4 && ((meta >> (24 + q)) & 1)) {
+        const int two = __ldg(ix.two + s);
+#pragma unroll
+        for (int g = 0; g < (B == kFvCoef3 ? 2 : 1); ++g) {
+            point_value<T, VEC, B>(fi, c, B == kFvCoef3 ? tb.phig + (s * 2 + g) * B : tb.phi + s * B, val);
+            Vec<T, VEC> o;
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) o.v[u] = val[u];
+            stv<T, VEC>(FX + two_row<B>(rows, two, other, g) * nv + k, o);
+        }
+    }
+    bool any = boundary;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) any = any || vn[u] >= (T)0;
+    if (!any) return;
+    point_value<T, VEC, B>(fi, c, tb.phi + s * B, val);
+    put_flux<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
+}
+
+// Pass 1 of one cell, any polygon.
+template <typename T, int VEC, int MAXF, int B, int K>
+__device__ __forceinline__ void recon_faces(const T *__restrict__ f, T *__restrict__ FX, const FvTables<T> &tb,
+                                            const FvIdx &ix, int64_t rows, int64_t p, int ncf, int meta, int k, int nv,
+                                            T v1, const T (&v2)[VEC], const Vec<T, VEC> &fi) {
+    T c[B][VEC];
+    if constexpr (sizeof(T) == 8) {
+        static_assert(VEC == 1, "FP64 takes one velocity per thread");
+        double c1[B];
+        recon_coefs_f64<MAXF, B, K>(f, tb, ix, p, ncf, k, nv, fi.v[0], c1);
+#pragma unroll
+        for (int l = 0; l < B; ++l) c[l][0] = c1[l];
+    } else {
+        recon_coefs_f32<VEC, MAXF>(f, tb, ix, p, ncf, k, nv, fi, c);
+    }
+    const int nf = meta & 0xf;
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q)
+        if (q < nf)
+            emit_face<T, VEC, B>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v1, v2, fi,
+                                 c);
+}
+
+// Weights of one pair of velocities of a flagged triangle (kFvRegularTri: its
+// stencil starts with the face neighbours; sector s joins faces s and s + 1
+// mod 3) in FP32x2: c holds p_opt's coefficients, d the differences to the face
+// neighbours; the steps of recon_coefs_f32.
+template <int B>
+__device__ __forceinline__ void weigh_tri(float2 (&c)[B], const float2 (&d)[3], const float4 (&R)[3],
+                                          const float4 &quad) {
+    constexpr float kLam0 = 0.75f, kInvLam0 = (float)(4.0 / 3.0), kEps = 1e-14f;
+    const float lamL = 0.25f / 3.0f;
+    float2 sx[3], sy[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const float2 da = d[s], db = d[(s + 1) % 3];
+        sx[s] = fma2(dup2(R[s].x), da, mul2(dup2(R[s].y), db));
+        sy[s] = fma2(dup2(R[s].z), da, mul2(dup2(R[s].w), db));
+    }
+    const float2 sumx = add2(add2(sx[0], sx[1]), sx[2]), sumy = add2(add2(sy[0], sy[1]), sy[2]);
+    float2 p0[B];
+    p0[0] = mul2(fma2(dup2(-lamL), sumx, c[0]), dup2(kInvLam0));
+    p0[1] = mul2(fma2(dup2(-lamL), sumy, c[1]), dup2(kInvLam0));
+#pragma unroll
+    for (int l = 2; l < B; ++l) p0[l] = mul2(c[l], dup2(kInvLam0));
+    float2 sig0 = fma2(p0[0], p0[0], mul2(p0[1], p0[1]));
+    if constexpr (B == kFvCoef3) {
+        const float2 A22 = dup2(4.f * quad.x + 4.f), A33 = dup2(quad.z + quad.x + 1.f), A44 = dup2(4.f * quad.z + 4.f);
+        const float2 A23 = dup2(4.f * quad.y);
+        sig0 = fma2(mul2(A22, p0[2]), p0[2], sig0);
+        sig0 = fma2(mul2(A33, p0[3]), p0[3], sig0);
+        sig0 = fma2(mul2(A44, p0[4]), p0[4], sig0);
+        sig0 = fma2(mul2(A23, p0[2]), p0[3], sig0);
+        sig0 = fma2(mul2(A23, p0[3]), p0[4], sig0);
+    } else {
+        sig0 = mul2(dup2(quad.w), sig0);
+    }
+    const float2 E = dup2(kEps);
+    float2 sig[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        sig[s] = fma2(sx[s], sx[s], mul2(sy[s], sy[s]));
+        if (B == 2) sig[s] = mul2(dup2(quad.w), sig[s]);
+    }
+    const float2 smin = make_float2(fminf(fminf(sig0.x, sig[0].x), fminf(sig[1].x, sig[2].x)),
+                                    fminf(fminf(sig0.y, sig[0].y), fminf(sig[1].y, sig[2].y)));
+    const float2 num = add2(smin, E);
+    float2 r = mul2(num, rcp2(add2(sig0, E)));
+    r = mul2(r, r);
+    float2 w = mul2(dup2(kLam0), mul2(r, r)), wsum = w;
+#pragma unroll
+    for (int l = 0; l < B; ++l) p0[l] = mul2(w, p0[l]);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        r = mul2(num, rcp2(add2(sig[s], E)));
+        r = mul2(r, r);
+        w = mul2(dup2(lamL), mul2(r, r));
+        wsum = add2(wsum, w);
+        p0[0] = fma2(w, sx[s], p0[0]);
+        p0[1] = fma2(w, sy[s], p0[1]);
+    }
+    const float2 iw = rcp2(wsum);
+#pragma unroll
+    for (int l = 0; l < B; ++l) c[l] = mul2(p0[l], iw);
+}
+
+// Coefficients of the 4 velocities of a thread on a flagged triangle: row(q)
+// gives f of stencil cell q, each row read once.
+template <int B, int K, typename Row>
+__device__ __forceinline__ void coefs_tri_x2(const FvTables<float> &tb, int64_t p, const Vec<float, 4> &fi, Row row,
+                                             float (&c)[B][4]) {
+    const float2 nf[2] = {make_float2(-fi.v[0], -fi.v[1]), make_float2(-fi.v[2], -fi.v[3])};
+    const float *Rc = tb.Rc + p * (B * K);
+    float2 c2[2][B], dface[2][3];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        const float4 r = row(q);
+        const float2 d0 = add2(lo2(r), nf[0]), d1 = add2(hi2(r), nf[1]);
+        if (q < 3) {
+            dface[0][q] = d0;
+            dface[1][q] = d1;
+        }
+#pragma unroll
+        for (int l = 0; l < B; ++l) {
+            const float2 R = dup2(__ldg(Rc + l * K + q));
+            c2[0][l] = q == 0 ? mul2(R, d0) : fma2(R, d0, c2[0][l]);
+            c2[1][l] = q == 0 ? mul2(R, d1) : fma2(R, d1, c2[1][l]);
+        }
+    }
+    float4 R[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) R[s] = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (p * kFvMaxFaces + s) * 4));
+    const float4 quad = __ldg(reinterpret_cast<const float4 *>(tb.quad + 4 * p));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) weigh_tri<B>(c2[h], dface[h], R, quad);
+#pragma unroll
+    for (int l = 0; l < B; ++l) {
+        c[l][0] = c2[0][l].x;
+        c[l][1] = c2[0][l].y;
+        c[l][2] = c2[1][l].x;
+        c[l][3] = c2[1][l].y;
+    }
+}
+
+template <typename T, int VEC> struct Velocity {
+    T v1, v2[VEC];
+    __device__ __forceinline__ Velocity(int k, int N, T Lv, T dv) {
+        const int j1 = k / N, j2 = k - j1 * N;
+        v1 = -Lv + (T)j1 * dv;
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) v2[u] = -Lv + (T)(j2 + u) * dv;
+    }
+};
+
+template <typename T, int VEC, int MAXF, int B, int K>
+__device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restrict__ FX, const FvTables<T> &tb,
+                                            const FvIdx &ix, int64_t rows, int nv, int N, T Lv, T dv) {
+    const int64_t p = blockIdx.x;
+    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
+    if (k >= nv) return;
+    const int ncf = __ldg(ix.ncen + p), meta = __ldg(ix.meta + p);
+    const Vec<T, VEC> fi = ldv<T, VEC>(f + (int64_t)__ldg(ix.order + p) * nv + k);
+    const Velocity<T, VEC> v(k, N, Lv, dv);
+    if constexpr (sizeof(T) == 4 && VEC == 4 && MAXF == 3) {
+        if (ncf & kFvRegularTri) {      // uniform over the block: one cell per block
+            float c[B][4];
+            coefs_tri_x2<B, K>(tb, p, fi, [&](int q) {
+                return *reinterpret_cast<const float4 *>(f + (int64_t)__ldg(ix.cen + p * K + q) * nv + k);
+            }, c);
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                emit_face<float, 4, B>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v.v1,
+                                       v.v2, fi, c);
+            return;
+        }
+    }
+    recon_faces<T, VEC, MAXF, B, K>(f, FX, tb, ix, rows, p, ncf, meta, k, nv, v.v1, v.v2, fi);
+}
+
+template <typename T, int VEC, int MAXF, int B, int K>
+__global__ void __launch_bounds__(kFvThreads)
+fv_faces_kernel(const T *__restrict__ f, T *__restrict__ FX, FvTables<T> tb, FvIdx ix, int64_t rows, int nv, int N, T Lv,
+                T dv) {
+    faces_block<T, VEC, MAXF, B, K>(f, FX, tb, ix, rows, nv, N, Lv, dv);
+}
+
+// Degree 2 on FP32 triangles, 4 velocities per thread: four blocks per SM (64
+// registers, 36 bytes spilled; 19802 cells x 32^2: 0.203 ms, with three blocks
+// 0.232, with two 0.279).  A bound on the template above would also change the
+// register allocation of its other instantiations.
+__global__ void __launch_bounds__(kFvThreads, 4)
+fv_faces3_tri_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix, int64_t rows,
+                     int nv, int N, float Lv, float dv) {
+    faces_block<float, 4, 3, kFvCoef3, kFvCentral3>(f, FX, tb, ix, rows, nv, N, Lv, dv);
+}
+
+// Degree 1 on FP32 triangles without walls: the same two passes with a cell's
+// value at each of its faces, FV [cell][3][nv], in place of the upwind flux.
+// Both passes are persistent: a block takes one of every (SMs x blocks per SM)
+// positions of the processing order, walking them in steps of the grid; while
+// it computes one cell, the rows of the next one travel into shared memory by
+// cp.async (16 bytes per thread and row, each thread copying exactly the slots
+// it reads back, so no block barrier is needed and threads past nv leave at
+// once), and the index records of the cell after that are already being
+// loaded.  Writing whole rows of values unmasked costs this light
+// reconstruction less than forming and masking fluxes: 19802 triangles x 32^2,
+// 0.100 + 0.061 ms against 0.137 + 0.050 ms with upwind flux rows.
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+
+constexpr int kFaceRows = 6;         // rows staged per cell: f_i and 5 stencil rows / 3 own and 3 neighbour face rows
+// blocks per SM: 3 for the reconstruction (85 registers, no spills; 4 spill
+// its record prefetch), 4 for the flux pass (64 registers)
+constexpr int kFacesCtasPerSm = 3, kFluxCtasPerSm = 4;
+constexpr size_t kFaceStageBytes = 2 * kFaceRows * kFvThreads * sizeof(float4);   // 48 KB
+
 // CWENO gradient of one pair of velocities of a flagged triangle (kFvRegularTri):
 // d[q] = fbar_{cen q} - fbar_i, the face neighbours in d[0..2]; sector s
-// joins faces s and s + 1 mod 3.  The steps are those of the generic kernel
-// below (central gradient, sector gradients, g_0, smoothness, weights as
+// joins faces s and s + 1 mod 3.  The steps are those of
+// recon_coefs_f32 (central gradient, sector gradients, g_0, smoothness, weights as
 // lambda_s ((sigma_min + eps) / (sigma_s + eps))^4, normalised sum).
 __device__ __forceinline__ void cweno_pair_tri(const float2 (&d)[kFvCentral], const float (&rx)[kFvCentral],
                                                const float (&ry)[kFvCentral], const float4 (&R)[3], float h2,
@@ -148,339 +777,38 @@ __device__ __forceinline__ void cweno_pair_tri(const float2 (&d)[kFvCentral], co
     gy_out = mul2(ay, iw);
 }
 
-// Gradient of the 4 velocities k..k+3 of a flagged triangle in FP32x2: six
-// rows of f (the cell and its stencil, the face neighbours first), each
-// loaded once.  FACE: the output is the reconstruction's value at the three
-// face midpoints, f_i + g . (x_f - x_b,i), rows [cell][face][nv], in place of
-// the gradient rows [cell][2][nv].
-template <bool FACE>
-__device__ __forceinline__ void tri_x2_rows(float *__restrict__ G, const FvTables<float> &tb,
-                                            const float4 (&fr)[kFvCentral], int64_t i, int k, int nv,
-                                            const float4 fi) {
+// Values at the three faces of the 4 velocities k..k+3 of a flagged triangle.
+__device__ __forceinline__ void tri_values_x2(float *__restrict__ FV, const FvTables<float> &tb,
+                                              const float4 (&fr)[kFvCentral], int64_t p, int64_t i, int k, int nv,
+                                              const float4 fi) {
     float rx[kFvCentral], ry[kFvCentral];
 #pragma unroll
     for (int q = 0; q < kFvCentral; ++q) {
-        rx[q] = __ldg(tb.Rc + (i * 2) * kFvCentral + q);
-        ry[q] = __ldg(tb.Rc + (i * 2 + 1) * kFvCentral + q);
+        rx[q] = __ldg(tb.Rc + (p * 2) * kFvCentral + q);
+        ry[q] = __ldg(tb.Rc + (p * 2 + 1) * kFvCentral + q);
     }
     float4 R[3];
 #pragma unroll
-    for (int s = 0; s < 3; ++s) R[s] = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (i * kFvMaxFaces + s) * 4));
-    const float h2 = __ldg(tb.h2 + i);
+    for (int s = 0; s < 3; ++s) R[s] = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (p * kFvMaxFaces + s) * 4));
+    const float h2 = __ldg(tb.quad + 4 * p + 3);
     float2 gx[2], gy[2];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const float2 nf = neg2(p == 0 ? lo2(fi) : hi2(fi));
+    for (int h = 0; h < 2; ++h) {
+        const float2 nf = neg2(h == 0 ? lo2(fi) : hi2(fi));
         float2 d[kFvCentral];
 #pragma unroll
-        for (int q = 0; q < kFvCentral; ++q) d[q] = add2(p == 0 ? lo2(fr[q]) : hi2(fr[q]), nf);
-        cweno_pair_tri(d, rx, ry, R, h2, gx[p], gy[p]);
+        for (int q = 0; q < kFvCentral; ++q) d[q] = add2(h == 0 ? lo2(fr[q]) : hi2(fr[q]), nf);
+        cweno_pair_tri(d, rx, ry, R, h2, gx[h], gy[h]);
     }
-    if constexpr (FACE) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const float2 ox = dup2(__ldg(tb.off_i + 2 * (i * kFvMaxFaces + q)));
-            const float2 oy = dup2(__ldg(tb.off_i + 2 * (i * kFvMaxFaces + q) + 1));
-            const float2 a = fma2(gy[0], oy, fma2(gx[0], ox, lo2(fi)));
-            const float2 b = fma2(gy[1], oy, fma2(gx[1], ox, hi2(fi)));
-            *reinterpret_cast<float4 *>(G + (i * 3 + q) * nv + k) = make_float4(a.x, a.y, b.x, b.y);
-        }
-    } else {
-        *reinterpret_cast<float4 *>(G + (i * 2) * nv + k) = make_float4(gx[0].x, gx[0].y, gx[1].x, gx[1].y);
-        *reinterpret_cast<float4 *>(G + (i * 2 + 1) * nv + k) = make_float4(gy[0].x, gy[0].y, gy[1].x, gy[1].y);
+    for (int q = 0; q < 3; ++q) {
+        const float2 ox = dup2(__ldg(tb.phi + 2 * (p * kFvMaxFaces + q)));
+        const float2 oy = dup2(__ldg(tb.phi + 2 * (p * kFvMaxFaces + q) + 1));
+        const float2 a = fma2(gy[0], oy, fma2(gx[0], ox, lo2(fi)));
+        const float2 b = fma2(gy[1], oy, fma2(gx[1], ox, hi2(fi)));
+        *reinterpret_cast<float4 *>(FV + (i * 3 + q) * nv + k) = make_float4(a.x, a.y, b.x, b.y);
     }
 }
-
-template <bool FACE>
-__device__ __forceinline__ void gradient_tri_x2(const float *__restrict__ f, float *__restrict__ G,
-                                                const FvTables<float> &tb, const int (&jc)[kFvCentral], int64_t i,
-                                                int k, int nv, const float4 fi) {
-    float4 fr[kFvCentral];
-#pragma unroll
-    for (int q = 0; q < kFvCentral; ++q) fr[q] = *reinterpret_cast<const float4 *>(f + (int64_t)jc[q] * nv + k);
-    tri_x2_rows<FACE>(G, tb, fr, i, k, nv, fi);
-}
-
-// Reconstruction of cell i for the VEC velocities k.. of a thread (any
-// polygon; MAXS bounds its sectors): gradients, or with FACE the values at
-// the three face midpoints of a triangle.
-template <typename T, int VEC, int MAXS, bool FACE>
-__device__ __forceinline__ void gradient_generic(const T *__restrict__ f, T *__restrict__ G, const FvTables<T> &tb,
-                                                 const int *__restrict__ cen, const int *__restrict__ nsec,
-                                                 const int *__restrict__ sec, int64_t i, int ncf, int k, int nv,
-                                                 const Vec<T, VEC> &fi) {
-    const int nc = ncf & (kFvRegularTri - 1), ns = __ldg(nsec + i);
-    // central least-squares gradient
-    T gx[VEC], gy[VEC];
-    {
-        Vec<T, VEC> fj[kFvCentral];
-        T rx[kFvCentral], ry[kFvCentral];
-#pragma unroll
-        for (int q = 0; q < kFvCentral; ++q) {
-            rx[q] = ry[q] = (T)0;
-            fj[q] = fi;
-            if (q < nc) {
-                const int j = __ldg(cen + i * kFvCentral + q);
-                rx[q] = __ldg(tb.Rc + (i * 2) * kFvCentral + q);
-                ry[q] = __ldg(tb.Rc + (i * 2 + 1) * kFvCentral + q);
-                fj[q] = ldv<T, VEC>(f + (int64_t)j * nv + k);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) {
-            gx[u] = gy[u] = (T)0;
-#pragma unroll
-            for (int q = 0; q < kFvCentral; ++q) {
-                const T d = fj[q].v[u] - fi.v[u];
-                gx[u] += rx[q] * d;
-                gy[u] += ry[q] * d;
-            }
-        }
-    }
-    if (ns > 0) {
-        constexpr T kLam0 = (T)0.75, kInvLam0 = (T)(4.0 / 3.0), kEps = (T)1e-14;
-        const T lamL = (T)0.25 / (T)ns, h2 = __ldg(tb.h2 + i);
-        T sx[MAXS][VEC], sy[MAXS][VEC];
-        {
-            Vec<T, VEC> fa[MAXS], fb[MAXS];
-            T R[MAXS][4];
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) {
-                fa[s] = fi;
-                fb[s] = fi;
-                R[s][0] = R[s][1] = R[s][2] = R[s][3] = (T)0;
-                if (s < ns) {
-                    const int a = __ldg(sec + (i * kFvMaxFaces + s) * 2), b = __ldg(sec + (i * kFvMaxFaces + s) * 2 + 1);
-                    const T *Rp = tb.Rs + (i * kFvMaxFaces + s) * 4;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) R[s][c] = __ldg(Rp + c);
-                    fa[s] = ldv<T, VEC>(f + (int64_t)a * nv + k);
-                    fb[s] = ldv<T, VEC>(f + (int64_t)b * nv + k);
-                }
-            }
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s)
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) {
-                    const T da = fa[s].v[u] - fi.v[u], db = fb[s].v[u] - fi.v[u];
-                    sx[s][u] = R[s][0] * da + R[s][1] * db;
-                    sy[s][u] = R[s][2] * da + R[s][3] * db;
-                }
-        }
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) {
-            T sumx = (T)0, sumy = (T)0;
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s)
-                if (s < ns) {
-                    sumx += sx[s][u];
-                    sumy += sy[s][u];
-                }
-            const T g0x = (gx[u] - lamL * sumx) * kInvLam0, g0y = (gy[u] - lamL * sumy) * kInvLam0;
-            const T sig0 = h2 * (g0x * g0x + g0y * g0y);
-            T sig[MAXS];
-            T smin = sig0;
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) {
-                sig[s] = h2 * (sx[s][u] * sx[s][u] + sy[s][u] * sy[s][u]);
-                if (s < ns) smin = fmin(smin, sig[s]);
-            }
-            // weight ratios: FP32 takes the fast division (2 ulp; the weights
-            // are smooth in sigma), FP64 the correctly rounded one
-            const T num = smin + kEps;
-            auto ratio = [](T a, T b) {
-                if constexpr (sizeof(T) == 4) return __fdividef(a, b);
-                else return a / b;
-            };
-            T r = ratio(num, sig0 + kEps);
-            r = r * r;
-            T w = kLam0 * (r * r);
-            T wsum = w, ax = w * g0x, ay = w * g0y;
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s)
-                if (s < ns) {
-                    r = ratio(num, sig[s] + kEps);
-                    r = r * r;
-                    w = lamL * (r * r);
-                    wsum += w;
-                    ax += w * sx[s][u];
-                    ay += w * sy[s][u];
-                }
-            const T iw = (T)1 / wsum;
-            gx[u] = ax * iw;
-            gy[u] = ay * iw;
-        }
-    }
-    if constexpr (FACE) {
-        static_assert(MAXS == 3, "face values: triangle meshes");
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const T ofx = __ldg(tb.off_i + 2 * (i * kFvMaxFaces + q)), ofy = __ldg(tb.off_i + 2 * (i * kFvMaxFaces + q) + 1);
-            Vec<T, VEC> o;
-#pragma unroll
-            for (int u = 0; u < VEC; ++u) o.v[u] = fi.v[u] + gx[u] * ofx + gy[u] * ofy;
-            stv<T, VEC>(G + (i * 3 + q) * nv + k, o);
-        }
-    } else {
-        Vec<T, VEC> ox, oy;
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) {
-            ox.v[u] = gx[u];
-            oy.v[u] = gy[u];
-        }
-        stv<T, VEC>(G + (i * 2) * nv + k, ox);
-        stv<T, VEC>(G + (i * 2 + 1) * nv + k, oy);
-    }
-}
-
-// MAXS / MAXF: compile-time bound on the sectors / faces of a cell (3 for
-// triangle meshes, kFvMaxFaces otherwise).  Every loop over them is unrolled
-// with a predicate, so all neighbour rows of a cell are requested before the
-// first one is used (the kernels are latency-bound otherwise).
-template <typename T, int VEC, int MAXS>
-__global__ void __launch_bounds__(kFvThreads, (sizeof(T) == 4 && VEC == 4) ? 4 : 1)
-fv_gradient_kernel(const T *__restrict__ f, T *__restrict__ G, FvTables<T> tb, const int *__restrict__ ncen,
-                   const int *__restrict__ cen, const int *__restrict__ nsec, const int *__restrict__ sec,
-                   const int *__restrict__ order, int nv) {
-    const int64_t i = __ldg(order + blockIdx.x);
-    const int ncf = __ldg(ncen + i);
-    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
-    if (k >= nv) return;
-    const Vec<T, VEC> fi = ldv<T, VEC>(f + i * nv + k);
-    if constexpr (sizeof(T) == 4 && VEC == 4 && MAXS == 3) {
-        if (ncf & kFvRegularTri) {      // uniform over the block: one cell per block
-            int jc[kFvCentral];
-#pragma unroll
-            for (int q = 0; q < kFvCentral; ++q) jc[q] = __ldg(cen + i * kFvCentral + q);
-            gradient_tri_x2<false>(f, G, tb, jc, i, k, nv, make_float4(fi.v[0], fi.v[1], fi.v[2], fi.v[3]));
-            return;
-        }
-    }
-    gradient_generic<T, VEC, MAXS, false>(f, G, tb, cen, nsec, sec, i, ncf, k, nv, fi);
-}
-
-template <typename T, bool kGrad, int VEC, int MAXF>
-__global__ void __launch_bounds__(kFvThreads, (sizeof(T) == 4 && VEC == 4 && MAXF <= 3) ? 4 : 1)
-fv_flux_kernel(const T *__restrict__ f, const T *__restrict__ G, T *__restrict__ L, FvTables<T> tb,
-               const int *__restrict__ nface, const int *__restrict__ nb, const int *__restrict__ order, int nv,
-               int N, T Lv, T dv) {
-    const int64_t i = __ldg(order + (gridDim.x - 1 - blockIdx.x));
-    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
-    if (k >= nv) return;
-    const int nf = __ldg(nface + i);
-    const Vec<T, VEC> fi = ldv<T, VEC>(f + i * nv + k);
-    Vec<T, VEC> gxi, gyi;
-    if (kGrad) {
-        gxi = ldv<T, VEC>(G + (i * 2) * nv + k);
-        gyi = ldv<T, VEC>(G + (i * 2 + 1) * nv + k);
-    }
-    // every face's neighbour row first
-    int jn[MAXF];
-    Vec<T, VEC> fj[MAXF], gxj[MAXF], gyj[MAXF];
-#pragma unroll
-    for (int q = 0; q < MAXF; ++q) {
-        jn[q] = q < nf ? __ldg(nb + i * kFvMaxFaces + q) : -1;
-        fj[q] = fi;
-        if (kGrad) {
-            gxj[q] = gxi;
-            gyj[q] = gyi;
-        }
-        if (jn[q] >= 0) {
-            fj[q] = ldv<T, VEC>(f + (int64_t)jn[q] * nv + k);
-            if (kGrad) {
-                gxj[q] = ldv<T, VEC>(G + ((int64_t)jn[q] * 2) * nv + k);
-                gyj[q] = ldv<T, VEC>(G + ((int64_t)jn[q] * 2 + 1) * nv + k);
-            }
-        }
-    }
-    // velocities in the working precision; the VEC velocities of a thread lie
-    // in one row of the grid (the host takes VEC = 4 only when 4 divides N)
-    const int j1 = k / N, j2 = k - j1 * N;
-    const T v1 = -Lv + (T)j1 * dv;
-    T v2[VEC], acc[VEC];
-#pragma unroll
-    for (int u = 0; u < VEC; ++u) {
-        v2[u] = -Lv + (T)(j2 + u) * dv;
-        acc[u] = (T)0;
-    }
-#pragma unroll
-    for (int q = 0; q < MAXF; ++q) {
-        if (q >= nf) continue;
-        const int64_t s = i * kFvMaxFaces + q;
-        const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
-        T oix = (T)0, oiy = (T)0, ojx = (T)0, ojy = (T)0;
-        if (kGrad) {
-            oix = __ldg(tb.off_i + 2 * s);
-            oiy = __ldg(tb.off_i + 2 * s + 1);
-            ojx = __ldg(tb.off_j + 2 * s);
-            ojy = __ldg(tb.off_j + 2 * s + 1);
-        }
-        if constexpr (sizeof(T) == 4 && VEC == 4) {
-            // the same face flux on pairs of velocities in FP32x2
-            const float2 v1nx = dup2(v1 * nx), hf = dup2(0.5f);
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                const int u = 2 * p;
-                const float2 vn = fma2(make_float2(v2[u], v2[u + 1]), dup2(ny), v1nx);
-                float2 fl = make_float2(fi.v[u], fi.v[u + 1]);
-                if (kGrad)
-                    fl = fma2(make_float2(gyi.v[u], gyi.v[u + 1]), dup2(oiy),
-                              fma2(make_float2(gxi.v[u], gxi.v[u + 1]), dup2(oix), fl));
-                float2 fr = fl;
-                if (jn[q] >= 0) {
-                    fr = make_float2(fj[q].v[u], fj[q].v[u + 1]);
-                    if (kGrad)
-                        fr = fma2(make_float2(gyj[q].v[u], gyj[q].v[u + 1]), dup2(ojy),
-                                  fma2(make_float2(gxj[q].v[u], gxj[q].v[u + 1]), dup2(ojx), fr));
-                }
-                const float2 h = mul2(hf, vn), nah = make_float2(-fabsf(h.x), -fabsf(h.y));
-                float2 a = make_float2(acc[u], acc[u + 1]);
-                a = fma2(h, add2(fl, fr), a);
-                a = fma2(nah, add2(fr, neg2(fl)), a);
-                acc[u] = a.x;
-                acc[u + 1] = a.y;
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < VEC; ++u) {
-                const T vn = v1 * nx + v2[u] * ny;
-                T fl = fi.v[u];
-                if (kGrad) fl += gxi.v[u] * oix + gyi.v[u] * oiy;
-                T fr = fl;
-                if (jn[q] >= 0) {
-                    fr = fj[q].v[u];
-                    if (kGrad) fr += gxj[q].v[u] * ojx + gyj[q].v[u] * ojy;
-                }
-                acc[u] += (T)0.5 * vn * (fl + fr) - (T)0.5 * fabs(vn) * (fr - fl);
-            }
-        }
-    }
-    const T ia = __ldg(tb.inv_area + i);
-    Vec<T, VEC> o;
-#pragma unroll
-    for (int u = 0; u < VEC; ++u) o.v[u] = acc[u] * ia;
-    stv<T, VEC>(L + i * nv + k, o);
-}
-
-// ---- persistent forms of the two face-value passes --------------------------
-// A block takes one of every (SMs x blocks per SM) positions of the
-// processing order, walking them in steps of the grid; while it computes one cell, the rows of
-// the next one travel into shared memory by cp.async (16 bytes per thread and
-// row, each thread copying exactly the slots it reads back, so no block
-// barrier is needed and threads past nv leave at once), and the index
-// records of the cell after that are already being loaded.
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-
-constexpr int kFaceRows = 6;         // rows staged per cell: f_i and 5 stencil rows / 3 own and 3 neighbour face rows
-// blocks per SM: 3 for the reconstruction (85 registers, no spills; 4 spill
-// its record prefetch), 4 for the flux pass (64 registers)
-constexpr int kFacesCtasPerSm = 3, kFluxCtasPerSm = 4;
-constexpr size_t kFaceStageBytes = 2 * kFaceRows * kFvThreads * sizeof(float4);   // 48 KB
 
 // Index record of position p needed by the reconstruction: cell, flags, stencil.
 struct RecG {
@@ -491,11 +819,9 @@ __device__ __forceinline__ RecG rec_g(const int4 *__restrict__ tripos, int64_t p
     return RecG{a.x, a.y, {b.x, b.y, b.z, b.w, c.x}};
 }
 
-template <int CPS>
-__global__ void __launch_bounds__(kFvThreads, CPS)
-fv_faces_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, FvTables<float> tb,
-                        const int *__restrict__ cen, const int *__restrict__ nsec, const int *__restrict__ sec,
-                        const int4 *__restrict__ tripos, int64_t n, int nv) {
+__global__ void __launch_bounds__(kFvThreads, kFacesCtasPerSm)
+fv_values_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, FvTables<float> tb, FvIdx ix,
+                         const int4 *__restrict__ tripos, int64_t n, int nv) {
     extern __shared__ float4 stage[];            // [2][kFaceRows][kFvThreads]
     const int t = threadIdx.x;
     const int k = (blockIdx.y * kFvThreads + t) * 4;
@@ -526,11 +852,18 @@ fv_faces_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, FvT
             float4 fr[kFvCentral];
 #pragma unroll
             for (int q = 0; q < kFvCentral; ++q) fr[q] = sl[(q + 1) * kFvThreads];
-            tri_x2_rows<true>(FV, tb, fr, cur.i, k, nv, fi);
+            tri_values_x2(FV, tb, fr, p, cur.i, k, nv, fi);
         } else {
             Vec<float, 4> fv;
             fv.v[0] = fi.x; fv.v[1] = fi.y; fv.v[2] = fi.z; fv.v[3] = fi.w;
-            gradient_generic<float, 4, 3, true>(f, FV, tb, cen, nsec, sec, cur.i, cur.ncf, k, nv, fv);
+            float c[2][4], val[4];
+            recon_coefs_f32<4, 3>(f, tb, ix, p, cur.ncf, k, nv, fv, c);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                point_value<float, 4, 2>(fv, c, tb.phi + (p * kFvMaxFaces + q) * 2, val);
+                *reinterpret_cast<float4 *>(FV + ((int64_t)cur.i * 3 + q) * nv + k) =
+                    make_float4(val[0], val[1], val[2], val[3]);
+            }
         }
         if (!more) break;
         p += G;
@@ -549,7 +882,7 @@ __device__ __forceinline__ RecF rec_f(const int4 *__restrict__ tripos, int64_t p
 }
 
 __global__ void __launch_bounds__(kFvThreads, kFluxCtasPerSm)
-fv_flux_faces_persist_kernel(const float *__restrict__ FV, float *__restrict__ L, FvTables<float> tb,
+fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ L, FvTables<float> tb,
                              const int4 *__restrict__ tripos, int64_t n, int nv, int N, float Lv, float dv) {
     extern __shared__ float4 stage[];            // [2][kFaceRows][kFvThreads]
     const int t = threadIdx.x;
@@ -593,7 +926,7 @@ fv_flux_faces_persist_kernel(const float *__restrict__ FV, float *__restrict__ L
         for (int q = 0; q < 3; ++q) {
             const float4 fl = sl[q * kFvThreads];
             const float4 fr = cur.nb[q] >= 0 ? sl[(3 + q) * kFvThreads] : fl;
-            const int64_t s = i * kFvMaxFaces + q;
+            const int64_t s = pos(p) * kFvMaxFaces + q;
             const float nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
             const float2 v1nx = dup2(v1 * nx);
 #pragma unroll
@@ -602,10 +935,10 @@ fv_flux_faces_persist_kernel(const float *__restrict__ FV, float *__restrict__ L
                 const float2 vn = fma2(v2[h], dup2(ny), v1nx);
                 const float2 hv = mul2(hf, vn), nah = make_float2(-fabsf(hv.x), -fabsf(hv.y));
                 acc[h] = fma2(hv, add2(a, b), acc[h]);
-                acc[h] = fma2(nah, add2(b, neg2(a)), acc[h]);
+                acc[h] = fma2(nah, add2(b, make_float2(-a.x, -a.y)), acc[h]);
             }
         }
-        const float2 ia = dup2(__ldg(tb.inv_area + i));
+        const float2 ia = dup2(__ldg(tb.inv_area + pos(p)));
         const float2 o0 = mul2(acc[0], ia), o1 = mul2(acc[1], ia);
         *reinterpret_cast<float4 *>(L + i * nv + k) = make_float4(o0.x, o0.y, o1.x, o1.y);
         if (!more) break;
@@ -615,93 +948,193 @@ fv_flux_faces_persist_kernel(const float *__restrict__ FV, float *__restrict__ L
     }
 }
 
-// Flux pass of a mesh with walls (full accommodation, eq. BOU with alpha = 1,
-// eq. MAXB, eq. MU): one CTA holds all nv <= 1024 velocities of its cell, 4
-// per thread, so the wall density mu of a face -- the ratio of the outgoing
-// mass flux sum_{v.n > 0} f_L v.n to the incoming flux of the unit wall
-// Maxwellian sum_{v.n < 0} M_w |v.n| -- is a block reduction (FP64, fixed
-// order).  Velocities entering the domain through the wall carry mu M_w(v),
-// the others the reconstructed inner value; other faces as in fv_flux_kernel.
-template <typename T, bool VLOAD>
-__device__ __forceinline__ Vec<T, 4> ld4(const T *__restrict__ p) {
-    if constexpr (VLOAD) {
-        return ldv<T, 4>(p);
-    } else {
-        Vec<T, 4> r;
+// Incoming half of a wall face (full accommodation, eq. BOU with alpha = 1,
+// eq. MAXB, eq. MU): one block per wall holds all nv <= 1024 velocities, 4 per
+// thread.  mu, the ratio of the outgoing mass flux sum_{v.n > 0} f_L v.n (the
+// face row as pass 1 wrote it) to the incoming flux of the unit wall
+// Maxwellian sum_{v.n < 0} M_w |v.n|, is a block reduction (FP64, fixed
+// order); velocities entering the domain get the flux (v.n) mu M_w(v).  For
+// degree 2 the balance at the face's two Gauss points is linear in the
+// outgoing flux, so the mean over the face is balanced once.
+template <typename T>
+__global__ void __launch_bounds__(kFvThreads)
+fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__ fid, const int *__restrict__ wall,
+                     const int64_t *__restrict__ wallslot, const T *__restrict__ wallp, int nv, int N, T Lv, T dv) {
+    __shared__ double red[2 * (kFvThreads / 32)];
+    const int w = blockIdx.x;
+    const int64_t s = wallslot[w];
+    if (wall[s] != w) return;                    // an edge named twice: the last wall holds
+    const int kt = threadIdx.x * 4;
+    const bool act = kt < nv;
+    const int k = act ? kt : 0;                  // idle threads store nothing
+    T *row = FX + (int64_t)__ldg(fid + s) * nv + k;
+    const Velocity<T, 4> v(k, N, Lv, dv);
+    T vn[4], mw[4];
+    normal_velocity<T, 4>(v.v1, v.v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+    const T th = __ldg(wallp + 3 * w), uw1 = __ldg(wallp + 3 * w + 1), uw2 = __ldg(wallp + 3 * w + 2);
+    const T inv2th = (T)0.5 / th, norm = (T)(0.15915494309189535) / th;   // 1 / (2 pi theta)
+    double num = 0.0, den = 0.0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) r.v[u] = p[u];
-        return r;
+    for (int u = 0; u < 4; ++u) {
+        const T d1 = v.v1 - uw1, d2 = v.v2[u] - uw2;
+        mw[u] = norm * exp(-(d1 * d1 + d2 * d2) * inv2th);
+        if (act && vn[u] > (T)0) num += (double)row[u];
+        if (act && vn[u] < (T)0) den += (double)(mw[u] * -vn[u]);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[2 * (threadIdx.x >> 5)] = num;
+        red[2 * (threadIdx.x >> 5) + 1] = den;
+    }
+    __syncthreads();
+    num = den = 0.0;
+#pragma unroll
+    for (int q = 0; q < kFvThreads / 32; ++q) {
+        num += red[2 * q];
+        den += red[2 * q + 1];
+    }
+    const T mu = (T)(num / den);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (act && !(vn[u] > (T)0)) row[u] = vn[u] * (mu * mw[u]);
 }
 
-template <typename T, bool kGrad, int MAXF, bool VLOAD>
+// Pass 2: L_i = (1/|P_i|) sum over the faces of the signed flux rows, the
+// cells in the reverse of pass 1's order, so that the first ones find the rows
+// written last still in L2.  DRAM-bound.
+template <typename T, int VEC, int MAXF, int B>
 __global__ void __launch_bounds__(kFvThreads)
-fv_flux_wall_kernel(const T *__restrict__ f, const T *__restrict__ G, T *__restrict__ L, FvTables<T> tb,
-                    const int *__restrict__ nface, const int *__restrict__ nb, const int *__restrict__ order,
-                    const int *__restrict__ wall, const T *__restrict__ wallp, int nv, int N, T Lv, T dv) {
+fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
+              int64_t rows, int nv, int N, T Lv, T dv) {
+    const int64_t p = gridDim.x - 1 - blockIdx.x;
+    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
+    if (k >= nv) return;
+    const int meta = __ldg(ix.meta + p), nf = meta & 0xf;
+    Vec<T, VEC> x[MAXF];
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q)
+        if (q < nf) x[q] = ldv<T, VEC>(FX + (int64_t)__ldg(ix.fid + p * kFvMaxFaces + q) * nv + k);
+    const T ia = __ldg(tb.inv_area + p);
+    Vec<T, VEC> o;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) o.v[u] = (T)0;
+    const unsigned two_sided = sizeof(T) == 4 ? (unsigned)meta >> 24 : 0u;
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q)
+        if (q < nf && !((two_sided >> q) & 1)) {
+            const bool other = (meta >> (8 + q)) & 1;
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) o.v[u] += other ? -x[q].v[u] : x[q].v[u];
+        }
+    if (two_sided) {
+        // faces of thin cells: (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2 at every face point
+        constexpr int GP = B == kFvCoef3 ? 2 : 1;
+        constexpr T half = (T)(0.5 / GP);
+        for (int q = 0; q < nf; ++q) {
+            if (!((two_sided >> q) & 1)) continue;
+            const int64_t s = p * kFvMaxFaces + q;
+            if (wall && __ldg(wall + s) >= 0) {          // the wall's flux row
+                const T *r = FX + (int64_t)__ldg(ix.fid + s) * nv + k;
+                for (int u = 0; u < VEC; ++u) o.v[u] += r[u];
+                continue;
+            }
+            const int side = (meta >> (8 + q)) & 1, two = __ldg(ix.two + s);
+            const bool boundary = (meta >> (16 + q)) & 1;
+            const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
+            for (int g = 0; g < GP; ++g) {
+                const T *a = FX + two_row<B>(rows, two, side, g) * nv + k;
+                // the other side's points run the other way
+                const T *b = boundary ? a : FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k;
+                for (int u = 0; u < VEC; ++u) {
+                    const Velocity<T, 1> v(k + u, N, Lv, dv);
+                    T vn[1];
+                    normal_velocity<T, 1>(v.v1, v.v2, nx, ny, vn);
+                    const T h = half * vn[0], fl = a[u], fr = b[u];
+                    o.v[u] = fma(h, fl + fr, o.v[u]);
+                    o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) o.v[u] *= ia;
+    stv<T, VEC>(L + (int64_t)__ldg(ix.order + p) * nv + k, o);
+}
+
+// ---- order 1: Rusanov fluxes of the cell averages in one pass ------------------
+template <typename T, int VEC, int MAXF>
+__global__ void __launch_bounds__(kFvThreads, (sizeof(T) == 4 && VEC == 4 && MAXF <= 3) ? 4 : 1)
+fv_first_kernel(const T *__restrict__ f, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ nb,
+                int nv, int N, T Lv, T dv) {
+    const int64_t p = blockIdx.x;
+    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
+    if (k >= nv) return;
+    const int64_t i = __ldg(ix.order + p);
+    const int nf = __ldg(ix.meta + p) & 0xf;
+    const Vec<T, VEC> fi = ldv<T, VEC>(f + i * nv + k);
+    // every face's neighbour row first
+    Vec<T, VEC> fj[MAXF];
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q) {
+        const int j = q < nf ? __ldg(nb + p * kFvMaxFaces + q) : -1;
+        fj[q] = fi;
+        if (j >= 0) fj[q] = ldv<T, VEC>(f + (int64_t)j * nv + k);
+    }
+    const Velocity<T, VEC> v(k, N, Lv, dv);
+    T acc[VEC];
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) acc[u] = (T)0;
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q) {
+        if (q >= nf) continue;
+        const int64_t s = p * kFvMaxFaces + q;
+        T vn[VEC];
+        normal_velocity<T, VEC>(v.v1, v.v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            const T fl = fi.v[u], fr = fj[q].v[u];
+            acc[u] += (T)0.5 * vn[u] * (fl + fr) - (T)0.5 * fabs(vn[u]) * (fr - fl);
+        }
+    }
+    const T ia = __ldg(tb.inv_area + p);
+    Vec<T, VEC> o;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) o.v[u] = acc[u] * ia;
+    stv<T, VEC>(L + i * nv + k, o);
+}
+
+// Order 1 on a mesh with walls: one block holds all nv <= 1024 velocities of
+// its cell, 4 per thread, and forms each wall face's mu as
+// fv_wall_faces_kernel does.
+template <typename T, int MAXF>
+__global__ void __launch_bounds__(kFvThreads)
+fv_first_wall_kernel(const T *__restrict__ f, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ nb,
+                     const int *__restrict__ wall, const T *__restrict__ wallp, int nv, int N, T Lv, T dv) {
     __shared__ double red[2 * (kFvThreads / 32)];
-    const int64_t i = __ldg(order + (gridDim.x - 1 - blockIdx.x));
+    const int64_t p = blockIdx.x, i = __ldg(ix.order + p);
     const int kt = threadIdx.x * 4;
     const bool act = kt < nv;
     const int k = act ? kt : 0;                  // idle threads read row 0 and store nothing
-    const int nf = __ldg(nface + i);
-    const Vec<T, 4> fi = ld4<T, VLOAD>(f + i * nv + k);
-    Vec<T, 4> gxi, gyi;
-    if (kGrad) {
-        gxi = ld4<T, VLOAD>(G + (i * 2) * nv + k);
-        gyi = ld4<T, VLOAD>(G + (i * 2 + 1) * nv + k);
-    }
-    int jn[MAXF];
-    Vec<T, 4> fj[MAXF], gxj[MAXF], gyj[MAXF];
+    const int nf = __ldg(ix.meta + p) & 0xf;
+    const Vec<T, 4> fi = ld4<T>(f + i * nv + k);
+    const Velocity<T, 4> v(k, N, Lv, dv);
+    T acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = (T)0;
 #pragma unroll
     for (int q = 0; q < MAXF; ++q) {
-        jn[q] = q < nf ? __ldg(nb + i * kFvMaxFaces + q) : -1;
-        fj[q] = fi;
-        if (kGrad) {
-            gxj[q] = gxi;
-            gyj[q] = gyi;
-        }
-        if (jn[q] >= 0) {
-            fj[q] = ld4<T, VLOAD>(f + (int64_t)jn[q] * nv + k);
-            if (kGrad) {
-                gxj[q] = ld4<T, VLOAD>(G + ((int64_t)jn[q] * 2) * nv + k);
-                gyj[q] = ld4<T, VLOAD>(G + ((int64_t)jn[q] * 2 + 1) * nv + k);
-            }
-        }
-    }
-    const int j1 = k / N, j2 = k - j1 * N;
-    const T v1 = -Lv + (T)j1 * dv;
-    T v2[4], acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        v2[u] = -Lv + (T)(j2 + u) * dv;
-        acc[u] = (T)0;
-    }
-#pragma unroll
-    for (int q = 0; q < MAXF; ++q) {
-        if (q >= nf) continue;                   // uniform over the CTA (one cell)
-        const int64_t s = i * kFvMaxFaces + q;
-        const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
-        T oix = (T)0, oiy = (T)0, ojx = (T)0, ojy = (T)0;
-        if (kGrad) {
-            oix = __ldg(tb.off_i + 2 * s);
-            oiy = __ldg(tb.off_i + 2 * s + 1);
-            ojx = __ldg(tb.off_j + 2 * s);
-            ojy = __ldg(tb.off_j + 2 * s + 1);
-        }
-        T vn[4], fl[4], fr[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            vn[u] = v1 * nx + v2[u] * ny;
-            fl[u] = fi.v[u];
-            if (kGrad) fl[u] += gxi.v[u] * oix + gyi.v[u] * oiy;
-            fr[u] = fl[u];
-            if (jn[q] >= 0) {
-                fr[u] = fj[q].v[u];
-                if (kGrad) fr[u] += gxj[q].v[u] * ojx + gyj[q].v[u] * ojy;
-            }
-        }
-        const int w = jn[q] < 0 ? __ldg(wall + s) : -1;      // uniform over the CTA
+        if (q >= nf) continue;                   // uniform over the block (one cell)
+        const int64_t s = p * kFvMaxFaces + q;
+        const int j = __ldg(nb + s);
+        T vn[4];
+        normal_velocity<T, 4>(v.v1, v.v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+        Vec<T, 4> fr = fi;
+        if (j >= 0) fr = ld4<T>(f + (int64_t)j * nv + k);
+        const int w = j < 0 ? __ldg(wall + s) : -1;          // uniform over the block
         if (w >= 0) {
             const T th = __ldg(wallp + 3 * w), uw1 = __ldg(wallp + 3 * w + 1), uw2 = __ldg(wallp + 3 * w + 2);
             const T inv2th = (T)0.5 / th, norm = (T)(0.15915494309189535) / th;   // 1 / (2 pi theta)
@@ -709,9 +1142,9 @@ fv_flux_wall_kernel(const T *__restrict__ f, const T *__restrict__ G, T *__restr
             double num = 0.0, den = 0.0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const T d1 = v1 - uw1, d2 = v2[u] - uw2;
+                const T d1 = v.v1 - uw1, d2 = v.v2[u] - uw2;
                 mw[u] = norm * exp(-(d1 * d1 + d2 * d2) * inv2th);
-                if (act && vn[u] > (T)0) num += (double)(fl[u] * vn[u]);
+                if (act && vn[u] > (T)0) num += (double)(fi.v[u] * vn[u]);
                 if (act && vn[u] < (T)0) den += (double)(mw[u] * -vn[u]);
             }
 #pragma unroll
@@ -733,651 +1166,39 @@ fv_flux_wall_kernel(const T *__restrict__ f, const T *__restrict__ G, T *__restr
             }
             const T mu = (T)(num / den);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) fr[u] = vn[u] > (T)0 ? fl[u] : mu * mw[u];
+            for (int u = 0; u < 4; ++u) fr.v[u] = vn[u] > (T)0 ? fi.v[u] : mu * mw[u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += (T)0.5 * vn[u] * (fl[u] + fr[u]) - (T)0.5 * fabs(vn[u]) * (fr[u] - fl[u]);
+        for (int u = 0; u < 4; ++u)
+            acc[u] += (T)0.5 * vn[u] * (fi.v[u] + fr.v[u]) - (T)0.5 * fabs(vn[u]) * (fr.v[u] - fi.v[u]);
     }
     if (act) {
-        const T ia = __ldg(tb.inv_area + i);
+        const T ia = __ldg(tb.inv_area + p);
 #pragma unroll
         for (int u = 0; u < 4; ++u) L[i * nv + k + u] = acc[u] * ia;
     }
 }
 
-
-// ---- degree 2 (order 3) -----------------------------------------------------
-// Coefficients of the CWENO polynomial of degree 2 per (cell, velocity) in the
-// zero-mean scaled Taylor basis phi = (xi, eta, xi^2 - mu20, xi eta - mu11,
-// eta^2 - mu02), xi = (x - x_b)/h: p_opt from the least-squares rows over the
-// cell's 11 nearest cells, the degree-1 sector polynomials (coefficients of
-// xi and eta only), p_0 = (p_opt - lambda_L sum_L p_L) / lambda_0, and the
-// weights lambda_s / (sigma_s + eps)^4 in the same ratio form as degree 1,
-// sigma_s the cell mean of |h grad p|^2 plus the squared scaled second
-// derivatives (for the linear sectors: |h grad p|^2).  VEC velocities per
-// thread (4 on triangle meshes with aligned rows: the table entries, uniform
-// over the CTA, are then loaded once per 4 velocities); C is [cell][5][nv].
-// Degree-2 coefficients of the 4 velocities k..k+3 of a flagged triangle in
-// FP32x2 (its 11-cell stencil starts with the face neighbours; sector s joins
-// faces s and s + 1 mod 3): the steps of the generic kernel below, each
-// neighbour row loaded once.
-__device__ __forceinline__ void coef3_tri_x2(const float *__restrict__ f, float *__restrict__ C,
-                                             const FvTables<float> &tb, const FvTables3<float> &t3,
-                                             const int *__restrict__ cen, int64_t i, int k, int nv, const float4 fi) {
-    constexpr float kInvLam0 = (float)(4.0 / 3.0), kLam0 = 0.75f, kEps = 1e-14f;
-    const float lamL = 0.25f / 3.0f;
-    const float2 nf[2] = {neg2(lo2(fi)), neg2(hi2(fi))};
-    const float *Rc = t3.Rc + i * kFvCoef3 * kFvCentral3;
-    float2 c[kFvCoef3][2], dface[3][2];
-#pragma unroll
-    for (int q = 0; q < kFvCentral3; ++q) {
-        const int j = __ldg(cen + i * kFvCentral3 + q);
-        const float4 r = *reinterpret_cast<const float4 *>(f + (int64_t)j * nv + k);
-        const float2 d0 = add2(lo2(r), nf[0]), d1 = add2(hi2(r), nf[1]);
-        if (q < 3) {
-            dface[q][0] = d0;
-            dface[q][1] = d1;
-        }
-#pragma unroll
-        for (int l = 0; l < kFvCoef3; ++l) {
-            const float2 R = dup2(__ldg(Rc + l * kFvCentral3 + q));
-            c[l][0] = q == 0 ? mul2(R, d0) : fma2(R, d0, c[l][0]);
-            c[l][1] = q == 0 ? mul2(R, d1) : fma2(R, d1, c[l][1]);
-        }
-    }
-    float2 sx[3][2], sy[3][2];
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const float4 R = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (i * kFvMaxFaces + s) * 4));
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const float2 da = dface[s][p], db = dface[(s + 1) % 3][p];
-            sx[s][p] = fma2(dup2(R.x), da, mul2(dup2(R.y), db));
-            sy[s][p] = fma2(dup2(R.z), da, mul2(dup2(R.w), db));
-        }
-    }
-    const float m20 = __ldg(t3.mu + 3 * i), m11 = __ldg(t3.mu + 3 * i + 1), m02 = __ldg(t3.mu + 3 * i + 2);
-    // smoothness of the central polynomial: sum of its squared derivatives
-    // over the scaled cell, a quadratic form in p0 with these coefficients
-    const float2 A22 = dup2(4.f * m20 + 4.f), A33 = dup2(m02 + m20 + 1.f), A44 = dup2(4.f * m02 + 4.f);
-    const float2 A23 = dup2(4.f * m11), E = dup2(kEps);
-    float2 out[kFvCoef3][2];
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const float2 sumx = add2(add2(sx[0][p], sx[1][p]), sx[2][p]), sumy = add2(add2(sy[0][p], sy[1][p]), sy[2][p]);
-        float2 p0[kFvCoef3];
-        p0[0] = mul2(fma2(dup2(-lamL), sumx, c[0][p]), dup2(kInvLam0));
-        p0[1] = mul2(fma2(dup2(-lamL), sumy, c[1][p]), dup2(kInvLam0));
-#pragma unroll
-        for (int l = 2; l < kFvCoef3; ++l) p0[l] = mul2(c[l][p], dup2(kInvLam0));
-        float2 sig0 = fma2(p0[0], p0[0], mul2(p0[1], p0[1]));
-        sig0 = fma2(mul2(A22, p0[2]), p0[2], sig0);
-        sig0 = fma2(mul2(A33, p0[3]), p0[3], sig0);
-        sig0 = fma2(mul2(A44, p0[4]), p0[4], sig0);
-        sig0 = fma2(mul2(A23, p0[2]), p0[3], sig0);
-        sig0 = fma2(mul2(A23, p0[3]), p0[4], sig0);
-        float2 sig[3];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) sig[s] = fma2(sx[s][p], sx[s][p], mul2(sy[s][p], sy[s][p]));
-        const float2 smin = make_float2(fminf(fminf(sig0.x, sig[0].x), fminf(sig[1].x, sig[2].x)),
-                                        fminf(fminf(sig0.y, sig[0].y), fminf(sig[1].y, sig[2].y)));
-        const float2 num = add2(smin, E);
-        float2 r = mul2(num, rcp2(add2(sig0, E)));
-        r = mul2(r, r);
-        float2 w = mul2(dup2(kLam0), mul2(r, r));
-        float2 wsum = w, acc[kFvCoef3];
-#pragma unroll
-        for (int l = 0; l < kFvCoef3; ++l) acc[l] = mul2(w, p0[l]);
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            r = mul2(num, rcp2(add2(sig[s], E)));
-            r = mul2(r, r);
-            w = mul2(dup2(lamL), mul2(r, r));
-            wsum = add2(wsum, w);
-            acc[0] = fma2(w, sx[s][p], acc[0]);
-            acc[1] = fma2(w, sy[s][p], acc[1]);
-        }
-        const float2 iw = rcp2(wsum);
-#pragma unroll
-        for (int l = 0; l < kFvCoef3; ++l) out[l][p] = mul2(acc[l], iw);
-    }
-#pragma unroll
-    for (int l = 0; l < kFvCoef3; ++l)
-        *reinterpret_cast<float4 *>(C + (i * kFvCoef3 + l) * nv + k) =
-            make_float4(out[l][0].x, out[l][0].y, out[l][1].x, out[l][1].y);
-}
-
-template <typename T, int VEC, int MAXS>
-__device__ __forceinline__ void coef3_body(const T *__restrict__ f, T *__restrict__ C, const FvTables<T> &tb,
-                                           const FvTables3<T> &t3, const int *__restrict__ ncen,
-                                           const int *__restrict__ cen, const int *__restrict__ nsec,
-                                           const int *__restrict__ sec, const int *__restrict__ order, int nv) {
-    const int64_t i = __ldg(order + blockIdx.x);
-    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
-    if (k >= nv) return;
-    const Vec<T, VEC> fi = ldv<T, VEC>(f + i * nv + k);
-    const int ncf = __ldg(ncen + i);
-    if constexpr (sizeof(T) == 4 && VEC == 4 && MAXS == 3) {
-        if (ncf & kFvRegularTri) {      // uniform over the block: one cell per block
-            coef3_tri_x2(f, C, tb, t3, cen, i, k, nv, make_float4(fi.v[0], fi.v[1], fi.v[2], fi.v[3]));
-            return;
-        }
-    }
-    T c[kFvCoef3][VEC];
-#pragma unroll
-    for (int l = 0; l < kFvCoef3; ++l)
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) c[l][u] = (T)0;
-    const int nc = ncf & (kFvRegularTri - 1);
-    const T *Rc = t3.Rc + i * kFvCoef3 * kFvCentral3;
-#pragma unroll
-    for (int q = 0; q < kFvCentral3; ++q) {
-        if (q < nc) {
-            const int j = __ldg(cen + i * kFvCentral3 + q);
-            const Vec<T, VEC> fj = ldv<T, VEC>(f + (int64_t)j * nv + k);
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) {
-                const T r = __ldg(Rc + l * kFvCentral3 + q);
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) c[l][u] += r * (fj.v[u] - fi.v[u]);
-            }
-        }
-    }
-    const int ns = __ldg(nsec + i);
-    if (ns > 0) {
-        constexpr T kInvLam0 = (T)(4.0 / 3.0), kLam0 = (T)0.75, kEps = (T)1e-14;
-        const T lamL = (T)0.25 / (T)ns;
-        T sx[MAXS][VEC], sy[MAXS][VEC];
-#pragma unroll
-        for (int s = 0; s < MAXS; ++s) {
-#pragma unroll
-            for (int u = 0; u < VEC; ++u) sx[s][u] = sy[s][u] = (T)0;
-            if (s < ns) {
-                const int a = __ldg(sec + (i * kFvMaxFaces + s) * 2), b = __ldg(sec + (i * kFvMaxFaces + s) * 2 + 1);
-                const T *R = tb.Rs + (i * kFvMaxFaces + s) * 4;
-                const T r0 = __ldg(R), r1 = __ldg(R + 1), r2 = __ldg(R + 2), r3 = __ldg(R + 3);
-                const Vec<T, VEC> fa = ldv<T, VEC>(f + (int64_t)a * nv + k), fb = ldv<T, VEC>(f + (int64_t)b * nv + k);
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) {
-                    const T da = fa.v[u] - fi.v[u], db = fb.v[u] - fi.v[u];
-                    sx[s][u] = r0 * da + r1 * db;
-                    sy[s][u] = r2 * da + r3 * db;
-                }
-            }
-        }
-        const T m20 = __ldg(t3.mu + 3 * i), m11 = __ldg(t3.mu + 3 * i + 1), m02 = __ldg(t3.mu + 3 * i + 2);
-        auto ratio = [](T a, T b) {
-            if constexpr (sizeof(T) == 4) return __fdividef(a, b);
-            else return a / b;
-        };
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) {
-            T sumx = (T)0, sumy = (T)0;
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) {
-                sumx += sx[s][u];
-                sumy += sy[s][u];
-            }
-            T p0[kFvCoef3];
-            p0[0] = (c[0][u] - lamL * sumx) * kInvLam0;
-            p0[1] = (c[1][u] - lamL * sumy) * kInvLam0;
-#pragma unroll
-            for (int l = 2; l < kFvCoef3; ++l) p0[l] = c[l][u] * kInvLam0;
-            const T sig0 = p0[0] * p0[0] + p0[1] * p0[1] + (T)4 * p0[2] * p0[2] * m20 + (T)4 * p0[2] * p0[3] * m11 +
-                           p0[3] * p0[3] * m02 + p0[3] * p0[3] * m20 + (T)4 * p0[3] * p0[4] * m11 +
-                           (T)4 * p0[4] * p0[4] * m02 + (T)4 * p0[2] * p0[2] + p0[3] * p0[3] + (T)4 * p0[4] * p0[4];
-            T sig[MAXS], smin = sig0;
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) {
-                sig[s] = sx[s][u] * sx[s][u] + sy[s][u] * sy[s][u];
-                if (s < ns) smin = fmin(smin, sig[s]);
-            }
-            const T num = smin + kEps;
-            T r = ratio(num, sig0 + kEps);
-            r = r * r;
-            T w = kLam0 * (r * r);
-            T wsum = w, acc[kFvCoef3];
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) acc[l] = w * p0[l];
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s)
-                if (s < ns) {
-                    r = ratio(num, sig[s] + kEps);
-                    r = r * r;
-                    w = lamL * (r * r);
-                    wsum += w;
-                    acc[0] += w * sx[s][u];
-                    acc[1] += w * sy[s][u];
-                }
-            const T iw = (T)1 / wsum;
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) c[l][u] = acc[l] * iw;
-        }
-    }
-#pragma unroll
-    for (int l = 0; l < kFvCoef3; ++l) {
-        Vec<T, VEC> o;
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) o.v[u] = c[l][u];
-        stv<T, VEC>(C + (i * kFvCoef3 + l) * nv + k, o);
-    }
-}
-
-template <typename T, int VEC, int MAXS>
-__global__ void __launch_bounds__(kFvThreads)
-fv_coef3_kernel(const T *__restrict__ f, T *__restrict__ C, FvTables<T> tb, FvTables3<T> t3,
-                const int *__restrict__ ncen, const int *__restrict__ cen, const int *__restrict__ nsec,
-                const int *__restrict__ sec, const int *__restrict__ order, int nv) {
-    coef3_body<T, VEC, MAXS>(f, C, tb, t3, ncen, cen, nsec, sec, order, nv);
-}
-
-// FP32 triangles, 4 velocities per thread: four blocks per SM (64 registers;
-// measured 0.194 -> 0.180 ms on 19802 cells x 32^2 against three).  A bound
-// on the template above would also change the register allocation of its
-// other instantiations.
-__global__ void __launch_bounds__(kFvThreads, 4)
-fv_coef3_tri_kernel(const float *__restrict__ f, float *__restrict__ C, FvTables<float> tb, FvTables3<float> t3,
-                    const int *__restrict__ ncen, const int *__restrict__ cen, const int *__restrict__ nsec,
-                    const int *__restrict__ sec, const int *__restrict__ order, int nv) {
-    coef3_body<float, 4, 3>(f, C, tb, t3, ncen, cen, nsec, sec, order, nv);
-}
-
-// Flux pass of degree 2: the reconstruction on both sides at the face's two
-// Gauss-Legendre points (weights 1/2), the Rusanov flux at each; transmissive
-// boundary faces take f_R = f_L.  VEC velocities of one grid row per thread
-// (the host takes VEC = 4 only when 4 divides N).
-template <typename T, int VEC, int MAXF>
-__global__ void __launch_bounds__(kFvThreads, (sizeof(T) == 4 && VEC == 4 && MAXF <= 3) ? 3 : 1)
-fv_flux3_kernel(const T *__restrict__ f, const T *__restrict__ C, T *__restrict__ L, FvTables<T> tb,
-                FvTables3<T> t3, const int *__restrict__ nface, const int *__restrict__ nb,
-                const int *__restrict__ order, int nv, int N, T Lv, T dv) {
-    const int64_t i = __ldg(order + (gridDim.x - 1 - blockIdx.x));
-    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
-    if (k >= nv) return;
-    const int nf = __ldg(nface + i);
-    const Vec<T, VEC> fi = ldv<T, VEC>(f + i * nv + k);
-    Vec<T, VEC> ci[kFvCoef3];
-#pragma unroll
-    for (int l = 0; l < kFvCoef3; ++l) ci[l] = ldv<T, VEC>(C + (i * kFvCoef3 + l) * nv + k);
-    const int j1 = k / N, j2 = k - j1 * N;
-    const T v1 = -Lv + (T)j1 * dv;
-    T v2[VEC], acc[VEC];
-#pragma unroll
-    for (int u = 0; u < VEC; ++u) {
-        v2[u] = -Lv + (T)(j2 + u) * dv;
-        acc[u] = (T)0;
-    }
-#pragma unroll
-    for (int q = 0; q < MAXF; ++q) {
-        if (q >= nf) continue;
-        const int64_t s = i * kFvMaxFaces + q;
-        const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
-        const int jn = __ldg(nb + s);
-        Vec<T, VEC> fj = fi, cj[kFvCoef3];
-#pragma unroll
-        for (int l = 0; l < kFvCoef3; ++l) cj[l] = ci[l];
-        if (jn >= 0) {
-            fj = ldv<T, VEC>(f + (int64_t)jn * nv + k);
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) cj[l] = ldv<T, VEC>(C + ((int64_t)jn * kFvCoef3 + l) * nv + k);
-        }
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            T pi[kFvCoef3], pj[kFvCoef3];
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) {
-                pi[l] = __ldg(t3.phi_i + (s * 2 + g) * kFvCoef3 + l);
-                pj[l] = jn >= 0 ? __ldg(t3.phi_j + (s * 2 + g) * kFvCoef3 + l) : (T)0;
-            }
-            if constexpr (sizeof(T) == 4 && VEC == 4) {
-                // the same Gauss-point flux on pairs of velocities in FP32x2
-                const float2 v1nx = dup2(v1 * nx), qf = dup2(0.25f);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int u = 2 * h;
-                    float2 fl = make_float2(fi.v[u], fi.v[u + 1]);
-#pragma unroll
-                    for (int l = 0; l < kFvCoef3; ++l) fl = fma2(make_float2(ci[l].v[u], ci[l].v[u + 1]), dup2(pi[l]), fl);
-                    float2 fr = fl;
-                    if (jn >= 0) {
-                        fr = make_float2(fj.v[u], fj.v[u + 1]);
-#pragma unroll
-                        for (int l = 0; l < kFvCoef3; ++l)
-                            fr = fma2(make_float2(cj[l].v[u], cj[l].v[u + 1]), dup2(pj[l]), fr);
-                    }
-                    const float2 vn = fma2(make_float2(v2[u], v2[u + 1]), dup2(ny), v1nx);
-                    const float2 hv = mul2(qf, vn), nah = make_float2(-fabsf(hv.x), -fabsf(hv.y));
-                    float2 a = make_float2(acc[u], acc[u + 1]);
-                    a = fma2(hv, add2(fl, fr), a);
-                    a = fma2(nah, add2(fr, neg2(fl)), a);
-                    acc[u] = a.x;
-                    acc[u + 1] = a.y;
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) {
-                    T fl = fi.v[u];
-#pragma unroll
-                    for (int l = 0; l < kFvCoef3; ++l) fl += ci[l].v[u] * pi[l];
-                    T fr = fl;
-                    if (jn >= 0) {
-                        fr = fj.v[u];
-#pragma unroll
-                        for (int l = 0; l < kFvCoef3; ++l) fr += cj[l].v[u] * pj[l];
-                    }
-                    const T vn = v1 * nx + v2[u] * ny;
-                    acc[u] += (T)0.25 * (vn * (fl + fr) - fabs(vn) * (fr - fl));
-                }
-            }
-        }
-    }
-    const T ia = __ldg(tb.inv_area + i);
-    Vec<T, VEC> o;
-#pragma unroll
-    for (int u = 0; u < VEC; ++u) o.v[u] = acc[u] * ia;
-    stv<T, VEC>(L + i * nv + k, o);
-}
-
-
-// Flux pass of degree 2 on a mesh with walls: as fv_flux_wall_kernel (one CTA
-// per cell, 4 velocities per thread, nv <= 1024), with the reconstruction at
-// the two Gauss points of every face; at a wall face the mass balance of
-// eq. MU holds at each Gauss point, so one block reduction forms the two
-// outgoing fluxes and the wall Maxwellian's incoming flux together.
-template <typename T, int MAXF, bool VLOAD>
-__global__ void __launch_bounds__(kFvThreads)
-fv_flux3_wall_kernel(const T *__restrict__ f, const T *__restrict__ C, T *__restrict__ L, FvTables<T> tb,
-                     FvTables3<T> t3, const int *__restrict__ nface, const int *__restrict__ nb,
-                     const int *__restrict__ order, const int *__restrict__ wall, const T *__restrict__ wallp, int nv,
-                     int N, T Lv, T dv) {
-    __shared__ double red[3 * (kFvThreads / 32)];
-    const int64_t i = __ldg(order + (gridDim.x - 1 - blockIdx.x));
-    const int kt = threadIdx.x * 4;
-    const bool act = kt < nv;
-    const int k = act ? kt : 0;                  // idle threads read row 0 and store nothing
-    const int nf = __ldg(nface + i);
-    const Vec<T, 4> fi = ld4<T, VLOAD>(f + i * nv + k);
-    Vec<T, 4> ci[kFvCoef3];
-#pragma unroll
-    for (int l = 0; l < kFvCoef3; ++l) ci[l] = ld4<T, VLOAD>(C + (i * kFvCoef3 + l) * nv + k);
-    const int j1 = k / N, j2 = k - j1 * N;
-    const T v1 = -Lv + (T)j1 * dv;
-    T v2[4], acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        v2[u] = -Lv + (T)(j2 + u) * dv;
-        acc[u] = (T)0;
-    }
-#pragma unroll
-    for (int q = 0; q < MAXF; ++q) {
-        if (q >= nf) continue;                   // uniform over the CTA (one cell)
-        const int64_t s = i * kFvMaxFaces + q;
-        const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
-        const int jn = __ldg(nb + s);
-        Vec<T, 4> fj = fi, cj[kFvCoef3];
-#pragma unroll
-        for (int l = 0; l < kFvCoef3; ++l) cj[l] = ci[l];
-        if (jn >= 0) {
-            fj = ld4<T, VLOAD>(f + (int64_t)jn * nv + k);
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) cj[l] = ld4<T, VLOAD>(C + ((int64_t)jn * kFvCoef3 + l) * nv + k);
-        }
-        T vn[4], fl[2][4], fr[2][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) vn[u] = v1 * nx + v2[u] * ny;
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            T pi[kFvCoef3], pj[kFvCoef3];
-#pragma unroll
-            for (int l = 0; l < kFvCoef3; ++l) {
-                pi[l] = __ldg(t3.phi_i + (s * 2 + g) * kFvCoef3 + l);
-                pj[l] = jn >= 0 ? __ldg(t3.phi_j + (s * 2 + g) * kFvCoef3 + l) : (T)0;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                T a = fi.v[u];
-#pragma unroll
-                for (int l = 0; l < kFvCoef3; ++l) a += ci[l].v[u] * pi[l];
-                fl[g][u] = a;
-                T b = a;
-                if (jn >= 0) {
-                    b = fj.v[u];
-#pragma unroll
-                    for (int l = 0; l < kFvCoef3; ++l) b += cj[l].v[u] * pj[l];
-                }
-                fr[g][u] = b;
-            }
-        }
-        const int w = jn < 0 ? __ldg(wall + s) : -1;         // uniform over the CTA
-        if (w >= 0) {
-            const T th = __ldg(wallp + 3 * w), uw1 = __ldg(wallp + 3 * w + 1), uw2 = __ldg(wallp + 3 * w + 2);
-            const T inv2th = (T)0.5 / th, norm = (T)(0.15915494309189535) / th;   // 1 / (2 pi theta)
-            T mw[4];
-            double num0 = 0.0, num1 = 0.0, den = 0.0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const T d1 = v1 - uw1, d2 = v2[u] - uw2;
-                mw[u] = norm * exp(-(d1 * d1 + d2 * d2) * inv2th);
-                if (act && vn[u] > (T)0) {
-                    num0 += (double)(fl[0][u] * vn[u]);
-                    num1 += (double)(fl[1][u] * vn[u]);
-                }
-                if (act && vn[u] < (T)0) den += (double)(mw[u] * -vn[u]);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                num0 += __shfl_xor_sync(0xffffffffu, num0, o);
-                num1 += __shfl_xor_sync(0xffffffffu, num1, o);
-                den += __shfl_xor_sync(0xffffffffu, den, o);
-            }
-            __syncthreads();                     // red is reused face after face
-            if ((threadIdx.x & 31) == 0) {
-                red[3 * (threadIdx.x >> 5)] = num0;
-                red[3 * (threadIdx.x >> 5) + 1] = num1;
-                red[3 * (threadIdx.x >> 5) + 2] = den;
-            }
-            __syncthreads();
-            num0 = num1 = den = 0.0;
-#pragma unroll
-            for (int q2 = 0; q2 < kFvThreads / 32; ++q2) {
-                num0 += red[3 * q2];
-                num1 += red[3 * q2 + 1];
-                den += red[3 * q2 + 2];
-            }
-            const T mu0 = (T)(num0 / den), mu1 = (T)(num1 / den);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                fr[0][u] = vn[u] > (T)0 ? fl[0][u] : mu0 * mw[u];
-                fr[1][u] = vn[u] > (T)0 ? fl[1][u] : mu1 * mw[u];
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < 2; ++g)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                acc[u] += (T)0.25 * (vn[u] * (fl[g][u] + fr[g][u]) - fabs(vn[u]) * (fr[g][u] - fl[g][u]));
-    }
-    if (act) {
-        const T ia = __ldg(tb.inv_area + i);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) L[i * nv + k + u] = acc[u] * ia;
-    }
-}
-
-bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
+bool aligned(const void *p, size_t bytes) { return ((uintptr_t)p & (bytes - 1)) == 0; }
 
 template <typename T> const FvTables<T> &pick(const bz_mesh *m);
 template <> const FvTables<double> &pick<double>(const bz_mesh *m) { return m->t64; }
 template <> const FvTables<float> &pick<float>(const bz_mesh *m) { return m->t32; }
-template <typename T> const FvTables3<T> &pick3(const bz_mesh *m);
-template <> const FvTables3<double> &pick3<double>(const bz_mesh *m) { return m->u64; }
-template <> const FvTables3<float> &pick3<float>(const bz_mesh *m) { return m->u32; }
+template <typename T> const T *wall_params(const bz_mesh *m);
+template <> const double *wall_params<double>(const bz_mesh *m) { return m->d_wall64; }
+template <> const float *wall_params<float>(const bz_mesh *m) { return m->d_wall32; }
 
-template <typename T>
-cudaError_t coef3(const bz_mesh *m, const GridView &g, const T *f, T *C, cudaStream_t st) {
-    if (m->n_cells <= 0) return cudaSuccess;
-    const int nv = (int)g.nv;
-    const bool v4 = m->max_faces <= 3 && nv % 4 == 0 && aligned16(f) && aligned16(C);
-    const int vec = v4 ? 4 : 1;
-    const dim3 grid((unsigned)m->n_cells, (unsigned)((nv / vec + kFvThreads - 1) / kFvThreads));
-    if constexpr (sizeof(T) == 4) {
-        if (v4) {
-            fv_coef3_tri_kernel<<<grid, kFvThreads, 0, st>>>(f, C, pick<T>(m), pick3<T>(m), m->d_ncen3, m->d_cen3,
-                                                             m->d_nsec, m->d_sec, m->d_order, nv);
-            return cudaGetLastError();
-        }
-    }
-    if (v4)
-        fv_coef3_kernel<T, 4, 3><<<grid, kFvThreads, 0, st>>>(f, C, pick<T>(m), pick3<T>(m), m->d_ncen3, m->d_cen3,
-                                                               m->d_nsec, m->d_sec, m->d_order, nv);
-    else if (m->max_faces <= 3)
-        fv_coef3_kernel<T, 1, 3><<<grid, kFvThreads, 0, st>>>(f, C, pick<T>(m), pick3<T>(m), m->d_ncen3, m->d_cen3,
-                                                               m->d_nsec, m->d_sec, m->d_order, nv);
-    else
-        fv_coef3_kernel<T, 1, kFvMaxFaces><<<grid, kFvThreads, 0, st>>>(f, C, pick<T>(m), pick3<T>(m), m->d_ncen3,
-                                                                         m->d_cen3, m->d_nsec, m->d_sec, m->d_order,
-                                                                         nv);
-    return cudaGetLastError();
+FvIdx indices(const bz_mesh *m) {
+    return FvIdx{m->d_order, m->d_meta, m->d_fid, m->d_two, m->d_ncen, m->d_cen, m->d_nsec, m->d_sec};
 }
 
-template <typename T>
-cudaError_t flux3(const bz_mesh *m, const GridView &g, const T *f, const T *C, T *L, cudaStream_t st) {
-    if (m->n_cells <= 0) return cudaSuccess;
-    const int nv = (int)g.nv;
-    if (m->n_walls > 0) {
-        if (!fv_walls_supported(m, g)) return cudaErrorInvalidValue;
-        const T *wp = static_cast<const T *>(sizeof(T) == 8 ? static_cast<const void *>(m->d_wall64)
-                                                            : static_cast<const void *>(m->d_wall32));
-        const bool al = aligned16(f) && aligned16(C) && aligned16(L);
-        const unsigned grid = (unsigned)m->n_cells;
-        if (m->max_faces <= 3 && al)
-            fv_flux3_wall_kernel<T, 3, true><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m), m->d_nface,
-                                                                          m->d_nb, m->d_order, m->d_wall, wp, nv, g.N,
-                                                                          (T)g.L, (T)g.dv);
-        else if (m->max_faces <= 3)
-            fv_flux3_wall_kernel<T, 3, false><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m),
-                                                                           m->d_nface, m->d_nb, m->d_order, m->d_wall,
-                                                                           wp, nv, g.N, (T)g.L, (T)g.dv);
-        else if (al)
-            fv_flux3_wall_kernel<T, kFvMaxFaces, true><<<grid, kFvThreads, 0, st>>>(
-                f, C, L, pick<T>(m), pick3<T>(m), m->d_nface, m->d_nb, m->d_order, m->d_wall, wp, nv, g.N, (T)g.L,
-                (T)g.dv);
-        else
-            fv_flux3_wall_kernel<T, kFvMaxFaces, false><<<grid, kFvThreads, 0, st>>>(
-                f, C, L, pick<T>(m), pick3<T>(m), m->d_nface, m->d_nb, m->d_order, m->d_wall, wp, nv, g.N, (T)g.L,
-                (T)g.dv);
-        return cudaGetLastError();
-    }
-    const bool al = g.N % 4 == 0 && aligned16(f) && aligned16(C) && aligned16(L);
-    // polygons in FP32 also take 4 velocities per thread here (measured: 0.082 -> 0.064 ms on a
-    // 2603-cell Voronoi mesh; the reconstruction passes lose occupancy to registers and keep 1)
-    const bool v4 = m->max_faces <= 3 && al, p4 = m->max_faces > 3 && al && sizeof(T) == 4;
-    const int vec = (v4 || p4) ? 4 : 1;
-    const dim3 grid((unsigned)m->n_cells, (unsigned)((nv / vec + kFvThreads - 1) / kFvThreads));
-    if (v4)
-        fv_flux3_kernel<T, 4, 3><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m), m->d_nface, m->d_nb,
-                                                               m->d_order, nv, g.N, (T)g.L, (T)g.dv);
-    else if (m->max_faces <= 3)
-        fv_flux3_kernel<T, 1, 3><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m), m->d_nface, m->d_nb,
-                                                               m->d_order, nv, g.N, (T)g.L, (T)g.dv);
-    else if (p4) {
-        if constexpr (sizeof(T) == 4)
-            fv_flux3_kernel<T, 4, kFvMaxFaces><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m),
-                                                                             m->d_nface, m->d_nb, m->d_order, nv,
-                                                                             g.N, (T)g.L, (T)g.dv);
-    } else
-        fv_flux3_kernel<T, 1, kFvMaxFaces><<<grid, kFvThreads, 0, st>>>(f, C, L, pick<T>(m), pick3<T>(m),
-                                                                         m->d_nface, m->d_nb, m->d_order, nv, g.N,
-                                                                         (T)g.L, (T)g.dv);
-    return cudaGetLastError();
+int64_t flux_rows(const bz_mesh *m) { return m->n_faces_interior + m->n_faces_boundary; }
+
+dim3 cell_grid(const bz_mesh *m, int nv, int vec) {
+    return dim3((unsigned)m->n_cells, (unsigned)((nv / vec + kFvThreads - 1) / kFvThreads));
 }
 
-template <typename T, int VEC, int MAXS>
-void gradient_launch(const bz_mesh *m, int nv, const T *f, T *G, cudaStream_t st) {
-    const dim3 grid((unsigned)m->n_cells, (unsigned)((nv / VEC + kFvThreads - 1) / kFvThreads));
-    fv_gradient_kernel<T, VEC, MAXS><<<grid, kFvThreads, 0, st>>>(f, G, pick<T>(m), m->d_ncen, m->d_cen, m->d_nsec,
-                                                                  m->d_sec, m->d_order, nv);
-}
-
-template <typename T, bool kGrad, int VEC, int MAXF>
-void flux_launch(const bz_mesh *m, const GridView &g, const T *f, const T *G, T *L, cudaStream_t st) {
-    const int nv = (int)g.nv;
-    const dim3 grid((unsigned)m->n_cells, (unsigned)((nv / VEC + kFvThreads - 1) / kFvThreads));
-    fv_flux_kernel<T, kGrad, VEC, MAXF><<<grid, kFvThreads, 0, st>>>(f, G, L, pick<T>(m), m->d_nface, m->d_nb,
-                                                                     m->d_order, nv, g.N, (T)g.L, (T)g.dv);
-}
-
-// Triangle meshes with 16-byte aligned rows take 4 velocities per thread and
-// unrolled 3-face loops; other meshes one velocity per thread and 8-face loops.
-template <typename T>
-cudaError_t gradient(const bz_mesh *m, const GridView &g, const T *f, T *G, cudaStream_t st) {
-    if (m->n_cells <= 0) return cudaSuccess;
-    const int nv = (int)g.nv;
-    if (m->max_faces <= 3 && nv % 4 == 0 && aligned16(f) && aligned16(G))
-        gradient_launch<T, 4, 3>(m, nv, f, G, st);
-    else if (m->max_faces <= 3)
-        gradient_launch<T, 1, 3>(m, nv, f, G, st);
-    else
-        gradient_launch<T, 1, kFvMaxFaces>(m, nv, f, G, st);
-    return cudaGetLastError();
-}
-
-template <typename T, bool kGrad, int MAXF, bool VLOAD>
-void flux_wall_launch(const bz_mesh *m, const GridView &g, const T *f, const T *G, T *L, cudaStream_t st) {
-    const T *wp = static_cast<const T *>(sizeof(T) == 8 ? static_cast<const void *>(m->d_wall64)
-                                                        : static_cast<const void *>(m->d_wall32));
-    fv_flux_wall_kernel<T, kGrad, MAXF, VLOAD><<<(unsigned)m->n_cells, kFvThreads, 0, st>>>(
-        f, G, L, pick<T>(m), m->d_nface, m->d_nb, m->d_order, m->d_wall, wp, (int)g.nv, g.N, (T)g.L, (T)g.dv);
-}
-
-template <typename T>
-cudaError_t flux_walls(const bz_mesh *m, const GridView &g, const T *f, const T *G, T *L, cudaStream_t st) {
-    const bool al = aligned16(f) && aligned16(L) && (!G || aligned16(G));
-    const bool tri = m->max_faces <= 3;
-    if (G) {
-        if (tri && al) flux_wall_launch<T, true, 3, true>(m, g, f, G, L, st);
-        else if (tri) flux_wall_launch<T, true, 3, false>(m, g, f, G, L, st);
-        else if (al) flux_wall_launch<T, true, kFvMaxFaces, true>(m, g, f, G, L, st);
-        else flux_wall_launch<T, true, kFvMaxFaces, false>(m, g, f, G, L, st);
-    } else {
-        if (tri && al) flux_wall_launch<T, false, 3, true>(m, g, f, G, L, st);
-        else if (tri) flux_wall_launch<T, false, 3, false>(m, g, f, G, L, st);
-        else if (al) flux_wall_launch<T, false, kFvMaxFaces, true>(m, g, f, G, L, st);
-        else flux_wall_launch<T, false, kFvMaxFaces, false>(m, g, f, G, L, st);
-    }
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t flux(const bz_mesh *m, const GridView &g, const T *f, const T *G, T *L, cudaStream_t st) {
-    if (m->n_cells <= 0) return cudaSuccess;
-    if (m->n_walls > 0) {
-        if (!fv_walls_supported(m, g)) return cudaErrorInvalidValue;
-        return flux_walls<T>(m, g, f, G, L, st);
-    }
-    const bool tri = m->max_faces <= 3;
-    const bool v4 = tri && g.N % 4 == 0 && aligned16(f) && aligned16(L) && (!G || aligned16(G));
-    if (G) {
-        if (v4) flux_launch<T, true, 4, 3>(m, g, f, G, L, st);
-        else if (tri) flux_launch<T, true, 1, 3>(m, g, f, G, L, st);
-        else flux_launch<T, true, 1, kFvMaxFaces>(m, g, f, G, L, st);
-    } else {
-        if (v4) flux_launch<T, false, 4, 3>(m, g, f, G, L, st);
-        else if (tri) flux_launch<T, false, 1, 3>(m, g, f, G, L, st);
-        else flux_launch<T, false, 1, kFvMaxFaces>(m, g, f, G, L, st);
-    }
-    return cudaGetLastError();
-}
-
-}  // namespace
-
-bool fv_face_mode(const bz_mesh *m, const GridView &g, const void *f, const void *L, const void *FV) {
-    return m->order == 2 && m->max_faces <= 3 && m->d_tripos && m->n_walls == 0 && g.N % 4 == 0 && aligned16(f) &&
-           aligned16(L) &&
-           aligned16(FV);
-}
-
-static int fv_sm_count() {
+int fv_sm_count() {
     static std::atomic<int> cache[64];
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1391,26 +1212,139 @@ static int fv_sm_count() {
     return n;
 }
 
-// persistent grid: cps blocks per SM over the velocity blocks
-static dim3 faces_grid(const bz_mesh *m, int nv, int cps) {
+template <typename T, int VEC, int MAXF>
+void faces_launch(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaStream_t st) {
+    const int nv = (int)g.nv;
+    const dim3 grid = cell_grid(m, nv, VEC);
+    if (m->order == 3)
+        fv_faces_kernel<T, VEC, MAXF, kFvCoef3, kFvCentral3><<<grid, kFvThreads, 0, st>>>(
+            f, FX, pick<T>(m), indices(m), flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+    else
+        fv_faces_kernel<T, VEC, MAXF, 2, kFvCentral><<<grid, kFvThreads, 0, st>>>(
+            f, FX, pick<T>(m), indices(m), flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+}
+
+// persistent grid of the value passes: cps blocks per SM over the velocity blocks
+dim3 values_grid(const bz_mesh *m, int nv, int cps) {
     const int gy = (nv / 4 + kFvThreads - 1) / kFvThreads;
     const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(m->n_cells, (int64_t)fv_sm_count() * cps / gy));
     return dim3((unsigned)gx, (unsigned)gy);
 }
 
-cudaError_t launch_fv_faces_f32(const bz_mesh *m, const GridView &g, const float *f, float *FV, cudaStream_t st) {
+// FP64 takes one velocity per thread (the FP64 pipe is the bound, so loads per
+// velocity cost nothing); FP32 two, and four on triangles with 4 | N, as far
+// as the alignment of the caller's f allows (FX is the library's).
+template <typename T>
+cudaError_t faces(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
     const int nv = (int)g.nv;
-    fv_faces_persist_kernel<kFacesCtasPerSm><<<faces_grid(m, nv, kFacesCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
-        f, FV, m->t32, m->d_cen, m->d_nsec, m->d_sec, m->d_tripos, m->n_cells, nv);
+    const bool tri = m->max_faces <= 3;
+    if constexpr (sizeof(T) == 8) {
+        if (tri) faces_launch<T, 1, 3>(m, g, f, FX, st);
+        else faces_launch<T, 1, kFvMaxFaces>(m, g, f, FX, st);
+    } else {
+        if (tri && g.N % 4 == 0 && aligned(f, 16)) {
+            if (m->order == 3)
+                fv_faces3_tri_kernel<<<cell_grid(m, nv, 4), kFvThreads, 0, st>>>(
+                    f, FX, m->t32, indices(m), flux_rows(m), nv, g.N, (float)g.L, (float)g.dv);
+            else
+                fv_faces_kernel<T, 4, 3, 2, kFvCentral><<<cell_grid(m, nv, 4), kFvThreads, 0, st>>>(
+                    f, FX, m->t32, indices(m), flux_rows(m), nv, g.N, (float)g.L, (float)g.dv);
+        } else if (aligned(f, 8)) {
+            if (tri) faces_launch<T, 2, 3>(m, g, f, FX, st);
+            else faces_launch<T, 2, kFvMaxFaces>(m, g, f, FX, st);
+        } else {
+            if (tri) faces_launch<T, 1, 3>(m, g, f, FX, st);
+            else faces_launch<T, 1, kFvMaxFaces>(m, g, f, FX, st);
+        }
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && m->n_walls > 0) {
+        if (!fv_walls_supported(m, g)) return cudaErrorInvalidValue;
+        fv_wall_faces_kernel<T><<<(unsigned)m->n_walls, kFvThreads, 0, st>>>(
+            FX, pick<T>(m), m->d_fid, m->d_wall, m->d_wallslot, wall_params<T>(m), nv, g.N, (T)g.L, (T)g.dv);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+template <typename T, int VEC, int MAXF>
+void sum_launch(const bz_mesh *m, const GridView &g, const T *FX, T *L, cudaStream_t st) {
+    const int nv = (int)g.nv;
+    const dim3 grid = cell_grid(m, nv, VEC);
+    const int *wall = m->n_walls > 0 ? m->d_wall : nullptr;
+    if (m->order == 3)
+        fv_sum_kernel<T, VEC, MAXF, kFvCoef3><<<grid, kFvThreads, 0, st>>>(FX, L, pick<T>(m), indices(m), wall,
+                                                                           flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+    else
+        fv_sum_kernel<T, VEC, MAXF, 2><<<grid, kFvThreads, 0, st>>>(FX, L, pick<T>(m), indices(m), wall, flux_rows(m),
+                                                                    nv, g.N, (T)g.L, (T)g.dv);
+}
+
+// 16-byte rows where L allows (N^2 is a multiple of 4)
+template <typename T>
+cudaError_t sum(const bz_mesh *m, const GridView &g, const T *FX, T *L, cudaStream_t st) {
+    if (m->n_cells <= 0) return cudaSuccess;
+    constexpr int V = 16 / (int)sizeof(T);
+    const bool tri = m->max_faces <= 3, al = aligned(L, 16);
+    if (tri && al) sum_launch<T, V, 3>(m, g, FX, L, st);
+    else if (tri) sum_launch<T, 1, 3>(m, g, FX, L, st);
+    else if (al) sum_launch<T, V, kFvMaxFaces>(m, g, FX, L, st);
+    else sum_launch<T, 1, kFvMaxFaces>(m, g, FX, L, st);
     return cudaGetLastError();
 }
 
-cudaError_t launch_fv_flux_faces_f32(const bz_mesh *m, const GridView &g, const float *FV, float *L,
-                                     cudaStream_t st) {
+template <typename T, int VEC, int MAXF>
+void first_launch(const bz_mesh *m, const GridView &g, const T *f, T *L, cudaStream_t st) {
+    fv_first_kernel<T, VEC, MAXF><<<cell_grid(m, (int)g.nv, VEC), kFvThreads, 0, st>>>(
+        f, L, pick<T>(m), indices(m), m->d_nb, (int)g.nv, g.N, (T)g.L, (T)g.dv);
+}
+
+template <typename T>
+cudaError_t first(const bz_mesh *m, const GridView &g, const T *f, T *L, cudaStream_t st) {
+    if (m->n_cells <= 0) return cudaSuccess;
+    const bool tri = m->max_faces <= 3;
+    if (m->n_walls > 0) {
+        if (!fv_walls_supported(m, g)) return cudaErrorInvalidValue;
+        const unsigned grid = (unsigned)m->n_cells;
+        if (tri)
+            fv_first_wall_kernel<T, 3><<<grid, kFvThreads, 0, st>>>(f, L, pick<T>(m), indices(m), m->d_nb, m->d_wall,
+                                                                    wall_params<T>(m), (int)g.nv, g.N, (T)g.L, (T)g.dv);
+        else
+            fv_first_wall_kernel<T, kFvMaxFaces><<<grid, kFvThreads, 0, st>>>(
+                f, L, pick<T>(m), indices(m), m->d_nb, m->d_wall, wall_params<T>(m), (int)g.nv, g.N, (T)g.L, (T)g.dv);
+        return cudaGetLastError();
+    }
+    if (tri && g.N % 4 == 0 && aligned(f, 16) && aligned(L, 16)) first_launch<T, 4, 3>(m, g, f, L, st);
+    else if (tri) first_launch<T, 1, 3>(m, g, f, L, st);
+    else first_launch<T, 1, kFvMaxFaces>(m, g, f, L, st);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool fv_value_mode(const bz_mesh *m, const GridView &g, const void *f, const void *L) {
+    return m->d_tripos && m->n_walls == 0 && g.N % 4 == 0 && aligned(f, 16) && aligned(L, 16);
+}
+
+int64_t fv_scratch_rows(const bz_mesh *m, bool f32) {
+    if (m->order == 1) return 0;
+    const int64_t flux = flux_rows(m) + (f32 ? m->n_two * (m->order == 3 ? 4 : 2) : 0);
+    return f32 && m->d_tripos ? std::max<int64_t>(flux, 3 * m->n_cells) : flux;
+}
+
+cudaError_t launch_fv_values_f32(const bz_mesh *m, const GridView &g, const float *f, float *FV, cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
     const int nv = (int)g.nv;
-    fv_flux_faces_persist_kernel<<<faces_grid(m, nv, kFluxCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
+    fv_values_persist_kernel<<<values_grid(m, nv, kFacesCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
+        f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
+    return cudaGetLastError();
+}
+cudaError_t launch_fv_flux_values_f32(const bz_mesh *m, const GridView &g, const float *FV, float *L,
+                                      cudaStream_t st) {
+    if (m->n_cells <= 0) return cudaSuccess;
+    const int nv = (int)g.nv;
+    fv_flux_values_persist_kernel<<<values_grid(m, nv, kFluxCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
         FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
     return cudaGetLastError();
 }
@@ -1419,34 +1353,23 @@ bool fv_walls_supported(const bz_mesh *m, const GridView &g) {
     return m->n_walls == 0 || (g.N % 4 == 0 && g.nv <= 4 * kFvThreads);
 }
 
-cudaError_t launch_fv_gradient_f64(const bz_mesh *m, const GridView &g, const double *f, double *G, cudaStream_t st) {
-    return gradient<double>(m, g, f, G, st);
+cudaError_t launch_fv_first_f64(const bz_mesh *m, const GridView &g, const double *f, double *L, cudaStream_t st) {
+    return first<double>(m, g, f, L, st);
 }
-cudaError_t launch_fv_gradient_f32(const bz_mesh *m, const GridView &g, const float *f, float *G, cudaStream_t st) {
-    return gradient<float>(m, g, f, G, st);
+cudaError_t launch_fv_first_f32(const bz_mesh *m, const GridView &g, const float *f, float *L, cudaStream_t st) {
+    return first<float>(m, g, f, L, st);
 }
-cudaError_t launch_fv_flux_f64(const bz_mesh *m, const GridView &g, const double *f, const double *G, double *L,
-                               cudaStream_t st) {
-    return flux<double>(m, g, f, G, L, st);
+cudaError_t launch_fv_faces_f64(const bz_mesh *m, const GridView &g, const double *f, double *FX, cudaStream_t st) {
+    return faces<double>(m, g, f, FX, st);
 }
-cudaError_t launch_fv_flux_f32(const bz_mesh *m, const GridView &g, const float *f, const float *G, float *L,
-                               cudaStream_t st) {
-    return flux<float>(m, g, f, G, L, st);
+cudaError_t launch_fv_faces_f32(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
+    return faces<float>(m, g, f, FX, st);
 }
-
-cudaError_t launch_fv_coef3_f64(const bz_mesh *m, const GridView &g, const double *f, double *C, cudaStream_t st) {
-    return coef3<double>(m, g, f, C, st);
+cudaError_t launch_fv_sum_f64(const bz_mesh *m, const GridView &g, const double *FX, double *L, cudaStream_t st) {
+    return sum<double>(m, g, FX, L, st);
 }
-cudaError_t launch_fv_coef3_f32(const bz_mesh *m, const GridView &g, const float *f, float *C, cudaStream_t st) {
-    return coef3<float>(m, g, f, C, st);
-}
-cudaError_t launch_fv_flux3_f64(const bz_mesh *m, const GridView &g, const double *f, const double *C, double *L,
-                                cudaStream_t st) {
-    return flux3<double>(m, g, f, C, L, st);
-}
-cudaError_t launch_fv_flux3_f32(const bz_mesh *m, const GridView &g, const float *f, const float *C, float *L,
-                                cudaStream_t st) {
-    return flux3<float>(m, g, f, C, L, st);
+cudaError_t launch_fv_sum_f32(const bz_mesh *m, const GridView &g, const float *FX, float *L, cudaStream_t st) {
+    return sum<float>(m, g, FX, L, st);
 }
 
 }  // namespace bz
