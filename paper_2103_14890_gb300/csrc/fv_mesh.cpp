@@ -183,7 +183,6 @@ void fv_mesh_destroy(bz_mesh *m) {
     dev_free(m->d_sec);
     dev_free(m->d_order);
     dev_free(m->d_wall);
-    dev_free(m->d_wallslot);
     dev_free(m->d_wall64);
     dev_free(m->d_wall32);
     free(m->h_ptr);
@@ -679,7 +678,6 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
 
 static void drop_walls(bz_mesh *m) {
     dev_free(m->d_wall);
-    dev_free(m->d_wallslot);
     dev_free(m->d_wall64);
     dev_free(m->d_wall32);
     m->d_wall = nullptr;
@@ -722,8 +720,11 @@ int fv_mesh_set_walls(bz_mesh *m, int64_t n_edges, const int64_t *edges, const d
     }
     std::vector<float> p32(p64.size());
     for (size_t q = 0; q < p64.size(); ++q) p32[q] = (float)p64[q];
+    // the slots follow the per-face table in one block
+    wall.resize(wall.size() + 2 * slot.size());
+    memcpy(wall.data() + (size_t)n * kFvMaxFaces, slot.data(), sizeof(int64_t) * slot.size());
     cudaError_t err = upload(&m->d_wall, wall);
-    if (err == cudaSuccess) err = upload(&m->d_wallslot, slot);
+    if (err == cudaSuccess) m->d_wallslot = reinterpret_cast<int64_t *>(m->d_wall + n * kFvMaxFaces);
     if (err == cudaSuccess) err = upload(&m->d_wall64, p64);
     if (err == cudaSuccess) err = upload(&m->d_wall32, p32);
     if (err != cudaSuccess) {
