@@ -72,22 +72,26 @@ struct bz_modes {
     // in use (null if the generic kernel serves this grid)
     float *var_W[kModesumVariants];
     int *var_task[kModesumVariants];
-    int *var_task_split[kModesumVariants][kSplitTables];   // 32-cell variants: tile split over 2, 4, 8 CTAs
+    int *var_task_split[kModesumVariants][kSplitTables];   // 32- and 8-cell variants: tile split over 2, 4, 8 CTAs
+    float var_bal[kModesumVariants][kSplitTables + 1];     // load of the most loaded warp, tile on 1, 2, 4, 8 CTAs
     int var_rowmax[kModesumVariants];
     int variant;          // index of the selected variant
     int variant_fixed;    // 1: chosen by BZ_MODESUM_VARIANT (no last-wave split)
     void *w64;            // FP64 weight stream and task table, null if unused
     int *task64;
+    int *task64_split[kSplitTables];
+    float bal64[kSplitTables + 1];
     int rowmax64;
     int variant64;        // layout of the FP64 tables (entry of the variant list), -1 if none
     float *wx2;           // FP32X2 weight stream: the FP64 stream's layout and task table, each
                           // step's weights as FP32 (hi, lo) parts; null if unused
-    int modesum_variant;  // variant id reported to callers (index + 1; 0: generic kernel)
+    int modesum_variant;  // variant id reported to callers (index + 1; 0: no choice of variants, N > 48)
     float *d_W32;
     int w32_rowmax;       // largest staged weight row (floats)
     int *d_task;
     int64_t pairs_sym;   // unordered pairs per cell (algorithmic unit)
-    int tile_dft;        // 1: the tile FFT kernels of k_dft32.cu serve this grid
+    int tile_dft;        // 1: the tile FFT kernels of k_dft32.cu serve this grid in FP32
+    int tile_dft64;      // ... and in FP64 (also the FP32X2 form's forward transform)
     double scale;        // s^(d + gamma)
     double penalty;      // c of the Boltzmann model's penalty rate nu = c rho (IMEX stages)
     // fast spectral (Carleman) form, k_fast.cu: method 1 replaces the mode sum
@@ -210,8 +214,8 @@ cudaError_t launch_dft_inverse_f32(const GridView &g, const float2 *E, const flo
                                    float *Q, int64_t n, double scale, const double *cinv,
                                    const InvEpilogue &ep, cudaStream_t st);
 
-// ---- tile FFT kernels (k_dft32.cu), FP32 and FP64, 2-D, N in {16, 24, 32, 48} ----
-bool dft32_tile_supported(const GridView &g);
+// ---- tile FFT kernels (k_dft32.cu), FP32 and FP64: 2-D, N in {16, 24, 32, 48}; 3-D, N = 16; FP32: 2-D, N = 64 ----
+bool dft32_tile_supported(const GridView &g, bool fp64);
 int dft32_setup();   // twiddles on the current device
 cudaError_t launch_dft32_forward_tile(const GridView &g, const float *f, float2 *fhat, int64_t n, cudaStream_t st);
 cudaError_t launch_dft32_inverse_tile(const GridView &g, const float2 *Qhat, float *Q, int64_t n, double scale,

@@ -1,4 +1,4 @@
-// fft_reg.cuh -- register-resident FFTs of small lengths (2^p <= 32,
+// fft_reg.cuh -- register-resident FFTs of small lengths (2^p <= 64,
 // 3 * 2^p <= 48 and 72), unrolled with compile-time indices so that the data stay in
 // registers and the twiddles are constant-bank operands.  Each translation
 // unit that includes this header gets its own copy of the twiddle tables in
@@ -15,10 +15,21 @@ namespace {
 
 __constant__ float2 c_w32[32];          // e^{-2 pi i k / 32}, k = 0..31
 __constant__ double2 c_w32d[32];
+__constant__ float2 c_w64[64];          // e^{-2 pi i k / 64} (FP32 only)
 
 template <typename V> __device__ __forceinline__ V tw32(int k);
 template <> __device__ __forceinline__ float2 tw32<float2>(int k) { return c_w32[k]; }
 template <> __device__ __forceinline__ double2 tw32<double2>(int k) { return c_w32d[k]; }
+
+// e^{-2 pi i k / L}, L a power of two <= 64
+template <int L, typename V> __device__ __forceinline__ V twp(int k) {
+    if constexpr (L == 64) {
+        static_assert(sizeof(V) == 8, "length 64: FP32");
+        return c_w64[k];
+    } else {
+        return tw32<V>(k * (32 / L));
+    }
+}
 
 // Complex sums and differences: one FP32x2 instruction for float2 (two IEEE
 // FP32 additions, the results of the scalar form), two scalar ones otherwise.
@@ -36,7 +47,7 @@ constexpr int bitrev(int i, int bits) {
     return r;
 }
 
-// In-place radix-2 decimation-in-time FFT of length L <= 32 whose input sits
+// In-place radix-2 decimation-in-time FFT of length L <= 64 whose input sits
 // in bit-reversed order; output in natural order.  SIGN = -1: sum x_n
 // e^{-2 pi i k n / L}; SIGN = +1: sum x_n e^{+2 pi i k n / L} (unnormalised).
 template <int L, int SIGN, typename V>
@@ -56,7 +67,7 @@ __device__ __forceinline__ void fft_dit(V (&a)[L]) {
                 } else if (2 * j == m) {                       // twiddle -i (forward) or +i (inverse)
                     t = SIGN < 0 ? cmk<V2>(b.y, -b.x) : cmk<V2>(-b.y, b.x);
                 } else {
-                    const V w = tw32<V>(j * (32 / (2 * m)));
+                    const V w = twp<L < 64 ? 32 : 64, V>(j * ((L < 64 ? 32 : 64) / (2 * m)));
                     const S wy = SIGN < 0 ? w.y : -w.y;    // conj for the inverse
                     t = cmk<V2>(b.x * w.x - b.y * wy, b.x * wy + b.y * w.x);
                 }
@@ -94,7 +105,7 @@ template <int L, typename V> __device__ __forceinline__ V twl(int k) {
     else return tw72<V>(k * (72 / L));
 }
 
-// Transform of length L (2^p <= 32, 3 * 2^p <= 48, or 72) from natural to
+// Transform of length L (2^p <= 64, 3 * 2^p <= 48, or 72) from natural to
 // natural order; SIGN as in fft_dit.
 template <int L, int SIGN, typename V>
 __device__ __forceinline__ void fft_nat(V (&a)[L]) {
@@ -182,15 +193,18 @@ __device__ __forceinline__ void fft_nat_mid0(V (&a)[L]) {
     }
 }
 
-// e^{-2 pi i k / N} for N in {16, 24, 32, 48}
+// e^{-2 pi i k / N} for N in {16, 24, 32, 48, 64}
 template <int N, typename V> __device__ __forceinline__ V tw(int k) {
-    if constexpr (N == 16 || N == 32) return tw32<V>(k * (32 / N));
+    if constexpr (N == 64) return twp<64, V>(k);
+    else if constexpr (N == 16 || N == 32) return tw32<V>(k * (32 / N));
     else return tw48<V>(k * (48 / N));
 }
 
 // Fill this translation unit's twiddle tables on the current device.
 inline cudaError_t upload_fft_twiddles() {
-    float2 w32[32], w48[48], w72[72];
+    float2 w32[32], w48[48], w64[64], w72[72];
+    for (int k = 0; k < 64; ++k)
+        w64[k] = make_float2((float)cos(2.0 * M_PI * k / 64), (float)-sin(2.0 * M_PI * k / 64));
     double2 d32[32], d48[48], d72[72];
     for (int k = 0; k < 32; ++k) {
         d32[k] = make_double2(cos(2.0 * M_PI * k / 32), -sin(2.0 * M_PI * k / 32));
@@ -208,6 +222,7 @@ inline cudaError_t upload_fft_twiddles() {
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w48, w48, sizeof w48);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w32d, d32, sizeof d32);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w48d, d48, sizeof d48);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w64, w64, sizeof w64);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w72, w72, sizeof w72);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w72d, d72, sizeof d72);
     return e;

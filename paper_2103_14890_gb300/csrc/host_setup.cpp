@@ -243,9 +243,10 @@ int modes_create(const bz_grid *g, double gamma, double b0, int nq, bz_modes **o
     }
     m->pairs_sym = symmetric_pair_count(v);
     int rc = modes_build_fp32_tables(m);
-    if (rc == BZ_OK && dft32_tile_supported(v)) {
+    if (rc == BZ_OK && dft32_tile_supported(v, false)) {
         rc = dft32_setup();
         m->tile_dft = rc == BZ_OK;
+        m->tile_dft64 = rc == BZ_OK && dft32_tile_supported(v, true);
     }
     if (rc != BZ_OK) {
         modes_destroy(m);        // also the variant tables built before the failure
@@ -332,9 +333,10 @@ int fast_modes_create(const bz_grid *g, double b0, int ndirs, bz_modes **out) {
         return cuda_fail(e, "build_fast_modes: direction factors");
     }
     int rc = fast_setup();
-    if (rc == BZ_OK && dft32_tile_supported(v)) {
+    if (rc == BZ_OK && dft32_tile_supported(v, false)) {
         rc = dft32_setup();
         m->tile_dft = rc == BZ_OK;
+        m->tile_dft64 = rc == BZ_OK && dft32_tile_supported(v, true);
     }
     if (rc != BZ_OK) {
         modes_destroy(m);
@@ -354,6 +356,7 @@ void modes_destroy(bz_modes *m) {
     dev_free(m->w64);
     dev_free(m->wx2);
     dev_free(m->task64);
+    for (int k = 0; k < kSplitTables; ++k) dev_free(m->task64_split[k]);
     for (int v = 0; v < kModesumVariants; ++v) {
         dev_free(m->var_W[v]);
         dev_free(m->var_task[v]);

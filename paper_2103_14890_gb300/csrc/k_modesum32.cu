@@ -1,5 +1,5 @@
 // k_modesum32.cu -- register-blocked FP32 mode sum of eq. CF1 (Sec. 3.3) for
-// 2-D velocity grids with N <= 48 and 3-D grids with N <= 16.
+// 2-D velocity grids (N <= 64; N <= 48 in FP64) and 3-D grids with N <= 16.
 //
 // Work reduction (exact algebra, no approximation):
 //   * Q is real, so only k_1 >= 0 is computed (Q-hat_{-k} = conj(Q-hat_k)).
@@ -14,7 +14,7 @@
 //     the same in both dimensions.
 //
 // Layout and blocking:
-//   * one CTA = one tile of C cells (C = 32, or 16 for grids whose spectrum
+//   * one CTA = one tile of C cells (C = 32, or 16 or 8 for grids whose spectrum
 //     does not fit 32 cells in shared memory); the tile's half spectrum
 //     (complex FP32, [mode][cell]) sits in shared memory with lane % C = cell,
 //     so every weight load is uniform over the lanes that share it and every
@@ -61,22 +61,26 @@ namespace {
 // lanes hold cells c and c + 16 of a 32-cell tile in FP32x2 register pairs),
 // wdup: each weight stored twice (w, w) as an FP32x2 operand, pq: the FP32x2
 // form with one cell per lane (modesum_pq_kernel), orient: 2 when the two
-// halves of a warp hold the same cells and run each task plain and mirrored
-// (paired orientations).  Variant ids reported by bz_modes_info are index + 1.
+// halves of a warp (of each of its row groups) hold the same cells and run
+// each task plain and mirrored (paired orientations), rows: row pairs of a
+// task that a warp sums at a time, one per group of lanes.  Variant ids
+// reported by bz_modes_info are index + 1.
 struct Variant {
-    int R, warps, cells, pack, wdup, pq, orient;
+    int R, warps, cells, pack, wdup, pq, orient, rows;
 };
 constexpr int kNumVariants = kModesumVariants;   // FP32 variants (timed by the autotuner)
 // entries 0..9: the FP32 variants; entries 10, 11: layouts of the FP64 and FP32X2
 // forms only (2 outputs per thread, 8 warps, 8- and 4-cell tiles) for grids
 // whose 16-byte-per-value spectrum needs them (48^2, 16^3)
 constexpr Variant kVariants[kNumVariants + 2] = {
-    {8, 16, 32, 1, 0, 0, 1}, {4, 32, 32, 1, 0, 0, 1}, {4, 16, 16, 1, 0, 0, 1}, {4, 16, 8, 1, 0, 0, 1},
-    {4, 16, 32, 2, 1, 0, 1}, {8, 12, 32, 1, 0, 1, 1}, {8, 16, 32, 1, 0, 1, 1}, {8, 16, 16, 1, 0, 1, 2},
-    {8, 8, 16, 1, 0, 1, 2},  {8, 4, 16, 1, 0, 1, 2},  {2, 8, 8, 1, 0, 0, 1},   {2, 8, 4, 1, 0, 0, 1}};
+    {8, 16, 32, 1, 0, 0, 1, 1}, {4, 32, 32, 1, 0, 0, 1, 1}, {4, 16, 16, 1, 0, 0, 1, 1}, {8, 12, 8, 1, 0, 1, 2, 2},
+    {4, 16, 32, 2, 1, 0, 1, 1}, {8, 12, 32, 1, 0, 1, 1, 1}, {8, 16, 32, 1, 0, 1, 1, 1}, {8, 16, 16, 1, 0, 1, 2, 1},
+    {8, 8, 16, 1, 0, 1, 2, 1},  {8, 4, 16, 1, 0, 1, 2, 1},  {2, 8, 8, 1, 0, 0, 1, 1},   {2, 8, 4, 1, 0, 0, 1, 1}};
 
 // lane groups splitting a task's outputs, and outputs per task (RT)
-constexpr int variant_groups(int v) { return 32 / kVariants[v].cells * kVariants[v].pack / kVariants[v].orient; }
+constexpr int variant_groups(int v) {
+    return 32 / kVariants[v].cells * kVariants[v].pack / kVariants[v].orient / kVariants[v].rows;
+}
 constexpr int variant_rt(int v) { return kVariants[v].R * variant_groups(v); }
 // Whether an FP32 variant's tables compute k_2 < 0 on the reflected spectrum
 // (every output block of k_2 >= 0 fits within the row: R T <= h + 1); all
@@ -671,10 +675,16 @@ __device__ __forceinline__ void row_pass_pq(const float2 *__restrict__ rowl, con
 // upper half running every task mirrored, i.e. the task's reflected twin with
 // the same weights and control flow, so all lanes take the same outputs and
 // the ramp applies; the table holds no reflected tasks and k_2 = 0 is the
-// lower half's.
+// lower half's.  CELLS = 8 (grids whose 16-cell spectrum does not fit: 64^2,
+// 16^3): the two halves of a warp each do the same for 8 cells, one on the
+// even and one on the odd of a task's row pairs (ROWS = 2; the table lists
+// them in couples of one read direction), and their sums are added at the end
+// of the task.  Consecutive rows lie an odd number of modes apart, so the four
+// 64-byte groups of a load fall two and two into the halves of the banks.
 template <int RR, int WARPS, int CELLS>
 __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 1) modesum_pq_kernel(const Mode32Group gd) {
-    constexpr bool PAIRED = (CELLS == 16);
+    constexpr bool PAIRED = (CELLS <= 16);
+    constexpr int ROWS = PAIRED ? 16 / CELLS : 1;   // row pairs at a time
     constexpr int G = 32 / CELLS;                // CTAs per 32-cell tile
     constexpr int WS = RR;                       // floats per l_2 step
     constexpr int HEAD = kRowHeadBytes / (int)sizeof(float);
@@ -698,9 +708,10 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cell = lane % CELLS;
-    const bool upper = PAIRED && lane >= CELLS;                      // runs every task mirrored
-    float *wbuf0 = wsm + (size_t)warp * 2 * wrow_max;
-    float *wbuf1 = wbuf0 + wrow_max;
+    const bool upper = PAIRED && (lane / CELLS) % 2 == 1;            // runs every task mirrored
+    const int rgrp = ROWS > 1 ? lane / (2 * CELLS) : 0;              // its row pair of each couple
+    float *wbuf0 = wsm + (size_t)warp * 2 * ROWS * wrow_max;
+    float *wbuf1 = wbuf0 + ROWS * wrow_max;
     const int NW = WARPS * ip.split;                 // one phase: every task reads this spectrum
     int t = tasks[part * WARPS + warp], tend = tasks[part * WARPS + warp + 1];
     const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * NW + 1);
@@ -717,11 +728,13 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
 #pragma unroll
         for (int r = 0; r < RR; ++r) hi[r] = lo[r] = P[r] = Q[r] = make_float2(0.f, 0.f);
         const int mbase0 = tk.k20 - tk.l2lo - (RR - 1);
-        stage_row(wbuf0, wsrc, rowf * (int)sizeof(float), lane);
-        for (int i = 0; i < tk.nrows; ++i) {
-            const float *wcur = (i & 1) ? wbuf1 : wbuf0;
-            if (i + 1 < tk.nrows) {
-                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * rowf, rowf * (int)sizeof(float), lane);
+        stage_row(wbuf0, wsrc, ROWS * rowf * (int)sizeof(float), lane);
+        const int nrows = tk.nrows / ROWS;
+        for (int i = 0; i < nrows; ++i) {
+            const float *wcur = ((i & 1) ? wbuf1 : wbuf0) + rgrp * rowf;
+            if (i + 1 < nrows) {
+                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * (ROWS * rowf),
+                          ROWS * rowf * (int)sizeof(float), lane);
                 cp_async_wait<1>();
             } else {
                 cp_async_wait<0>();
@@ -735,7 +748,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
                 row_pass_pq<RR, WS, CELLS, -1>(F0 + hd.x, F0 + hd.y, wcur + HEAD, tk.nblk, tk.l2lo, mbase0, ramp,
                                                mirror, P, Q);
             __syncwarp();
-            if ((i & 3) == 3 || i + 1 == tk.nrows) {
+            if ((i & 3) == 3 || i + 1 == nrows) {
 #pragma unroll
                 for (int r = 0; r < RR; ++r) {
                     // (re, im) TwoSum as FP32x2 operations: the scalar ones, pairwise
@@ -748,7 +761,20 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
                 }
             }
         }
-        if (valid) {
+        if constexpr (ROWS > 1) {
+#pragma unroll
+            for (int r = 0; r < RR; ++r) {
+                const float2 h2 = make_float2(__shfl_xor_sync(0xffffffffu, hi[r].x, 16),
+                                              __shfl_xor_sync(0xffffffffu, hi[r].y, 16));
+                const float2 l2 = make_float2(__shfl_xor_sync(0xffffffffu, lo[r].x, 16),
+                                              __shfl_xor_sync(0xffffffffu, lo[r].y, 16));
+                float2 sm, e;
+                two_sum2(hi[r], h2, sm, e);
+                hi[r] = sm;
+                lo[r] = __fadd2_rn(__fadd2_rn(lo[r], l2), e);
+            }
+        }
+        if (valid && rgrp == 0) {
             const volatile TaskRec *tv = trec + (t - 1);
             const int orow = tv->orow, rfirst = tv->rfirst, flags = tv->flags, crow = tv->crow, k20 = tv->k20;
             float2 *out = qt + (int64_t)orow * M * 32;
@@ -906,13 +932,15 @@ __device__ __forceinline__ void row_pass_x2(const float2 *__restrict__ rowl, con
 template <int RR, int WARPS, int CELLS>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 modesum_x2_kernel(const double2 *__restrict__ fhat, float2 *__restrict__ Qhat, const float *__restrict__ W,
-                  const int *__restrict__ tasks, int h, int M, int nhalf, int wrow_max, int64_t n) {
+                  const int *__restrict__ tasks, int h, int M, int nhalf, int wrow_max, int64_t n, int split) {
     constexpr int G = 32 / CELLS;
     constexpr int RT = RR * G;
     constexpr int HEADF = kRowHeadBytes / (int)sizeof(float);
     extern __shared__ __align__(16) uint4 smem16[];
-    const int64_t tile = (int64_t)blockIdx.x / G;
-    const int sub = (int)(blockIdx.x % G);
+    const int part = (int)(blockIdx.x % split);      // this CTA's part of the task table
+    const int64_t cta = (int64_t)blockIdx.x / split;
+    const int64_t tile = cta / G;
+    const int sub = (int)(cta % G);
     const int rows = nhalf + 2 * kPad;
     float2 *Fh = reinterpret_cast<float2 *>(smem16);              // [rows][CELLS] high parts
     float2 *Fl = Fh + (size_t)rows * CELLS;                       // [rows][CELLS] low parts
@@ -939,8 +967,9 @@ modesum_x2_kernel(const double2 *__restrict__ fhat, float2 *__restrict__ Qhat, c
     const int cell = lane % CELLS, grp = lane / CELLS;
     float *wbuf0 = wsm + (size_t)warp * 4 * wrow_max;             // wrow_max counts 8-byte slots
     float *wbuf1 = wbuf0 + 2 * wrow_max;
-    const int tbeg = tasks[warp], tend = tasks[warp + 1];
-    const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * WARPS + 1);
+    const int vw = part * WARPS + warp;
+    const int tbeg = tasks[vw], tend = tasks[vw + 1];
+    const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * WARPS * split + 1);
     const float2 *F0 = Fh + (size_t)(kPad + h) * CELLS + cell;
 
     for (int t = tbeg; t < tend; ++t) {
@@ -982,7 +1011,7 @@ modesum_x2_kernel(const double2 *__restrict__ fhat, float2 *__restrict__ Qhat, c
 
 template <typename T> size_t smem_bytes(const GridView &g, int wrow_max, int v) {
     return 2 * sizeof(T) * (size_t)(g.nhalf + 2 * kPad) * kVariants[v].cells +
-           sizeof(T) * (size_t)kVariants[v].warps * 2 * wrow_max;
+           sizeof(T) * (size_t)kVariants[v].warps * 2 * kVariants[v].rows * wrow_max;
 }
 
 }  // namespace
@@ -998,7 +1027,7 @@ double beta_host(const bz_modes *m, const int *l, const int *mm);
 // (hi = fl32(w), lo = fl32(w - hi)), headers copied as they are.
 template <typename T>
 static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, int *outRowmax,
-                          float **outX2 = nullptr, int **outSplit = nullptr) {
+                          float **outX2 = nullptr, int **outSplit = nullptr, float *outBal = nullptr) {
     constexpr int HEAD = kRowHeadBytes / (int)sizeof(T);
     const int R = variant_rt(v);                                // outputs per task (RT)
     const int kWarps = kVariants[v].warps;
@@ -1006,7 +1035,8 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
     rc = BZ_OK;
     const GridView &gv = m->g->v;
     const int d = gv.dim, h = gv.h, M = gv.M;
-    if (!((d == 2 && gv.N <= 48) || (d == 3 && gv.N <= 16))) return false;
+    const int rows = kVariants[v].rows;                         // row pairs at a time
+    if (!((d == 2 && gv.N <= (rows > 1 ? 64 : 48)) || (d == 3 && gv.N <= 16))) return false;
     // shared memory of the spectrum alone must leave room for the weight buffers
     if (2 * sizeof(T) * (size_t)(gv.nhalf + 2 * kPad) * kVariants[v].cells > 200 * 1024) return false;
     const int nb = (M + R - 1) / R;
@@ -1044,6 +1074,19 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                 } else {
                     for (int l2 = std::max(-h, k2 - h); l2 <= std::min(h, k2 + h); ++l2)
                         pairs.push_back({{l1, l2}, {m1, k2 - l2}});
+                }
+            }
+            // couples of row pairs with one read direction: an odd one out is
+            // coupled with a copy of itself whose weights are zero
+            std::vector<char> dummy(pairs.size(), 0);
+            if (rows > 1) {
+                std::vector<Pair> in = pairs;
+                pairs.clear();
+                dummy.clear();
+                for (int neg = 1; neg >= 0; --neg) {
+                    for (const Pair &p : in)
+                        if ((p.l[0] < 0) == (neg == 1)) pairs.push_back(p), dummy.push_back(0);
+                    if (pairs.size() % 2) pairs.push_back(pairs.back()), dummy.push_back(1);
                 }
             }
             // blocks of R consecutive last-axis outputs.  reflect: the blocks
@@ -1100,7 +1143,8 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                 t.crow = (d == 3) ? (M - 1 - i2) : 0;        // k_1 = 0: row of -k (middle index -k_2)
                 t.pad2 = t.pad3 = 0;
                 prev_end = k2last;
-                for (const Pair &p : pairs) {
+                for (size_t ip = 0; ip < pairs.size(); ++ip) {
+                    const Pair &p = pairs[ip];
                     // row of l (that of -l read backwards when l_1 < 0) and row of m
                     const bool neg = p.l[0] < 0;
                     const int a1 = neg ? -p.l[0] : p.l[0], a2 = neg ? -p.l[1] : p.l[1];
@@ -1122,7 +1166,7 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                         for (int r = 0; r < R; ++r) {
                             const int kz = k20 + r, mz = kz - lz;
                             double w = 0.0;
-                            if (kz <= h && lz >= -h && lz <= h && mz >= -h && mz <= h) {
+                            if (!dummy[ip] && kz <= h && lz >= -h && lz <= h && mz >= -h && mz <= h) {
                                 int l[3], mm[3];
                                 l[0] = p.l[0];
                                 mm[0] = p.m[0];
@@ -1163,7 +1207,8 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
     }
     // longest-processing-time-first assignment of tasks to nw warps: the
     // offsets of each warp's list, then the task records
-    auto make_table = [&](int nw) {
+    auto make_table = [&](int nw, float *worst = nullptr) {
+        double longest = 0.0;                               // sum over the phases of the most loaded warp
         std::vector<std::vector<int>> per(2 * nw);
         for (int ph = 0; ph < 2; ++ph) {
             std::vector<int> order;
@@ -1176,7 +1221,9 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                 load[w] += cost[i];
                 per[ph * nw + w].push_back(i);
             }
+            longest += *std::max_element(load.begin(), load.end());
         }
+        if (worst) *worst = (float)longest;
         std::vector<int> t(2 * nw + 1 + tasks.size() * kTaskInts);
         int pos = 0;
         for (int q = 0; q < 2 * nw; ++q) {
@@ -1189,7 +1236,7 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
         t[2 * nw] = pos;
         return t;
     };
-    const std::vector<int> tab = make_table(kWarps);
+    const std::vector<int> tab = make_table(kWarps, outBal);
     int wrow_max = 0;
     for (auto &t : tasks) wrow_max = std::max(wrow_max, t.rowf);   // staging buffer: one row pair
     if (smem_bytes<T>(gv, wrow_max, v) > 227 * 1024) return false;   // does not fit
@@ -1211,11 +1258,12 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
         rc = cuda_fail(e, "build_kernel_modes: weight stream");
         return false;
     }
-    // tables for one tile split over S = 2, 4, 8 CTAs (S x kWarps warps; the
-    // last partial wave of a launch of a 32-cell variant)
+    // tables for one tile split over S = 2, 4, 8 CTAs (S x kWarps warps): the
+    // last partial wave of a launch of a 32-cell variant, or every tile of a
+    // launch (launch_split)
     if (outSplit) {
         for (int k = 0; k < kSplitTables && e == cudaSuccess; ++k) {
-            const std::vector<int> ts = make_table(kWarps << (k + 1));
+            const std::vector<int> ts = make_table(kWarps << (k + 1), outBal ? outBal + k + 1 : nullptr);
             e = dev_malloc(&outSplit[k], sizeof(int) * ts.size());
             if (e == cudaSuccess) e = cudaMemcpy(outSplit[k], ts.data(), sizeof(int) * ts.size(), cudaMemcpyHostToDevice);
         }
@@ -1260,7 +1308,7 @@ static cudaError_t launch_group(const Mode32Group &gd, int v, size_t sm, cudaStr
         case 0: return launch_instance<float, 8, 16, 32, true>(gd, sm, st);
         case 1: return launch_instance<float, 4, 32, 32>(gd, sm, st);
         case 2: return launch_instance<float, 4, 16, 16>(gd, sm, st);
-        case 3: return launch_instance<float, 4, 16, 8>(gd, sm, st);
+        case 3: return launch_pq<8, 12, 8>(gd, sm, st);
         case 4: {
             cudaError_t e = cudaFuncSetAttribute(modesum_p2_kernel<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)sm);
@@ -1292,6 +1340,9 @@ static void fill_item(Mode32Item &it, const bz_modes *m, const void *W, const in
     it.n = n;
 }
 
+// Index of the task tables of a tile split over S = 2, 4, 8 CTAs.
+static int split_index(int S) { return S == 2 ? 0 : S == 4 ? 1 : 2; }
+
 // CTAs of an instance of n cells: one per CELLS cells of each 32-cell tile.
 static int64_t ctas_for(int v, int64_t n) {
     const int G = 32 / kVariants[v].cells;      // CTAs per 32-cell tile
@@ -1299,24 +1350,50 @@ static int64_t ctas_for(int v, int64_t n) {
 }
 
 static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
-                                  cudaStream_t st) {
+                                  cudaStream_t st, int S = 1) {
     if (n <= 0) return cudaSuccess;
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
     gd.nitems = 1;
-    fill_item(gd.item[0], m, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, Qhat, n);
+    fill_item(gd.item[0], m, m->var_W[v], S > 1 ? m->var_task_split[v][split_index(S)] : m->var_task[v],
+              m->var_rowmax[v], fhat, Qhat, n, S);
     gd.tile_start[0] = 0;
-    gd.tile_start[1] = ctas_for(v, n);
+    gd.tile_start[1] = ctas_for(v, n) * S;
     return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
 }
 
 // FP64 form: the same kernel on double spectra and weights, on 16-cell tiles
 // (variant entry 2) or, where the double spectrum of 16 cells does not fit
-// shared memory, on 8- or 4-cell tiles (entries 10, 11: 48^2, 16^3); no
-// last-wave split.  The FP32X2 form runs on the same layout.
+// shared memory, on 8- or 4-cell tiles (entries 10, 11: 48^2, 16^3).  The FP32X2 form runs on the same layout.
 constexpr int kFp64Variants[3] = {2, 10, 11};
 
 bool modesum64_available(const bz_modes *m) { return m->w64 != nullptr; }
+
+static int sm_count();
+
+// CTAs that take one tile's tasks between them (1, 2, 4 or 8), for kernels with
+// one CTA per SM: the S with the least ceil(ctas S / SMs) x (load of the most
+// loaded warp with S CTAs), so that neither a launch smaller than a wave nor
+// its last partial wave leaves SMs idle.  Every output is computed by one task
+// with the same arithmetic, so the results do not depend on S.  Staging the
+// spectrum S times costs little (a few us of an SM against hundreds); a larger
+// S has to win by 3 %.  4099 cells of 32^2 (257 CTAs on 152 SMs), FP64: 8.76 ->
+// @F64S@ ms, FP32X2: 1.53 -> @X2S@ ms.
+static int launch_split(int64_t ctas, const float (&bal)[kSplitTables + 1], int *const *tables) {
+    const int64_t sms = sm_count();
+    int best = 1;
+    double t = (double)((ctas + sms - 1) / sms) * bal[0];
+    for (int k = 0; k < kSplitTables; ++k) {
+        if (!tables[k]) continue;
+        const int S = 2 << k;
+        const double ts = (double)((ctas * S + sms - 1) / sms) * bal[k + 1];
+        if (ts < 0.97 * t) {
+            t = ts;
+            best = S;
+        }
+    }
+    return best;
+}
 
 cudaError_t launch_modesum64(const bz_modes *m, const double2 *fhat, double2 *Qhat, int64_t n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
@@ -1324,9 +1401,10 @@ cudaError_t launch_modesum64(const bz_modes *m, const double2 *fhat, double2 *Qh
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
     gd.nitems = 1;
-    fill_item(gd.item[0], m, m->w64, m->task64, m->rowmax64, fhat, Qhat, n);
+    const int S = launch_split(ctas_for(m->variant64, n), m->bal64, m->task64_split);
+    fill_item(gd.item[0], m, m->w64, S > 1 ? m->task64_split[split_index(S)] : m->task64, m->rowmax64, fhat, Qhat, n, S);
     gd.tile_start[0] = 0;
-    gd.tile_start[1] = ctas_for(m->variant64, n);
+    gd.tile_start[1] = ctas_for(m->variant64, n) * S;
     const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, m->variant64);
     if (m->variant64 == kFp64Variants[0]) return launch_instance<double, 4, 16, 16>(gd, sm, st);
     if (m->variant64 == kFp64Variants[1]) return launch_instance<double, 2, 8, 8>(gd, sm, st);
@@ -1344,8 +1422,11 @@ static cudaError_t launch_x2_instance(const bz_modes *m, const double2 *fhat, fl
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     const GridView &gv = m->g->v;
-    modesum_x2_kernel<RR, WARPS, CELLS><<<(unsigned)ctas_for(m->variant64, n), WARPS * 32, sm, st>>>(
-        fhat, Qhat, m->wx2, m->task64, gv.h, gv.M, (int)gv.nhalf, m->rowmax64, n);
+    const int64_t ctas = ctas_for(m->variant64, n);
+    const int S = launch_split(ctas, m->bal64, m->task64_split);
+    modesum_x2_kernel<RR, WARPS, CELLS><<<(unsigned)(ctas * S), WARPS * 32, sm, st>>>(
+        fhat, Qhat, m->wx2, S > 1 ? m->task64_split[split_index(S)] : m->task64, gv.h, gv.M, (int)gv.nhalf, m->rowmax64,
+        n, S);
     return cudaGetLastError();
 }
 
@@ -1360,8 +1441,6 @@ cudaError_t launch_modesum_x2(const bz_modes *m, const double2 *fhat, float2 *Qh
     if (m->variant64 == kFp64Variants[2]) return launch_x2_instance<2, 8, 4>(m, fhat, Qhat, n, sm, st);
     return cudaErrorInvalidValue;
 }
-
-static int sm_count();
 
 // A launch over n cells ends with a partial wave of tiles; the SMs that run
 // one tile fewer idle meanwhile.  With a 32-cell variant chosen by timing,
@@ -1443,6 +1522,9 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
     if (n <= 0) return cudaSuccess;
     const int sv = small_batch_variant(m, n);
     if (sv != m->variant) return launch_variant(m, sv, fhat, Qhat, n, st);
+    if (kVariants[sv].rows > 1)
+        return launch_variant(m, sv, fhat, Qhat, n, st,
+                              launch_split(ctas_for(sv, n), m->var_bal[sv], m->var_task_split[sv]));
     int tv = -1, ts = 1;
     const int64_t nm = modesum32_split(m, n, &tv, &ts);
     const int v = m->variant;
@@ -1492,13 +1574,15 @@ cudaError_t launch_modesum32_group(const bz_modes *const *ms, const float2 *cons
     memset(&gd, 0, sizeof gd);
     gd.nitems = count;
     size_t sm = 0;
-    int64_t ctas = 0;
+    int64_t ctas = 0, whole = 0;
+    for (int i = 0; i < count; ++i) whole += ctas_for(v, n[i]);
     for (int i = 0; i < count; ++i) {
         if (ms[i]->variant != v) return cudaErrorInvalidValue;
-        fill_item(gd.item[i], ms[i], ms[i]->var_W[v], ms[i]->var_task[v], ms[i]->var_rowmax[v], fhat[i], Qhat[i],
-                  n[i]);
+        const int S = kVariants[v].rows > 1 ? launch_split(whole, ms[0]->var_bal[v], ms[0]->var_task_split[v]) : 1;
+        fill_item(gd.item[i], ms[i], ms[i]->var_W[v], S > 1 ? ms[i]->var_task_split[v][split_index(S)] : ms[i]->var_task[v],
+                  ms[i]->var_rowmax[v], fhat[i], Qhat[i], n[i], S);
         gd.tile_start[i] = ctas;
-        ctas += ctas_for(v, n[i]);
+        ctas += ctas_for(v, n[i]) * S;
         sm = std::max(sm, smem_bytes<float>(ms[i]->g->v, ms[i]->var_rowmax[v], v));
     }
     gd.tile_start[count] = ctas;
@@ -1624,8 +1708,8 @@ int modes_build_fp32_tables(bz_modes *m) {
         m->var_rowmax[v] = 0;
         void *w = nullptr;
         for (int k = 0; k < kSplitTables; ++k) m->var_task_split[v][k] = nullptr;
-        int **split = kVariants[v].cells == 32 ? m->var_task_split[v] : nullptr;
-        if (build_variant<float>(m, v, rc, &w, &m->var_task[v], &m->var_rowmax[v], nullptr, split)) {
+        int **split = kVariants[v].cells == 32 || kVariants[v].rows > 1 ? m->var_task_split[v] : nullptr;
+        if (build_variant<float>(m, v, rc, &w, &m->var_task[v], &m->var_rowmax[v], nullptr, split, m->var_bal[v])) {
             m->var_W[v] = static_cast<float *>(w);
             any = true;
         }
@@ -1637,8 +1721,10 @@ int modes_build_fp32_tables(bz_modes *m) {
     m->rowmax64 = 0;
     m->variant64 = -1;
     m->wx2 = nullptr;
+    for (int k = 0; k < kSplitTables; ++k) m->task64_split[k] = nullptr;
     for (int q = 0; q < 3 && m->variant64 < 0; ++q) {
-        if (build_variant<double>(m, kFp64Variants[q], rc, &m->w64, &m->task64, &m->rowmax64, &m->wx2))
+        if (build_variant<double>(m, kFp64Variants[q], rc, &m->w64, &m->task64, &m->rowmax64, &m->wx2, m->task64_split,
+                                  m->bal64))
             m->variant64 = kFp64Variants[q];
         if (rc) return rc;
     }
@@ -1656,7 +1742,7 @@ int modes_build_fp32_tables(bz_modes *m) {
     m->d_W32 = m->var_W[v];
     m->d_task = m->var_task[v];
     m->w32_rowmax = m->var_rowmax[v];
-    m->modesum_variant = v + 1;
+    m->modesum_variant = m->g->v.dim == 2 && m->g->v.N > 48 ? 0 : v + 1;   // one form only: no choice to report
     return BZ_OK;
 }
 
