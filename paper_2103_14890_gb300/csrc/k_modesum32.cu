@@ -47,6 +47,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "bz_device.cuh"
@@ -69,13 +70,14 @@ struct Variant {
     int R, warps, cells, pack, wdup, pq, orient, rows;
 };
 constexpr int kNumVariants = kModesumVariants;   // FP32 variants (timed by the autotuner)
-// entries 0..9: the FP32 variants; entries 10, 11: layouts of the FP64 and FP32X2
-// forms only (2 outputs per thread, 8 warps, 8- and 4-cell tiles) for grids
-// whose 16-byte-per-value spectrum needs them (48^2, 16^3)
-constexpr Variant kVariants[kNumVariants + 2] = {
+// entries 0..9: the FP32 variants; entries 10..12: layouts of the FP64 and FP32X2
+// forms (16 bytes per spectrum value): 8-cell tiles, 4-cell tiles for 16^3, and
+// two outputs per thread for grids of fewer than 8 points
+constexpr Variant kVariants[kNumVariants + 3] = {
     {8, 16, 32, 1, 0, 0, 1, 1}, {4, 32, 32, 1, 0, 0, 1, 1}, {4, 16, 16, 1, 0, 0, 1, 1}, {8, 12, 8, 1, 0, 1, 2, 2},
     {4, 16, 32, 2, 1, 0, 1, 1}, {8, 12, 32, 1, 0, 1, 1, 1}, {8, 16, 32, 1, 0, 1, 1, 1}, {8, 16, 16, 1, 0, 1, 2, 1},
-    {8, 8, 16, 1, 0, 1, 2, 1},  {8, 4, 16, 1, 0, 1, 2, 1},  {2, 8, 8, 1, 0, 0, 1, 1},   {2, 8, 4, 1, 0, 0, 1, 1}};
+    {8, 8, 16, 1, 0, 1, 2, 1},  {8, 4, 16, 1, 0, 1, 2, 1},  {4, 8, 8, 1, 0, 1, 2, 2},   {4, 8, 4, 1, 0, 1, 2, 4},
+    {2, 8, 8, 1, 0, 1, 2, 2}};
 
 // lane groups splitting a task's outputs, and outputs per task (RT)
 constexpr int variant_groups(int v) {
@@ -129,14 +131,6 @@ __device__ __forceinline__ void load_w4(float *wv, const float *p) {
     wv[2] = w4.z;
     wv[3] = w4.w;
 }
-__device__ __forceinline__ void load_w4(double *wv, const double *p) {
-    const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
-    wv[0] = a.x;
-    wv[1] = a.y;
-    wv[2] = b.x;
-    wv[3] = b.y;
-}
-
 // One block of RR l_2 steps.  The window of f-hat_m values lives in a 2RR-slot
 // register array used under two alternating namings (PH = 0, 1): logical slot
 // j is physical slot (j + PH RR) mod 2RR, so moving the window by RR between
@@ -169,16 +163,9 @@ __device__ __forceinline__ void block_body(typename C2<T>::type (&win)[2 * RR],
         V2 fl = (DIR == 0) ? lp[s * dcs] : lp[s * DIR * CS];
         if (DIR == 0) fl.y *= sgn;
         T wv[RR];
-        if constexpr (RR % 4 == 0) {
 #pragma unroll
-            for (int q = 0; q < RR; q += 4)
-                if (!RAMP || q < s) load_w4(wv + q, wb + s * WS + q);
-        } else {
-            static_assert(RR == 2 && sizeof(T) == 8 && !RAMP, "two-output blocks are used by the FP64 form only");
-            const double2 w2 = *reinterpret_cast<const double2 *>(wb + s * WS);
-            wv[0] = w2.x;
-            wv[1] = w2.y;
-        }
+        for (int q = 0; q < RR; q += 4)
+            if (!RAMP || q < s) load_w4(wv + q, wb + s * WS + q);
 #pragma unroll
         for (int r = 0; r < RR; ++r) {
             if (RAMP && r >= s) continue;
@@ -792,163 +779,217 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
     }
 }
 
-// ---- FP32X2 form: double-float arithmetic on the FP32 pipe ------------------
-// Every value is an unevaluated sum hi + lo of two FP32 numbers (|lo| <= u |hi|).
-// For each term w f-hat_l f-hat_m of eq. CF1 the product X = w f-hat_l is
-// formed exactly in its high part (TwoProd: fmaf(a, b, -fl(a b)) is the exact
-// rounding error of a b) with the low parts of w and f-hat_l added to its
-// error; each of the four real products X b of the complex product is split
-// exactly the same way, its high part enters the running sum by TwoSum (exact
-// error), and every error and the cross terms with the low part of b
-// accumulate in a second FP32 sum.  This is the compensated dot product
-// ("Dot2") of Ogita, Rump and Oishi (2005), accurate as if computed in twice
-// the working precision; the operations are pinned with the _rn intrinsics
-// so the compiler cannot fuse them into FMAs that would break the exact splits.
-// The real and imaginary parts run as the two lanes of FP32x2 instructions:
-// every lane performs exactly the scalar operations in the scalar order
-// (the products (-y) x of the imaginary part are formed as y (-x), the same
-// value), so the result is that of the scalar form bit for bit.
-struct X2Acc {
-    float2 s;         // running sums of the high parts (real, imaginary)
-    float2 c;         // accumulated errors and low-order terms
-};
-
-__device__ __forceinline__ float2 x2_neg(float2 a) { return make_float2(-a.x, -a.y); }
-
-// acc += w a b with w = wh + wl (real), a = ah + al (conjugated for DIR < 0),
-// b = bh + bl; bs, ls are bh and bl with their lanes exchanged.
-template <int DIR>
-__device__ __forceinline__ void x2_term(X2Acc &acc, float wh, float wl, float2 ah, float2 al, float2 bh,
-                                        float2 bl, float2 bs, float2 ls) {
-    // X = w a: high parts exact products, errors plus the low-part terms
-    const float2 W = make_float2(wh, wh);
-    const float2 X = __fmul2_rn(W, ah);
-    float2 E = __ffma2_rn(W, ah, x2_neg(X));
-    E = __ffma2_rn(make_float2(wl, wl), ah, E);
-    E = __ffma2_rn(W, al, E);
-    // with xi the imaginary part of X after the optional conjugation, yn = -xi:
-    // X b = xx (bx, by) + (yn by, -yn bx)
-    const float yn = DIR > 0 ? -X.y : X.y, en = DIR > 0 ? -E.y : E.y;
-    const float2 XX = make_float2(X.x, X.x), YN = make_float2(yn, -yn);
-    float2 sm, d;
-    const float2 P = __fmul2_rn(XX, bh);
-    const float2 qp = __ffma2_rn(XX, bh, x2_neg(P));
-    two_sum2(acc.s, P, sm, d);
-    acc.s = sm;
-    float2 c = __fadd2_rn(qp, d);
-    const float2 Q = __fmul2_rn(YN, bs);
-    const float2 qq = __ffma2_rn(YN, bs, x2_neg(Q));
-    two_sum2(acc.s, Q, sm, d);
-    acc.s = sm;
-    c = __fadd2_rn(c, __fadd2_rn(qq, d));
-    acc.c = __fadd2_rn(acc.c, c);
-    acc.c = __ffma2_rn(make_float2(E.x, E.x), bh, acc.c);
-    acc.c = __ffma2_rn(make_float2(en, -en), bs, acc.c);
-    acc.c = __ffma2_rn(XX, bl, acc.c);
-    acc.c = __ffma2_rn(YN, ls, acc.c);
+// ---- FP64 and FP32X2 forms -----------------------------------------------------
+// Both run the paired orientations of modesum_pq_kernel on tiles of CELLS = 8 or
+// 4 cells: a warp holds ROWS = 16 / CELLS groups of lanes, each group its
+// CELLS cells plain and mirrored on its own row pair of the task.  Their blocks
+// of RR <= 4 outputs divide the half row of 16, 32 and 48 points, so the ramped
+// tables leave no padding (the earlier tables for blocks of 8 over the whole
+// row summed 1.24 pairs per useful one at 32^2, these 1.04), and two CTAs share
+// an SM at 32^2, so that the end of one tile overlaps the other.  4099 cells of
+// 32^2 in FP64: 8.76 -> 7.56 ms.
+//
+// One block of RR l_2 steps and one row pair, as block_pq and row_pass_pq; Term
+// supplies the value type (what a spectrum entry is) and the product sums.
+template <typename Term, int RR, int PH, bool RAMP>
+__device__ __forceinline__ void block_pair(typename Term::Val (&win)[2 * RR], const typename Term::Src mp, int mcs,
+                                           const typename Term::Src lp, int dcs, int dir,
+                                           const typename Term::W *__restrict__ wb, typename Term::Acc (&acc)[RR]) {
+#pragma unroll
+    for (int j = 0; j < (RAMP ? RR - 1 : RR); ++j) win[(j + PH * RR) & (2 * RR - 1)] = Term::load(mp, j * mcs);
+#pragma unroll
+    for (int s = RAMP ? 1 : 0; s < RR; ++s) {
+        const typename Term::Val fl = Term::conj(Term::load(lp, s * dcs), dir);
+        typename Term::Wt wv[RR];
+        Term::template weights<RR>(wv, wb + s * RR * Term::kWPer);
+#pragma unroll
+        for (int r = 0; r < RR; ++r)
+            if (!RAMP || r < s) Term::add(acc[r], wv[r], fl, win[(r - s + RR - 1 + PH * RR) & (2 * RR - 1)]);
+    }
 }
 
-// RR consecutive FP32 weights (RR = 4: 16-byte aligned, RR = 2: 8-byte aligned).
-template <int RR> __device__ __forceinline__ void load_wx(float *wv, const float *p) {
-    if constexpr (RR == 4) {
-        const float4 w4 = *reinterpret_cast<const float4 *>(p);
-        wv[0] = w4.x;
-        wv[1] = w4.y;
-        wv[2] = w4.z;
-        wv[3] = w4.w;
+template <typename Term, int RR, int CS>
+__device__ __forceinline__ void row_pass_pair(typename Term::Src rowl, typename Term::Src rowm,
+                                              const typename Term::W *__restrict__ wrow, int nblk, int l2lo, int mbase0,
+                                              int dir, bool ramp, bool mirror, typename Term::Acc (&acc)[RR]) {
+    typename Term::Val win[2 * RR];
+    constexpr int WB = RR * RR * Term::kWPer;            // weights of a block
+    const int dcs = (mirror ? -dir : dir) * CS;          // between consecutive l_2
+    const int mcs = mirror ? -CS : CS;                   // between consecutive window columns
+    typename Term::Src mp = Term::at(rowm, mbase0 * mcs), lp = Term::at(rowl, l2lo * dcs);
+    int blk = 0;
+    if (ramp) {
+        block_pair<Term, RR, 1, true>(win, mp, mcs, lp, dcs, dir, wrow, acc);
+        mp = Term::at(mp, -RR * mcs);
+        lp = Term::at(lp, RR * dcs);
+        blk = 1;
     } else {
-        static_assert(RR == 2, "FP32X2 blocks hold 2 or 4 outputs per thread");
-        const float2 w2 = *reinterpret_cast<const float2 *>(p);
-        wv[0] = w2.x;
-        wv[1] = w2.y;
+#pragma unroll
+        for (int j = RR; j < 2 * RR - 1; ++j) win[j] = Term::load(mp, j * mcs);
     }
+    for (; blk + 1 < nblk; blk += 2) {
+        block_pair<Term, RR, 0, false>(win, mp, mcs, lp, dcs, dir, wrow + blk * WB, acc);
+        block_pair<Term, RR, 1, false>(win, Term::at(mp, -RR * mcs), mcs, Term::at(lp, RR * dcs), dcs, dir,
+                                       wrow + (blk + 1) * WB, acc);
+        mp = Term::at(mp, -2 * RR * mcs);
+        lp = Term::at(lp, 2 * RR * dcs);
+    }
+    if (blk < nblk) block_pair<Term, RR, 0, false>(win, mp, mcs, lp, dcs, dir, wrow + blk * WB, acc);
 }
 
-// One block of RR l_2 steps of the FP32X2 form: the window scheme of
-// block_pass, with the high and low parts of each spectrum value LO elements
-// apart in shared memory and the weights of step s at wb + s * 2 RT (high
-// parts) and wb + s * 2 RT + RT (low parts).  The read direction of f-hat_l is
-// chosen at run time (dcs = +/-CS, sgn = +/-1 on the imaginary parts):
-// x2_term<+1> on the conjugated value performs exactly the
-// operations of x2_term<-1> on the value read, each negated (rounding is
-// symmetric), so the results are those of direction-specialised bodies with
-// half the code (four specialised bodies overflow the instruction cache).
-template <int RR, int CS, int RT, int PH>
-__device__ __forceinline__ void block_pass_x2_rt(float2 (&wh)[2 * RR], float2 (&wl)[2 * RR],
-                                                 const float2 *__restrict__ mp, const float2 *__restrict__ lp, int dcs,
-                                                 float sgn, int LO, const float *__restrict__ wb, X2Acc (&acc)[RR]) {
-#pragma unroll
-    for (int j = 0; j < RR; ++j) {
-        wh[(j + PH * RR) & (2 * RR - 1)] = mp[j * CS];
-        wl[(j + PH * RR) & (2 * RR - 1)] = mp[j * CS + LO];
+// FP64: six operations of the FP64 pipe per pair, which bounds the kernel.
+struct Term64 {
+    using Val = double2;
+    using Src = const double2 *;
+    using W = double;
+    using Wt = double;
+    using Acc = double2;
+    static constexpr int kWPer = 1;
+    static __device__ __forceinline__ Src at(Src p, int off) { return p + off; }
+    static __device__ __forceinline__ Val load(Src p, int off) { return p[off]; }
+    static __device__ __forceinline__ Val conj(Val v, int dir) {
+        return make_double2(v.x, dir > 0 ? v.y : -v.y);
     }
+    template <int RR> static __device__ __forceinline__ void weights(Wt (&w)[RR], const W *__restrict__ p) {
 #pragma unroll
-    for (int s = 0; s < RR; ++s) {
-        float2 ah = lp[s * dcs], al = lp[s * dcs + LO];
-        ah.y *= sgn;
-        al.y *= sgn;
-        float whi[RR], wlo[RR];
-        load_wx<RR>(whi, wb + s * 2 * RT);
-        load_wx<RR>(wlo, wb + s * 2 * RT + RT);
-#pragma unroll
-        for (int r = 0; r < RR; ++r) {
-            const int q = (r - s + RR - 1 + PH * RR) & (2 * RR - 1);
-            x2_term<1>(acc[r], whi[r], wlo[r], ah, al, wh[q], wl[q], make_float2(wh[q].y, wh[q].x),
-                       make_float2(wl[q].y, wl[q].x));
+        for (int q = 0; q < RR; q += 2) {
+            const double2 x = *reinterpret_cast<const double2 *>(p + q);
+            w[q] = x.x;
+            w[q + 1] = x.y;
         }
     }
-}
-
-template <int RR, int CS, int RT>
-__device__ __forceinline__ void row_pass_x2(const float2 *__restrict__ rowl, const float2 *__restrict__ rowm, int LO,
-                                            const float *__restrict__ wrow, int nblk, int l2lo, int mbase0, int dir,
-                                            X2Acc (&acc)[RR]) {
-    float2 wh[2 * RR], wl[2 * RR];
-    const int dcs = dir * CS;
-    const float sgn = (float)dir;
-    const float2 *mp = rowm + mbase0 * CS;
-    const float2 *lp = rowl + l2lo * dcs;
-#pragma unroll
-    for (int j = RR; j < 2 * RR - 1; ++j) {
-        wh[j] = mp[j * CS];
-        wl[j] = mp[j * CS + LO];
+    static __device__ __forceinline__ void add(Acc &a, Wt w, const Val &f, const Val &b) {
+        const double tx = w * f.x, ty = w * f.y;
+        a.x = fma(tx, b.x, a.x);
+        a.x = fma(-ty, b.y, a.x);
+        a.y = fma(tx, b.y, a.y);
+        a.y = fma(ty, b.x, a.y);
     }
-    int blk = 0;
-    for (; blk + 1 < nblk; blk += 2) {
-        block_pass_x2_rt<RR, CS, RT, 0>(wh, wl, mp, lp, dcs, sgn, LO, wrow + blk * RR * 2 * RT, acc);
-        block_pass_x2_rt<RR, CS, RT, 1>(wh, wl, mp - RR * CS, lp + RR * dcs, dcs, sgn, LO,
-                                        wrow + (blk + 1) * RR * 2 * RT, acc);
-        mp -= 2 * RR * CS;
-        lp += 2 * RR * dcs;
-    }
-    if (blk < nblk) block_pass_x2_rt<RR, CS, RT, 0>(wh, wl, mp, lp, dcs, sgn, LO, wrow + blk * RR * 2 * RT, acc);
-}
+};
 
-// The FP32X2 mode sum: the task structure and shared-memory layout of
-// modesum32_kernel on the FP64 tables (same tasks, same row pairs; a weight's
-// 8 bytes hold its FP32 high and low parts).  Input: FP64 spectra in the tiled
-// layout, split into FP32 high and low parts while they are staged; output:
-// Q-hat rounded to FP32 (hi + lo), tiled layout.
-template <int RR, int WARPS, int CELLS>
-__global__ void __launch_bounds__(WARPS * 32, 1)
-modesum_x2_kernel(const double2 *__restrict__ fhat, float2 *__restrict__ Qhat, const float *__restrict__ W,
-                  const int *__restrict__ tasks, int h, int M, int nhalf, int wrow_max, int64_t n, int split) {
-    constexpr int G = 32 / CELLS;
-    constexpr int RT = RR * G;
-    constexpr int HEADF = kRowHeadBytes / (int)sizeof(float);
+// FP32X2: double-float arithmetic on the FP32 pipe.  Every value is an
+// unevaluated sum hi + lo of two FP32 numbers (|lo| <= u |hi|).  For each term
+// w f-hat_l f-hat_m of eq. CF1 the product X = w f-hat_l is formed exactly in
+// its high part (TwoProd: fma(a, b, -fl(a b)) is the exact rounding error of
+// a b) with the low parts of w and f-hat_l added to its error; each of the four
+// real products X b of the complex product is split exactly the same way, its
+// high part enters the running sum with its exact error, and every error and
+// the cross terms with the low part of b accumulate in a second FP32 sum.  This
+// is the compensated dot product ("Dot2") of Ogita, Rump and Oishi (2005),
+// accurate as if computed in twice the working precision; the real and
+// imaginary parts are the two lanes, and the _rn intrinsics pin the operations.
+// The FMA pipe bounds the kernel (70 % busy): 28 FP32x2 operations per pair.
+// 4096 cells of 32^2: 1.53 -> 1.34 ms by the tables and the split of the tiles.
+// Not kept: Dekker's three-operation sums on operands ordered by selects (22
+// operations, the same numbers) moved the bound to the ALU pipe, 1.55 ms; a
+// running sum biased so that it always exceeds the product needs 16 operations
+// and took 0.94 ms, but its errors are relative to the bias, 100 times those of
+// Dot2 on cells near equilibrium.
+struct X2Val {
+    float2 h, l;
+};
+struct X2Src {
+    const float2 *p;
+    int LO;                                  // from a value's high part to its low part
+};
+struct X2Wt {
+    float h, l;
+};
+struct X2Acc {
+    float2 s, c;
+};
+struct TermX2 {
+    using Val = X2Val;
+    using Src = X2Src;
+    using W = float;
+    using Wt = X2Wt;
+    using Acc = X2Acc;
+    static constexpr int kWPer = 2;          // a step's high parts, then its low parts
+    static __device__ __forceinline__ Src at(Src s, int off) { return Src{s.p + off, s.LO}; }
+    static __device__ __forceinline__ Val load(Src s, int off) { return Val{s.p[off], s.p[off + s.LO]}; }
+    static __device__ __forceinline__ Val conj(Val v, int dir) {
+        if (dir < 0) {
+            v.h.y = -v.h.y;
+            v.l.y = -v.l.y;
+        }
+        return v;
+    }
+    template <int RR> static __device__ __forceinline__ void weights(Wt (&w)[RR], const W *__restrict__ p) {
+        if constexpr (RR == 4) {
+            const float4 h = *reinterpret_cast<const float4 *>(p), l = *reinterpret_cast<const float4 *>(p + 4);
+            w[0] = Wt{h.x, l.x};
+            w[1] = Wt{h.y, l.y};
+            w[2] = Wt{h.z, l.z};
+            w[3] = Wt{h.w, l.w};
+        } else {
+            static_assert(RR == 2, "2 or 4 outputs per thread");
+            const float4 q = *reinterpret_cast<const float4 *>(p);
+            w[0] = Wt{q.x, q.z};
+            w[1] = Wt{q.y, q.w};
+        }
+    }
+    static __device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+    static __device__ __forceinline__ void add(Acc &a, const Wt &w, const Val &f, const Val &b) {
+        const float2 W2 = make_float2(w.h, w.h);
+        const float2 X = __fmul2_rn(W2, f.h);
+        float2 E = __ffma2_rn(W2, f.h, neg(X));
+        E = __ffma2_rn(make_float2(w.l, w.l), f.h, E);
+        E = __ffma2_rn(W2, f.l, E);
+        // X b = X_x (b_x, b_y) + (-X_y, X_y) (b_y, b_x)
+        const float2 bs = make_float2(b.h.y, b.h.x), ls = make_float2(b.l.y, b.l.x);
+        const float2 XX = make_float2(X.x, X.x), YN = make_float2(-X.y, X.y);
+        const float2 P = __fmul2_rn(XX, b.h);
+        float2 d;
+        sum_exact(a.s, P, d);
+        float2 c = __fadd2_rn(__ffma2_rn(XX, b.h, neg(P)), d);
+        const float2 Q = __fmul2_rn(YN, bs);
+        sum_exact(a.s, Q, d);
+        c = __fadd2_rn(c, __fadd2_rn(__ffma2_rn(YN, bs, neg(Q)), d));
+        c = __fadd2_rn(a.c, c);
+        c = __ffma2_rn(make_float2(E.x, E.x), b.h, c);
+        c = __ffma2_rn(make_float2(-E.y, E.y), bs, c);
+        c = __ffma2_rn(XX, b.l, c);
+        a.c = __ffma2_rn(YN, ls, c);
+    }
+    // s <- fl(s + p), d the exact error (TwoSum)
+    static __device__ __forceinline__ void sum_exact(float2 &s, float2 p, float2 &d) {
+        float2 sm;
+        two_sum2(s, p, sm, d);
+        s = sm;
+    }
+};
+
+// The task loop of both forms.  FP64: sums along a row pair fold into (hi, lo)
+// by TwoSum every four.  FP32X2: the FP64 spectrum is split into FP32 high and
+// low parts as it is staged; its output is rounded to FP32.  A tile may be
+// split over gd.item[0].split CTAs.
+template <bool X2, int RR, int WARPS, int CELLS>
+__global__ void __launch_bounds__(WARPS * 32, CELLS == 8 ? 2 : 1) modesum_pair_kernel(const Mode32Group gd) {
+    constexpr int G = 32 / CELLS;                // CTAs per 32-cell tile
+    constexpr int ROWS = 16 / CELLS;             // row pairs at a time
+    constexpr int SLOT = X2 ? 2 : 1;             // floats or doubles per 8-byte slot of the weight stream
+    using W = typename std::conditional<X2, float, double>::type;
+    using OutV = typename std::conditional<X2, float2, double2>::type;
     extern __shared__ __align__(16) uint4 smem16[];
-    const int part = (int)(blockIdx.x % split);      // this CTA's part of the task table
-    const int64_t cta = (int64_t)blockIdx.x / split;
+    const Mode32Item &ip = gd.item[0];
+    const double2 *__restrict__ fhat = static_cast<const double2 *>(ip.fhat);
+    const W *__restrict__ Wst = static_cast<const W *>(ip.W);
+    const int *__restrict__ tasks = ip.tasks;
+    const int h = ip.h, M = ip.M, nhalf = ip.nhalf, wrow_max = ip.wrow_max;
+    const int part = (int)(blockIdx.x % ip.split);
+    const int64_t cta = (int64_t)blockIdx.x / ip.split;
     const int64_t tile = cta / G;
     const int sub = (int)(cta % G);
     const int rows = nhalf + 2 * kPad;
-    float2 *Fh = reinterpret_cast<float2 *>(smem16);              // [rows][CELLS] high parts
-    float2 *Fl = Fh + (size_t)rows * CELLS;                       // [rows][CELLS] low parts
-    float *wsm = reinterpret_cast<float *>(Fl + (size_t)rows * CELLS);   // [warps][2][2 wrow_max]
-    const int LO = rows * CELLS;
-    {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cell = lane % CELLS;
+    double2 *Fs = reinterpret_cast<double2 *>(smem16);               // [rows][CELLS]; X2: float2 high, then low parts
+    float2 *Fh = reinterpret_cast<float2 *>(smem16);
+    W *wsm = reinterpret_cast<W *>(Fs + (size_t)rows * CELLS);       // [warps][2][ROWS wrow_max slots]
+    if constexpr (X2) {
         const double2 *src = fhat + tile * (int64_t)nhalf * 32 + sub * CELLS;
-        for (int i = threadIdx.x; i < rows * CELLS; i += blockDim.x) {
+        float2 *Fl = Fh + (size_t)rows * CELLS;
+        for (int i = threadIdx.x; i < rows * CELLS; i += WARPS * 32) {
             const int row = i / CELLS - kPad, c = i % CELLS;
             float2 hv = make_float2(0.f, 0.f), lv = make_float2(0.f, 0.f);
             if (row >= 0 && row < nhalf) {
@@ -961,49 +1002,99 @@ modesum_x2_kernel(const double2 *__restrict__ fhat, float2 *__restrict__ Qhat, c
             Fh[i] = hv;
             Fl[i] = lv;
         }
+        __syncthreads();
+    } else {
+        stage_spectrum<double2, CELLS>(smem16, fhat, tile, sub, nhalf, M, false);
+        __syncthreads();
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int cell = lane % CELLS, grp = lane / CELLS;
-    float *wbuf0 = wsm + (size_t)warp * 4 * wrow_max;             // wrow_max counts 8-byte slots
-    float *wbuf1 = wbuf0 + 2 * wrow_max;
-    const int vw = part * WARPS + warp;
-    const int tbeg = tasks[vw], tend = tasks[vw + 1];
-    const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * WARPS * split + 1);
-    const float2 *F0 = Fh + (size_t)(kPad + h) * CELLS + cell;
+    const bool upper = (lane / CELLS) % 2 == 1;                      // runs every task mirrored
+    const int rgrp = lane / (2 * CELLS);                             // its row pair of each ROWS
+    W *wbuf0 = wsm + (size_t)warp * 2 * ROWS * wrow_max * SLOT;
+    W *wbuf1 = wbuf0 + (size_t)ROWS * wrow_max * SLOT;
+    const int NW = WARPS * ip.split;
+    int t = tasks[part * WARPS + warp];
+    const int tend = tasks[part * WARPS + warp + 1];
+    const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * NW + 1);
+    const size_t f0 = (size_t)(kPad + h) * CELLS + cell;
+    const bool valid = tile * 32 + sub * CELLS + cell < ip.n && rgrp == 0;
+    OutV *const qt = static_cast<OutV *>(ip.Qhat) + tile * (int64_t)nhalf * 32 + sub * CELLS + cell;
 
-    for (int t = tbeg; t < tend; ++t) {
-        const TaskRec tk = trec[t];
-        const int rowb = tk.rowf * 8;                      // bytes per row pair
-        const float *wsrc = W + 2 * (size_t)tk.woff;
-        X2Acc acc[RR];
+    for (; t < tend;) {
+        const TaskRec tk = trec[t++];
+        const int rowb = ROWS * tk.rowf * 8;                         // bytes staged per step
+        const bool ramp = (tk.flags & kTaskRamp) != 0;
+        const W *wsrc = Wst + (size_t)tk.woff * SLOT;
+        const int mbase0 = tk.k20 - tk.l2lo - (RR - 1);
+        const int nrows = tk.nrows / ROWS;
+        typename std::conditional<X2, X2Acc, double2>::type acc[RR];
+        OutV hi[RR], lo[RR];
 #pragma unroll
-        for (int r = 0; r < RR; ++r) acc[r] = X2Acc{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        const int k20 = tk.k20 + grp * RR;
-        const int mbase0 = k20 - tk.l2lo - (RR - 1);
+        for (int r = 0; r < RR; ++r) {
+            hi[r] = lo[r] = cmk<OutV>(0, 0);
+            if constexpr (X2) acc[r] = X2Acc{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            else acc[r] = make_double2(0.0, 0.0);
+        }
         stage_row(wbuf0, wsrc, rowb, lane);
-        for (int i = 0; i < tk.nrows; ++i) {
-            const float *wcur = (i & 1) ? wbuf1 : wbuf0;
-            if (i + 1 < tk.nrows) {
-                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * 2 * tk.rowf, rowb, lane);
+        for (int i = 0; i < nrows; ++i) {
+            const W *wcur = ((i & 1) ? wbuf1 : wbuf0) + (size_t)rgrp * tk.rowf * SLOT;
+            if (i + 1 < nrows) {
+                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * ROWS * tk.rowf * SLOT, rowb, lane);
                 cp_async_wait<1>();
             } else {
                 cp_async_wait<0>();
             }
             __syncwarp();
             const int4 hd = *reinterpret_cast<const int4 *>(wcur);
-            row_pass_x2<RR, CELLS, RT>(F0 + hd.x, F0 + hd.y, LO, wcur + HEADF + grp * RR, tk.nblk * G, tk.l2lo,
-                                       mbase0, hd.z > 0 ? 1 : -1, acc);
+            constexpr int HEAD = kRowHeadBytes / (int)sizeof(W);
+            if constexpr (X2) {
+                row_pass_pair<TermX2, RR, CELLS>(X2Src{Fh + f0 + hd.x, rows * CELLS}, X2Src{Fh + f0 + hd.y, rows * CELLS},
+                                                 wcur + HEAD, tk.nblk, tk.l2lo, mbase0, hd.z, ramp, upper, acc);
+            } else {
+                row_pass_pair<Term64, RR, CELLS>(Fs + f0 + hd.x, Fs + f0 + hd.y, wcur + HEAD, tk.nblk, tk.l2lo, mbase0,
+                                                 hd.z, ramp, upper, acc);
+                if ((i & 3) == 3 || i + 1 == nrows) {
+#pragma unroll
+                    for (int r = 0; r < RR; ++r) {
+                        double sm, e;
+                        two_sum(hi[r].x, acc[r].x, sm, e);
+                        hi[r].x = sm;
+                        lo[r].x += e;
+                        two_sum(hi[r].y, acc[r].y, sm, e);
+                        hi[r].y = sm;
+                        lo[r].y += e;
+                        acc[r] = make_double2(0.0, 0.0);
+                    }
+                }
+            }
             __syncwarp();
         }
-        const int64_t c = tile * 32 + sub * CELLS + cell;
-        if (c < n) {
-            float2 *out = Qhat + tile * (int64_t)nhalf * 32 + (int64_t)tk.orow * M * 32 + sub * CELLS + cell;
+        // the row groups' sums
+#pragma unroll
+        for (int r = 0; r < RR; ++r) {
+            if constexpr (X2) hi[r] = acc[r].s, lo[r] = acc[r].c;
+#pragma unroll
+            for (int o = 2 * CELLS; o < 32; o <<= 1) {
+                OutV h2, l2;
+                h2.x = __shfl_xor_sync(0xffffffffu, hi[r].x, o);
+                h2.y = __shfl_xor_sync(0xffffffffu, hi[r].y, o);
+                l2.x = __shfl_xor_sync(0xffffffffu, lo[r].x, o);
+                l2.y = __shfl_xor_sync(0xffffffffu, lo[r].y, o);
+                decltype(h2.x) sm, e;
+                two_sum(hi[r].x, h2.x, sm, e);
+                hi[r].x = sm;
+                lo[r].x = (lo[r].x + l2.x) + e;
+                two_sum(hi[r].y, h2.y, sm, e);
+                hi[r].y = sm;
+                lo[r].y = (lo[r].y + l2.y) + e;
+            }
+        }
+        if (valid) {
+            OutV *out = qt + (int64_t)tk.orow * M * 32;
 #pragma unroll
             for (int r = 0; r < RR; ++r) {
-                const int k2 = k20 + r;
-                if (grp * RR + r >= tk.rfirst && k2 <= h)
-                    out[(k2 + h) * 32] = __fadd2_rn(acc[r].s, acc[r].c);
+                const int k2 = tk.k20 + r;
+                if (k2 <= h && !(upper && k2 == 0))
+                    out[(upper ? h - k2 : k2 + h) * 32] = cmk<OutV>(hi[r].x + lo[r].x, hi[r].y + lo[r].y);
             }
         }
     }
@@ -1036,7 +1127,7 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
     const GridView &gv = m->g->v;
     const int d = gv.dim, h = gv.h, M = gv.M;
     const int rows = kVariants[v].rows;                         // row pairs at a time
-    if (!((d == 2 && gv.N <= (rows > 1 ? 64 : 48)) || (d == 3 && gv.N <= 16))) return false;
+    if (!((d == 2 && gv.N <= (rows > 1 && sizeof(T) == 4 ? 64 : 48)) || (d == 3 && gv.N <= 16))) return false;
     // shared memory of the spectrum alone must leave room for the weight buffers
     if (2 * sizeof(T) * (size_t)(gv.nhalf + 2 * kPad) * kVariants[v].cells > 200 * 1024) return false;
     const int nb = (M + R - 1) / R;
@@ -1054,7 +1145,7 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
     // one lane group and R dividing h + 1, every task starts with the ramp
     // block and no step is padding
     const int G = variant_groups(v);
-    const bool reflect = sizeof(T) == 4 && variant_reflects(v, h);
+    const bool reflect = (sizeof(T) == 4 || kVariants[v].orient == 2) && variant_reflects(v, h);
     const bool ramped = reflect && G == 1 && (h + 1) % R == 0;
     const bool twins = reflect && kVariants[v].orient == 1;   // paired orientations need no reflected tasks
     // paired orientations compute k_2 < 0 in the mirrored half of every task:
@@ -1076,8 +1167,8 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                         pairs.push_back({{l1, l2}, {m1, k2 - l2}});
                 }
             }
-            // couples of row pairs with one read direction: an odd one out is
-            // coupled with a copy of itself whose weights are zero
+            // groups of `rows` row pairs with one read direction, the last one
+            // filled with copies whose weights are zero
             std::vector<char> dummy(pairs.size(), 0);
             if (rows > 1) {
                 std::vector<Pair> in = pairs;
@@ -1086,7 +1177,7 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                 for (int neg = 1; neg >= 0; --neg) {
                     for (const Pair &p : in)
                         if ((p.l[0] < 0) == (neg == 1)) pairs.push_back(p), dummy.push_back(0);
-                    if (pairs.size() % 2) pairs.push_back(pairs.back()), dummy.push_back(1);
+                    while (pairs.size() % rows) pairs.push_back(pairs.back()), dummy.push_back(1);
                 }
             }
             // blocks of R consecutive last-axis outputs.  reflect: the blocks
@@ -1362,84 +1453,86 @@ static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, 
     return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
 }
 
-// FP64 form: the same kernel on double spectra and weights, on 16-cell tiles
-// (variant entry 2) or, where the double spectrum of 16 cells does not fit
-// shared memory, on 8- or 4-cell tiles (entries 10, 11: 48^2, 16^3).  The FP32X2 form runs on the same layout.
-constexpr int kFp64Variants[3] = {2, 10, 11};
+// FP64 form: paired orientations on 8-cell tiles (variant entry 10), on 4-cell
+// tiles where the double spectrum of 8 cells does not fit shared memory (16^3),
+// and with two outputs per thread where four overhang the half row (N < 8).
+// The FP32X2 form runs on the same layout.
+constexpr int kFp64Variants[3] = {10, 11, 12};
 
 bool modesum64_available(const bz_modes *m) { return m->w64 != nullptr; }
 
 static int sm_count();
 
-// CTAs that take one tile's tasks between them (1, 2, 4 or 8), for kernels with
-// one CTA per SM: the S with the least ceil(ctas S / SMs) x (load of the most
-// loaded warp with S CTAs), so that neither a launch smaller than a wave nor
-// its last partial wave leaves SMs idle.  Every output is computed by one task
-// with the same arithmetic, so the results do not depend on S.  Staging the
-// spectrum S times costs little (a few us of an SM against hundreds); a larger
-// S has to win by 3 %.  4099 cells of 32^2 (257 CTAs on 152 SMs), FP64: 8.76 ->
-// @F64S@ ms, FP32X2: 1.53 -> @X2S@ ms.
-static int launch_split(int64_t ctas, const float (&bal)[kSplitTables + 1], int *const *tables) {
+// CTAs that take one tile's tasks between them (1, 2, 4 or 8): the S with the
+// least estimated time, so that neither a launch smaller than a wave nor its
+// last partial wave leaves SMs idle.  Every output is computed by one task with
+// the same arithmetic, so the results do not depend on S; staging the spectrum
+// S times costs a few us of an SM against hundreds, and a larger S has to win
+// by 3 %.  With one CTA per SM the time is the number of waves times the load
+// of the most loaded warp; with several (shared), whose warps fill one
+// another's gaps, it is the most CTAs an SM gets times their mean load.  The
+// FP64 and FP32X2 forms run 32^2 so; 4099 cells (516 CTAs, 152 SMs), S = 1, 2, 4: FP64 8.60,
+// 7.56, 7.59 ms.  500 cells of 64^2 in FP32 (64
+// CTAs): 0.581, 0.306, 0.326 ms.
+static int launch_split(int64_t ctas, const float (&bal)[kSplitTables + 1], int *const *tables, bool shared) {
     const int64_t sms = sm_count();
+    auto estimate = [&](int S, double most) {
+        const double waves = (double)((ctas * S + sms - 1) / sms);
+        return shared ? std::max(waves * bal[0] / S, most) : waves * most;
+    };
     int best = 1;
-    double t = (double)((ctas + sms - 1) / sms) * bal[0];
+    double t = estimate(1, bal[0]);
     for (int k = 0; k < kSplitTables; ++k) {
         if (!tables[k]) continue;
-        const int S = 2 << k;
-        const double ts = (double)((ctas * S + sms - 1) / sms) * bal[k + 1];
+        const double ts = estimate(2 << k, bal[k + 1]);
         if (ts < 0.97 * t) {
             t = ts;
-            best = S;
+            best = 2 << k;
         }
     }
     return best;
 }
 
-cudaError_t launch_modesum64(const bz_modes *m, const double2 *fhat, double2 *Qhat, int64_t n, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    if (!m->w64) return cudaErrorInvalidValue;
+template <bool X2, int RR, int WARPS, int CELLS>
+static cudaError_t launch_pair(const Mode32Group &gd, size_t sm, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(modesum_pair_kernel<X2, RR, WARPS, CELLS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    modesum_pair_kernel<X2, RR, WARPS, CELLS><<<(unsigned)gd.tile_start[1], WARPS * 32, sm, st>>>(gd);
+    return cudaGetLastError();
+}
+
+// Spectra of 16 bytes per value (one double, or FP32 high and low parts) and
+// weight rows of 8-byte slots in both forms.
+template <bool X2>
+static cudaError_t launch_pairs(const bz_modes *m, const double2 *fhat, void *Qhat, int64_t n, cudaStream_t st) {
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
     gd.nitems = 1;
-    const int S = launch_split(ctas_for(m->variant64, n), m->bal64, m->task64_split);
-    fill_item(gd.item[0], m, m->w64, S > 1 ? m->task64_split[split_index(S)] : m->task64, m->rowmax64, fhat, Qhat, n, S);
-    gd.tile_start[0] = 0;
-    gd.tile_start[1] = ctas_for(m->variant64, n) * S;
+    const int64_t ctas = ctas_for(m->variant64, n);
+    const int S = launch_split(ctas, m->bal64, m->task64_split, true);
+    fill_item(gd.item[0], m, X2 ? static_cast<const void *>(m->wx2) : m->w64,
+              S > 1 ? m->task64_split[split_index(S)] : m->task64, m->rowmax64, fhat, Qhat, n, S);
+    gd.tile_start[1] = ctas * S;
     const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, m->variant64);
-    if (m->variant64 == kFp64Variants[0]) return launch_instance<double, 4, 16, 16>(gd, sm, st);
-    if (m->variant64 == kFp64Variants[1]) return launch_instance<double, 2, 8, 8>(gd, sm, st);
-    if (m->variant64 == kFp64Variants[2]) return launch_instance<double, 2, 8, 4>(gd, sm, st);
+    if (m->variant64 == kFp64Variants[0]) return launch_pair<X2, 4, 8, 8>(gd, sm, st);
+    if (m->variant64 == kFp64Variants[1]) return launch_pair<X2, 4, 8, 4>(gd, sm, st);
+    if (m->variant64 == kFp64Variants[2]) return launch_pair<X2, 2, 8, 8>(gd, sm, st);
     return cudaErrorInvalidValue;
 }
 
-// FP32X2 form on the FP64 layout (the entries of kFp64Variants).
-bool modesum_x2_available(const bz_modes *m) { return m->wx2 != nullptr && m->variant64 >= 0; }
-
-template <int RR, int WARPS, int CELLS>
-static cudaError_t launch_x2_instance(const bz_modes *m, const double2 *fhat, float2 *Qhat, int64_t n, size_t sm,
-                                      cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(modesum_x2_kernel<RR, WARPS, CELLS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    const GridView &gv = m->g->v;
-    const int64_t ctas = ctas_for(m->variant64, n);
-    const int S = launch_split(ctas, m->bal64, m->task64_split);
-    modesum_x2_kernel<RR, WARPS, CELLS><<<(unsigned)(ctas * S), WARPS * 32, sm, st>>>(
-        fhat, Qhat, m->wx2, S > 1 ? m->task64_split[split_index(S)] : m->task64, gv.h, gv.M, (int)gv.nhalf, m->rowmax64,
-        n, S);
-    return cudaGetLastError();
+cudaError_t launch_modesum64(const bz_modes *m, const double2 *fhat, double2 *Qhat, int64_t n, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    if (!m->w64) return cudaErrorInvalidValue;
+    return launch_pairs<false>(m, fhat, Qhat, n, st);
 }
+
+bool modesum_x2_available(const bz_modes *m) { return m->wx2 != nullptr && m->variant64 >= 0; }
 
 cudaError_t launch_modesum_x2(const bz_modes *m, const double2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     if (!modesum_x2_available(m)) return cudaErrorInvalidValue;
-    // the FP64 layout's shared memory: spectra of 16 bytes per value (hi, lo
-    // parts of FP32 instead of one double) and weight rows of 8-byte slots
-    const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, m->variant64);
-    if (m->variant64 == kFp64Variants[0]) return launch_x2_instance<4, 16, 16>(m, fhat, Qhat, n, sm, st);
-    if (m->variant64 == kFp64Variants[1]) return launch_x2_instance<2, 8, 8>(m, fhat, Qhat, n, sm, st);
-    if (m->variant64 == kFp64Variants[2]) return launch_x2_instance<2, 8, 4>(m, fhat, Qhat, n, sm, st);
-    return cudaErrorInvalidValue;
+    return launch_pairs<true>(m, fhat, Qhat, n, st);
 }
 
 // A launch over n cells ends with a partial wave of tiles; the SMs that run
@@ -1524,7 +1617,7 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
     if (sv != m->variant) return launch_variant(m, sv, fhat, Qhat, n, st);
     if (kVariants[sv].rows > 1)
         return launch_variant(m, sv, fhat, Qhat, n, st,
-                              launch_split(ctas_for(sv, n), m->var_bal[sv], m->var_task_split[sv]));
+                              launch_split(ctas_for(sv, n), m->var_bal[sv], m->var_task_split[sv], false));
     int tv = -1, ts = 1;
     const int64_t nm = modesum32_split(m, n, &tv, &ts);
     const int v = m->variant;
@@ -1578,7 +1671,7 @@ cudaError_t launch_modesum32_group(const bz_modes *const *ms, const float2 *cons
     for (int i = 0; i < count; ++i) whole += ctas_for(v, n[i]);
     for (int i = 0; i < count; ++i) {
         if (ms[i]->variant != v) return cudaErrorInvalidValue;
-        const int S = kVariants[v].rows > 1 ? launch_split(whole, ms[0]->var_bal[v], ms[0]->var_task_split[v]) : 1;
+        const int S = kVariants[v].rows > 1 ? launch_split(whole, ms[0]->var_bal[v], ms[0]->var_task_split[v], false) : 1;
         fill_item(gd.item[i], ms[i], ms[i]->var_W[v], S > 1 ? ms[i]->var_task_split[v][split_index(S)] : ms[i]->var_task[v],
                   ms[i]->var_rowmax[v], fhat[i], Qhat[i], n[i], S);
         gd.tile_start[i] = ctas;
