@@ -6,8 +6,10 @@
 
 #include <algorithm>
 #include <atomic>
+#include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "bz_internal.h"
@@ -49,6 +51,20 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
 
 void dev_free(void *p) {
     if (p && cudaFree(p) == cudaSuccess) g_live_blocks.fetch_sub(1);
+}
+
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, size_t> allowed;   // never lowered: other threads may rely on it
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    size_t &have = allowed[{kernel, dev}];
+    if (bytes <= have) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) have = bytes;
+    return e;
 }
 
 int grid_create(int dim, int N, double L, bz_grid **out);
@@ -260,7 +276,8 @@ int phase_forward(const bz_modes *m, int precision, const void *f, void *fh, int
     return BZ_OK;
 }
 
-int phase_modesum(const bz_modes *m, int precision, const void *fh, void *qh, int64_t n, cudaStream_t st) {
+int phase_modesum(const bz_modes *m, int precision, const void *fh, void *qh, int64_t n, cudaStream_t st,
+                  bool pdl = false) {
     const GridView &v = m->g->v;
     if (precision == BZ_FP32X2) {
         BZ_LAUNCH("modesum_x2", st,
@@ -287,7 +304,7 @@ int phase_modesum(const bz_modes *m, int precision, const void *fh, void *qh, in
         // whole waves on the selected variant, the last partial wave split
         // (one launch), or on the 16-cell variant (a second launch)
         BZ_LAUNCH("modesum_f32", st,
-                  launch_modesum32(m, static_cast<const float2 *>(fh), static_cast<float2 *>(qh), n, st),
+                  launch_modesum32(m, static_cast<const float2 *>(fh), static_cast<float2 *>(qh), n, st, pdl),
                   "collide: mode sum");
     } else {
         BZ_LAUNCH("modesum_f32_generic", st,
@@ -299,7 +316,7 @@ int phase_modesum(const bz_modes *m, int precision, const void *fh, void *qh, in
 }
 
 int phase_inverse(const bz_modes *m, int precision, int flags, const void *qh, void *Q, const void *P, int64_t n,
-                  cudaStream_t st) {
+                  cudaStream_t st, bool pdl = false) {
     const bz_grid *g = m->g;
     const GridView &v = g->v;
     InvEpilogue ep;
@@ -319,7 +336,7 @@ int phase_inverse(const bz_modes *m, int precision, int flags, const void *qh, v
     } else if (m->tile_dft) {
         BZ_LAUNCH("dft_inverse_f32", st,
                   launch_dft32_inverse_tile(v, static_cast<const float2 *>(qh), static_cast<float *>(Q), n, m->scale,
-                                            g->cinv, ep, st),
+                                            g->cinv, ep, st, pdl),
                   "collide: inverse DFT");
     } else {
         BZ_LAUNCH("dft_inverse_f32_generic", st,
@@ -353,9 +370,13 @@ int collide_chain(const bz_modes *m, int precision, int flags, const void *f, vo
     Scratch s;
     if (!ext) BZ_TRY(s.alloc(bytes, st), "collide: scratch");
     char *fh = static_cast<char *>(ext ? ext : s.p), *qh = fh + spectrum_bytes(m, precision, n);
+    // a batch of few CTAs is bound by latency: its mode sum and inverse transform
+    // start their prologues while the kernel before them ends (64 cells of
+    // 16^2: 20.2 -> 15.0 us a call); larger ones gain nothing from it
+    const bool pdl = precision == BZ_FP32 && m->tile_dft && n <= 1024;
     int rc = phase_forward(m, precision, f, fh, n, st);
-    if (!rc) rc = phase_modesum(m, precision, fh, qh, n, st);
-    if (!rc) rc = phase_inverse(m, precision, flags, qh, Q, P, n, st);
+    if (!rc) rc = phase_modesum(m, precision, fh, qh, n, st, pdl);
+    if (!rc) rc = phase_inverse(m, precision, flags, qh, Q, P, n, st, pdl);
     return rc;
 }
 

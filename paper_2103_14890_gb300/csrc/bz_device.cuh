@@ -53,6 +53,32 @@ template <int K> __device__ __forceinline__ void block_sum(double (&v)[K], doubl
     __syncthreads();
 }
 
+// Programmatic dependent launch.  griddep_launch: the next kernel of the stream,
+// if launched with the attribute (launch_after), may start its prologue once
+// every CTA of this grid has called it; griddep_wait: returns when the kernel
+// before has completed and its writes are visible (at once without the
+// attribute).  A kernel launched that way waits before it touches anything the
+// kernels before it read or write.
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch `kernel`; pdl: as a programmatic dependent of the kernel before it.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
+                         A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Velocity of flat grid index `idx` along dimension i (j_1 slowest).
 __device__ __forceinline__ double grid_velocity(int64_t idx, int i, int dim, int N, double L,
                                                 double dv) {

@@ -31,6 +31,11 @@ template <typename X> cudaError_t dev_malloc(X **p, size_t bytes) {
 void dev_free(void *p);
 bool alloc_fault_due();
 
+// Let `kernel` launch with `bytes` of dynamic shared memory on the current
+// device: the attribute call, made only when the kernel needs more than it has
+// been allowed so far (it costs about half a microsecond of every launch).
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes);
+
 // Device error word (one per device context), latched by kernels.
 enum DeviceError : int { kDevOk = 0, kDevNonFinite = 1, kDevTimeout = 2 };
 
@@ -77,6 +82,11 @@ struct bz_modes {
     int var_rowmax[kModesumVariants];
     int variant;          // index of the selected variant
     int variant_fixed;    // 1: chosen by BZ_MODESUM_VARIANT (no last-wave split)
+    float *small_W;       // weight stream and task tables of the small-launch variant (two outputs per thread)
+    int *small_task;
+    int *small_task_split[kSplitTables];
+    float small_bal[kSplitTables + 1];
+    int small_rowmax;
     void *w64;            // FP64 weight stream and task table, null if unused
     int *task64;
     int *task64_split[kSplitTables];
@@ -219,7 +229,7 @@ bool dft32_tile_supported(const GridView &g, bool fp64);
 int dft32_setup();   // twiddles on the current device
 cudaError_t launch_dft32_forward_tile(const GridView &g, const float *f, float2 *fhat, int64_t n, cudaStream_t st);
 cudaError_t launch_dft32_inverse_tile(const GridView &g, const float2 *Qhat, float *Q, int64_t n, double scale,
-                                      const double *cinv, const InvEpilogue &ep, cudaStream_t st);
+                                      const double *cinv, const InvEpilogue &ep, cudaStream_t st, bool pdl = false);
 cudaError_t launch_dft64_forward_tile(const GridView &g, const double *f, double2 *fhat, int64_t n,
                                       cudaStream_t st);
 cudaError_t launch_dft64_forward_tile_f32in(const GridView &g, const float *f, double2 *fhat, int64_t n,
@@ -244,7 +254,8 @@ struct Mode32Group {
     Mode32Item item[kMaxGroup];
 };
 bool modesum32_available(const bz_modes *m);
-cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st);
+cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st,
+                             bool pdl = false);
 int64_t modesum32_split(const bz_modes *m, int64_t n, int *tail_v, int *tail_split);
 // Cells one SM holds at a time in the handle's FP32 mode-sum kernel (CTAs per
 // SM x cells per CTA; 32 where the register-blocked kernels do not serve it).

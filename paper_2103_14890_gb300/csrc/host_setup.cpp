@@ -353,6 +353,9 @@ void modes_destroy(bz_modes *m) {
     free(m->h_fast);
     dev_free(m->d_F64);
     dev_free(m->d_F32);
+    dev_free(m->small_W);
+    dev_free(m->small_task);
+    for (int k = 0; k < kSplitTables; ++k) dev_free(m->small_task_split[k]);
     dev_free(m->w64);
     dev_free(m->wx2);
     dev_free(m->task64);

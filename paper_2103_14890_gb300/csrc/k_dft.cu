@@ -223,7 +223,7 @@ cudaError_t forward(const GridView &g, const typename C2<T>::type *E, const TI *
     if (n <= 0) return cudaSuccess;
     size_t sm = fwd_smem<T>(g);
     cudaError_t e =
-        cudaFuncSetAttribute(dft_forward_kernel<T, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_dynamic_smem((const void *)dft_forward_kernel<T, TI>, sm);
     if (e != cudaSuccess) return e;
     dft_forward_kernel<T, TI><<<(unsigned)n, kThreads, sm, st>>>(g, E, f, fhat);
     return cudaGetLastError();
@@ -235,7 +235,7 @@ cudaError_t inverse(const GridView &g, const typename C2<T>::type *E, const type
                     cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     size_t sm = inv_smem<T>(g);
-    cudaError_t e = cudaFuncSetAttribute(dft_inverse_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_dynamic_smem((const void *)dft_inverse_kernel<T>, sm);
     if (e != cudaSuccess) return e;
     Cinv ci;
     for (int i = 0; i < 25; ++i) ci.v[i] = cinv[i];

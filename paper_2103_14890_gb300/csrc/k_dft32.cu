@@ -115,6 +115,7 @@ fft_fwd32_kernel(const TI *__restrict__ f, typename C2<T>::type *__restrict__ fh
     constexpr int NW = C / 2, P = C + 1;                // warps; cell pitch of the shared rows
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V2 *As = reinterpret_cast<V2 *>(smem_raw);        // [H][N][P]
+    griddep_launch();
     const int64_t tile = blockIdx.x / (32 / C);
     const int sub = (int)(blockIdx.x % (32 / C)) * C;   // first cell of this CTA within the tile
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -181,6 +182,7 @@ fft_inv32_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ 
     constexpr int NW = C / 2, P = C + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V2 *Bs = reinterpret_cast<V2 *>(smem_raw);        // [H][N][P]
+    griddep_wait();
     const int64_t tile = blockIdx.x / (32 / C);
     const int sub = (int)(blockIdx.x % (32 / C)) * C;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -271,6 +273,7 @@ fftg_fwd_kernel(const TI *__restrict__ f, typename C2<T>::type *__restrict__ fha
     constexpr int H = N / 2, M = N - 1, NV = N * N, P = C + 1, NT = C * threads_per_cell<N>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V2 *As = reinterpret_cast<V2 *>(smem_raw);        // [H][N][P], rows RS apart
+    griddep_launch();
     constexpr int RS = row_pitch<N, P>();
     const int64_t tile = blockIdx.x / (32 / C);
     const int sub = (int)(blockIdx.x % (32 / C)) * C;
@@ -409,6 +412,7 @@ fftg_inv_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ Q
     constexpr int RS = row_pitch<N, P>();
     V2 *Bs = reinterpret_cast<V2 *>(smem_raw);        // [H][N][P], rows RS apart, then NT/32 * 4 doubles
     double *red = reinterpret_cast<double *>(Bs + (size_t)H * RS);
+    griddep_wait();
     const int64_t tile = blockIdx.x / (32 / C);
     const int sub = (int)(blockIdx.x % (32 / C)) * C;
     // ---- stage 1: thread = (cell, row k1); inverse complex transform over k2 ----
@@ -490,14 +494,12 @@ cudaError_t fwd_tile(const TI *f, typename C2<T>::type *fhat, int64_t n, cudaStr
     cudaError_t e;
     if constexpr (N == 16 || N == 32) {
         const size_t sm = fft_smem<T, N, C>();
-        e = cudaFuncSetAttribute(fft_fwd32_kernel<T, N, C, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
+        e = allow_dynamic_smem((const void *)fft_fwd32_kernel<T, N, C, TI>, sm);
         if (e != cudaSuccess) return e;
         fft_fwd32_kernel<T, N, C, TI><<<grid, C * 16, sm, st>>>(f, fhat, n);
     } else {
         const size_t sm = fftg_smem<T, N, C>();
-        e = cudaFuncSetAttribute(fftg_fwd_kernel<T, N, C, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
+        e = allow_dynamic_smem((const void *)fftg_fwd_kernel<T, N, C, TI>, sm);
         if (e != cudaSuccess) return e;
         fftg_fwd_kernel<T, N, C, TI><<<grid, C * threads_per_cell<N>(), sm, st>>>(f, fhat, n);
     }
@@ -506,25 +508,24 @@ cudaError_t fwd_tile(const TI *f, typename C2<T>::type *fhat, int64_t n, cudaStr
 
 template <typename T, int N>
 cudaError_t inv_tile(const GridView &g, const typename C2<T>::type *Qhat, T *Q, int64_t n, double scale,
-                     const Cinv &ci, const InvEpilogue &ep, cudaStream_t st) {
+                     const Cinv &ci, const InvEpilogue &ep, cudaStream_t st, bool pdl) {
     constexpr int C = ifft_cells<T, N>();
     const unsigned grid = (unsigned)(((n + 31) / 32) * (32 / C));
     const T *P = static_cast<const T *>(ep.P);
     cudaError_t e;
     if constexpr (N == 16 || N == 32) {
         const size_t sm = fft_smem<T, N, C>();
-        e = cudaFuncSetAttribute(fft_inv32_kernel<T, N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_dynamic_smem((const void *)fft_inv32_kernel<T, N, C>, sm);
         if (e != cudaSuccess) return e;
-        fft_inv32_kernel<T, N, C><<<grid, C * 16, sm, st>>>(Qhat, Q, (T)scale, ci, ep.conserve, P, (T)g.L, (T)g.dv,
-                                                             n);
+        return launch_after(fft_inv32_kernel<T, N, C>, grid, C * 16, sm, st, pdl, Qhat, Q, scale, ci, ep.conserve, P,
+                            g.L, g.dv, n);
     } else {
         const size_t sm = fftg_smem<T, N, C>();
-        e = cudaFuncSetAttribute(fftg_inv_kernel<T, N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_dynamic_smem((const void *)fftg_inv_kernel<T, N, C>, sm);
         if (e != cudaSuccess) return e;
-        fftg_inv_kernel<T, N, C><<<grid, C * threads_per_cell<N>(), sm, st>>>(Qhat, Q, (T)scale, ci, ep.conserve,
-                                                                             P, (T)g.L, (T)g.dv, n);
+        return launch_after(fftg_inv_kernel<T, N, C>, grid, C * threads_per_cell<N>(), sm, st, pdl, Qhat, Q, scale, ci,
+                            ep.conserve, P, g.L, g.dv, n);
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -741,8 +742,7 @@ fft3_inv_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ Q
 
 template <typename T, typename TI = T>
 cudaError_t fwd3(const TI *f, typename C2<T>::type *fhat, int64_t n, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(fft3_fwd_kernel<T, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Fft3<T>::smem);
+    cudaError_t e = allow_dynamic_smem((const void *)fft3_fwd_kernel<T, TI>, Fft3<T>::smem);
     if (e != cudaSuccess) return e;
     fft3_fwd_kernel<T, TI><<<(unsigned)((n + 31) / 32 * (32 / Fft3<T>::C)), 256, Fft3<T>::smem, st>>>(f, fhat, n);
     return cudaGetLastError();
@@ -751,8 +751,7 @@ cudaError_t fwd3(const TI *f, typename C2<T>::type *fhat, int64_t n, cudaStream_
 template <typename T>
 cudaError_t inv3(const GridView &g, const typename C2<T>::type *Qhat, T *Q, int64_t n, double scale, const Cinv &ci,
                  const InvEpilogue &ep, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(fft3_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Fft3<T>::smem);
+    cudaError_t e = allow_dynamic_smem((const void *)fft3_inv_kernel<T>, Fft3<T>::smem);
     if (e != cudaSuccess) return e;
     fft3_inv_kernel<T><<<(unsigned)((n + 31) / 32 * (32 / Fft3<T>::C)), 256, Fft3<T>::smem, st>>>(
         Qhat, Q, (T)scale, ci, ep.conserve, static_cast<const T *>(ep.P), (T)g.L, (T)g.dv, n);
@@ -776,18 +775,18 @@ cudaError_t fwd_any(const GridView &g, const TI *f, typename C2<T>::type *fhat, 
 
 template <typename T>
 cudaError_t inv_any(const GridView &g, const typename C2<T>::type *Qhat, T *Q, int64_t n, double scale,
-                    const double *cinv, const InvEpilogue &ep, cudaStream_t st) {
+                    const double *cinv, const InvEpilogue &ep, cudaStream_t st, bool pdl = false) {
     if (n <= 0) return cudaSuccess;
     Cinv ci;
     for (int i = 0; i < 25; ++i) ci.v[i] = cinv[i];
     if (g.dim == 3) return g.N == 16 ? inv3<T>(g, Qhat, Q, n, scale, ci, ep, st) : cudaErrorInvalidValue;
     if constexpr (sizeof(T) == 4)
-        if (g.N == 64) return inv_tile<T, 64>(g, Qhat, Q, n, scale, ci, ep, st);
+        if (g.N == 64) return inv_tile<T, 64>(g, Qhat, Q, n, scale, ci, ep, st, pdl);
     switch (g.N) {
-        case 16: return inv_tile<T, 16>(g, Qhat, Q, n, scale, ci, ep, st);
-        case 24: return inv_tile<T, 24>(g, Qhat, Q, n, scale, ci, ep, st);
-        case 32: return inv_tile<T, 32>(g, Qhat, Q, n, scale, ci, ep, st);
-        case 48: return inv_tile<T, 48>(g, Qhat, Q, n, scale, ci, ep, st);
+        case 16: return inv_tile<T, 16>(g, Qhat, Q, n, scale, ci, ep, st, pdl);
+        case 24: return inv_tile<T, 24>(g, Qhat, Q, n, scale, ci, ep, st, pdl);
+        case 32: return inv_tile<T, 32>(g, Qhat, Q, n, scale, ci, ep, st, pdl);
+        case 48: return inv_tile<T, 48>(g, Qhat, Q, n, scale, ci, ep, st, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -819,8 +818,8 @@ cudaError_t launch_dft64_forward_tile_f32in(const GridView &g, const float *f, d
     return fwd_any<double, float>(g, f, fhat, n, st);
 }
 cudaError_t launch_dft32_inverse_tile(const GridView &g, const float2 *Qhat, float *Q, int64_t n, double scale,
-                                      const double *cinv, const InvEpilogue &ep, cudaStream_t st) {
-    return inv_any<float>(g, Qhat, Q, n, scale, cinv, ep, st);
+                                      const double *cinv, const InvEpilogue &ep, cudaStream_t st, bool pdl) {
+    return inv_any<float>(g, Qhat, Q, n, scale, cinv, ep, st, pdl);
 }
 cudaError_t launch_dft64_inverse_tile(const GridView &g, const double2 *Qhat, double *Q, int64_t n, double scale,
                                       const double *cinv, const InvEpilogue &ep, cudaStream_t st) {

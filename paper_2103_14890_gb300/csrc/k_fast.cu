@@ -249,8 +249,7 @@ cudaError_t launch_fast_n(const GridView &g, const typename C2<T>::type *fh, typ
     constexpr int C = FastShape<T, N>::C;
     const int64_t blocks = (n + C - 1) / C;
     if (blocks > INT_MAX) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fast_collide_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+    cudaError_t e = allow_dynamic_smem((const void *)fast_collide_kernel<T, N>, sm);
     if (e != cudaSuccess) return e;
     fast_collide_kernel<T, N><<<(unsigned)blocks, FastShape<T, N>::NT, sm, st>>>(fh, qh, coef, nconv, g.nhalf, n);
     return cudaGetLastError();

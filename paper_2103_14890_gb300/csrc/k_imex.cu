@@ -286,7 +286,7 @@ cudaError_t stage(const GridView &g, const StageCoef &c, const T *fn, T *F, cons
     }
     const size_t sm = sizeof(double) * (32 * 5 + g.N) + sizeof(T) * ((size_t)g.nv + 3 * g.N);
     auto *kern = g.dim == 2 ? imex_stage_kernel<T, 2> : imex_stage_kernel<T, 3>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n, kThreads, sm, st>>>(g, c, fn, F, G, P, Lres, stride);
     return cudaGetLastError();

@@ -72,12 +72,14 @@ struct Variant {
 constexpr int kNumVariants = kModesumVariants;   // FP32 variants (timed by the autotuner)
 // entries 0..9: the FP32 variants; entries 10..12: layouts of the FP64 and FP32X2
 // forms (16 bytes per spectrum value): 8-cell tiles, 4-cell tiles for 16^3, and
-// two outputs per thread for grids of fewer than 8 points
-constexpr Variant kVariants[kNumVariants + 3] = {
+// two outputs per thread for grids of fewer than 8 points; entry 13: the paired
+// 16-cell FP32 variants with two outputs per thread, for small launches
+constexpr int kSmallVariant = kNumVariants + 3;
+constexpr Variant kVariants[kNumVariants + 4] = {
     {8, 16, 32, 1, 0, 0, 1, 1}, {4, 32, 32, 1, 0, 0, 1, 1}, {4, 16, 16, 1, 0, 0, 1, 1}, {8, 12, 8, 1, 0, 1, 2, 2},
     {4, 16, 32, 2, 1, 0, 1, 1}, {8, 12, 32, 1, 0, 1, 1, 1}, {8, 16, 32, 1, 0, 1, 1, 1}, {8, 16, 16, 1, 0, 1, 2, 1},
     {8, 8, 16, 1, 0, 1, 2, 1},  {8, 4, 16, 1, 0, 1, 2, 1},  {4, 8, 8, 1, 0, 1, 2, 2},   {4, 8, 4, 1, 0, 1, 2, 4},
-    {2, 8, 8, 1, 0, 1, 2, 2}};
+    {2, 8, 8, 1, 0, 1, 2, 2},   {2, 16, 16, 1, 0, 1, 2, 1}};
 
 // lane groups splitting a task's outputs, and outputs per task (RT)
 constexpr int variant_groups(int v) {
@@ -607,9 +609,15 @@ __device__ __forceinline__ void block_pq(float2 (&win)[2 * RR], const float2 *__
         // all products U first, then the P and then the Q updates: no FMA
         // waits on the multiply issued just before it
         float wv[RR];
+        if constexpr (RR == 2) {
+            const float2 w2 = *reinterpret_cast<const float2 *>(wb + s * WS);
+            wv[0] = w2.x;
+            wv[1] = w2.y;
+        } else {
 #pragma unroll
-        for (int q = 0; q < RR; q += 4)
-            if (!RAMP || q < s) load_w4(wv + q, wb + s * WS + q);   // outputs q .. q + 3 before the ramp
+            for (int q = 0; q < RR; q += 4)
+                if (!RAMP || q < s) load_w4(wv + q, wb + s * WS + q);   // outputs q .. q + 3 before the ramp
+        }
         float2 u[RR];
 #pragma unroll
         for (int r = 0; r < RR; ++r)
@@ -669,7 +677,7 @@ __device__ __forceinline__ void row_pass_pq(const float2 *__restrict__ rowl, con
 // of the task.  Consecutive rows lie an odd number of modes apart, so the four
 // 64-byte groups of a load fall two and two into the halves of the banks.
 template <int RR, int WARPS, int CELLS>
-__global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 1) modesum_pq_kernel(const Mode32Group gd) {
+__global__ void __launch_bounds__(WARPS * 32, RR == 2 ? 2 : WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 1) modesum_pq_kernel(const Mode32Group gd) {
     constexpr bool PAIRED = (CELLS <= 16);
     constexpr int ROWS = PAIRED ? 16 / CELLS : 1;   // row pairs at a time
     constexpr int G = 32 / CELLS;                // CTAs per 32-cell tile
@@ -691,8 +699,6 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
     const int sub = (int)(cta % G);
     float2 *Fs = reinterpret_cast<float2 *>(smem16);                 // [kPad + nhalf + kPad][CELLS]
     float *wsm = reinterpret_cast<float *>(Fs + (size_t)(nhalf + 2 * kPad) * CELLS);
-    stage_spectrum<float2, CELLS>(smem16, fhat, tile, sub, nhalf, M, false);
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cell = lane % CELLS;
     const bool upper = PAIRED && (lane / CELLS) % 2 == 1;            // runs every task mirrored
@@ -702,6 +708,17 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
     const int NW = WARPS * ip.split;                 // one phase: every task reads this spectrum
     int t = tasks[part * WARPS + warp], tend = tasks[part * WARPS + warp + 1];
     const TaskRec *trec = reinterpret_cast<const TaskRec *>(tasks + 2 * NW + 1);
+    bool staged = false;
+    if constexpr (RR == 2) {
+        // small launches: the first task's first weights travel while the
+        // kernel before this one ends and the spectrum is staged
+        griddep_launch();
+        staged = t < tend;
+        if (staged) stage_row(wbuf0, W + trec[t].woff, ROWS * trec[t].rowf * (int)sizeof(float), lane);
+        griddep_wait();
+    }
+    stage_spectrum<float2, CELLS>(smem16, fhat, tile, sub, nhalf, M, false);
+    __syncthreads();
     const float2 *F0 = Fs + (size_t)(kPad + h) * CELLS + cell;
     const bool valid = tile * 32 + sub * CELLS + cell < ip.n;
     float2 *const qt = Qhat + tile * (int64_t)nhalf * 32 + sub * CELLS + cell;
@@ -715,13 +732,13 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS <= 4 ? 3 : WARPS <= 8 ? 2 : 
 #pragma unroll
         for (int r = 0; r < RR; ++r) hi[r] = lo[r] = P[r] = Q[r] = make_float2(0.f, 0.f);
         const int mbase0 = tk.k20 - tk.l2lo - (RR - 1);
-        stage_row(wbuf0, wsrc, ROWS * rowf * (int)sizeof(float), lane);
-        const int nrows = tk.nrows / ROWS;
+        const int nrows = tk.nrows / ROWS, rowb = ROWS * rowf * (int)sizeof(float);
+        if (!staged) stage_row(wbuf0, wsrc, rowb, lane);
+        staged = false;
         for (int i = 0; i < nrows; ++i) {
             const float *wcur = ((i & 1) ? wbuf1 : wbuf0) + rgrp * rowf;
             if (i + 1 < nrows) {
-                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * (ROWS * rowf),
-                          ROWS * rowf * (int)sizeof(float), lane);
+                stage_row((i & 1) ? wbuf0 : wbuf1, wsrc + (size_t)(i + 1) * (ROWS * rowf), rowb, lane);
                 cp_async_wait<1>();
             } else {
                 cp_async_wait<0>();
@@ -1378,31 +1395,31 @@ bool modesum32_available(const bz_modes *m) { return m->d_W32 != nullptr; }
 
 template <typename T, int RR, int WARPS, int CELLS, bool RTDIR = false>
 static cudaError_t launch_instance(const Mode32Group &gd, size_t sm, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(modesum32_kernel<T, RR, WARPS, CELLS, RTDIR>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_dynamic_smem((const void *)modesum32_kernel<T, RR, WARPS, CELLS, RTDIR>, sm);
     if (e != cudaSuccess) return e;
     modesum32_kernel<T, RR, WARPS, CELLS, RTDIR><<<(unsigned)gd.tile_start[gd.nitems], WARPS * 32, sm, st>>>(gd);
     return cudaGetLastError();
 }
 
 template <int RR, int WARPS, int CELLS>
-static cudaError_t launch_pq(const Mode32Group &gd, size_t sm, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(modesum_pq_kernel<RR, WARPS, CELLS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+static cudaError_t launch_pq(const Mode32Group &gd, size_t sm, cudaStream_t st, bool pdl = false) {
+    cudaError_t e = allow_dynamic_smem((const void *)modesum_pq_kernel<RR, WARPS, CELLS>, sm);
     if (e != cudaSuccess) return e;
+    if constexpr (RR == 2)
+        return launch_after(modesum_pq_kernel<RR, WARPS, CELLS>, (unsigned)gd.tile_start[gd.nitems], WARPS * 32, sm, st,
+                            pdl, gd);
     modesum_pq_kernel<RR, WARPS, CELLS><<<(unsigned)gd.tile_start[gd.nitems], WARPS * 32, sm, st>>>(gd);
     return cudaGetLastError();
 }
 
-static cudaError_t launch_group(const Mode32Group &gd, int v, size_t sm, cudaStream_t st) {
+static cudaError_t launch_group(const Mode32Group &gd, int v, size_t sm, cudaStream_t st, bool pdl = false) {
     switch (v) {
         case 0: return launch_instance<float, 8, 16, 32, true>(gd, sm, st);
         case 1: return launch_instance<float, 4, 32, 32>(gd, sm, st);
         case 2: return launch_instance<float, 4, 16, 16>(gd, sm, st);
         case 3: return launch_pq<8, 12, 8>(gd, sm, st);
         case 4: {
-            cudaError_t e = cudaFuncSetAttribute(modesum_p2_kernel<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)sm);
+            cudaError_t e = allow_dynamic_smem((const void *)modesum_p2_kernel<4, 16>, sm);
             if (e != cudaSuccess) return e;
             modesum_p2_kernel<4, 16><<<(unsigned)gd.tile_start[gd.nitems], 16 * 32, sm, st>>>(gd);
             return cudaGetLastError();
@@ -1412,6 +1429,7 @@ static cudaError_t launch_group(const Mode32Group &gd, int v, size_t sm, cudaStr
         case 7: return launch_pq<8, 16, 16>(gd, sm, st);
         case 8: return launch_pq<8, 8, 16>(gd, sm, st);
         case 9: return launch_pq<8, 4, 16>(gd, sm, st);
+        case kSmallVariant: return launch_pq<2, 16, 16>(gd, sm, st, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1495,8 +1513,7 @@ static int launch_split(int64_t ctas, const float (&bal)[kSplitTables + 1], int 
 
 template <bool X2, int RR, int WARPS, int CELLS>
 static cudaError_t launch_pair(const Mode32Group &gd, size_t sm, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(modesum_pair_kernel<X2, RR, WARPS, CELLS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_dynamic_smem((const void *)modesum_pair_kernel<X2, RR, WARPS, CELLS>, sm);
     if (e != cudaSuccess) return e;
     modesum_pair_kernel<X2, RR, WARPS, CELLS><<<(unsigned)gd.tile_start[1], WARPS * 32, sm, st>>>(gd);
     return cudaGetLastError();
@@ -1600,6 +1617,25 @@ static int small_batch_variant(const bz_modes *m, int64_t n) {
     return v;
 }
 
+// A launch that would give less than one CTA to every SM is bound by the chain
+// of one warp's tasks.  The small variant runs the paired 16-cell variants' sums
+// (the same terms in the same order, bit-identical results) with two outputs
+// per thread: four times the tasks, a third of the chain each, spread over up
+// to eight CTAs per tile.  Its steps do fewer FMAs per load, so it is taken where
+// the loads of the most loaded warps say that it is faster by a tenth.  64 cells
+// of 16^2: 14.6 -> 12.5 us, of 32^2: 82 -> 31 us, of 48^2: 375 -> 93 us.  Returns the CTAs per
+// tile, 0 where the other variants are better.
+static int small_split(const bz_modes *m, int v, int64_t n) {
+    const Variant &k = kVariants[v];
+    if (m->variant_fixed || !m->small_W || !k.pq || k.cells != 16 || k.R != 8) return 0;
+    const int64_t ctas = ctas_for(kSmallVariant, n), sms = sm_count();
+    if (ctas > sms) return 0;
+    const int S = launch_split(ctas, m->small_bal, m->small_task_split, true);
+    const int ix = S > 1 ? split_index(S) + 1 : 0;
+    const double t = std::max((double)((ctas * S + sms - 1) / sms) * m->small_bal[0] / S, (double)m->small_bal[ix]);
+    return t < 0.9 * m->var_bal[v][0] ? S : 0;
+}
+
 bool modesum32_small_batches_fast(const bz_modes *m) {
     return m->method == 0 && modesum32_available(m) && small_batch_variant(m, 1) != m->variant;
 }
@@ -1611,9 +1647,19 @@ int modesum32_wave_cells_per_sm(const bz_modes *m) {
 
 // One launch for the whole batch: the main part (one tile per CTA) and the
 // last partial wave (split tiles, or the 16-cell variant) as two items.
-cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st) {
+cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st,
+                             bool pdl) {
     if (n <= 0) return cudaSuccess;
     const int sv = small_batch_variant(m, n);
+    if (const int S = small_split(m, sv, n)) {
+        Mode32Group gd;
+        memset(&gd, 0, sizeof gd);
+        gd.nitems = 1;
+        fill_item(gd.item[0], m, m->small_W, S > 1 ? m->small_task_split[split_index(S)] : m->small_task,
+                  m->small_rowmax, fhat, Qhat, n, S);
+        gd.tile_start[1] = ctas_for(kSmallVariant, n) * S;
+        return launch_group(gd, kSmallVariant, smem_bytes<float>(m->g->v, m->small_rowmax, kSmallVariant), st, pdl);
+    }
     if (sv != m->variant) return launch_variant(m, sv, fhat, Qhat, n, st);
     if (kVariants[sv].rows > 1)
         return launch_variant(m, sv, fhat, Qhat, n, st,
@@ -1808,7 +1854,18 @@ int modes_build_fp32_tables(bz_modes *m) {
         }
         if (rc) return rc;
     }
-    // FP64 tables (16-cell tiles) where the double spectrum fits shared memory
+    // the small variant's tables beside those of the 16-warp paired variant
+    m->small_W = nullptr;
+    m->small_task = nullptr;
+    for (int k = 0; k < kSplitTables; ++k) m->small_task_split[k] = nullptr;
+    if (m->var_W[7]) {
+        void *w = nullptr;
+        if (build_variant<float>(m, kSmallVariant, rc, &w, &m->small_task, &m->small_rowmax, nullptr,
+                                 m->small_task_split, m->small_bal))
+            m->small_W = static_cast<float *>(w);
+        if (rc) return rc;
+    }
+    // FP64 tables where the double spectrum fits shared memory
     m->w64 = nullptr;
     m->task64 = nullptr;
     m->rowmax64 = 0;
