@@ -466,6 +466,7 @@ int run_stage(const bz_modes *m, const Tableau &t, int l, int model, double dt, 
     c.dt = dt;
     c.eps = eps;
     c.nuf = (model == BZ_BOLTZMANN) ? m->penalty : 1.0;
+    c.coef = dt * c.all * c.nuf / eps;
     const bool f0 = in_step && l == 0 && c.all == 0.0;     // F_0 = f^n
     const bool needG = model == BZ_BOLTZMANN && explicit_used(t, l);
     c.store_F = f0 ? 0 : 1;

@@ -25,6 +25,24 @@ template <typename V> __device__ __forceinline__ void cmac(V &acc, V a, V b) {
     acc.y = fma(a.y, b.x, acc.y);
 }
 
+// FP64 quotients that spare the FP64 pipe, on which a warp instruction takes 16
+// cycles of an SM.  rcp64: the hardware's approximate reciprocal y of b (relative
+// error e below 2^-17) and one step of the cubic iteration y (1 + e + e^2), e = 1 -
+// b y: three operations, error below 2^-51 plus a rounding.  div64: a / b from y =
+// rcp64(b) with the remainder's correction (Markstein), three more, within half
+// an ulp in all but rare cases.  The full division takes about three times as many.
+__device__ __forceinline__ double rcp64(double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    double e = fma(-b, y, 1.0);
+    e = fma(e, e, e);
+    return fma(y, e, y);
+}
+__device__ __forceinline__ double div64(double a, double b, double y) {
+    const double q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+
 // Tiled half-spectrum layout: [cell / 32][mode][cell % 32].
 __host__ __device__ __forceinline__ int64_t tiled_index(int64_t cell, int64_t mode, int64_t nhalf) {
     return (cell >> 5) * nhalf * 32 + mode * 32 + (cell & 31);

@@ -301,6 +301,7 @@ struct StageCoef {
     double all;                // A[l][l]
     double dt, eps;
     double nuf;                // penalty rate nu = nuf * rho
+    double coef;               // dt A_ll nuf / eps: c = coef * rho
     int store_F;               // 0: F_l equals f^n exactly (stage 0 of a step) and is not written
     int store_P;               // 0: no later stage reads P_l
     int use_G;                 // 0: every G is zero (a whole step of the BGK model) and none is read

@@ -113,21 +113,27 @@ __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageC
     }
 }
 
-// 2-D, N <= 32: one warp per cell, lane = column j2, loop over rows j1, 8 cells
-// per CTA.  (With N = 30 in FP64 on 2603 cells the block-per-cell form above it
-// took 552 us a stage, an exponential and index arithmetic per point on the
-// FP64 pipe; this one 139 us.)  FP64 work is what limits this kernel on a GPU
-// whose FP64 rate is 1/74 of FP32, so it is arranged to keep the FP64 pipe's
-// lanes busy with distinct work:
+// 2-D, N <= 32: one warp per cell, lane = column j2, loop over rows j1.  (With
+// N = 30 in FP64 on 2603 cells the block-per-cell form above took 552 us a
+// stage, an exponential and index arithmetic per point on the FP64 pipe.)  FP64
+// work is what limits this kernel on a GPU whose FP64 rate is 1/74 of FP32, so
+// it is arranged to keep the FP64 pipe's lanes busy with distinct work:
 //   * per lane, sums along j1 in the state precision (FP32: with a TwoSum
-//     error term), turned into FP64 once (S0, S1, S3 and the v2 products);
+//     error term), turned into FP64 once (S0, S1, S3 and the v2 products; the
+//     error terms stay in FP32);
 //   * the 32 lane partials of each cell are summed in FP64 by four threads per
 //     (cell, moment) from shared memory, not by a shuffle tree on every lane;
-//   * the Maxwellian parameters (rho, u, theta, ...) of the CTA's 8 cells are
-//     computed by 8 lanes of one warp, one cell per lane;
+//   * the Maxwellian parameters (rho, u, theta, ...) of the CTA's cells are
+//     computed by one warp, one cell per lane, with div64 for the quotients (in
+//     FP32 full divisions were the larger part of the kernel's FP64 time);
 //   * the Maxwellian of a 2-D grid factorises, M(v1, v2) = pref e1(v1) e2(v2):
 //     each lane forms its row and column offsets v - u in FP64 and the rest of
 //     the exponent and the exponential in the state precision.
+// Mean of a step's stages: FP32 N = 32 on 23160 cells 112 us with full divisions,
+// the error terms in FP64 and 8 cells a CTA, 95.5 us now; FP64 N = 30 on 2603
+// cells 139 -> 124 us (the row nodes from shared memory, not an FP64 fma per
+// row).  Four cells a CTA, so that the warps that wait for the parameters are
+// few: 8 cells take 107.6 and 130.5 us.
 template <typename T>
 __device__ __forceinline__ void acc2(T &s, T &e, T x) {
     if constexpr (sizeof(T) == 4) {
@@ -139,7 +145,7 @@ __device__ __forceinline__ void acc2(T &s, T &e, T x) {
     }
 }
 
-constexpr int kStageCells = 8;    // cells (warps) per CTA of the 2-D stage kernel (two CTAs per SM)
+constexpr int kStageCells = 4;    // cells (warps) per CTA of the 2-D stage kernel
 
 // NMAX rows in registers; FIXED: N = NMAX at compile time, else any N <= NMAX.
 template <typename T, int NMAX, bool FIXED>
@@ -148,8 +154,21 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
                                                                        const T *__restrict__ G, T *__restrict__ P,
                                                                        const T *__restrict__ Lres, int64_t stride,
                                                                        int64_t n) {
+    constexpr bool F32 = sizeof(T) == 4;
     __shared__ double part[kStageCells][4][33];   // per-lane moment partials (pitch 33: no bank conflicts)
-    __shared__ double par[kStageCells][8];        // nu, u1, u2, inv2t, pref, c, 1/(1+c)
+    __shared__ T perr[F32 ? kStageCells : 1][F32 ? 4 : 1][33];   // FP32: the partials' error terms
+    __shared__ double par[kStageCells][3];        // u1, u2, inv2t
+    __shared__ T parT[kStageCells][5];            // nu, inv2t, pref, c, 1/(1+c)
+    __shared__ double vd[32];                     // nodes
+    __shared__ T vt[F32 ? 1 : 2][F32 ? 1 : NMAX]; // FP64: v1 and v1^2 of the rows
+    if (threadIdx.x < 32) {
+        vd[threadIdx.x] = -g.L + threadIdx.x * g.dv;
+        if (!F32 && threadIdx.x < NMAX) {
+            const T v = fma((T)threadIdx.x, (T)g.dv, -(T)g.L);
+            vt[0][threadIdx.x] = v;
+            vt[!F32][threadIdx.x] = v * v;
+        }
+    }
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t cell = (int64_t)blockIdx.x * kStageCells + wib;
     const bool live = cell < n;
@@ -181,22 +200,36 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
         }
     }
     // this lane's partial moments (column j2 = lane)
+    __syncthreads();
     {
         T s0 = 0, e0 = 0, s1 = 0, e1 = 0, s3 = 0, e3 = 0;
         const T L = (T)g.L, dv = (T)g.dv;
 #pragma unroll
         for (int j = 0; j < NMAX; ++j) {
-            const T v1 = fma((T)j, dv, -L);
+            T v1, q1;
+            if constexpr (!F32) {
+                v1 = vt[0][j];
+                q1 = vt[1][j];
+            } else {
+                v1 = fma((T)j, dv, -L);
+                q1 = v1 * v1;
+            }
             acc2(s0, e0, R[j]);
             acc2(s1, e1, v1 * R[j]);
-            acc2(s3, e3, v1 * v1 * R[j]);
+            acc2(s3, e3, q1 * R[j]);
         }
-        const double vv = -g.L + lane * g.dv;
-        const double S0 = (double)s0 + (double)e0, S1 = (double)s1 + (double)e1, S3 = (double)s3 + (double)e3;
+        const double vv = vd[lane], S0 = (double)s0;
         part[wib][0][lane] = S0;
-        part[wib][1][lane] = S1;
+        part[wib][1][lane] = (double)s1;
         part[wib][2][lane] = vv * S0;
-        part[wib][3][lane] = S3 + vv * vv * S0;
+        part[wib][3][lane] = fma(vv * vv, S0, (double)s3);
+        if constexpr (F32) {                 // of relative size 2^-24: their sums in FP32 lose nothing
+            const T v = (T)vv;
+            perr[wib][0][lane] = e0;
+            perr[wib][1][lane] = e1;
+            perr[wib][2][lane] = v * e0;
+            perr[wib][3][lane] = fma(v * v, e0, e3);
+        }
     }
     __syncthreads();
     // sums over the 32 lanes of each cell: four threads per (cell, moment) sum
@@ -206,6 +239,12 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
         double tot = 0.0;
 #pragma unroll
         for (int l = 0; l < 8; ++l) tot += part[cc][q][pp * 8 + l];
+        if constexpr (F32) {
+            T te = (T)0;
+#pragma unroll
+            for (int l = 0; l < 8; ++l) te += perr[cc][q][pp * 8 + l];
+            tot += (double)te;
+        }
         tot += __shfl_xor_sync(0xffffffffu, tot, 1);
         tot += __shfl_xor_sync(0xffffffffu, tot, 2);
         if (pp == 0) part[cc][q][32] = tot;
@@ -214,39 +253,40 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
     // Maxwellian parameters, one cell per lane of warp 0
     if (threadIdx.x < kStageCells) {
         const int cc = threadIdx.x;
-        const double w = g.dv * g.dv;
-        const double rho = w * part[cc][0][32];
-        const double u1 = w * part[cc][1][32] / rho, u2 = w * part[cc][2][32] / rho;
+        const double w = g.dv * g.dv, coef = c.coef;
+        const double rho = w * part[cc][0][32], yr = rcp64(rho);
+        const double u1 = div64(w * part[cc][1][32], rho, yr), u2 = div64(w * part[cc][2][32], rho, yr);
         const double E = 0.5 * w * part[cc][3][32];
-        const double theta = (2.0 * E / rho - (u1 * u1 + u2 * u2)) / 2.0;
-        const double cst = c.dt * c.all * c.nuf * rho / c.eps;
-        par[cc][0] = c.nuf * rho;          // penalty rate nu
-        par[cc][1] = u1;
-        par[cc][2] = u2;
-        par[cc][3] = 0.5 / theta;
-        par[cc][4] = rho / (2.0 * M_PI * theta);
-        par[cc][5] = cst;
-        par[cc][6] = 1.0 / (1.0 + cst);
+        const double theta = (div64(2.0 * E, rho, yr) - (u1 * u1 + u2 * u2)) * 0.5, yt = rcp64(theta);
+        const double cst = coef * rho, c1 = 1.0 + cst;
+        par[cc][0] = u1;
+        par[cc][1] = u2;
+        par[cc][2] = div64(0.5, theta, yt);
+        parT[cc][0] = (T)(c.nuf * rho);    // penalty rate nu
+        parT[cc][1] = (T)par[cc][2];
+        parT[cc][2] = (T)div64(rho * (0.5 / M_PI), theta, yt);
+        parT[cc][3] = (T)cst;
+        parT[cc][4] = (T)div64(1.0, c1, rcp64(c1));
     }
     __syncthreads();
     if (!live) return;
     // separable Maxwellian: this lane's column factor and row factor j1 = lane;
     // offsets v - u in FP64, the rest of the exponent and the exp in T
-    const double vl = -g.L + lane * g.dv;
     // (any other N: the whole exponent in FP64)
-    const double d2 = vl - par[wib][2], d1 = vl - par[wib][1];
+    const double vl = vd[lane];
+    const double d2 = vl - par[wib][1], d1 = vl - par[wib][0];
     T x1, x2;
     if constexpr (FIXED) {
-        const T i2t = (T)par[wib][3], t1 = (T)d1, t2 = (T)d2;
+        const T i2t = parT[wib][1], t1 = (T)d1, t2 = (T)d2;
         x1 = -t1 * t1 * i2t;
         x2 = -t2 * t2 * i2t;
     } else {
-        x1 = (T)(-d1 * d1 * par[wib][3]);
-        x2 = (T)(-d2 * d2 * par[wib][3]);
+        x1 = (T)(-d1 * d1 * par[wib][2]);
+        x2 = (T)(-d2 * d2 * par[wib][2]);
     }
-    const T fcol = (T)par[wib][4] * exp(x2);
+    const T fcol = parT[wib][2] * exp(x2);
     const T frow_l = exp(x1);
-    const T cT = (T)par[wib][5], denom = (T)par[wib][6], nuT = (T)par[wib][0];
+    const T cT = parT[wib][3], denom = parT[wib][4], nuT = parT[wib][0];
     T *Fo = F + base;
     T *Po = P + (int64_t)c.stage * stride + base;
 #pragma unroll

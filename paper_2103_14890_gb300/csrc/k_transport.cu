@@ -129,22 +129,10 @@ struct FvIdx {
     const int *order, *meta, *fid, *two, *ncen, *cen, *nsec, *sec;
 };
 
-// FP64 forms that spare the FP64 pipe, on which a warp instruction takes 16
-// cycles of an SM.  min of two non-negative numbers as integers (the same
-// order; a NaN operand ends in NaN weights either way).  1 / b for b > 0: the
-// hardware's approximate reciprocal y (relative error e below 2^-17) and one
-// step of the cubic iteration y (1 + e + e^2), e = 1 - b y: three operations,
-// error below 2^-51 plus a rounding; the full division takes about three times
-// as many.
+// min of two non-negative numbers as integers (the same order; a NaN operand
+// ends in NaN weights either way): it leaves the FP64 pipe alone.
 __device__ __forceinline__ double min_nonneg(double a, double b) {
     return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
-}
-__device__ __forceinline__ double rcp_pos(double b) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    double e = fma(-b, y, 1.0);
-    e = fma(e, e, e);
-    return fma(y, e, y);
 }
 
 // Write the flux of VEC velocities through a face: vn (outward normal velocity
@@ -243,13 +231,13 @@ __device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, co
             sig[s] = fma(sx[s], sx[s], fma(sy[s], sy[s], kEps));
             num = min_nonneg(num, sig[s]);
         }
-    double r = num * rcp_pos(s0);
+    double r = num * rcp64(s0);
     r = r * r;
     double w = kLam0 * (r * r), wl = 0.0, ax = 0.0, ay = 0.0;
 #pragma unroll
     for (int s = 0; s < MAXS; ++s)
         if (s < ns) {
-            r = num * rcp_pos(sig[s]);
+            r = num * rcp64(sig[s]);
             r = r * r;
             r = r * r;
             wl += r;
@@ -257,7 +245,7 @@ __device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, co
             ay = fma(r, sy[s], ay);
         }
     // (lambda_0 w_0 p_0 + lambda_L sum w_L p_L) / (lambda_0 w_0 + lambda_L sum w_L)
-    const double iw = rcp_pos(fma(lamL, wl, w)), wL = lamL * iw;
+    const double iw = rcp64(fma(lamL, wl, w)), wL = lamL * iw;
     w *= iw;
 #pragma unroll
     for (int l = 0; l < B; ++l) c[l] *= w;
