@@ -61,7 +61,15 @@ struct bz_grid {
 };
 
 constexpr int kModesumVariants = 10;   // register-blocked FP32 mode-sum kernel variants
-constexpr int kSplitTables = 3;       // task tables for a tile split over 2, 4, 8 CTAs
+constexpr int kMaxSplit = 8;          // most CTAs that share a tile's tasks
+
+// Task tables of one layout, for a tile on S = 1 .. kMaxSplit CTAs, in one block.
+struct TaskTables {
+    int *block;
+    int off[kMaxSplit];      // ints before the table of S CTAs, at S - 1
+    float bal[kMaxSplit];    // its most loaded warp's load
+    float work;              // load of all tasks
+};
 
 struct bz_modes {
     const bz_grid *g;
@@ -73,24 +81,18 @@ struct bz_modes {
     double *d_F64;
     float *d_F32;
     // symmetric weight streams and task tables of the FP32 2-D kernel, one per
-    // variant (k_modesum32.cu); d_W32 / d_task / w32_rowmax alias the variant
+    // variant (k_modesum32.cu); d_W32 / w32_rowmax alias the variant
     // in use (null if the generic kernel serves this grid)
     float *var_W[kModesumVariants];
-    int *var_task[kModesumVariants];
-    int *var_task_split[kModesumVariants][kSplitTables];   // 32- and 8-cell variants: tile split over 2, 4, 8 CTAs
-    float var_bal[kModesumVariants][kSplitTables + 1];     // load of the most loaded warp, tile on 1, 2, 4, 8 CTAs
+    TaskTables var_task[kModesumVariants];
     int var_rowmax[kModesumVariants];
     int variant;          // index of the selected variant
     int variant_fixed;    // 1: chosen by BZ_MODESUM_VARIANT (no last-wave split)
     float *small_W;       // weight stream and task tables of the small-launch variant (two outputs per thread)
-    int *small_task;
-    int *small_task_split[kSplitTables];
-    float small_bal[kSplitTables + 1];
+    TaskTables small_task;
     int small_rowmax;
     void *w64;            // FP64 weight stream and task table, null if unused
-    int *task64;
-    int *task64_split[kSplitTables];
-    float bal64[kSplitTables + 1];
+    TaskTables task64;
     int rowmax64;
     int variant64;        // layout of the FP64 tables (entry of the variant list), -1 if none
     float *wx2;           // FP32X2 weight stream: the FP64 stream's layout and task table, each
@@ -98,7 +100,6 @@ struct bz_modes {
     int modesum_variant;  // variant id reported to callers (index + 1; 0: no choice of variants, N > 48)
     float *d_W32;
     int w32_rowmax;       // largest staged weight row (floats)
-    int *d_task;
     int64_t pairs_sym;   // unordered pairs per cell (algorithmic unit)
     int tile_dft;        // 1: the tile FFT kernels of k_dft32.cu serve this grid in FP32
     int tile_dft64;      // ... and in FP64 (also the FP32X2 form's forward transform)
@@ -246,7 +247,7 @@ struct Mode32Item {
     const int *tasks;     // task table for WARPS x split warps
     int h, M, nhalf, wrow_max;
     int64_t n;
-    int split;            // CTAs per tile (1, or 2, 4, 8 for a last partial wave)
+    int split;            // CTAs that share a tile's tasks
 };
 struct Mode32Group {
     int nitems;
@@ -256,7 +257,6 @@ struct Mode32Group {
 bool modesum32_available(const bz_modes *m);
 cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat, int64_t n, cudaStream_t st,
                              bool pdl = false);
-int64_t modesum32_split(const bz_modes *m, int64_t n, int *tail_v, int *tail_split);
 // Cells one SM holds at a time in the handle's FP32 mode-sum kernel (CTAs per
 // SM x cells per CTA; 32 where the register-blocked kernels do not serve it).
 int modesum32_wave_cells_per_sm(const bz_modes *m);

@@ -354,16 +354,13 @@ void modes_destroy(bz_modes *m) {
     dev_free(m->d_F64);
     dev_free(m->d_F32);
     dev_free(m->small_W);
-    dev_free(m->small_task);
-    for (int k = 0; k < kSplitTables; ++k) dev_free(m->small_task_split[k]);
+    dev_free(m->small_task.block);
     dev_free(m->w64);
     dev_free(m->wx2);
-    dev_free(m->task64);
-    for (int k = 0; k < kSplitTables; ++k) dev_free(m->task64_split[k]);
+    dev_free(m->task64.block);
     for (int v = 0; v < kModesumVariants; ++v) {
         dev_free(m->var_W[v]);
-        dev_free(m->var_task[v]);
-        for (int k = 0; k < kSplitTables; ++k) dev_free(m->var_task_split[v][k]);
+        dev_free(m->var_task[v].block);
     }
     free(m->h_F);
     free(m);

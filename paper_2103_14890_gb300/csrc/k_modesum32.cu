@@ -896,7 +896,7 @@ struct Term64 {
 // accurate as if computed in twice the working precision; the real and
 // imaginary parts are the two lanes, and the _rn intrinsics pin the operations.
 // The FMA pipe bounds the kernel (70 % busy): 28 FP32x2 operations per pair.
-// 4096 cells of 32^2: 1.53 -> 1.34 ms by the tables and the split of the tiles.
+// 4096 cells of 32^2: 1.53 -> 1.27 ms by the tables and the split of the last tiles.
 // Not kept: Dekker's three-operation sums on operands ordered by selects (22
 // operations, the same numbers) moved the bound to the ALU pipe, 1.55 ms; a
 // running sum biased so that it always exceeds the product needs 16 operations
@@ -979,7 +979,7 @@ struct TermX2 {
 // The task loop of both forms.  FP64: sums along a row pair fold into (hi, lo)
 // by TwoSum every four.  FP32X2: the FP64 spectrum is split into FP32 high and
 // low parts as it is staged; its output is rounded to FP32.  A tile may be
-// split over gd.item[0].split CTAs.
+// shared by `split` CTAs.
 template <bool X2, int RR, int WARPS, int CELLS>
 __global__ void __launch_bounds__(WARPS * 32, CELLS == 8 ? 2 : 1) modesum_pair_kernel(const Mode32Group gd) {
     constexpr int G = 32 / CELLS;                // CTAs per 32-cell tile
@@ -988,13 +988,16 @@ __global__ void __launch_bounds__(WARPS * 32, CELLS == 8 ? 2 : 1) modesum_pair_k
     using W = typename std::conditional<X2, float, double>::type;
     using OutV = typename std::conditional<X2, float2, double2>::type;
     extern __shared__ __align__(16) uint4 smem16[];
-    const Mode32Item &ip = gd.item[0];
+    int it = 0;
+    while (it + 1 < gd.nitems && (int64_t)blockIdx.x >= gd.tile_start[it + 1]) ++it;
+    const Mode32Item &ip = gd.item[it];
     const double2 *__restrict__ fhat = static_cast<const double2 *>(ip.fhat);
     const W *__restrict__ Wst = static_cast<const W *>(ip.W);
     const int *__restrict__ tasks = ip.tasks;
     const int h = ip.h, M = ip.M, nhalf = ip.nhalf, wrow_max = ip.wrow_max;
-    const int part = (int)(blockIdx.x % ip.split);
-    const int64_t cta = (int64_t)blockIdx.x / ip.split;
+    const int64_t cta0 = (int64_t)blockIdx.x - gd.tile_start[it];
+    const int part = (int)(cta0 % ip.split);
+    const int64_t cta = cta0 / ip.split;
     const int64_t tile = cta / G;
     const int sub = (int)(cta % G);
     const int rows = nhalf + 2 * kPad;
@@ -1117,6 +1120,37 @@ __global__ void __launch_bounds__(WARPS * 32, CELLS == 8 ? 2 : 1) modesum_pair_k
     }
 }
 
+// Moves a task of the most loaded warp to another, or swaps it for a shorter
+// one, while that lowers the larger of the two loads, the best such step first.
+static void even_out(const std::vector<double> &cost, std::vector<int> *per, std::vector<double> &load) {
+    const int nw = (int)load.size();
+    for (int step = 0; step < 256; ++step) {
+        const int a = (int)(std::max_element(load.begin(), load.end()) - load.begin());
+        double best = load[a] * (1.0 - 1e-9);
+        int bb = -1, bx = -1, by = -1;
+        for (int b = 0; b < nw; ++b)
+            for (int x = 0; b != a && x < (int)per[a].size(); ++x)
+                for (int y = -1; y < (int)per[b].size(); ++y) {
+                    const double d = cost[per[a][x]] - (y >= 0 ? cost[per[b][y]] : 0.0);
+                    const double m = std::max(load[a] - d, load[b] + d);
+                    if (m < best) best = m, bb = b, bx = x, by = y;
+                }
+        if (bb < 0) break;
+        const int i = per[a][bx];
+        const double d = cost[i] - (by >= 0 ? cost[per[bb][by]] : 0.0);
+        if (by >= 0) {
+            std::swap(per[a][bx], per[bb][by]);
+        } else {
+            per[a].erase(per[a].begin() + bx);
+            per[bb].push_back(i);
+        }
+        load[a] -= d;
+        load[bb] += d;
+    }
+    for (int w = 0; w < nw; ++w)
+        std::stable_sort(per[w].begin(), per[w].end(), [&](int x, int y) { return cost[x] > cost[y]; });
+}
+
 template <typename T> size_t smem_bytes(const GridView &g, int wrow_max, int v) {
     return 2 * sizeof(T) * (size_t)(g.nhalf + 2 * kPad) * kVariants[v].cells +
            sizeof(T) * (size_t)kVariants[v].warps * 2 * kVariants[v].rows * wrow_max;
@@ -1134,8 +1168,8 @@ double beta_host(const bz_modes *m, const int *l, const int *mm);
 // each l_2 step become RT FP32 high parts followed by RT FP32 low parts
 // (hi = fl32(w), lo = fl32(w - hi)), headers copied as they are.
 template <typename T>
-static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, int *outRowmax,
-                          float **outX2 = nullptr, int **outSplit = nullptr, float *outBal = nullptr) {
+static bool build_variant(bz_modes *m, int v, int &rc, void **outW, TaskTables *outT, int *outRowmax,
+                          float **outX2 = nullptr) {
     constexpr int HEAD = kRowHeadBytes / (int)sizeof(T);
     const int R = variant_rt(v);                                // outputs per task (RT)
     const int kWarps = kVariants[v].warps;
@@ -1313,9 +1347,9 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
             }
         }
     }
-    // longest-processing-time-first assignment of tasks to nw warps: the
-    // offsets of each warp's list, then the task records
-    auto make_table = [&](int nw, float *worst = nullptr) {
+    // assignment of tasks to nw warps: longest first to the least loaded, then
+    // even_out; the offsets of each warp's list, then the task records
+    auto make_table = [&](int nw, float &worst) {
         double longest = 0.0;                               // sum over the phases of the most loaded warp
         std::vector<std::vector<int>> per(2 * nw);
         for (int ph = 0; ph < 2; ++ph) {
@@ -1329,9 +1363,10 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
                 load[w] += cost[i];
                 per[ph * nw + w].push_back(i);
             }
+            even_out(cost, &per[ph * nw], load);
             longest += *std::max_element(load.begin(), load.end());
         }
-        if (worst) *worst = (float)longest;
+        worst = (float)longest;
         std::vector<int> t(2 * nw + 1 + tasks.size() * kTaskInts);
         int pos = 0;
         for (int q = 0; q < 2 * nw; ++q) {
@@ -1344,10 +1379,19 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
         t[2 * nw] = pos;
         return t;
     };
-    const std::vector<int> tab = make_table(kWarps, outBal);
     int wrow_max = 0;
     for (auto &t : tasks) wrow_max = std::max(wrow_max, t.rowf);   // staging buffer: one row pair
     if (smem_bytes<T>(gv, wrow_max, v) > 227 * 1024) return false;   // does not fit
+    TaskTables tt;
+    std::vector<int> tab;
+    for (int S = 1; S <= kMaxSplit; ++S) {
+        const std::vector<int> t = make_table(kWarps * S, tt.bal[S - 1]);
+        tt.off[S - 1] = (int)tab.size();
+        tab.insert(tab.end(), t.begin(), t.end());
+    }
+    double work = 0.0;
+    for (double c : cost) work += c;
+    tt.work = (float)work;
     T *dW = nullptr;
     int *dT = nullptr;
     float *dX = nullptr;
@@ -1366,26 +1410,9 @@ static bool build_variant(bz_modes *m, int v, int &rc, void **outW, int **outT, 
         rc = cuda_fail(e, "build_kernel_modes: weight stream");
         return false;
     }
-    // tables for one tile split over S = 2, 4, 8 CTAs (S x kWarps warps): the
-    // last partial wave of a launch of a 32-cell variant, or every tile of a
-    // launch (launch_split)
-    if (outSplit) {
-        for (int k = 0; k < kSplitTables && e == cudaSuccess; ++k) {
-            const std::vector<int> ts = make_table(kWarps << (k + 1), outBal ? outBal + k + 1 : nullptr);
-            e = dev_malloc(&outSplit[k], sizeof(int) * ts.size());
-            if (e == cudaSuccess) e = cudaMemcpy(outSplit[k], ts.data(), sizeof(int) * ts.size(), cudaMemcpyHostToDevice);
-        }
-        if (e != cudaSuccess) {
-            for (int k = 0; k < kSplitTables; ++k) dev_free(outSplit[k]), outSplit[k] = nullptr;
-            dev_free(dW);
-            dev_free(dT);
-            dev_free(dX);
-            rc = cuda_fail(e, "build_kernel_modes: split task tables");
-            return false;
-        }
-    }
+    tt.block = dT;
     *outW = dW;
-    *outT = dT;
+    *outT = tt;
     *outRowmax = wrow_max;
     if (want_x2) *outX2 = dX;
     return true;
@@ -1434,14 +1461,14 @@ static cudaError_t launch_group(const Mode32Group &gd, int v, size_t sm, cudaStr
     }
 }
 
-static void fill_item(Mode32Item &it, const bz_modes *m, const void *W, const int *tasks, int rowmax,
+static void fill_item(Mode32Item &it, const bz_modes *m, const void *W, const TaskTables &tasks, int rowmax,
                       const void *fhat, void *Qhat, int64_t n, int split = 1) {
     it.split = split;
     const GridView &gv = m->g->v;
     it.fhat = fhat;
     it.Qhat = Qhat;
     it.W = W;
-    it.tasks = tasks;
+    it.tasks = tasks.block + tasks.off[split - 1];
     it.h = gv.h;
     it.M = gv.M;
     it.nhalf = (int)gv.nhalf;
@@ -1449,13 +1476,85 @@ static void fill_item(Mode32Item &it, const bz_modes *m, const void *W, const in
     it.n = n;
 }
 
-// Index of the task tables of a tile split over S = 2, 4, 8 CTAs.
-static int split_index(int S) { return S == 2 ? 0 : S == 4 ? 1 : 2; }
-
 // CTAs of an instance of n cells: one per CELLS cells of each 32-cell tile.
 static int64_t ctas_for(int v, int64_t n) {
     const int G = 32 / kVariants[v].cells;      // CTAs per 32-cell tile
     return ((n + 31) / 32) * G;
+}
+
+// CTAs per SM of a variant's kernel (its launch bounds: the FP32x2 kernels
+// with 8 or 4 warps are built for 2 or 3 resident CTAs, the 8-cell FP64 and
+// FP32X2 kernels for 2).
+static int variant_ctas_per_sm(int v) {
+    if (!kVariants[v].pq || (v >= kNumVariants && kVariants[v].cells == 4)) return 1;
+    return kVariants[v].warps <= 4 ? 3 : kVariants[v].warps <= 8 ? 2 : 1;
+}
+
+// How a launch ends: its first `full` CTAs take a tile each, the tiles after
+// them are shared by S CTAs.
+struct Tail {
+    int64_t full;
+    int S;
+};
+
+static int sm_count();
+
+// The whole waves of a launch run one CTA per tile; the T CTAs left over would
+// keep a part of the SMs busy for as long as a whole wave, so S CTAs share each
+// of their tiles.  Every output is computed by one task with the same
+// arithmetic, so the results do not depend on S.  S has the least estimated
+// time, in units of a CTA's time on a full SM: an SM gets q of the T S CTAs,
+// each taking the mean of its share of the work (what counts where other CTAs
+// fill its gaps) and of its most loaded warp's part (where they do not), and o
+// for its start, chiefly the staged spectrum: `stage` loads per mode.  With several CTAs per SM the last ones end
+// apart, by `ragged` times a CTA's length on the mean.  Measured, S = 1 and the
+// S taken here: 32^2 in FP32 on 5000, 9000, 19802, 32768 cells 246, 322, 687,
+// 1054 us and 185, 290, 632, 1014 (S = 4); 48^2 on 3000, 6000, 13632 cells 735,
+// 1110, 2233 us and 497 (4), 938 (2), 2154 (3); 64^2 on 500 and 1500 cells 577,
+// 1153 us and 297 (2), 736 (4); 16^3 on 700 and 1400 cells 446, 871 us and
+// 295 (5), 528 (6); 32^2 in FP64 on 4099 cells 8.60 ms and 7.54 (2).
+static Tail tail_split(const bz_modes *m, int v, const TaskTables &t, int64_t ctas, size_t sm, double stage,
+                       double ragged) {
+    const int64_t fit = std::max<int64_t>(1, 228 * 1024 / (int64_t)(sm + 1024));
+    const int64_t per_sm = std::min<int64_t>(variant_ctas_per_sm(v), fit), sms = sm_count(), wave = sms * per_sm;
+    if (per_sm == 1) ragged = 0.0;
+    const int G = 32 / kVariants[v].cells;
+    int64_t full = ctas / wave * wave;
+    full -= full % G;
+    const int64_t T = ctas - full;
+    if (T == 0) return {ctas, 1};
+    const double o = stage * (double)m->g->v.nhalf / t.work;
+    auto estimate = [&](int S) {
+        const double q = (double)((T * S + sms - 1) / sms);
+        return q * (0.5 * (1.0 / S + t.bal[S - 1] / t.bal[0]) + o) + ragged / S;
+    };
+    Tail r{full, 1};
+    double best = estimate(1);
+    for (int S = 2; S <= kMaxSplit; ++S)
+        if (estimate(S) < (r.S == 1 ? 0.97 : 0.99) * best) {
+            best = estimate(S);
+            r.S = S;
+        }
+    return r;
+}
+// `stage` and `ragged` of the FP32 forms, fitted to the times above; FP64 and
+// FP32X2 tasks take 30 and 5 times as long for the same staged bytes, and the
+// FP64 pipe is full to the end
+constexpr double kStage32 = 4.3, kRagged32 = 0.45, kStage64 = 0.15, kStageX2 = 0.8;
+
+// Appends an instance of n cells to a launch: the cells of its first `full`
+// CTAs, then those whose tiles S CTAs share.  fsize, qsize: bytes per value.
+static void add_items(Mode32Group &gd, const bz_modes *m, int v, const void *W, const TaskTables &t, int rowmax,
+                      const void *fhat, size_t fsize, void *Qhat, size_t qsize, int64_t n, Tail tail) {
+    const int64_t nm = std::min(n, tail.full * kVariants[v].cells);
+    for (int p = 0; p < 2; ++p) {
+        const int64_t first = p ? nm : 0, cnt = p ? n - nm : nm, off = first / 32 * m->g->v.nhalf * 32;
+        if (cnt <= 0) continue;
+        const int S = p ? tail.S : 1, k = gd.nitems++;
+        fill_item(gd.item[k], m, W, t, rowmax, static_cast<const char *>(fhat) + off * fsize,
+                  static_cast<char *>(Qhat) + off * qsize, cnt, S);
+        gd.tile_start[k + 1] = gd.tile_start[k] + ctas_for(v, cnt) * S;
+    }
 }
 
 static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
@@ -1463,11 +1562,8 @@ static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, 
     if (n <= 0) return cudaSuccess;
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
-    gd.nitems = 1;
-    fill_item(gd.item[0], m, m->var_W[v], S > 1 ? m->var_task_split[v][split_index(S)] : m->var_task[v],
-              m->var_rowmax[v], fhat, Qhat, n, S);
-    gd.tile_start[0] = 0;
-    gd.tile_start[1] = ctas_for(v, n) * S;
+    add_items(gd, m, v, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, sizeof(float2), Qhat, sizeof(float2), n,
+              {S > 1 ? 0 : ctas_for(v, n), S});
     return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
 }
 
@@ -1479,43 +1575,11 @@ constexpr int kFp64Variants[3] = {10, 11, 12};
 
 bool modesum64_available(const bz_modes *m) { return m->w64 != nullptr; }
 
-static int sm_count();
-
-// CTAs that take one tile's tasks between them (1, 2, 4 or 8): the S with the
-// least estimated time, so that neither a launch smaller than a wave nor its
-// last partial wave leaves SMs idle.  Every output is computed by one task with
-// the same arithmetic, so the results do not depend on S; staging the spectrum
-// S times costs a few us of an SM against hundreds, and a larger S has to win
-// by 3 %.  With one CTA per SM the time is the number of waves times the load
-// of the most loaded warp; with several (shared), whose warps fill one
-// another's gaps, it is the most CTAs an SM gets times their mean load.  The
-// FP64 and FP32X2 forms run 32^2 so; 4099 cells (516 CTAs, 152 SMs), S = 1, 2, 4: FP64 8.60,
-// 7.56, 7.59 ms.  500 cells of 64^2 in FP32 (64
-// CTAs): 0.581, 0.306, 0.326 ms.
-static int launch_split(int64_t ctas, const float (&bal)[kSplitTables + 1], int *const *tables, bool shared) {
-    const int64_t sms = sm_count();
-    auto estimate = [&](int S, double most) {
-        const double waves = (double)((ctas * S + sms - 1) / sms);
-        return shared ? std::max(waves * bal[0] / S, most) : waves * most;
-    };
-    int best = 1;
-    double t = estimate(1, bal[0]);
-    for (int k = 0; k < kSplitTables; ++k) {
-        if (!tables[k]) continue;
-        const double ts = estimate(2 << k, bal[k + 1]);
-        if (ts < 0.97 * t) {
-            t = ts;
-            best = 2 << k;
-        }
-    }
-    return best;
-}
-
 template <bool X2, int RR, int WARPS, int CELLS>
 static cudaError_t launch_pair(const Mode32Group &gd, size_t sm, cudaStream_t st) {
     cudaError_t e = allow_dynamic_smem((const void *)modesum_pair_kernel<X2, RR, WARPS, CELLS>, sm);
     if (e != cudaSuccess) return e;
-    modesum_pair_kernel<X2, RR, WARPS, CELLS><<<(unsigned)gd.tile_start[1], WARPS * 32, sm, st>>>(gd);
+    modesum_pair_kernel<X2, RR, WARPS, CELLS><<<(unsigned)gd.tile_start[gd.nitems], WARPS * 32, sm, st>>>(gd);
     return cudaGetLastError();
 }
 
@@ -1525,13 +1589,11 @@ template <bool X2>
 static cudaError_t launch_pairs(const bz_modes *m, const double2 *fhat, void *Qhat, int64_t n, cudaStream_t st) {
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
-    gd.nitems = 1;
-    const int64_t ctas = ctas_for(m->variant64, n);
-    const int S = launch_split(ctas, m->bal64, m->task64_split, true);
-    fill_item(gd.item[0], m, X2 ? static_cast<const void *>(m->wx2) : m->w64,
-              S > 1 ? m->task64_split[split_index(S)] : m->task64, m->rowmax64, fhat, Qhat, n, S);
-    gd.tile_start[1] = ctas * S;
-    const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, m->variant64);
+    const int v = m->variant64;
+    const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, v);
+    add_items(gd, m, v, X2 ? static_cast<const void *>(m->wx2) : m->w64, m->task64, m->rowmax64, fhat, sizeof(double2),
+              Qhat, X2 ? sizeof(float2) : sizeof(double2), n,
+              tail_split(m, v, m->task64, ctas_for(v, n), sm, X2 ? kStageX2 : kStage64, 0.0));
     if (m->variant64 == kFp64Variants[0]) return launch_pair<X2, 4, 8, 8>(gd, sm, st);
     if (m->variant64 == kFp64Variants[1]) return launch_pair<X2, 4, 8, 4>(gd, sm, st);
     if (m->variant64 == kFp64Variants[2]) return launch_pair<X2, 2, 8, 8>(gd, sm, st);
@@ -1552,51 +1614,8 @@ cudaError_t launch_modesum_x2(const bz_modes *m, const double2 *fhat, float2 *Qh
     return launch_pairs<true>(m, fhat, Qhat, n, st);
 }
 
-// A launch over n cells ends with a partial wave of tiles; the SMs that run
-// one tile fewer idle meanwhile.  With a 32-cell variant chosen by timing,
-// the whole waves run one tile per CTA and the T remaining tiles are split
-// over S = 2, 4 or 8 CTAs each (each CTA takes one part of the tile's tasks),
-// S the largest with T S <= SM count; when no such S exists (T > SMs / 2)
-// and the 16-cell variant fits the grid, the remaining tiles run on it (twice
-// the CTAs, each half as long).  Every output is computed by one task in
-// either case, with the same arithmetic (the one-cell-per-lane variants sum
-// each output over the same terms in the same order), so the results do not
-// depend on the split.  Returns the cells of the main part; *tail_v is the tail's variant
-// (-1: no tail) and *tail_split its split.
-int64_t modesum32_split(const bz_modes *m, int64_t n, int *tail_v, int *tail_split) {
-    *tail_v = -1;
-    *tail_split = 1;
-    if (m->variant_fixed || kVariants[m->variant].cells != 32) return n;
-    const int64_t sms = sm_count();
-    const int64_t ntiles = (n + 31) / 32, full = (ntiles / sms) * sms;
-    const int64_t T = ntiles - full;
-    if (T == 0) return n;
-    for (int k = kSplitTables - 1; k >= 0; --k) {
-        const int S = 2 << k;
-        if (T * S <= sms && m->var_task_split[m->variant][k]) {
-            *tail_v = m->variant;
-            *tail_split = S;
-            return full * 32;
-        }
-    }
-    // the 16-cell variant, if it sums every output in the order of this one
-    if (!m->var_W[2] || kVariants[m->variant].pq ||
-        variant_reflects(2, m->g->v.h) != variant_reflects(m->variant, m->g->v.h))
-        return n;
-    *tail_v = 2;
-    return full * 32;
-}
-
-// CTAs per SM of a variant's kernel (its launch bounds: the FP32x2 kernels
-// with 8 or 4 warps are built for 2 or 3 resident CTAs).
-static int variant_ctas_per_sm(int v) {
-    if (!kVariants[v].pq) return 1;
-    return kVariants[v].warps <= 4 ? 3 : kVariants[v].warps <= 8 ? 2 : 1;
-}
-
 bool modesum32_tail_splits(const bz_modes *m) {
-    return m->method == 0 && modesum32_available(m) && !m->variant_fixed && kVariants[m->variant].cells == 32 &&
-           m->var_task_split[m->variant][0] != nullptr;
+    return m->method == 0 && modesum32_available(m) && !m->variant_fixed && kVariants[m->variant].cells == 32;
 }
 
 // A variant that holds several CTAs per SM fills only part of each SM in a
@@ -1630,10 +1649,17 @@ static int small_split(const bz_modes *m, int v, int64_t n) {
     if (m->variant_fixed || !m->small_W || !k.pq || k.cells != 16 || k.R != 8) return 0;
     const int64_t ctas = ctas_for(kSmallVariant, n), sms = sm_count();
     if (ctas > sms) return 0;
-    const int S = launch_split(ctas, m->small_bal, m->small_task_split, true);
-    const int ix = S > 1 ? split_index(S) + 1 : 0;
-    const double t = std::max((double)((ctas * S + sms - 1) / sms) * m->small_bal[0] / S, (double)m->small_bal[ix]);
-    return t < 0.9 * m->var_bal[v][0] ? S : 0;
+    const float *bal = m->small_task.bal;
+    int best = 0;
+    double t = 0.9 * m->var_task[v].bal[0];
+    for (int S = 1; S <= kMaxSplit; ++S) {
+        const double ts = std::max((double)((ctas * S + sms - 1) / sms) * bal[0] / S, (double)bal[S - 1]);
+        if (ts < (best ? 0.97 : 1.0) * t) {
+            t = ts;
+            best = S;
+        }
+    }
+    return best;
 }
 
 bool modesum32_small_batches_fast(const bz_modes *m) {
@@ -1651,49 +1677,36 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
                              bool pdl) {
     if (n <= 0) return cudaSuccess;
     const int sv = small_batch_variant(m, n);
-    if (const int S = small_split(m, sv, n)) {
-        Mode32Group gd;
-        memset(&gd, 0, sizeof gd);
-        gd.nitems = 1;
-        fill_item(gd.item[0], m, m->small_W, S > 1 ? m->small_task_split[split_index(S)] : m->small_task,
-                  m->small_rowmax, fhat, Qhat, n, S);
-        gd.tile_start[1] = ctas_for(kSmallVariant, n) * S;
-        return launch_group(gd, kSmallVariant, smem_bytes<float>(m->g->v, m->small_rowmax, kSmallVariant), st, pdl);
-    }
-    if (sv != m->variant) return launch_variant(m, sv, fhat, Qhat, n, st);
-    if (kVariants[sv].rows > 1)
-        return launch_variant(m, sv, fhat, Qhat, n, st,
-                              launch_split(ctas_for(sv, n), m->var_bal[sv], m->var_task_split[sv], false));
-    int tv = -1, ts = 1;
-    const int64_t nm = modesum32_split(m, n, &tv, &ts);
-    const int v = m->variant;
-    if (tv >= 0 && tv != v) {
-        // tail on another variant: two launches (different kernels)
-        cudaError_t e = nm > 0 ? launch_variant(m, v, fhat, Qhat, nm, st) : cudaSuccess;
-        const size_t off = (size_t)(nm / 32) * m->g->v.nhalf * 32;
-        if (e == cudaSuccess) e = launch_variant(m, tv, fhat + off, Qhat + off, n - nm, st);
-        return e;
-    }
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
-    gd.tile_start[0] = 0;
-    int k = 0;
-    if (nm > 0) {
-        fill_item(gd.item[k], m, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, Qhat, nm);
-        gd.tile_start[k + 1] = gd.tile_start[k] + ctas_for(v, nm);
-        ++k;
+    if (const int S = small_split(m, sv, n)) {
+        add_items(gd, m, kSmallVariant, m->small_W, m->small_task, m->small_rowmax, fhat, sizeof(float2), Qhat,
+                  sizeof(float2), n, {0, S});
+        return launch_group(gd, kSmallVariant, smem_bytes<float>(m->g->v, m->small_rowmax, kSmallVariant), st, pdl);
     }
-    if (tv >= 0 && n > nm) {
-        const size_t off = (size_t)(nm / 32) * m->g->v.nhalf * 32;
-        int lg = 0;
-        while ((2 << lg) != ts) ++lg;
-        fill_item(gd.item[k], m, m->var_W[v], m->var_task_split[v][lg], m->var_rowmax[v], fhat + off, Qhat + off,
-                  n - nm, ts);
-        gd.tile_start[k + 1] = gd.tile_start[k] + ctas_for(v, n - nm) * ts;
-        ++k;
+    const Variant &k = kVariants[sv];
+    const int64_t ctas = ctas_for(sv, n);
+    const size_t sm = smem_bytes<float>(m->g->v, m->var_rowmax[sv], sv);
+    const Tail tail = m->variant_fixed && k.rows == 1 ? Tail{ctas, 1}
+                                                      : tail_split(m, sv, m->var_task[sv], ctas, sm, kStage32, kRagged32);
+    // scalar 32-cell variants: the tiles left over run on the 16-cell variant
+    // (twice the CTAs, bit-identical where it sums in the same order), itself with
+    // its last ones split: 24^2 on 1949, 7000, 40000 cells 72, 143, 646 us with split
+    // 32-cell tiles, 56, 128, 633 so
+    if (k.cells == 32 && !m->variant_fixed && tail.full < ctas && !k.pq && k.pack == 1 && m->var_W[2] &&
+        variant_reflects(2, m->g->v.h) == variant_reflects(sv, m->g->v.h)) {
+        const int64_t nm = tail.full * 32;
+        const size_t off = (size_t)nm * m->g->v.nhalf;
+        const cudaError_t e = launch_variant(m, sv, fhat, Qhat, nm, st);
+        if (e != cudaSuccess) return e;
+        const size_t s2 = smem_bytes<float>(m->g->v, m->var_rowmax[2], 2);
+        add_items(gd, m, 2, m->var_W[2], m->var_task[2], m->var_rowmax[2], fhat + off, sizeof(float2), Qhat + off,
+                  sizeof(float2), n - nm, tail_split(m, 2, m->var_task[2], ctas_for(2, n - nm), s2, kStage32, kRagged32));
+        return launch_group(gd, 2, s2, st);
     }
-    gd.nitems = k;
-    return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
+    add_items(gd, m, sv, m->var_W[sv], m->var_task[sv], m->var_rowmax[sv], fhat, sizeof(float2), Qhat, sizeof(float2), n,
+              tail);
+    return launch_group(gd, sv, sm, st);
 }
 
 cudaError_t launch_modesum32_part(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
@@ -1713,19 +1726,23 @@ cudaError_t launch_modesum32_group(const bz_modes *const *ms, const float2 *cons
     memset(&gd, 0, sizeof gd);
     gd.nitems = count;
     size_t sm = 0;
-    int64_t ctas = 0, whole = 0;
-    for (int i = 0; i < count; ++i) whole += ctas_for(v, n[i]);
+    int64_t whole = 0;
     for (int i = 0; i < count; ++i) {
         if (ms[i]->variant != v) return cudaErrorInvalidValue;
-        const int S = kVariants[v].rows > 1 ? launch_split(whole, ms[0]->var_bal[v], ms[0]->var_task_split[v], false) : 1;
-        fill_item(gd.item[i], ms[i], ms[i]->var_W[v], S > 1 ? ms[i]->var_task_split[v][split_index(S)] : ms[i]->var_task[v],
-                  ms[i]->var_rowmax[v], fhat[i], Qhat[i], n[i], S);
-        gd.tile_start[i] = ctas;
-        ctas += ctas_for(v, n[i]) * S;
+        whole += ctas_for(v, n[i]);
         sm = std::max(sm, smem_bytes<float>(ms[i]->g->v, ms[i]->var_rowmax[v], v));
     }
-    gd.tile_start[count] = ctas;
-    if (ctas == 0) return cudaSuccess;
+    for (int i = 0; i < count; ++i) {
+        // the launch's last partial wave, as far as it lies in the last instance
+        Tail tail{ctas_for(v, n[i]), 1};
+        if (i == count - 1 && count < kMaxGroup && (!ms[i]->variant_fixed || kVariants[v].rows > 1)) {
+            const Tail all = tail_split(ms[i], v, ms[i]->var_task[v], whole, sm, kStage32, kRagged32);
+            if (all.S > 1) tail = {tail.full - std::min(whole - all.full, tail.full), all.S};
+        }
+        add_items(gd, ms[i], v, ms[i]->var_W[v], ms[i]->var_task[v], ms[i]->var_rowmax[v], fhat[i], sizeof(float2),
+                  Qhat[i], sizeof(float2), n[i], tail);
+    }
+    if (gd.nitems == 0) return cudaSuccess;
     if (sm > 227 * 1024) return cudaErrorInvalidValue;
     return launch_group(gd, v, sm, st);
 }
@@ -1835,7 +1852,6 @@ static int autotune(bz_modes *m, int &rc) {
 
 int modes_build_fp32_tables(bz_modes *m) {
     m->d_W32 = nullptr;
-    m->d_task = nullptr;
     m->variant = 0;
     m->variant_fixed = 0;
     m->modesum_variant = 0;
@@ -1843,12 +1859,10 @@ int modes_build_fp32_tables(bz_modes *m) {
     bool any = false;
     for (int v = 0; v < kNumVariants; ++v) {
         m->var_W[v] = nullptr;
-        m->var_task[v] = nullptr;
+        m->var_task[v].block = nullptr;
         m->var_rowmax[v] = 0;
         void *w = nullptr;
-        for (int k = 0; k < kSplitTables; ++k) m->var_task_split[v][k] = nullptr;
-        int **split = kVariants[v].cells == 32 || kVariants[v].rows > 1 ? m->var_task_split[v] : nullptr;
-        if (build_variant<float>(m, v, rc, &w, &m->var_task[v], &m->var_rowmax[v], nullptr, split, m->var_bal[v])) {
+        if (build_variant<float>(m, v, rc, &w, &m->var_task[v], &m->var_rowmax[v])) {
             m->var_W[v] = static_cast<float *>(w);
             any = true;
         }
@@ -1856,25 +1870,21 @@ int modes_build_fp32_tables(bz_modes *m) {
     }
     // the small variant's tables beside those of the 16-warp paired variant
     m->small_W = nullptr;
-    m->small_task = nullptr;
-    for (int k = 0; k < kSplitTables; ++k) m->small_task_split[k] = nullptr;
+    m->small_task.block = nullptr;
     if (m->var_W[7]) {
         void *w = nullptr;
-        if (build_variant<float>(m, kSmallVariant, rc, &w, &m->small_task, &m->small_rowmax, nullptr,
-                                 m->small_task_split, m->small_bal))
+        if (build_variant<float>(m, kSmallVariant, rc, &w, &m->small_task, &m->small_rowmax))
             m->small_W = static_cast<float *>(w);
         if (rc) return rc;
     }
     // FP64 tables where the double spectrum fits shared memory
     m->w64 = nullptr;
-    m->task64 = nullptr;
+    m->task64.block = nullptr;
     m->rowmax64 = 0;
     m->variant64 = -1;
     m->wx2 = nullptr;
-    for (int k = 0; k < kSplitTables; ++k) m->task64_split[k] = nullptr;
     for (int q = 0; q < 3 && m->variant64 < 0; ++q) {
-        if (build_variant<double>(m, kFp64Variants[q], rc, &m->w64, &m->task64, &m->rowmax64, &m->wx2, m->task64_split,
-                                  m->bal64))
+        if (build_variant<double>(m, kFp64Variants[q], rc, &m->w64, &m->task64, &m->rowmax64, &m->wx2))
             m->variant64 = kFp64Variants[q];
         if (rc) return rc;
     }
@@ -1890,7 +1900,6 @@ int modes_build_fp32_tables(bz_modes *m) {
     if (rc) return rc;
     m->variant = v;
     m->d_W32 = m->var_W[v];
-    m->d_task = m->var_task[v];
     m->w32_rowmax = m->var_rowmax[v];
     m->modesum_variant = m->g->v.dim == 2 && m->g->v.N > 48 ? 0 : v + 1;   // one form only: no choice to report
     return BZ_OK;

@@ -42,3 +42,18 @@ def test_eight_cell_form(bz, dim, N, n):
     want = k.collide(fin, conserve=True)
     got = got.double().cpu().numpy()
     check_fp32_cells(k, fin, got, want, what="%dd N=%d" % (dim, N))
+
+
+@pytest.mark.parametrize("dim,N,precision,sizes", [
+    (2, 24, "fp32", (500, 1949, 7000)), (2, 32, "fp32", (2500, 5000, 9001)), (2, 48, "fp32", (1300, 3000, 6001)),
+    (2, 64, "fp32", (100, 700, 1501)), (3, 16, "fp32", (100, 700, 1401)), (2, 32, "fp64", (300, 2000)),
+    (2, 48, "fp32x2", (301, 1000))])
+def test_shared_tail_tiles(bz, dim, N, precision, sizes):
+    """Batches whose last tiles are shared by 2 to 8 CTAs: the bits of a batch that ends elsewhere."""
+    import torch
+    f = to_dev(workloads.bi_maxwellian(max(sizes), dim, N, 10.0, seed=N + 1), precision)
+    m = bz.Modes(bz.Grid(dim, N, 10.0), 1.0)
+    want = torch.cat([bz.collide_batch(m, part.contiguous(), precision=precision) for part in f.split(487)])
+    for n in sizes:
+        assert torch.equal(bz.collide_batch(m, f[:n].contiguous(), precision=precision), want[:n]), n
+    bz.check()
