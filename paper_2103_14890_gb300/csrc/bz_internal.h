@@ -325,6 +325,7 @@ cudaError_t launch_fill_zero(void *p, int64_t bytes, cudaStream_t st);
 // values at its three faces, FV [cell][3][nv], and the flux pass reads those
 // of the cell and its neighbours.  Scratch: fv_scratch_rows() rows of nv.
 bool fv_value_mode(const bz_mesh *mesh, const GridView &g, const void *f, const void *L);
+cudaError_t fv_values_setup();      // once per mesh: lets the value passes take their shared memory
 int64_t fv_scratch_rows(const bz_mesh *mesh, bool f32);
 cudaError_t launch_fv_values_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FV, cudaStream_t st);
 cudaError_t launch_fv_flux_values_f32(const bz_mesh *mesh, const GridView &g, const float *FV, float *L,

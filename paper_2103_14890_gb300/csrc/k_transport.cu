@@ -695,11 +695,12 @@ fv_faces3_tri_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTabl
 // positions of the processing order, walking them in steps of the grid; while
 // it computes one cell, the rows of the next one travel into shared memory by
 // cp.async (16 bytes per thread and row, each thread copying exactly the slots
-// it reads back, so no block barrier is needed and threads past nv leave at
+// it reads back, so no block barrier is needed and warps past nv leave at
 // once), and the index records of the cell after that are already being
 // loaded.  Writing whole rows of values unmasked costs this light
 // reconstruction less than forming and masking fluxes: 19802 triangles x 32^2,
-// 0.100 + 0.061 ms against 0.137 + 0.050 ms with upwind flux rows.
+// 0.094 + 0.055 ms (0.109 + 0.057 with table values loaded where they are
+// used) against 0.137 + 0.050 ms with upwind flux rows.
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
@@ -707,11 +708,22 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
+// The table values of a cell travel the same way, 4 bytes per lane into a buffer
+// of the warp (read in the order of processing they come from DRAM, and a block
+// that loads them when it needs them waits at every cell).
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
 constexpr int kFaceRows = 6;         // rows staged per cell: f_i and 5 stencil rows / 3 own and 3 neighbour face rows
 // blocks per SM: 3 for the reconstruction (85 registers, no spills; 4 spill
 // its record prefetch), 4 for the flux pass (64 registers)
 constexpr int kFacesCtasPerSm = 3, kFluxCtasPerSm = 4;
-constexpr size_t kFaceStageBytes = 2 * kFaceRows * kFvThreads * sizeof(float4);   // 48 KB
+// staged rows, then the warps' table values: 50 KB for 256 threads
+constexpr size_t face_stage_bytes(int threads) {
+    return 2 * kFaceRows * threads * sizeof(float4) + 2 * threads * sizeof(float);
+}
 
 // CWENO gradient of one pair of velocities of a flagged triangle (kFvRegularTri):
 // d[q] = fbar_{cen q} - fbar_i, the face neighbours in d[0..2]; sector s
@@ -765,20 +777,21 @@ __device__ __forceinline__ void cweno_pair_tri(const float2 (&d)[kFvCentral], co
     gy_out = mul2(ay, iw);
 }
 
-// Values at the three faces of the 4 velocities k..k+3 of a flagged triangle.
-__device__ __forceinline__ void tri_values_x2(float *__restrict__ FV, const FvTables<float> &tb,
-                                              const float4 (&fr)[kFvCentral], int64_t p, int64_t i, int k, int nv,
-                                              const float4 fi) {
+// Values at the three faces of the 4 velocities k..k+3 of a flagged triangle;
+// tab: its table values (kTabRs ...).
+constexpr int kTabRs = 0, kTabRc = 12, kTabPhi = 22, kTabH2 = 28, kTabValues = 29;
+__device__ __forceinline__ void tri_values_x2(float *__restrict__ FV, const float *tab, const float4 (&fr)[kFvCentral],
+                                              int64_t i, int k, int nv, const float4 fi, bool act) {
     float rx[kFvCentral], ry[kFvCentral];
 #pragma unroll
     for (int q = 0; q < kFvCentral; ++q) {
-        rx[q] = __ldg(tb.Rc + (p * 2) * kFvCentral + q);
-        ry[q] = __ldg(tb.Rc + (p * 2 + 1) * kFvCentral + q);
+        rx[q] = tab[kTabRc + q];
+        ry[q] = tab[kTabRc + kFvCentral + q];
     }
     float4 R[3];
 #pragma unroll
-    for (int s = 0; s < 3; ++s) R[s] = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (p * kFvMaxFaces + s) * 4));
-    const float h2 = __ldg(tb.quad + 4 * p + 3);
+    for (int s = 0; s < 3; ++s) R[s] = *reinterpret_cast<const float4 *>(tab + kTabRs + 4 * s);
+    const float h2 = tab[kTabH2];
     float2 gx[2], gy[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -790,11 +803,10 @@ __device__ __forceinline__ void tri_values_x2(float *__restrict__ FV, const FvTa
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        const float2 ox = dup2(__ldg(tb.phi + 2 * (p * kFvMaxFaces + q)));
-        const float2 oy = dup2(__ldg(tb.phi + 2 * (p * kFvMaxFaces + q) + 1));
+        const float2 ox = dup2(tab[kTabPhi + 2 * q]), oy = dup2(tab[kTabPhi + 2 * q + 1]);
         const float2 a = fma2(gy[0], oy, fma2(gx[0], ox, lo2(fi)));
         const float2 b = fma2(gy[1], oy, fma2(gx[1], ox, hi2(fi)));
-        *reinterpret_cast<float4 *>(FV + (i * 3 + q) * nv + k) = make_float4(a.x, a.y, b.x, b.y);
+        if (act) *reinterpret_cast<float4 *>(FV + (i * 3 + q) * nv + k) = make_float4(a.x, a.y, b.x, b.y);
     }
 }
 
@@ -807,40 +819,50 @@ __device__ __forceinline__ RecG rec_g(const int4 *__restrict__ tripos, int64_t p
     return RecG{a.x, a.y, {b.x, b.y, b.z, b.w, c.x}};
 }
 
-__global__ void __launch_bounds__(kFvThreads, kFacesCtasPerSm)
+template <int BT>
+__global__ void __launch_bounds__(BT, kFacesCtasPerSm * kFvThreads / BT)
 fv_values_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, FvTables<float> tb, FvIdx ix,
                          const int4 *__restrict__ tripos, int64_t n, int nv) {
-    extern __shared__ float4 stage[];            // [2][kFaceRows][kFvThreads]
-    const int t = threadIdx.x;
-    const int k = (blockIdx.y * kFvThreads + t) * 4;
-    if (k >= nv || (int64_t)blockIdx.x >= n) return;
+    extern __shared__ float4 stage[];            // [2][kFaceRows][BT], [2][warp][32] table values
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    float *const tabs = reinterpret_cast<float *>(stage + 2 * kFaceRows * BT) + warp * 32;
+    const int kt = (blockIdx.y * BT + t) * 4;
+    if (kt - 4 * lane >= nv || (int64_t)blockIdx.x >= n) return;   // warps past nv
+    const bool act = kt < nv;
+    const int k = act ? kt : 0;                  // the last warp's idle lanes store nothing
     const int64_t G = gridDim.x;
-    auto issue = [&](const RecG &r, int buf) {
-        float4 *sl = stage + buf * kFaceRows * kFvThreads + t;
+    // this lane's table value of position 0, and the distance between positions
+    const float *ts = lane < kTabRc ? tb.Rs + lane : lane < kTabPhi ? tb.Rc + (lane - kTabRc)
+                    : lane < kTabH2 ? tb.phi + (lane - kTabPhi) : tb.quad + 3;
+    const int td = lane < kTabRc ? kFvMaxFaces * 4 : lane < kTabPhi ? 2 * kFvCentral : lane < kTabH2 ? 2 * kFvMaxFaces : 4;
+    auto issue = [&](const RecG &r, int64_t pr, int buf) {
+        if (lane < kTabValues) cp_async4(tabs + buf * BT + lane, ts + pr * td);
+        float4 *sl = stage + buf * kFaceRows * BT + t;
         cp_async16(sl, f + (int64_t)r.i * nv + k);
 #pragma unroll
-        for (int q = 0; q < kFvCentral; ++q) cp_async16(sl + (q + 1) * kFvThreads, f + (int64_t)r.c[q] * nv + k);
+        for (int q = 0; q < kFvCentral; ++q) cp_async16(sl + (q + 1) * BT, f + (int64_t)r.c[q] * nv + k);
     };
     int64_t p = blockIdx.x;
     RecG cur = rec_g(tripos, p);
-    issue(cur, 0);
+    issue(cur, p, 0);
     cp_async_commit();
     RecG nxt = cur;
     if (p + G < n) nxt = rec_g(tripos, p + G);
     for (int it = 0;; ++it) {
         const bool more = p + G < n;
-        if (more) issue(nxt, (it + 1) & 1);
+        if (more) issue(nxt, p + G, (it + 1) & 1);
         cp_async_commit();
         RecG nn = nxt;
         if (p + 2 * G < n) nn = rec_g(tripos, p + 2 * G);
         cp_async_wait_prev();
-        const float4 *sl = stage + (it & 1) * kFaceRows * kFvThreads + t;
+        __syncwarp();
+        const float4 *sl = stage + (it & 1) * kFaceRows * BT + t;
         const float4 fi = sl[0];
         if (cur.ncf & kFvRegularTri) {
             float4 fr[kFvCentral];
 #pragma unroll
-            for (int q = 0; q < kFvCentral; ++q) fr[q] = sl[(q + 1) * kFvThreads];
-            tri_values_x2(FV, tb, fr, p, cur.i, k, nv, fi);
+            for (int q = 0; q < kFvCentral; ++q) fr[q] = sl[(q + 1) * BT];
+            tri_values_x2(FV, tabs + (it & 1) * BT, fr, cur.i, k, nv, fi, act);
         } else {
             Vec<float, 4> fv;
             fv.v[0] = fi.x; fv.v[1] = fi.y; fv.v[2] = fi.z; fv.v[3] = fi.w;
@@ -849,11 +871,13 @@ fv_values_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, Fv
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 point_value<float, 4, 2>(fv, c, tb.phi + (p * kFvMaxFaces + q) * 2, val);
-                *reinterpret_cast<float4 *>(FV + ((int64_t)cur.i * 3 + q) * nv + k) =
-                    make_float4(val[0], val[1], val[2], val[3]);
+                if (act)
+                    *reinterpret_cast<float4 *>(FV + ((int64_t)cur.i * 3 + q) * nv + k) =
+                        make_float4(val[0], val[1], val[2], val[3]);
             }
         }
         if (!more) break;
+        __syncwarp();
         p += G;
         cur = nxt;
         nxt = nn;
@@ -869,23 +893,29 @@ __device__ __forceinline__ RecF rec_f(const int4 *__restrict__ tripos, int64_t p
     return RecF{a.x, a.w, {c.y, c.z, c.w}};
 }
 
-__global__ void __launch_bounds__(kFvThreads, kFluxCtasPerSm)
+template <int BT>
+__global__ void __launch_bounds__(BT, kFluxCtasPerSm * kFvThreads / BT)
 fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ L, FvTables<float> tb,
                              const int4 *__restrict__ tripos, int64_t n, int nv, int N, float Lv, float dv) {
-    extern __shared__ float4 stage[];            // [2][kFaceRows][kFvThreads]
-    const int t = threadIdx.x;
-    const int k = (blockIdx.y * kFvThreads + t) * 4;
-    if (k >= nv || (int64_t)blockIdx.x >= n) return;
+    extern __shared__ float4 stage[];            // [2][kFaceRows][BT], [2][warp][32]: 3 (nx, ny), 1 / area
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    float *const tabs = reinterpret_cast<float *>(stage + 2 * kFaceRows * BT) + warp * 32;
+    const int kt = (blockIdx.y * BT + t) * 4;
+    if (kt - 4 * lane >= nv || (int64_t)blockIdx.x >= n) return;
+    const bool act = kt < nv;
+    const int k = act ? kt : 0;
     const int64_t G = gridDim.x;
     // positions from the end of the order (the rows the reconstruction wrote last are still in L2)
     auto pos = [&](int64_t p) { return n - 1 - p; };
-    auto issue = [&](const RecF &r, int buf) {
-        float4 *sl = stage + buf * kFaceRows * kFvThreads + t;
+    auto issue = [&](const RecF &r, int64_t pr, int buf) {
+        if (lane < 7)
+            cp_async4(tabs + buf * BT + lane, lane < 6 ? tb.fn + pos(pr) * kFvMaxFaces * 2 + lane : tb.inv_area + pos(pr));
+        float4 *sl = stage + buf * kFaceRows * BT + t;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            cp_async16(sl + q * kFvThreads, FV + ((int64_t)r.i * 3 + q) * nv + k);
+            cp_async16(sl + q * BT, FV + ((int64_t)r.i * 3 + q) * nv + k);
             if (r.nb[q] >= 0)
-                cp_async16(sl + (3 + q) * kFvThreads, FV + ((int64_t)r.nb[q] * 3 + ((r.qbits >> (2 * q)) & 3)) * nv + k);
+                cp_async16(sl + (3 + q) * BT, FV + ((int64_t)r.nb[q] * 3 + ((r.qbits >> (2 * q)) & 3)) * nv + k);
         }
     };
     const int j1 = k / N, j2 = k - j1 * N;
@@ -896,26 +926,27 @@ fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ 
     const float2 hf = dup2(0.5f);
     int64_t p = blockIdx.x;
     RecF cur = rec_f(tripos, pos(p));
-    issue(cur, 0);
+    issue(cur, p, 0);
     cp_async_commit();
     RecF nxt = cur;
     if (p + G < n) nxt = rec_f(tripos, pos(p + G));
     for (int it = 0;; ++it) {
         const bool more = p + G < n;
-        if (more) issue(nxt, (it + 1) & 1);
+        if (more) issue(nxt, p + G, (it + 1) & 1);
         cp_async_commit();
         RecF nn = nxt;
         if (p + 2 * G < n) nn = rec_f(tripos, pos(p + 2 * G));
         cp_async_wait_prev();
-        const float4 *sl = stage + (it & 1) * kFaceRows * kFvThreads + t;
+        __syncwarp();
+        const float *tab = tabs + (it & 1) * BT;
+        const float4 *sl = stage + (it & 1) * kFaceRows * BT + t;
         const int64_t i = cur.i;
         float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const float4 fl = sl[q * kFvThreads];
-            const float4 fr = cur.nb[q] >= 0 ? sl[(3 + q) * kFvThreads] : fl;
-            const int64_t s = pos(p) * kFvMaxFaces + q;
-            const float nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
+            const float4 fl = sl[q * BT];
+            const float4 fr = cur.nb[q] >= 0 ? sl[(3 + q) * BT] : fl;
+            const float nx = tab[2 * q], ny = tab[2 * q + 1];
             const float2 v1nx = dup2(v1 * nx);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -926,10 +957,11 @@ fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ 
                 acc[h] = fma2(nah, add2(b, make_float2(-a.x, -a.y)), acc[h]);
             }
         }
-        const float2 ia = dup2(__ldg(tb.inv_area + pos(p)));
+        const float2 ia = dup2(tab[6]);
         const float2 o0 = mul2(acc[0], ia), o1 = mul2(acc[1], ia);
-        *reinterpret_cast<float4 *>(L + i * nv + k) = make_float4(o0.x, o0.y, o1.x, o1.y);
+        if (act) *reinterpret_cast<float4 *>(L + i * nv + k) = make_float4(o0.x, o0.y, o1.x, o1.y);
         if (!more) break;
+        __syncwarp();
         p += G;
         cur = nxt;
         nxt = nn;
@@ -1212,11 +1244,31 @@ void faces_launch(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaSt
             f, FX, pick<T>(m), indices(m), flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
 }
 
-// persistent grid of the value passes: cps blocks per SM over the velocity blocks
+// Threads of a block of the value passes, no more than a row needs as far as
+// that goes (a row of 16^2 has 64), and their persistent grid: as many warps
+// per SM as cps blocks of kFvThreads.  Transport of 19802 triangles with 256
+// threads at every size and as here: 16^2 97 and 45 us, 24^2 117 and 97 us.
+// The flux pass takes two thirds of them while the value rows stay in L2 (64 MB of
+// 129): 24^2 on 4050 cells 26.8 and 25.7 us; on 12800, out of L2, 66.0 and 69.4.
+int values_threads(int nv) { return nv <= 256 ? 64 : nv <= 512 ? 128 : nv <= 640 ? 160 : kFvThreads; }
 dim3 values_grid(const bz_mesh *m, int nv, int cps) {
-    const int gy = (nv / 4 + kFvThreads - 1) / kFvThreads;
-    const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(m->n_cells, (int64_t)fv_sm_count() * cps / gy));
-    return dim3((unsigned)gx, (unsigned)gy);
+    const int bt = values_threads(nv), gy = (nv / 4 + bt - 1) / bt;
+    int b = cps * kFvThreads / bt;
+    if (cps == kFluxCtasPerSm && bt < kFvThreads && 12 * m->n_cells * nv <= (64 << 20)) b = b * 2 / 3;
+    const int64_t blocks = (int64_t)fv_sm_count() * b / gy;
+    return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(m->n_cells, blocks)), (unsigned)gy);
+}
+template <int BT>
+void values_launch(const bz_mesh *m, const GridView &g, const float *f, float *FV, cudaStream_t st) {
+    const int nv = (int)g.nv;
+    fv_values_persist_kernel<BT><<<values_grid(m, nv, kFacesCtasPerSm), BT, face_stage_bytes(BT), st>>>(
+        f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
+}
+template <int BT>
+void flux_values_launch(const bz_mesh *m, const GridView &g, const float *FV, float *L, cudaStream_t st) {
+    const int nv = (int)g.nv;
+    fv_flux_values_persist_kernel<BT><<<values_grid(m, nv, kFluxCtasPerSm), BT, face_stage_bytes(BT), st>>>(
+        FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
 }
 
 // FP64 takes one velocity per thread (the FP64 pipe is the bound, so loads per
@@ -1311,6 +1363,13 @@ cudaError_t first(const bz_mesh *m, const GridView &g, const T *f, T *L, cudaStr
 
 }  // namespace
 
+cudaError_t fv_values_setup() {
+    const cudaError_t e = allow_dynamic_smem((const void *)fv_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads));
+    return e != cudaSuccess ? e
+                            : allow_dynamic_smem((const void *)fv_flux_values_persist_kernel<kFvThreads>,
+                                                 face_stage_bytes(kFvThreads));
+}
+
 bool fv_value_mode(const bz_mesh *m, const GridView &g, const void *f, const void *L) {
     return m->d_tripos && m->n_walls == 0 && g.N % 4 == 0 && aligned(f, 16) && aligned(L, 16);
 }
@@ -1323,17 +1382,23 @@ int64_t fv_scratch_rows(const bz_mesh *m, bool f32) {
 
 cudaError_t launch_fv_values_f32(const bz_mesh *m, const GridView &g, const float *f, float *FV, cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
-    const int nv = (int)g.nv;
-    fv_values_persist_kernel<<<values_grid(m, nv, kFacesCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
-        f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
+    switch (values_threads((int)g.nv)) {
+        case 64: values_launch<64>(m, g, f, FV, st); break;
+        case 128: values_launch<128>(m, g, f, FV, st); break;
+        case 160: values_launch<160>(m, g, f, FV, st); break;
+        default: values_launch<kFvThreads>(m, g, f, FV, st);
+    }
     return cudaGetLastError();
 }
 cudaError_t launch_fv_flux_values_f32(const bz_mesh *m, const GridView &g, const float *FV, float *L,
                                       cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
-    const int nv = (int)g.nv;
-    fv_flux_values_persist_kernel<<<values_grid(m, nv, kFluxCtasPerSm), kFvThreads, kFaceStageBytes, st>>>(
-        FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+    switch (values_threads((int)g.nv)) {
+        case 64: flux_values_launch<64>(m, g, FV, L, st); break;
+        case 128: flux_values_launch<128>(m, g, FV, L, st); break;
+        case 160: flux_values_launch<160>(m, g, FV, L, st); break;
+        default: flux_values_launch<kFvThreads>(m, g, FV, L, st);
+    }
     return cudaGetLastError();
 }
 

@@ -71,3 +71,16 @@ def test_stage_kernels_fp64(bz, dim, N, scheme, model):
     bz.check()
     want = oracle.Kernel(dim, N, 8.0, 0.0).imex_step(f, 2e-3, 5e-2, scheme=scheme, model=model)
     assert relerr(got.cpu().numpy(), want) < 1e-12
+
+
+@pytest.mark.parametrize("N", [12, 16, 20, 24, 28])
+def test_value_pass_blocks(bz, fvo, N):
+    """The FP32 triangle passes of degree 1 with 64, 128, 160 and 256 threads, the last warp not always full, on more
+    cells than a thin mesh has and on none of the sizes of the passes' grids."""
+    pts, tri = workloads.sod_triangulation(18, jitter=0.2)
+    om = fvo.Mesh(pts, tri)
+    f = workloads.mesh_states(om.bary, N, 6.0)
+    fin = as_input(f, "fp32")
+    Lr = bz.transport_residual(bz.Mesh(pts, tri, order=2), bz.Grid(2, N, 6.0), to_dev(f, "fp32"), precision="fp32")
+    bz.check()
+    _check(Lr.double().cpu().numpy(), fvo.transport_residual(om, fin, N, 6.0, order=2), om, fin, N, 6.0, 2, fvo, U32, ETA32)
