@@ -127,7 +127,8 @@ constexpr int kFvMaxFaces = 8;
 constexpr int kFvCentral = 5;       // central stencil: the cell and its 5 nearest cells (2 x 3 cells)
 constexpr int kFvCentral3 = 11;     // degree 2: the cell and its 11 nearest cells (2 x 6 cells)
 constexpr int kFvCoef3 = 5;         // degree 2: coefficients of xi, eta, xi^2, xi eta, eta^2
-constexpr int kFvRegularTri = 0x100;  // flag in ncen: a triangle whose stencil starts with its 3 face neighbours
+constexpr int kFvRegular = 0x100;     // flag in ncen: a full stencil that starts with the neighbours of all the
+                                      // cell's faces in order, and a sector at every vertex
 
 // Tables of the transport step, one row per position p of the processing order
 // (cell order[p]).  Order 2 reconstructs a gradient (B = 2 coefficients from
@@ -135,7 +136,8 @@ constexpr int kFvRegularTri = 0x100;  // flag in ncen: a triangle whose stencil 
 // scaled Taylor basis phi = (xi, eta, xi^2 - mu20, xi eta - mu11, eta^2 -
 // mu02), xi = (x - x_b)/h, from K = kFvCentral3 cells.  The FP64 tables have
 // factors folded in that save FP64 operations: order 2 is scaled to xi, eta
-// too, and Rc is divided by lambda_0 where the cell has sectors.
+// too, Rc is divided by lambda_0 where the cell has sectors, and in cells
+// flagged kFvRegular the rows of Rc give p_0, the sectors' share taken off.
 template <typename T> struct FvTables {
     const T *Rs;            // [p][face][4]  sector inverses (row-major 2 x 2)
     const T *quad;          // [p][4]  FP32: (mu20, mu11, mu02, h^2); FP64: the degree-2 smoothness form's
@@ -167,7 +169,7 @@ struct bz_mesh {
     int *d_fid;             // [p][face] face index, numbered in the processing order of the owners
     int *d_two;             // [p][face] index of a two-sided face
     int64_t n_two;
-    int *d_ncen;            // [p] central stencil size (<= K), | kFvRegularTri for a triangle whose stencil
+    int *d_ncen;            // [p] central stencil size (<= K), | kFvRegular for a triangle whose stencil
                             // starts with its face neighbours, sector s on faces s, s+1
     int *d_cen;             // [p][K]
     int *d_nsec;            // [p] sectors

@@ -157,7 +157,25 @@ std::vector<double> fill_real(const HostMesh &h, bool folded) {
     put(h.fn, kFvMaxFaces * 2, one);
     put(h.phi, kFvMaxFaces * h.B, ih);
     put(h.phig, h.B == kFvCoef3 ? kFvMaxFaces * 2 * h.B : 0, one);
-    put(h.Rc, h.B * h.K, [&](int i) { return hc(i) * (h.nsec[i] > 0 ? 4.0 / 3.0 : 1.0); });
+    if (folded) {
+        // p_0 in place of p_opt: over lambda_0 and, in flagged cells, less the
+        // sectors' share (linear in the differences to the face neighbours)
+        std::vector<double> rc(h.Rc);
+        for (int64_t i = 0; h.B && i < h.n; ++i) {
+            const int ns = h.nsec[i];
+            double *R = &rc[(size_t)i * h.B * h.K];
+            for (int e = 0; e < h.B * h.K; ++e) R[e] *= hc((int)i) * (ns > 0 ? 4.0 / 3.0 : 1.0);
+            const double *S = &h.Rs[(size_t)i * kFvMaxFaces * 4];
+            for (int q = 0; (h.ncen[i] & kFvRegular) && q < ns; ++q) {
+                const double *Sa = S + 4 * q, *Sb = S + 4 * ((q + ns - 1) % ns), f = hc((int)i) / (3.0 * ns);
+                R[q] -= f * (Sa[0] + Sb[1]);
+                R[h.K + q] -= f * (Sa[2] + Sb[3]);
+            }
+        }
+        put(rc, h.B * h.K, one);
+    } else {
+        put(h.Rc, h.B * h.K, one);
+    }
     put(h.inv_area, 1, one);
     return out;
 }
@@ -473,18 +491,18 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                 ++ns;
             }
             h.nsec[i] = ns;
-            // A triangle with three sectors whose face neighbours all lie in
-            // its full central stencil (nearly every interior cell of a
-            // triangle mesh): the stencil is reordered to start with the face
-            // neighbours in face order and the cell is flagged, so that the
-            // FP32 reconstruction loads every neighbour row once for the
-            // central and the sector gradients (sector s joins faces s and
-            // s + 1 mod 3).
+            // A cell with a sector at every vertex whose face neighbours all lie
+            // in its full central stencil (nearly every interior cell): the
+            // stencil is reordered to start with the face neighbours in face
+            // order and the cell is flagged, so that the FP32 reconstruction
+            // of triangles and the FP64 one load every neighbour row once
+            // for the central and the sector gradients (sector s joins faces s
+            // and s + 1, cyclically).
             auto face_first = [&](int *cn, double *R) {
-                if (k != 3 || ns != 3 || h.ncen[i] != K) return;
+                if (ns != k || h.ncen[i] != K || k > K) return;
                 int perm[kFvCentral3];
                 bool used[kFvCentral3] = {};
-                for (int q = 0; q < 3; ++q) {
+                for (int q = 0; q < k; ++q) {
                     const int j = h.nb[(size_t)i * kFvMaxFaces + q];
                     int hit = -1;
                     for (int t = 0; t < K && hit < 0; ++t)
@@ -493,7 +511,7 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                     used[hit] = true;
                     perm[q] = hit;
                 }
-                for (int t = 0, p = 3; t < K; ++t)
+                for (int t = 0, p = k; t < K; ++t)
                     if (!used[t]) perm[p++] = t;
                 int c0[kFvCentral3];
                 double r0[kFvCoef3 * kFvCentral3];
@@ -503,7 +521,7 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                     cn[t] = c0[perm[t]];
                     for (int r = 0; r < B; ++r) R[r * K + t] = r0[r * K + perm[t]];
                 }
-                h.ncen[i] |= kFvRegularTri;
+                h.ncen[i] |= kFvRegular;
             };
             face_first(&h.cen[i * K], &h.Rc[(size_t)i * B * K]);
         }

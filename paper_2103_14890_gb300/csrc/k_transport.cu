@@ -34,8 +34,10 @@
 // cell in place of 5 and 24 for degree 2) and cuts the arithmetic that bounds
 // FP64 (the GB300 does 2 FP64 operations per clock and SM): per hexagon face
 // and velocity 9 operations in place of 34.  19802 triangles x 32^2, FP32,
-// degree 2: 0.382 -> 0.253 ms; 2603 Voronoi cells x
-// 30^2, FP64, degree 2: 2.13 -> 1.34 ms.
+// degree 2: 0.382 -> 0.253 ms; 2603 Voronoi cells x 30^2, FP64, degree 2: 2.13
+// -> 1.34 ms, 1.20 with p_0's rows and one difference per neighbour in the
+// cells flagged kFvRegular (about 227 FP64 operations per hexagon and velocity
+// for 260: pass 1 1.27 -> 1.13 ms, the FP64 pipe nine tenths busy).
 //
 // Reconstruction: the central (least-squares) coefficients and the sector
 // polynomials are linear in the averages (tables Rc, Rs of fv_mesh.cpp);
@@ -129,10 +131,16 @@ struct FvIdx {
     const int *order, *meta, *fid, *two, *ncen, *cen, *nsec, *sec;
 };
 
-// min of two non-negative numbers as integers (the same order; a NaN operand
-// ends in NaN weights either way): it leaves the FP64 pipe alone.
-__device__ __forceinline__ double min_nonneg(double a, double b) {
-    return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
+// 2^e / b for b > 0, e given as scale = e << 20: rcp64 with the power of two
+// added to the exponent of the first approximation, off the FP64 pipe.  The
+// result lies below 2^1022; below the normal range it is flushed to (nearly) 0.
+__device__ __forceinline__ double scaled_rcp(double b, int scale) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    double e = fma(-b, y, 1.0);
+    e = fma(e, e, e);
+    y = __hiloint2double(max(__double2hiint(y) + scale, 0), __double2loint(y));
+    return fma(y, e, y);
 }
 
 // Write the flux of VEC velocities through a face: vn (outward normal velocity
@@ -186,36 +194,55 @@ __device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, co
                                                 double (&c)[B]) {
 #pragma unroll
     for (int l = 0; l < B; ++l) c[l] = 0.0;
-    const int nc = ncf & (kFvRegularTri - 1), ns = __ldg(ix.nsec + p);
-    const double *Rc = tb.Rc + p * (B * K);
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-        if (q < nc) {
-            const double d = f[(int64_t)__ldg(ix.cen + p * K + q) * nv + k] - fi;
-#pragma unroll
-            for (int l = 0; l < B; ++l) c[l] = fma(__ldg(Rc + l * K + q), d, c[l]);
-        }
-    }
-    if (ns == 0) return;
+    const int nc = ncf & (kFvRegular - 1), ns = __ldg(ix.nsec + p);
+    const double *Rc = tb.Rc + p * (B * K), *Rs = tb.Rs + p * kFvMaxFaces * 4;
     constexpr double kLam0 = 0.75, kEps = 1e-14;
     const double lamL = 0.25 / (double)ns;
-    double sx[MAXS], sy[MAXS], sumx = 0.0, sumy = 0.0;
+    double sx[MAXS], sy[MAXS];
+    if (ncf & kFvRegular) {              // uniform over the block; the rows of p_0, the sectors' share included
+        double d[MAXS];
 #pragma unroll
-    for (int s = 0; s < MAXS; ++s) {
-        if (s < ns) {
-            const int a = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2), b = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2 + 1);
-            const double *R = tb.Rs + (p * kFvMaxFaces + s) * 4;
-            const double da = f[(int64_t)a * nv + k] - fi, db = f[(int64_t)b * nv + k] - fi;
-            sx[s] = fma(__ldg(R), da, __ldg(R + 1) * db);
-            sy[s] = fma(__ldg(R + 2), da, __ldg(R + 3) * db);
-            sumx += sx[s];
-            sumy += sy[s];
+        for (int q = 0; q < K; ++q) {
+            const double dq = f[(int64_t)__ldg(ix.cen + p * K + q) * nv + k] - fi;
+            if (q < MAXS) d[q] = dq;
+#pragma unroll
+            for (int l = 0; l < B; ++l) c[l] = fma(__ldg(Rc + l * K + q), dq, c[l]);
         }
+#pragma unroll
+        for (int s = 0; s < MAXS; ++s)
+            if (s < ns) {
+                const double db = s + 1 < ns ? d[(s + 1) % MAXS] : d[0];
+                sx[s] = fma(__ldg(Rs + 4 * s), d[s], __ldg(Rs + 4 * s + 1) * db);
+                sy[s] = fma(__ldg(Rs + 4 * s + 2), d[s], __ldg(Rs + 4 * s + 3) * db);
+            }
+    } else {
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            if (q < nc) {
+                const double d = f[(int64_t)__ldg(ix.cen + p * K + q) * nv + k] - fi;
+#pragma unroll
+                for (int l = 0; l < B; ++l) c[l] = fma(__ldg(Rc + l * K + q), d, c[l]);
+            }
+        }
+        if (ns == 0) return;
+        double sumx = 0.0, sumy = 0.0;
+#pragma unroll
+        for (int s = 0; s < MAXS; ++s) {
+            if (s < ns) {
+                const int a = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2), b = __ldg(ix.sec + (p * kFvMaxFaces + s) * 2 + 1);
+                const double da = f[(int64_t)a * nv + k] - fi, db = f[(int64_t)b * nv + k] - fi;
+                sx[s] = fma(__ldg(Rs + 4 * s), da, __ldg(Rs + 4 * s + 1) * db);
+                sy[s] = fma(__ldg(Rs + 4 * s + 2), da, __ldg(Rs + 4 * s + 3) * db);
+                sumx += sx[s];
+                sumy += sy[s];
+            }
+        }
+        // p_0's coefficients (1 / lambda_0 is in Rc)
+        const double lam10 = lamL * (4.0 / 3.0);
+        c[0] = fma(-lam10, sumx, c[0]);
+        c[1] = fma(-lam10, sumy, c[1]);
     }
-    // p_0's coefficients (1 / lambda_0 is in Rc), sigma + eps of every polynomial
-    const double lam10 = lamL * (4.0 / 3.0);
-    c[0] = fma(-lam10, sumx, c[0]);
-    c[1] = fma(-lam10, sumy, c[1]);
+    // sigma + eps of every polynomial
     double s0 = fma(c[0], c[0], fma(c[1], c[1], kEps));
     if constexpr (B == kFvCoef3) {
         const double *q = tb.quad + 4 * p;
@@ -224,20 +251,23 @@ __device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, co
         s0 = fma(c[3], fma(__ldg(q + 1), c[3], q3 * c[4]), s0);
         s0 = fma(c[4], __ldg(q + 2) * c[4], s0);
     }
-    double sig[MAXS], num = s0;
+    double sig[MAXS];
+    int least = __double2hiint(s0);
 #pragma unroll
     for (int s = 0; s < MAXS; ++s)
         if (s < ns) {
             sig[s] = fma(sx[s], sx[s], fma(sy[s], sy[s], kEps));
-            num = min_nonneg(num, sig[s]);
+            least = min(least, __double2hiint(sig[s]));
         }
-    double r = num * rcp64(s0);
+    // weights (2^e / (sigma + eps))^4, 2^e the power of two below the least of them
+    const int scale = (least & 0x7ff00000) - 0x3ff00000;
+    double r = scaled_rcp(s0, scale);
     r = r * r;
     double w = kLam0 * (r * r), wl = 0.0, ax = 0.0, ay = 0.0;
 #pragma unroll
     for (int s = 0; s < MAXS; ++s)
         if (s < ns) {
-            r = num * rcp64(sig[s]);
+            r = scaled_rcp(sig[s], scale);
             r = r * r;
             r = r * r;
             wl += r;
@@ -258,7 +288,7 @@ template <int VEC, int MAXS>
 __device__ __forceinline__ void recon_coefs_f32(const float *__restrict__ f, const FvTables<float> &tb, const FvIdx &ix,
                                                 int64_t p, int ncf, int k, int nv, const Vec<float, VEC> &fi,
                                                 float (&c)[2][VEC]) {
-    const int nc = ncf & (kFvRegularTri - 1), ns = __ldg(ix.nsec + p);
+    const int nc = ncf & (kFvRegular - 1), ns = __ldg(ix.nsec + p);
     // central least-squares gradient
     float gx[VEC], gy[VEC];
     {
@@ -369,7 +399,7 @@ __device__ __forceinline__ void recon_coefs_f32(const float *__restrict__ f, con
     for (int l = 0; l < kFvCoef3; ++l)
 #pragma unroll
         for (int u = 0; u < VEC; ++u) c[l][u] = 0.f;
-    const int nc = ncf & (kFvRegularTri - 1);
+    const int nc = ncf & (kFvRegular - 1);
     const float *Rc = tb.Rc + p * kFvCoef3 * kFvCentral3;
 #pragma unroll
     for (int q = 0; q < kFvCentral3; ++q) {
@@ -536,7 +566,7 @@ __device__ __forceinline__ void recon_faces(const T *__restrict__ f, T *__restri
                                  c);
 }
 
-// Weights of one pair of velocities of a flagged triangle (kFvRegularTri: its
+// Weights of one pair of velocities of a flagged triangle (kFvRegular: its
 // stencil starts with the face neighbours; sector s joins faces s and s + 1
 // mod 3) in FP32x2: c holds p_opt's coefficients, d the differences to the face
 // neighbours; the steps of recon_coefs_f32.
@@ -657,7 +687,7 @@ __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restri
     const Vec<T, VEC> fi = ldv<T, VEC>(f + (int64_t)__ldg(ix.order + p) * nv + k);
     const Velocity<T, VEC> v(k, N, Lv, dv);
     if constexpr (sizeof(T) == 4 && VEC == 4 && MAXF == 3) {
-        if (ncf & kFvRegularTri) {      // uniform over the block: one cell per block
+        if (ncf & kFvRegular) {      // uniform over the block: one cell per block
             float c[B][4];
             coefs_tri_x2<B, K>(tb, p, fi, [&](int q) {
                 return *reinterpret_cast<const float4 *>(f + (int64_t)__ldg(ix.cen + p * K + q) * nv + k);
@@ -725,7 +755,7 @@ constexpr size_t face_stage_bytes(int threads) {
     return 2 * kFaceRows * threads * sizeof(float4) + 2 * threads * sizeof(float);
 }
 
-// CWENO gradient of one pair of velocities of a flagged triangle (kFvRegularTri):
+// CWENO gradient of one pair of velocities of a flagged triangle (kFvRegular):
 // d[q] = fbar_{cen q} - fbar_i, the face neighbours in d[0..2]; sector s
 // joins faces s and s + 1 mod 3.  The steps are those of
 // recon_coefs_f32 (central gradient, sector gradients, g_0, smoothness, weights as
@@ -858,7 +888,7 @@ fv_values_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, Fv
         __syncwarp();
         const float4 *sl = stage + (it & 1) * kFaceRows * BT + t;
         const float4 fi = sl[0];
-        if (cur.ncf & kFvRegularTri) {
+        if (cur.ncf & kFvRegular) {
             float4 fr[kFvCentral];
 #pragma unroll
             for (int q = 0; q < kFvCentral; ++q) fr[q] = sl[(q + 1) * BT];
