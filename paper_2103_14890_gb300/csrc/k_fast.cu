@@ -32,7 +32,11 @@
 // pass B of direction p - 1 at the same time on a double-buffered Y (fewer
 // CTAs per SM, idle warps at the pipeline's fill and drain: +23 %), and one
 // shared FFT body for all passes with cp.async loads of the half spectrum
-// (the paired-cell pass C it needs runs on half the threads: +3 %).
+// (the paired-cell pass C it needs runs on half the threads: +3 %).  A third,
+// persistent CTAs that copy the next cells' spectra during the last pass B,
+// was slower at A = 8 (19802 cells: 398 us against 382).  The spectra come by
+// cp.async, every copy in flight at once: with plain loads, a few at a time,
+// 393 us at 32^2 and 2116 us at 48^2 (now 1715).
 #include <limits.h>
 
 #include "bz_device.cuh"
@@ -77,6 +81,12 @@ template <int BYTES> __device__ __forceinline__ void cp_async_val(void *smem, co
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
 }
+// The same, or zeros where !take (nothing is read).
+template <int BYTES> __device__ __forceinline__ void cp_async_val_or_zero(void *smem, const void *gmem, bool take) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    const int src = take ? BYTES : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gmem), "n"(BYTES), "r"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit_wait_all() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_all;\n" ::: "memory");
 }
@@ -105,9 +115,8 @@ fast_collide_kernel(const typename C2<T>::type *__restrict__ fh, typename C2<T>:
     };
     stage_cf(0);
     for (int i = tid; i < Sh::nF; i += Sh::NT) {
-        const int c = i % C, mode = i / C;
-        const int64_t cell = cell0 + c;
-        F[i] = cell < n ? fh[tiled_index(cell, mode, nhalf)] : cmk<V2>((S)0., (S)0.);
+        const int64_t cell = cell0 + i % C;
+        cp_async_val_or_zero<(int)sizeof(V2)>(F + i, fh + tiled_index(cell < n ? cell : cell0, i / C, nhalf), cell < n);
     }
     cp_async_commit_wait_all();
     __syncthreads();
