@@ -383,11 +383,12 @@ int collide_chain(const bz_modes *m, int precision, int flags, const void *f, vo
 // Transport residual L [cell][nv] of f over the mesh: one pass for order 1,
 // else the face fluxes or values into scratch (`ext` if given:
 // transport_scratch_bytes), then their sums.
-size_t transport_scratch_bytes(const bz_mesh *mesh, const bz_grid *g, int precision) {
-    return (size_t)fv_scratch_rows(mesh, precision != BZ_FP64) * g->v.nv *
+size_t transport_scratch_bytes(const bz_mesh *mesh, const bz_grid *g, int precision, bool step = false) {
+    return (size_t)fv_scratch_rows(mesh, precision != BZ_FP64, step) * g->v.nv *
            (precision == BZ_FP64 ? sizeof(double) : sizeof(float));
 }
 
+// ext: the scratch of a step (transport_scratch_bytes with step).
 int transport_chain(const bz_mesh *mesh, const bz_grid *g, int precision, const void *f, void *L, cudaStream_t st,
                     void *ext = nullptr) {
     const GridView &v = g->v;
@@ -410,6 +411,15 @@ int transport_chain(const bz_mesh *mesh, const bz_grid *g, int precision, const 
                   "transport: reconstruction");
         BZ_LAUNCH("fv_flux_values_f32", st,
                   launch_fv_flux_values_f32(mesh, v, static_cast<const float *>(FX), static_cast<float *>(L), st),
+                  "transport: fluxes");
+        return BZ_OK;
+    }
+    if (ext && fv_two_sided(mesh, !d)) {
+        BZ_LAUNCH("fv_faces_two_f32", st,
+                  launch_fv_faces_two_f32(mesh, v, static_cast<const float *>(f), static_cast<float *>(FX), st),
+                  "transport: reconstruction");
+        BZ_LAUNCH("fv_sum_two_f32", st,
+                  launch_fv_sum_two_f32(mesh, v, static_cast<const float *>(FX), static_cast<float *>(L), st),
                   "transport: fluxes");
         return BZ_OK;
     }
@@ -1000,7 +1010,8 @@ int imex_step_fv(const bz_modes *m, const bz_mesh *mesh, int scheme, int model, 
         if (rc) return rc;
     }
     const size_t step_bytes = (step_scratch_bytes(m, t, n, precision) + 255) / 256 * 256;
-    const size_t bytes = step_bytes + (size_t)t.s * n * m->g->v.nv * es + transport_scratch_bytes(mesh, m->g, precision);
+    const size_t bytes = step_bytes + (size_t)t.s * n * m->g->v.nv * es +
+                         transport_scratch_bytes(mesh, m->g, precision, true);
     Scratch s;
     BZ_TRY(s.alloc(bytes, st), "imex_step_fv: scratch");
     return step_sequence_fv(m, mesh, t, model, dt, eps, f_n, f_out, n, precision, flags, st, s.p, step_bytes);

@@ -82,10 +82,10 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 
 // Launch `kernel`; pdl: as a programmatic dependent of the kernel before it.
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
                          A... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

@@ -328,7 +328,15 @@ cudaError_t launch_fill_zero(void *p, int64_t bytes, cudaStream_t st);
 // of the cell and its neighbours.  Scratch: fv_scratch_rows() rows of nv.
 bool fv_value_mode(const bz_mesh *mesh, const GridView &g, const void *f, const void *L);
 cudaError_t fv_values_setup();      // once per mesh: lets the value passes take their shared memory
-int64_t fv_scratch_rows(const bz_mesh *mesh, bool f32);
+int64_t fv_scratch_rows(const bz_mesh *mesh, bool f32, bool step);
+// Whether an IMEX step takes every face as two-sided: FP32, degree 2, thin cells.
+// A step can be unstable in thin cells (their CFL limit is far below the
+// others'), and growth by many orders of magnitude within a step shows the
+// rounding of every cell around them: there the sums stay term by term those
+// of the two-sided Rusanov form.
+bool fv_two_sided(const bz_mesh *mesh, bool f32);
+cudaError_t launch_fv_faces_two_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FX, cudaStream_t st);
+cudaError_t launch_fv_sum_two_f32(const bz_mesh *mesh, const GridView &g, const float *FX, float *L, cudaStream_t st);
 cudaError_t launch_fv_values_f32(const bz_mesh *mesh, const GridView &g, const float *f, float *FV, cudaStream_t st);
 cudaError_t launch_fv_flux_values_f32(const bz_mesh *mesh, const GridView &g, const float *FV, float *L,
                                       cudaStream_t st);

@@ -660,8 +660,8 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                 tp[3 * p + 2] = make_int4(c[4], nb[0], nb[1], nb[2]);
             }
             e = upload(&m->d_tripos, tp);
-            if (e == cudaSuccess) e = fv_values_setup();
         }
+        if (e == cudaSuccess && maxf <= 3) e = fv_values_setup();
     }
     double *r64 = nullptr;
     float *r32 = nullptr;

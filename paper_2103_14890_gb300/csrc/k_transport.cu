@@ -483,15 +483,21 @@ __device__ __forceinline__ void recon_coefs_f32(const float *__restrict__ f, con
     }
 }
 
+// A table value: in global memory, or staged in shared memory (SM).
+template <bool SM, typename X> __device__ __forceinline__ X tab_load(const X *p) {
+    if constexpr (SM) return *p;
+    else return __ldg(p);
+}
+
 // f + sum_l c_l phi_l for VEC velocities.
-template <typename T, int VEC, int B>
+template <typename T, int VEC, int B, bool SM = false>
 __device__ __forceinline__ void point_value(const Vec<T, VEC> &fi, const T (&c)[B][VEC], const T *__restrict__ phi,
                                             T (&val)[VEC]) {
     if constexpr (sizeof(T) == 4 && VEC == 4) {
         float2 x = make_float2(fi.v[0], fi.v[1]), y = make_float2(fi.v[2], fi.v[3]);
 #pragma unroll
         for (int l = 0; l < B; ++l) {
-            const float2 ph = dup2(__ldg(phi + l));
+            const float2 ph = dup2(tab_load<SM>(phi + l));
             x = fma2(make_float2(c[l][0], c[l][1]), ph, x);
             y = fma2(make_float2(c[l][2], c[l][3]), ph, y);
         }
@@ -501,7 +507,7 @@ __device__ __forceinline__ void point_value(const Vec<T, VEC> &fi, const T (&c)[
         for (int u = 0; u < VEC; ++u) val[u] = fi.v[u];
 #pragma unroll
         for (int l = 0; l < B; ++l) {
-            const T ph = __ldg(phi + l);
+            const T ph = tab_load<SM>(phi + l);
 #pragma unroll
             for (int u = 0; u < VEC; ++u) val[u] = fma(c[l][u], ph, val[u]);
         }
@@ -515,17 +521,19 @@ template <int B> __device__ __forceinline__ int64_t two_row(int64_t rows, int tw
 }
 
 // Face q of the cell at position p: the upwind flux, and on a two-sided face
-// (FP32) the values at its points.
-template <typename T, int VEC, int B>
+// (FP32) the values at its points.  fn, phi: the face's entries of these tables.
+// TWO: only the values at its two points (every face taken as two-sided; the
+// rows number faces).
+template <typename T, int VEC, int B, bool SM, bool TWO = false>
 __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> &tb, const FvIdx &ix, int64_t rows,
                                           int64_t p, int q, int fid, int meta, int k, int nv, T v1,
-                                          const T (&v2)[VEC], const Vec<T, VEC> &fi, const T (&c)[B][VEC]) {
+                                          const T (&v2)[VEC], const Vec<T, VEC> &fi, const T (&c)[B][VEC],
+                                          const T *fn, const T *phi) {
     const int64_t s = p * kFvMaxFaces + q;
     T vn[VEC], val[VEC];
-    normal_velocity<T, VEC>(v1, v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
     const bool other = (meta >> (8 + q)) & 1, boundary = (meta >> (16 + q)) & 1;
-    if (sizeof(T) == 4 && ((meta >> (24 + q)) & 1)) {
-        const int two = __ldg(ix.two + s);
+    if (TWO || (sizeof(T) == 4 && ((meta >> (24 + q)) & 1))) {
+        const int two = TWO ? fid : __ldg(ix.two + s);
 #pragma unroll
         for (int g = 0; g < (B == kFvCoef3 ? 2 : 1); ++g) {
             point_value<T, VEC, B>(fi, c, B == kFvCoef3 ? tb.phig + (s * 2 + g) * B : tb.phi + s * B, val);
@@ -535,16 +543,18 @@ __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> 
             stv<T, VEC>(FX + two_row<B>(rows, two, other, g) * nv + k, o);
         }
     }
+    if constexpr (TWO) return;
+    normal_velocity<T, VEC>(v1, v2, tab_load<SM>(fn), tab_load<SM>(fn + 1), vn);
     bool any = boundary;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) any = any || vn[u] >= (T)0;
     if (!any) return;
-    point_value<T, VEC, B>(fi, c, tb.phi + s * B, val);
+    point_value<T, VEC, B, SM>(fi, c, phi, val);
     put_flux<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
 }
 
 // Pass 1 of one cell, any polygon.
-template <typename T, int VEC, int MAXF, int B, int K>
+template <typename T, int VEC, int MAXF, int B, int K, bool TWO>
 __device__ __forceinline__ void recon_faces(const T *__restrict__ f, T *__restrict__ FX, const FvTables<T> &tb,
                                             const FvIdx &ix, int64_t rows, int64_t p, int ncf, int meta, int k, int nv,
                                             T v1, const T (&v2)[VEC], const Vec<T, VEC> &fi) {
@@ -562,8 +572,8 @@ __device__ __forceinline__ void recon_faces(const T *__restrict__ f, T *__restri
 #pragma unroll
     for (int q = 0; q < MAXF; ++q)
         if (q < nf)
-            emit_face<T, VEC, B>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v1, v2, fi,
-                                 c);
+            emit_face<T, VEC, B, false, TWO>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v1,
+                                             v2, fi, c, tb.fn + 2 * (p * kFvMaxFaces + q), tb.phi + (p * kFvMaxFaces + q) * B);
 }
 
 // Weights of one pair of velocities of a flagged triangle (kFvRegular: its
@@ -630,12 +640,12 @@ __device__ __forceinline__ void weigh_tri(float2 (&c)[B], const float2 (&d)[3], 
 }
 
 // Coefficients of the 4 velocities of a thread on a flagged triangle: row(q)
-// gives f of stencil cell q, each row read once.
-template <int B, int K, typename Row>
-__device__ __forceinline__ void coefs_tri_x2(const FvTables<float> &tb, int64_t p, const Vec<float, 4> &fi, Row row,
-                                             float (&c)[B][4]) {
+// gives f of stencil cell q, each row read once; then rows_read() is called.
+// Rc, Rs, qd: the cell's table values.
+template <int B, int K, bool SM, typename Row, typename Done>
+__device__ __forceinline__ void coefs_tri_x2(const float *Rc, const float *Rs, const float *qd, const Vec<float, 4> &fi,
+                                             Row row, Done rows_read, float (&c)[B][4]) {
     const float2 nf[2] = {make_float2(-fi.v[0], -fi.v[1]), make_float2(-fi.v[2], -fi.v[3])};
-    const float *Rc = tb.Rc + p * (B * K);
     float2 c2[2][B], dface[2][3];
 #pragma unroll
     for (int q = 0; q < K; ++q) {
@@ -647,15 +657,16 @@ __device__ __forceinline__ void coefs_tri_x2(const FvTables<float> &tb, int64_t 
         }
 #pragma unroll
         for (int l = 0; l < B; ++l) {
-            const float2 R = dup2(__ldg(Rc + l * K + q));
+            const float2 R = dup2(tab_load<SM>(Rc + l * K + q));
             c2[0][l] = q == 0 ? mul2(R, d0) : fma2(R, d0, c2[0][l]);
             c2[1][l] = q == 0 ? mul2(R, d1) : fma2(R, d1, c2[1][l]);
         }
     }
+    rows_read();
     float4 R[3];
 #pragma unroll
-    for (int s = 0; s < 3; ++s) R[s] = __ldg(reinterpret_cast<const float4 *>(tb.Rs + (p * kFvMaxFaces + s) * 4));
-    const float4 quad = __ldg(reinterpret_cast<const float4 *>(tb.quad + 4 * p));
+    for (int s = 0; s < 3; ++s) R[s] = tab_load<SM>(reinterpret_cast<const float4 *>(Rs + 4 * s));
+    const float4 quad = tab_load<SM>(reinterpret_cast<const float4 *>(qd));
 #pragma unroll
     for (int h = 0; h < 2; ++h) weigh_tri<B>(c2[h], dface[h], R, quad);
 #pragma unroll
@@ -677,9 +688,10 @@ template <typename T, int VEC> struct Velocity {
     }
 };
 
-template <typename T, int VEC, int MAXF, int B, int K>
+template <typename T, int VEC, int MAXF, int B, int K, bool TWO>
 __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restrict__ FX, const FvTables<T> &tb,
                                             const FvIdx &ix, int64_t rows, int nv, int N, T Lv, T dv) {
+    griddep_launch();
     const int64_t p = blockIdx.x;
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
     if (k >= nv) return;
@@ -689,34 +701,25 @@ __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restri
     if constexpr (sizeof(T) == 4 && VEC == 4 && MAXF == 3) {
         if (ncf & kFvRegular) {      // uniform over the block: one cell per block
             float c[B][4];
-            coefs_tri_x2<B, K>(tb, p, fi, [&](int q) {
+            coefs_tri_x2<B, K, false>(tb.Rc + p * (B * K), tb.Rs + p * kFvMaxFaces * 4, tb.quad + 4 * p, fi, [&](int q) {
                 return *reinterpret_cast<const float4 *>(f + (int64_t)__ldg(ix.cen + p * K + q) * nv + k);
-            }, c);
+            }, [] {}, c);
 #pragma unroll
             for (int q = 0; q < 3; ++q)
-                emit_face<float, 4, B>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v.v1,
-                                       v.v2, fi, c);
+                emit_face<float, 4, B, false, TWO>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv,
+                                              v.v1, v.v2, fi, c, tb.fn + 2 * (p * kFvMaxFaces + q),
+                                              tb.phi + (p * kFvMaxFaces + q) * B);
             return;
         }
     }
-    recon_faces<T, VEC, MAXF, B, K>(f, FX, tb, ix, rows, p, ncf, meta, k, nv, v.v1, v.v2, fi);
+    recon_faces<T, VEC, MAXF, B, K, TWO>(f, FX, tb, ix, rows, p, ncf, meta, k, nv, v.v1, v.v2, fi);
 }
 
-template <typename T, int VEC, int MAXF, int B, int K>
+template <typename T, int VEC, int MAXF, int B, int K, bool TWO = false>
 __global__ void __launch_bounds__(kFvThreads)
 fv_faces_kernel(const T *__restrict__ f, T *__restrict__ FX, FvTables<T> tb, FvIdx ix, int64_t rows, int nv, int N, T Lv,
                 T dv) {
-    faces_block<T, VEC, MAXF, B, K>(f, FX, tb, ix, rows, nv, N, Lv, dv);
-}
-
-// Degree 2 on FP32 triangles, 4 velocities per thread: four blocks per SM (64
-// registers, 36 bytes spilled; 19802 cells x 32^2: 0.203 ms, with three blocks
-// 0.232, with two 0.279).  A bound on the template above would also change the
-// register allocation of its other instantiations.
-__global__ void __launch_bounds__(kFvThreads, 4)
-fv_faces3_tri_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix, int64_t rows,
-                     int nv, int N, float Lv, float dv) {
-    faces_block<float, 4, 3, kFvCoef3, kFvCentral3>(f, FX, tb, ix, rows, nv, N, Lv, dv);
+    faces_block<T, VEC, MAXF, B, K, TWO>(f, FX, tb, ix, rows, nv, N, Lv, dv);
 }
 
 // Degree 1 on FP32 triangles without walls: the same two passes with a cell's
@@ -737,6 +740,7 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // The table values of a cell travel the same way, 4 bytes per lane into a buffer
 // of the warp (read in the order of processing they come from DRAM, and a block
@@ -753,6 +757,111 @@ constexpr int kFacesCtasPerSm = 3, kFluxCtasPerSm = 4;
 // staged rows, then the warps' table values: 50 KB for 256 threads
 constexpr size_t face_stage_bytes(int threads) {
     return 2 * kFaceRows * threads * sizeof(float4) + 2 * threads * sizeof(float);
+}
+
+// Degree 2 on FP32 triangles with 4 | N: pass 1 persistent in the same way, with
+// the 12 rows of a stencil, the cell's table values and its indices staged, the
+// indices one cell further ahead, per warp.  The rows have one buffer: the next
+// cell's are asked for as soon as the differences have been formed, and arrive
+// while this one's weights and faces are computed.  Two blocks of 256 threads
+// per SM (58 KB and 128 registers a thread; three spill).
+constexpr int kFaces3CtasPerSm = 2, kRows3 = 1 + kFvCentral3;
+constexpr int kTab3Rs = 0, kTab3Quad = 12, kTab3Rc = 16, kTab3Phi = 71, kTab3Fn = 86, kTab3Values = 92;
+constexpr int kIdx3Cen = 0, kIdx3Fid = 11, kIdx3Order = 14, kIdx3Meta = 15, kIdx3Ncen = 16, kIdx3Values = 17;
+constexpr int kTab3Pitch = 96, kIdx3Pitch = 20;   // per warp and buffer
+constexpr size_t faces3_stage_bytes(int threads) {
+    return kRows3 * threads * sizeof(float4) +
+           threads / 32 * (2 * kTab3Pitch * sizeof(float) + 3 * kIdx3Pitch * sizeof(int));
+}
+
+template <int BT, bool TWO>
+__global__ void __launch_bounds__(BT, kFaces3CtasPerSm * kFvThreads / BT)
+fv_faces3_persist_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix,
+                         int64_t rows, int64_t n, int nv, int N, float Lv, float dv) {
+    constexpr int B = kFvCoef3, K = kFvCentral3, W = BT / 32;
+    extern __shared__ float4 stage[];            // [kRows3][BT], [2][W][kTab3Pitch], [3][W][kIdx3Pitch]
+    griddep_launch();
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int kt = (blockIdx.y * BT + t) * 4;
+    if (kt - 4 * lane >= nv || (int64_t)blockIdx.x >= n) return;   // warps past nv
+    const bool act = kt < nv;
+    const int k = act ? kt : 0;                  // the last warp's idle lanes store nothing
+    float *const tabs = reinterpret_cast<float *>(stage + kRows3 * BT) + warp * kTab3Pitch;
+    int *const idxs = reinterpret_cast<int *>(reinterpret_cast<float *>(stage + kRows3 * BT) + 2 * W * kTab3Pitch) +
+                      warp * kIdx3Pitch;
+    const int64_t G = gridDim.x;
+    // this lane's index word, and its three table values, of position 0 and the distances between positions
+    const int *is = lane < kIdx3Fid ? ix.cen + lane : lane < kIdx3Order ? ix.fid + (lane - kIdx3Fid)
+                  : lane == kIdx3Order ? ix.order : lane == kIdx3Meta ? ix.meta : ix.ncen;
+    const int id = lane < kIdx3Fid ? K : lane < kIdx3Order ? kFvMaxFaces : 1;
+    const float *ts[3];
+    int td[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const int e = lane + 32 * u;
+        ts[u] = e < kTab3Quad ? tb.Rs + e : e < kTab3Rc ? tb.quad + (e - kTab3Quad) : e < kTab3Phi ? tb.Rc + (e - kTab3Rc)
+              : e < kTab3Fn ? tb.phi + (e - kTab3Phi) : tb.fn + (e - kTab3Fn);
+        td[u] = e < kTab3Quad ? kFvMaxFaces * 4 : e < kTab3Rc ? 4 : e < kTab3Phi ? B * K
+              : e < kTab3Fn ? kFvMaxFaces * B : kFvMaxFaces * 2;
+    }
+    auto issue_idx = [&](int64_t pr, int slot) {
+        if (lane < kIdx3Values) cp_async4(idxs + slot * W * kIdx3Pitch + lane, is + pr * id);
+    };
+    float4 *const sl = stage + t;
+    auto issue = [&](int64_t pr, int slot, int buf) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (lane + 32 * u < kTab3Values) cp_async4(tabs + buf * W * kTab3Pitch + lane + 32 * u, ts[u] + pr * td[u]);
+        const int *x = idxs + slot * W * kIdx3Pitch;
+        cp_async16(sl, f + (int64_t)x[kIdx3Order] * nv + k);
+#pragma unroll
+        for (int q = 0; q < K; ++q)              // a short stencil's other entries are cell 0
+            cp_async16(sl + (q + 1) * BT, f + (int64_t)x[kIdx3Cen + q] * nv + k);
+    };
+    const Velocity<float, 4> v(k, N, Lv, dv);
+    int64_t p = blockIdx.x;
+    issue_idx(p, 0);
+    cp_async_commit();
+    cp_async_wait_all();
+    __syncwarp();
+    issue(p, 0, 0);
+    if (p + G < n) issue_idx(p + G, 1);
+    cp_async_commit();
+    int slot = 0;
+    for (int it = 0;; ++it) {
+        const bool more = p + G < n;
+        const int next = slot == 2 ? 0 : slot + 1, after = next == 2 ? 0 : next + 1;
+        cp_async_wait_all();
+        __syncwarp();
+        auto ahead = [&] {
+            if (more) issue(p + G, next, (it + 1) & 1);
+            if (p + 2 * G < n) issue_idx(p + 2 * G, after);
+            cp_async_commit();
+        };
+        const int *x = idxs + slot * W * kIdx3Pitch;
+        const float *tab = tabs + (it & 1) * W * kTab3Pitch;
+        const int meta = x[kIdx3Meta], ncf = x[kIdx3Ncen];
+        Vec<float, 4> fi;
+        const float4 f4 = sl[0];
+        fi.v[0] = f4.x; fi.v[1] = f4.y; fi.v[2] = f4.z; fi.v[3] = f4.w;
+        if (ncf & kFvRegular) {
+            float c[B][4];
+            coefs_tri_x2<B, K, true>(tab + kTab3Rc, tab + kTab3Rs, tab + kTab3Quad, fi,
+                                     [&](int q) { return sl[(q + 1) * BT]; }, ahead, c);
+#pragma unroll
+            for (int q = 0; act && q < 3; ++q)
+                emit_face<float, 4, B, true, TWO>(FX, tb, ix, rows, p, q, x[kIdx3Fid + q], meta, k, nv, v.v1, v.v2, fi, c,
+                                             tab + kTab3Fn + 2 * q, tab + kTab3Phi + B * q);
+        } else {
+            ahead();
+            if (act) recon_faces<float, 4, 3, B, K, TWO>(f, FX, tb, ix, rows, p, ncf, meta, k, nv, v.v1,
+                                                    v.v2, fi);
+        }
+        if (!more) break;
+        __syncwarp();
+        p += G;
+        slot = next;
+    }
 }
 
 // CWENO gradient of one pair of velocities of a flagged triangle (kFvRegular):
@@ -854,6 +963,7 @@ __global__ void __launch_bounds__(BT, kFacesCtasPerSm * kFvThreads / BT)
 fv_values_persist_kernel(const float *__restrict__ f, float *__restrict__ FV, FvTables<float> tb, FvIdx ix,
                          const int4 *__restrict__ tripos, int64_t n, int nv) {
     extern __shared__ float4 stage[];            // [2][kFaceRows][BT], [2][warp][32] table values
+    griddep_launch();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     float *const tabs = reinterpret_cast<float *>(stage + 2 * kFaceRows * BT) + warp * 32;
     const int kt = (blockIdx.y * BT + t) * 4;
@@ -956,6 +1066,7 @@ fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ 
     const float2 hf = dup2(0.5f);
     int64_t p = blockIdx.x;
     RecF cur = rec_f(tripos, pos(p));
+    griddep_wait();                              // launched while the reconstruction ends
     issue(cur, p, 0);
     cp_async_commit();
     RecF nxt = cur;
@@ -1064,11 +1175,15 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
     if (k >= nv) return;
     const int meta = __ldg(ix.meta + p), nf = meta & 0xf;
+    int row[MAXF];
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q) row[q] = q < nf ? __ldg(ix.fid + p * kFvMaxFaces + q) : 0;
+    const T ia = __ldg(tb.inv_area + p);
+    griddep_wait();                      // launched while pass 1 ends: its rows from here on
     Vec<T, VEC> x[MAXF];
 #pragma unroll
     for (int q = 0; q < MAXF; ++q)
-        if (q < nf) x[q] = ldv<T, VEC>(FX + (int64_t)__ldg(ix.fid + p * kFvMaxFaces + q) * nv + k);
-    const T ia = __ldg(tb.inv_area + p);
+        if (q < nf) x[q] = ldv<T, VEC>(FX + (int64_t)row[q] * nv + k);
     Vec<T, VEC> o;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] = (T)0;
@@ -1113,6 +1228,48 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] *= ia;
     stv<T, VEC>(L + (int64_t)__ldg(ix.order + p) * nv + k, o);
+}
+
+// Pass 2 where every face is two-sided (FP32, degree 2): the Rusanov form at
+// both points of every face, term by term as in the two-sided faces above.
+template <int VEC, int MAXF>
+__global__ void __launch_bounds__(kFvThreads)
+fv_sum_two_kernel(const float *__restrict__ FX, float *__restrict__ L, FvTables<float> tb, FvIdx ix, int nv, int N,
+                  float Lv, float dv) {
+    const int64_t p = gridDim.x - 1 - blockIdx.x;
+    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
+    if (k >= nv) return;
+    const int meta = __ldg(ix.meta + p), nf = meta & 0xf;
+    const Velocity<float, VEC> v(k, N, Lv, dv);
+    const float ia = __ldg(tb.inv_area + p);
+    griddep_wait();
+    Vec<float, VEC> o;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) o.v[u] = 0.f;
+#pragma unroll
+    for (int q = 0; q < MAXF; ++q) {
+        if (q >= nf) continue;
+        const int64_t s = p * kFvMaxFaces + q;
+        const int side = (meta >> (8 + q)) & 1, fid = __ldg(ix.fid + s);
+        const bool boundary = (meta >> (16 + q)) & 1;
+        float vn[VEC];
+        normal_velocity<float, VEC>(v.v1, v.v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const Vec<float, VEC> a = ldv<float, VEC>(FX + two_row<kFvCoef3>(0, fid, side, g) * nv + k);
+            const Vec<float, VEC> b =
+                boundary ? a : ldv<float, VEC>(FX + two_row<kFvCoef3>(0, fid, 1 - side, 1 - g) * nv + k);
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) {
+                const float h = 0.25f * vn[u];
+                o.v[u] = fma(h, a.v[u] + b.v[u], o.v[u]);
+                o.v[u] = fma(-fabsf(h), b.v[u] - a.v[u], o.v[u]);
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) o.v[u] *= ia;
+    stv<float, VEC>(L + (int64_t)__ldg(ix.order + p) * nv + k, o);
 }
 
 // ---- order 1: Rusanov fluxes of the cell averages in one pass ------------------
@@ -1294,11 +1451,31 @@ void values_launch(const bz_mesh *m, const GridView &g, const float *f, float *F
     fv_values_persist_kernel<BT><<<values_grid(m, nv, kFacesCtasPerSm), BT, face_stage_bytes(BT), st>>>(
         f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
 }
-template <int BT>
-void flux_values_launch(const bz_mesh *m, const GridView &g, const float *FV, float *L, cudaStream_t st) {
+template <int BT, bool TWO>
+void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     const int nv = (int)g.nv;
-    fv_flux_values_persist_kernel<BT><<<values_grid(m, nv, kFluxCtasPerSm), BT, face_stage_bytes(BT), st>>>(
-        FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+    fv_faces3_persist_kernel<BT, TWO><<<values_grid(m, nv, kFaces3CtasPerSm), BT, faces3_stage_bytes(BT), st>>>(
+        f, FX, m->t32, indices(m), TWO ? 0 : flux_rows(m), m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+}
+template <bool TWO>
+void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
+    switch (values_threads((int)g.nv)) {
+        case 64: return faces3_launch<64, TWO>(m, g, f, FX, st);
+        case 128: return faces3_launch<128, TWO>(m, g, f, FX, st);
+        case 160: return faces3_launch<160, TWO>(m, g, f, FX, st);
+        default: return faces3_launch<kFvThreads, TWO>(m, g, f, FX, st);
+    }
+}
+// The flux pass starts while the reconstruction's last blocks end (on 760 to
+// 19802 triangles x 32^2 it saves 2 to 3 us), except on meshes so small that the
+// host's part of a launch is the bound (the attribute takes it 1 us) and with
+// narrow blocks: beside those of the reconstruction they would be placed
+// unevenly (19802 triangles x 16^2: 45 us, 50 with it).
+template <int BT>
+cudaError_t flux_values_launch(const bz_mesh *m, const GridView &g, const float *FV, float *L, cudaStream_t st) {
+    const int nv = (int)g.nv;
+    return launch_after(fv_flux_values_persist_kernel<BT>, values_grid(m, nv, kFluxCtasPerSm), BT, face_stage_bytes(BT), st,
+                        BT == kFvThreads && m->n_cells * nv >= (1 << 19), FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
 }
 
 // FP64 takes one velocity per thread (the FP64 pipe is the bound, so loads per
@@ -1315,8 +1492,7 @@ cudaError_t faces(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaSt
     } else {
         if (tri && g.N % 4 == 0 && aligned(f, 16)) {
             if (m->order == 3)
-                fv_faces3_tri_kernel<<<cell_grid(m, nv, 4), kFvThreads, 0, st>>>(
-                    f, FX, m->t32, indices(m), flux_rows(m), nv, g.N, (float)g.L, (float)g.dv);
+                faces3_launch<false>(m, g, f, FX, st);
             else
                 fv_faces_kernel<T, 4, 3, 2, kFvCentral><<<cell_grid(m, nv, 4), kFvThreads, 0, st>>>(
                     f, FX, m->t32, indices(m), flux_rows(m), nv, g.N, (float)g.L, (float)g.dv);
@@ -1339,16 +1515,15 @@ cudaError_t faces(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaSt
 }
 
 template <typename T, int VEC, int MAXF>
-void sum_launch(const bz_mesh *m, const GridView &g, const T *FX, T *L, cudaStream_t st) {
+cudaError_t sum_launch(const bz_mesh *m, const GridView &g, const T *FX, T *L, cudaStream_t st) {
     const int nv = (int)g.nv;
     const dim3 grid = cell_grid(m, nv, VEC);
     const int *wall = m->n_walls > 0 ? m->d_wall : nullptr;
     if (m->order == 3)
-        fv_sum_kernel<T, VEC, MAXF, kFvCoef3><<<grid, kFvThreads, 0, st>>>(FX, L, pick<T>(m), indices(m), wall,
-                                                                           flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
-    else
-        fv_sum_kernel<T, VEC, MAXF, 2><<<grid, kFvThreads, 0, st>>>(FX, L, pick<T>(m), indices(m), wall, flux_rows(m),
-                                                                    nv, g.N, (T)g.L, (T)g.dv);
+        return launch_after(fv_sum_kernel<T, VEC, MAXF, kFvCoef3>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m),
+                            indices(m), wall, flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+    return launch_after(fv_sum_kernel<T, VEC, MAXF, 2>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m), indices(m),
+                        wall, flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
 }
 
 // 16-byte rows where L allows (N^2 is a multiple of 4)
@@ -1357,11 +1532,10 @@ cudaError_t sum(const bz_mesh *m, const GridView &g, const T *FX, T *L, cudaStre
     if (m->n_cells <= 0) return cudaSuccess;
     constexpr int V = 16 / (int)sizeof(T);
     const bool tri = m->max_faces <= 3, al = aligned(L, 16);
-    if (tri && al) sum_launch<T, V, 3>(m, g, FX, L, st);
-    else if (tri) sum_launch<T, 1, 3>(m, g, FX, L, st);
-    else if (al) sum_launch<T, V, kFvMaxFaces>(m, g, FX, L, st);
-    else sum_launch<T, 1, kFvMaxFaces>(m, g, FX, L, st);
-    return cudaGetLastError();
+    return tri && al ? sum_launch<T, V, 3>(m, g, FX, L, st)
+           : tri     ? sum_launch<T, 1, 3>(m, g, FX, L, st)
+           : al      ? sum_launch<T, V, kFvMaxFaces>(m, g, FX, L, st)
+                     : sum_launch<T, 1, kFvMaxFaces>(m, g, FX, L, st);
 }
 
 template <typename T, int VEC, int MAXF>
@@ -1393,19 +1567,51 @@ cudaError_t first(const bz_mesh *m, const GridView &g, const T *f, T *L, cudaStr
 
 }  // namespace
 
+// The two-sided passes (see fv_two_sided): FX rows [face][side][point].
+cudaError_t launch_fv_faces_two_f32(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
+    if (m->n_cells <= 0) return cudaSuccess;
+    const int nv = (int)g.nv;
+    if (m->max_faces <= 3 && g.N % 4 == 0 && aligned(f, 16))
+        faces3_launch<true>(m, g, f, FX, st);
+    else if (m->max_faces <= 3)
+        fv_faces_kernel<float, 1, 3, kFvCoef3, kFvCentral3, true><<<cell_grid(m, nv, 1), kFvThreads, 0, st>>>(
+            f, FX, m->t32, indices(m), 0, nv, g.N, (float)g.L, (float)g.dv);
+    else
+        fv_faces_kernel<float, 1, kFvMaxFaces, kFvCoef3, kFvCentral3, true><<<cell_grid(m, nv, 1), kFvThreads, 0, st>>>(
+            f, FX, m->t32, indices(m), 0, nv, g.N, (float)g.L, (float)g.dv);
+    return cudaGetLastError();
+}
+cudaError_t launch_fv_sum_two_f32(const bz_mesh *m, const GridView &g, const float *FX, float *L, cudaStream_t st) {
+    if (m->n_cells <= 0) return cudaSuccess;
+    const int nv = (int)g.nv;
+    if (m->max_faces <= 3 && g.N % 4 == 0 && aligned(L, 16))
+        return launch_after(fv_sum_two_kernel<4, 3>, cell_grid(m, nv, 4), kFvThreads, 0, st, true, FX, L, m->t32, indices(m),
+                            nv, g.N, (float)g.L, (float)g.dv);
+    return launch_after(fv_sum_two_kernel<1, kFvMaxFaces>, cell_grid(m, nv, 1), kFvThreads, 0, st, true, FX, L, m->t32,
+                        indices(m), nv, g.N, (float)g.L, (float)g.dv);
+}
+
 cudaError_t fv_values_setup() {
-    const cudaError_t e = allow_dynamic_smem((const void *)fv_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads));
-    return e != cudaSuccess ? e
-                            : allow_dynamic_smem((const void *)fv_flux_values_persist_kernel<kFvThreads>,
-                                                 face_stage_bytes(kFvThreads));
+    const std::pair<const void *, size_t> big[] = {
+        {(const void *)fv_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
+        {(const void *)fv_flux_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, false>, faces3_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, true>, faces3_stage_bytes(kFvThreads)}};
+    cudaError_t e = cudaSuccess;
+    for (const auto &[kernel, bytes] : big)
+        if (e == cudaSuccess) e = allow_dynamic_smem(kernel, bytes);
+    return e;
 }
 
 bool fv_value_mode(const bz_mesh *m, const GridView &g, const void *f, const void *L) {
     return m->d_tripos && m->n_walls == 0 && g.N % 4 == 0 && aligned(f, 16) && aligned(L, 16);
 }
 
-int64_t fv_scratch_rows(const bz_mesh *m, bool f32) {
+bool fv_two_sided(const bz_mesh *m, bool f32) { return f32 && m->order == 3 && m->n_two > 0 && m->n_walls == 0; }
+
+int64_t fv_scratch_rows(const bz_mesh *m, bool f32, bool step) {
     if (m->order == 1) return 0;
+    if (step && fv_two_sided(m, f32)) return 4 * flux_rows(m);
     const int64_t flux = flux_rows(m) + (f32 ? m->n_two * (m->order == 3 ? 4 : 2) : 0);
     return f32 && m->d_tripos ? std::max<int64_t>(flux, 3 * m->n_cells) : flux;
 }
@@ -1424,12 +1630,11 @@ cudaError_t launch_fv_flux_values_f32(const bz_mesh *m, const GridView &g, const
                                       cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
     switch (values_threads((int)g.nv)) {
-        case 64: flux_values_launch<64>(m, g, FV, L, st); break;
-        case 128: flux_values_launch<128>(m, g, FV, L, st); break;
-        case 160: flux_values_launch<160>(m, g, FV, L, st); break;
-        default: flux_values_launch<kFvThreads>(m, g, FV, L, st);
+        case 64: return flux_values_launch<64>(m, g, FV, L, st);
+        case 128: return flux_values_launch<128>(m, g, FV, L, st);
+        case 160: return flux_values_launch<160>(m, g, FV, L, st);
+        default: return flux_values_launch<kFvThreads>(m, g, FV, L, st);
     }
-    return cudaGetLastError();
 }
 
 bool fv_walls_supported(const bz_mesh *m, const GridView &g) {
