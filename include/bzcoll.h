@@ -108,17 +108,20 @@ int init_velocity_grid(int dim, int n_per_dim, double half_width_L, bz_grid **ou
  * integral over |q| <= 2 lambda pi, lambda = 2/(3+sqrt 2), and the weights
  * beta-hat(l,m) = B-hat(l,m) - B-hat(m,m) of the mode sum; uploads FP64 and
  * FP32 copies (plus the symmetrised weight tiles of the FP32 kernels).
- * For 2-D grids with N <= 48 the register-blocked FP32 mode-sum kernel has
- * several variants (see bz_modes_info); the first build for a (dim, N, SM count)
+ * For 2-D grids with N <= 48 and 3-D grids the register-blocked FP32 mode-sum
+ * kernel has several variants (see bz_modes_info); the first build for a (dim, N, SM count)
  * times those that fit the grid on the current device (a few ms, zero spectra)
  * and keeps the fastest.  The choice is cached in the process and, if the
  * environment variable BZ_TUNE_CACHE names a writable file, appended there as
  * lines "dim N sms variant" and read back by later processes.
- * BZ_MODESUM_VARIANT=1, 2, 3, 4 or 5 fixes the variant without timing (ignored
- * if that variant does not fit the grid).  With a 32-cell variant chosen by
- * timing, collide calls run the whole waves of CTAs on it and the last partial
- * wave on the 16-cell variant (a second launch); a fixed variant runs every
- * tile.  The call synchronises the current device.
+ * BZ_MODESUM_VARIANT=1 ... 10 fixes the variant without timing (ignored if
+ * that variant does not fit the grid).  With a variant chosen by timing,
+ * collide calls run the whole waves of CTAs on it; the tiles left over are
+ * shared by 2 to 8 CTAs each, or run on the 16-cell variant (scalar 32-cell
+ * variants, a second launch), and small batches on kernels of their own, all
+ * with the same results bit for bit.  A fixed variant runs every tile whole
+ * (8-cell tiles are shared in either case).  The call synchronises the current
+ * device.
  *   g          : grid handle (not consumed; must outlive the modes handle)
  *   gamma      : 0 = Maxwell molecules, 1 = hard spheres (VHS); 0 <= gamma <= 2
  *   b0         : kernel constant; <= 0 selects 1/(2 pi) in 2-D, 1/(4 pi) in 3-D
@@ -251,7 +254,7 @@ int imex_step(const bz_modes *m, int scheme, int model, double dt, double eps,
 /* group_collide -- one collision evaluation for several independent instances
  * (each its own grid N / dimension / kernel and cell batch) in one call.  The
  * FP32 mode sums of all instances served by the register-blocked kernel
- * (2-D N <= 48, 3-D N <= 16) share one launch per kernel variant (up to 16
+ * (2-D N <= 64, 3-D N <= 16) share one launch per kernel variant (up to 16
  * instances per launch, longest first by per-cell work); other instances
  * (and the FP64 and FP32X2 forms) use one launch each.  The instances of one
  * variant, with their forward and inverse DFTs, form a lane; the lanes run on
@@ -392,10 +395,13 @@ const char *bz_last_error(void);
  * per cell by the symmetric FP32 kernel (algorithmic work unit), out[7] =
  * register-blocked FP32 mode-sum variant in use: 1 = 8 outputs per thread,
  * 16 warps, 32-cell tiles; 2 = 4 outputs per thread, 32 warps, 32-cell tiles;
- * 3 = 4 outputs per thread, 16 warps, 16-cell tiles; 4 = 4 outputs per
- * thread, 16 warps, 8-cell tiles (3-D 16^3); 5 = two cells per thread in
- * FP32x2 register pairs, 4 outputs per thread, 16 warps, 32-cell tiles;
- * 0 = FP32 mode sums run on the generic kernel (2-D grids with N > 48). */
+ * 3 = 4 outputs per thread, 16 warps, 16-cell tiles; 4 = FP32x2, 8 outputs
+ * per thread, 12 warps, 8-cell tiles (3-D 16^3); 5 = two cells per thread in
+ * FP32x2 register pairs, 4 outputs per thread, 16 warps, 32-cell tiles; 6, 7 =
+ * FP32x2 with one cell per lane, 8 outputs per thread, 12 or 16 warps, 32-cell
+ * tiles; 8, 9, 10 = the same with paired orientations on 16-cell tiles, 16, 8
+ * or 4 warps; 0 = no choice of variants: 2-D grids with N > 48 (the 8-cell
+ * form), and grids that the register-blocked kernels do not serve. */
 int bz_modes_info(const bz_modes *m, int64_t out[8]);
 
 /* bz_fast_info -- out[0] = method of a modes handle (0: eq. KM / eq. CF1
