@@ -7,7 +7,7 @@ import pytest
 
 from paper_2103_14890_gb300 import workloads
 from gpu_util import as_input, bz_module, relerr, to_dev
-from test_gpu_transport import ETA32, ETA64, U32, U64, _check, _check3, _walls
+from test_gpu_transport import ETA32, ETA64, U32, U64, _check, _check3, _magnitude3, _walls
 
 pytestmark = pytest.mark.gpu
 
@@ -75,8 +75,7 @@ def test_stage_kernels_fp64(bz, dim, N, scheme, model):
 
 @pytest.mark.parametrize("N", [12, 16, 20, 24, 28])
 def test_value_pass_blocks(bz, fvo, N):
-    """The FP32 triangle passes of degree 1 with 64, 128, 160 and 256 threads, the last warp not always full, on more
-    cells than a thin mesh has and on none of the sizes of the passes' grids."""
+    """The FP32 triangle passes of degree 1 with 64, 128, 160 and 256 threads, the last warp not always full."""
     pts, tri = workloads.sod_triangulation(18, jitter=0.2)
     om = fvo.Mesh(pts, tri)
     f = workloads.mesh_states(om.bary, N, 6.0)
@@ -84,3 +83,36 @@ def test_value_pass_blocks(bz, fvo, N):
     Lr = bz.transport_residual(bz.Mesh(pts, tri, order=2), bz.Grid(2, N, 6.0), to_dev(f, "fp32"), precision="fp32")
     bz.check()
     _check(Lr.double().cpu().numpy(), fvo.transport_residual(om, fin, N, 6.0, order=2), om, fin, N, 6.0, 2, fvo, U32, ETA32)
+
+
+@pytest.mark.parametrize("N", [12, 16, 20, 24, 28])
+def test_degree2_pass_blocks(bz, fvo, N):
+    """As test_value_pass_blocks for the staged pass of degree 2."""
+    pts, tri = workloads.sod_triangulation(18, jitter=0.2)
+    om = fvo.Mesh(pts, tri)
+    f = workloads.mesh_states(om.bary, N, 6.0)
+    fin = as_input(f, "fp32")
+    Lr = bz.transport_residual(bz.Mesh(pts, tri, order=3), bz.Grid(2, N, 6.0), to_dev(f, "fp32"), precision="fp32")
+    bz.check()
+    _check3(Lr.double().cpu().numpy(), fvo.transport_residual(om, fin, N, 6.0, order=3), om, fin, N, 6.0, fvo, U32, ETA32)
+
+
+@pytest.mark.parametrize("N", [8, 6])
+def test_two_sided_step(bz, fvo, N):
+    """A step of degree 2 on a mesh with thin cells (every face two-sided), as good as without collisions (eps = 1e30):
+    f - dt L(f) of the oracle, within dt times the bound of L and four roundings of the terms."""
+    pts, tri = _thin_mesh()
+    om = fvo.Mesh(pts, tri)
+    f = workloads.mesh_states(om.bary, N, 6.0)
+    fin = as_input(f, "fp32")
+    dt = 2e-5
+    m = bz.Modes(bz.Grid(2, N, 6.0), 0.0)
+    got = bz.imex_step_fv(m, bz.Mesh(pts, tri, order=3), to_dev(f, "fp32"), dt, 1e30, scheme="euler", model="bgk",
+                          precision="fp32")
+    bz.check()
+    L = fvo.transport_residual(om, fin, N, 6.0, order=3)
+    M = _magnitude3(om, fin, N, 6.0, fvo, None)
+    bound = 64 * dt * (U32 * M + ETA32 * _magnitude3(om, np.ones_like(fin), N, 6.0, fvo, None))
+    bound += 4 * U32 * (np.abs(fin) + dt * np.abs(L)) + 4 * ETA32
+    err = np.abs(got.double().cpu().numpy() - (fin - dt * L))
+    assert (err <= bound).all(), float((err / bound).max())
