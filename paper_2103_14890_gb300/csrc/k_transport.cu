@@ -143,6 +143,19 @@ __device__ __forceinline__ double scaled_rcp(double b, int scale) {
     return fma(y, e, y);
 }
 
+// Signs and comparisons of finite FP64 values as integers, off the FP64 pipe.
+__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+__device__ __forceinline__ double negate_if(bool neg, double x) {
+    return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
+__device__ __forceinline__ float negate_if(bool neg, float x) { return neg ? -x : x; }
+// Not negative (-0 included), for a velocity, never a NaN.
+template <typename T> __device__ __forceinline__ bool leaves(T vn) {
+    if constexpr (sizeof(T) == 8) return !positive(negate_if(true, vn));
+    else return vn >= (T)0;
+}
+
 // Write the flux of VEC velocities through a face: vn (outward normal velocity
 // times |e|) times the reconstructed mean `val`, in the owner's orientation,
 // where this cell is upwind (everywhere on a boundary face).
@@ -154,8 +167,8 @@ __device__ __forceinline__ void put_flux(T *__restrict__ row, const T (&vn)[VEC]
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
         const T fl = vn[u] * val[u];
-        o.v[u] = other ? -fl : fl;
-        on[u] = boundary || (other ? vn[u] > (T)0 : vn[u] >= (T)0);
+        o.v[u] = negate_if(other, fl);
+        on[u] = boundary || (other ? positive(vn[u]) : leaves(vn[u]));
         all = all && on[u];
     }
     if (all) {
@@ -185,6 +198,11 @@ __device__ __forceinline__ void normal_velocity(T v1, const T (&v2)[VEC], T nx, 
     }
 }
 
+// lambda_L = 1/4 / #sectors (a division costs as much as ten FMAs)
+static_assert(kFvMaxFaces == 8, "entries of kLamSector");
+__constant__ double kLamSector[kFvMaxFaces + 1] = {0.0,      0.25,     0.25 / 2, 0.25 / 3, 0.25 / 4,
+                                                   0.25 / 5, 0.25 / 6, 0.25 / 7, 0.25 / 8};
+
 // Coefficients of a cell's CWENO polynomial in FP64, one velocity per thread
 // (any polygon).  B, K: coefficients and stencil cells (2, 5 or 5, 11); MAXS
 // bounds the sectors.  Loops are unrolled with block-uniform predicates.
@@ -197,7 +215,7 @@ __device__ __forceinline__ void recon_coefs_f64(const double *__restrict__ f, co
     const int nc = ncf & (kFvRegular - 1), ns = __ldg(ix.nsec + p);
     const double *Rc = tb.Rc + p * (B * K), *Rs = tb.Rs + p * kFvMaxFaces * 4;
     constexpr double kLam0 = 0.75, kEps = 1e-14;
-    const double lamL = 0.25 / (double)ns;
+    const double lamL = kLamSector[ns];
     double sx[MAXS], sy[MAXS];
     if (ncf & kFvRegular) {              // uniform over the block; the rows of p_0, the sectors' share included
         double d[MAXS];
@@ -547,7 +565,7 @@ __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> 
     normal_velocity<T, VEC>(v1, v2, tab_load<SM>(fn), tab_load<SM>(fn + 1), vn);
     bool any = boundary;
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) any = any || vn[u] >= (T)0;
+    for (int u = 0; u < VEC; ++u) any = any || leaves(vn[u]);
     if (!any) return;
     point_value<T, VEC, B, SM>(fi, c, phi, val);
     put_flux<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
@@ -1193,7 +1211,7 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
         if (q < nf && !((two_sided >> q) & 1)) {
             const bool other = (meta >> (8 + q)) & 1;
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) o.v[u] += other ? -x[q].v[u] : x[q].v[u];
+            for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, x[q].v[u]);
         }
     if (two_sided) {
         // faces of thin cells: (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2 at every face point
