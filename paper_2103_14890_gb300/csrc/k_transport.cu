@@ -36,8 +36,9 @@
 // and velocity 9 operations in place of 34.  19802 triangles x 32^2, FP32,
 // degree 2: 0.382 -> 0.253 ms; 2603 Voronoi cells x 30^2, FP64, degree 2: 2.13
 // -> 1.34 ms, 1.20 with p_0's rows and one difference per neighbour in the
-// cells flagged kFvRegular (about 227 FP64 operations per hexagon and velocity
-// for 260: pass 1 1.27 -> 1.13 ms, the FP64 pipe nine tenths busy).
+// cells flagged kFvRegular (pass 1 1.27 -> 1.13 ms, the FP64 pipe nine tenths
+// busy), 1.03 with signs, comparisons and 1 / #sectors off that pipe (pass 1
+// 0.98 ms, sums 0.070 -> 0.041).
 //
 // Reconstruction: the central (least-squares) coefficients and the sector
 // polynomials are linear in the averages (tables Rc, Rs of fv_mesh.cpp);
@@ -781,9 +782,12 @@ constexpr size_t face_stage_bytes(int threads) {
 // the 12 rows of a stencil, the cell's table values and its indices staged, the
 // indices one cell further ahead, per warp.  The rows have one buffer: the next
 // cell's are asked for as soon as the differences have been formed, and arrive
-// while this one's weights and faces are computed.  Two blocks of 256 threads
-// per SM (58 KB and 128 registers a thread; three spill).
-constexpr int kFaces3CtasPerSm = 2, kRows3 = 1 + kFvCentral3;
+// while this one's weights and faces are computed.  CPS: blocks per SM for 256
+// threads (58 KB each), as many threads with narrower ones.  Two have 128
+// registers a thread; three spill 36 bytes, but a small mesh takes fewer rounds
+// (faces3_per_sm), and narrower blocks gain by the warps (24^2 on 19802 cells
+// 165 -> 158 us, on 472 cells 19.0 -> 16.5).
+constexpr int kRows3 = 1 + kFvCentral3;
 constexpr int kTab3Rs = 0, kTab3Quad = 12, kTab3Rc = 16, kTab3Phi = 71, kTab3Fn = 86, kTab3Values = 92;
 constexpr int kIdx3Cen = 0, kIdx3Fid = 11, kIdx3Order = 14, kIdx3Meta = 15, kIdx3Ncen = 16, kIdx3Values = 17;
 constexpr int kTab3Pitch = 96, kIdx3Pitch = 20;   // per warp and buffer
@@ -792,8 +796,8 @@ constexpr size_t faces3_stage_bytes(int threads) {
            threads / 32 * (2 * kTab3Pitch * sizeof(float) + 3 * kIdx3Pitch * sizeof(int));
 }
 
-template <int BT, bool TWO>
-__global__ void __launch_bounds__(BT, kFaces3CtasPerSm * kFvThreads / BT)
+template <int BT, bool TWO, int CPS>
+__global__ void __launch_bounds__(BT, CPS * kFvThreads / BT)
 fv_faces3_persist_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix,
                          int64_t rows, int64_t n, int nv, int N, float Lv, float dv) {
     constexpr int B = kFvCoef3, K = kFvCentral3, W = BT / 32;
@@ -1469,20 +1473,30 @@ void values_launch(const bz_mesh *m, const GridView &g, const float *f, float *F
     fv_values_persist_kernel<BT><<<values_grid(m, nv, kFacesCtasPerSm), BT, face_stage_bytes(BT), st>>>(
         f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
 }
-template <int BT, bool TWO>
+template <int BT, bool TWO, int CPS>
 void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     const int nv = (int)g.nv;
-    fv_faces3_persist_kernel<BT, TWO><<<values_grid(m, nv, kFaces3CtasPerSm), BT, faces3_stage_bytes(BT), st>>>(
+    fv_faces3_persist_kernel<BT, TWO, CPS><<<values_grid(m, nv, CPS), BT, faces3_stage_bytes(BT), st>>>(
         f, FX, m->t32, indices(m), TWO ? 0 : flux_rows(m), m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+}
+// Blocks of 256 threads per SM: three where that saves rounds on a small mesh (a
+// round of three takes about 1.48 rounds of two, and a full one more).  Transport
+// of 32^2 with two and three: 338 cells 20.3 and 17.3 us, 450 cells 21.7 and
+// 22.9, 800 cells 22.9 and 21.4, 1150 cells 25.0 and 26.9, 1760 cells 34.7 and
+// 33.0, 19802 cells 237 and 240.
+int faces3_per_sm(const bz_mesh *m) {
+    const int64_t n = m->n_cells, sms = fv_sm_count(), two = (n + 2 * sms - 1) / (2 * sms), three = (n + 3 * sms - 1) / (3 * sms);
+    return n <= 20 * sms && 1.48 * three < two && n <= 0.95 * (3 * sms * three) ? 3 : 2;
 }
 template <bool TWO>
 void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     switch (values_threads((int)g.nv)) {
-        case 64: return faces3_launch<64, TWO>(m, g, f, FX, st);
-        case 128: return faces3_launch<128, TWO>(m, g, f, FX, st);
-        case 160: return faces3_launch<160, TWO>(m, g, f, FX, st);
-        default: return faces3_launch<kFvThreads, TWO>(m, g, f, FX, st);
+        case 64: return faces3_launch<64, TWO, 3>(m, g, f, FX, st);
+        case 128: return faces3_launch<128, TWO, 3>(m, g, f, FX, st);
+        case 160: return faces3_launch<160, TWO, 3>(m, g, f, FX, st);
     }
+    if (faces3_per_sm(m) == 3) return faces3_launch<kFvThreads, TWO, 3>(m, g, f, FX, st);
+    faces3_launch<kFvThreads, TWO, 2>(m, g, f, FX, st);
 }
 // The flux pass starts while the reconstruction's last blocks end (on 760 to
 // 19802 triangles x 32^2 it saves 2 to 3 us), except on meshes so small that the
@@ -1613,8 +1627,10 @@ cudaError_t fv_values_setup() {
     const std::pair<const void *, size_t> big[] = {
         {(const void *)fv_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
         {(const void *)fv_flux_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, false>, faces3_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, true>, faces3_stage_bytes(kFvThreads)}};
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, false, 2>, faces3_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, false, 3>, faces3_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, true, 2>, faces3_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, true, 3>, faces3_stage_bytes(kFvThreads)}};
     cudaError_t e = cudaSuccess;
     for (const auto &[kernel, bytes] : big)
         if (e == cudaSuccess) e = allow_dynamic_smem(kernel, bytes);
