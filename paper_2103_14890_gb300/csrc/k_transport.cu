@@ -1481,9 +1481,9 @@ void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *F
 }
 // Blocks of 256 threads per SM: three where that saves rounds on a small mesh (a
 // round of three takes about 1.48 rounds of two, and a full one more).  Transport
-// of 32^2 with two and three: 338 cells 20.3 and 17.3 us, 450 cells 21.7 and
-// 22.9, 800 cells 22.9 and 21.4, 1150 cells 25.0 and 26.9, 1760 cells 34.7 and
-// 33.0, 19802 cells 237 and 240.
+// of 32^2 with two and three: 312 cells 20.3 and 17.3 us, 472 cells 21.7 and
+// 22.9, 756 cells 22.9 and 21.4, 1105 cells 25.0 and 26.9, 19802 cells 237 and
+// 240.
 int faces3_per_sm(const bz_mesh *m) {
     const int64_t n = m->n_cells, sms = fv_sm_count(), two = (n + 2 * sms - 1) / (2 * sms), three = (n + 3 * sms - 1) / (3 * sms);
     return n <= 20 * sms && 1.48 * three < two && n <= 0.95 * (3 * sms * three) ? 3 : 2;
