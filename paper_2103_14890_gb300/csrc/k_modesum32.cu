@@ -1542,19 +1542,22 @@ static Tail tail_split(const bz_modes *m, int v, const TaskTables &t, int64_t ct
 // FP64 pipe is full to the end
 constexpr double kStage32 = 4.3, kRagged32 = 0.45, kStage64 = 0.15, kStageX2 = 0.8;
 
-// Appends an instance of n cells to a launch: the cells of its first `full`
-// CTAs, then those whose tiles S CTAs share.  fsize, qsize: bytes per value.
-static void add_items(Mode32Group &gd, const bz_modes *m, int v, const void *W, const TaskTables &t, int rowmax,
+// Appends an instance of n cells to a launch (gd.nitems counts its items): the
+// cells of its first `full` CTAs, then those whose tiles S CTAs share.  fsize,
+// qsize: bytes per value.  An error, and nothing written, past kMaxGroup items.
+static cudaError_t add_items(Mode32Group &gd, const bz_modes *m, int v, const void *W, const TaskTables &t, int rowmax,
                       const void *fhat, size_t fsize, void *Qhat, size_t qsize, int64_t n, Tail tail) {
     const int64_t nm = std::min(n, tail.full * kVariants[v].cells);
     for (int p = 0; p < 2; ++p) {
         const int64_t first = p ? nm : 0, cnt = p ? n - nm : nm, off = first / 32 * m->g->v.nhalf * 32;
         if (cnt <= 0) continue;
+        if (gd.nitems >= kMaxGroup) return cudaErrorInvalidValue;
         const int S = p ? tail.S : 1, k = gd.nitems++;
         fill_item(gd.item[k], m, W, t, rowmax, static_cast<const char *>(fhat) + off * fsize,
                   static_cast<char *>(Qhat) + off * qsize, cnt, S);
         gd.tile_start[k + 1] = gd.tile_start[k] + ctas_for(v, cnt) * S;
     }
+    return cudaSuccess;
 }
 
 static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
@@ -1562,8 +1565,9 @@ static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, 
     if (n <= 0) return cudaSuccess;
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
-    add_items(gd, m, v, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, sizeof(float2), Qhat, sizeof(float2), n,
-              {S > 1 ? 0 : ctas_for(v, n), S});
+    const cudaError_t e = add_items(gd, m, v, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, sizeof(float2), Qhat,
+                                    sizeof(float2), n, {S > 1 ? 0 : ctas_for(v, n), S});
+    if (e != cudaSuccess) return e;
     return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
 }
 
@@ -1591,9 +1595,10 @@ static cudaError_t launch_pairs(const bz_modes *m, const double2 *fhat, void *Qh
     memset(&gd, 0, sizeof gd);
     const int v = m->variant64;
     const size_t sm = smem_bytes<double>(m->g->v, m->rowmax64, v);
-    add_items(gd, m, v, X2 ? static_cast<const void *>(m->wx2) : m->w64, m->task64, m->rowmax64, fhat, sizeof(double2),
-              Qhat, X2 ? sizeof(float2) : sizeof(double2), n,
-              tail_split(m, v, m->task64, ctas_for(v, n), sm, X2 ? kStageX2 : kStage64, 0.0));
+    const cudaError_t e = add_items(gd, m, v, X2 ? static_cast<const void *>(m->wx2) : m->w64, m->task64, m->rowmax64, fhat,
+                                    sizeof(double2), Qhat, X2 ? sizeof(float2) : sizeof(double2), n,
+                                    tail_split(m, v, m->task64, ctas_for(v, n), sm, X2 ? kStageX2 : kStage64, 0.0));
+    if (e != cudaSuccess) return e;
     if (m->variant64 == kFp64Variants[0]) return launch_pair<X2, 4, 8, 8>(gd, sm, st);
     if (m->variant64 == kFp64Variants[1]) return launch_pair<X2, 4, 8, 4>(gd, sm, st);
     if (m->variant64 == kFp64Variants[2]) return launch_pair<X2, 2, 8, 8>(gd, sm, st);
@@ -1679,9 +1684,11 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
     const int sv = small_batch_variant(m, n);
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
+    cudaError_t e;
     if (const int S = small_split(m, sv, n)) {
-        add_items(gd, m, kSmallVariant, m->small_W, m->small_task, m->small_rowmax, fhat, sizeof(float2), Qhat,
-                  sizeof(float2), n, {0, S});
+        e = add_items(gd, m, kSmallVariant, m->small_W, m->small_task, m->small_rowmax, fhat, sizeof(float2), Qhat,
+                      sizeof(float2), n, {0, S});
+        if (e != cudaSuccess) return e;
         return launch_group(gd, kSmallVariant, smem_bytes<float>(m->g->v, m->small_rowmax, kSmallVariant), st, pdl);
     }
     const Variant &k = kVariants[sv];
@@ -1697,15 +1704,17 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
         variant_reflects(2, m->g->v.h) == variant_reflects(sv, m->g->v.h)) {
         const int64_t nm = tail.full * 32;
         const size_t off = (size_t)nm * m->g->v.nhalf;
-        const cudaError_t e = launch_variant(m, sv, fhat, Qhat, nm, st);
+        e = launch_variant(m, sv, fhat, Qhat, nm, st);
         if (e != cudaSuccess) return e;
         const size_t s2 = smem_bytes<float>(m->g->v, m->var_rowmax[2], 2);
-        add_items(gd, m, 2, m->var_W[2], m->var_task[2], m->var_rowmax[2], fhat + off, sizeof(float2), Qhat + off,
-                  sizeof(float2), n - nm, tail_split(m, 2, m->var_task[2], ctas_for(2, n - nm), s2, kStage32, kRagged32));
+        e = add_items(gd, m, 2, m->var_W[2], m->var_task[2], m->var_rowmax[2], fhat + off, sizeof(float2), Qhat + off,
+                      sizeof(float2), n - nm, tail_split(m, 2, m->var_task[2], ctas_for(2, n - nm), s2, kStage32, kRagged32));
+        if (e != cudaSuccess) return e;
         return launch_group(gd, 2, s2, st);
     }
-    add_items(gd, m, sv, m->var_W[sv], m->var_task[sv], m->var_rowmax[sv], fhat, sizeof(float2), Qhat, sizeof(float2), n,
-              tail);
+    e = add_items(gd, m, sv, m->var_W[sv], m->var_task[sv], m->var_rowmax[sv], fhat, sizeof(float2), Qhat, sizeof(float2),
+                  n, tail);
+    if (e != cudaSuccess) return e;
     return launch_group(gd, sv, sm, st);
 }
 
@@ -1724,7 +1733,6 @@ cudaError_t launch_modesum32_group(const bz_modes *const *ms, const float2 *cons
     const int v = ms[0]->variant;
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
-    gd.nitems = count;
     size_t sm = 0;
     int64_t whole = 0;
     for (int i = 0; i < count; ++i) {
@@ -1739,8 +1747,9 @@ cudaError_t launch_modesum32_group(const bz_modes *const *ms, const float2 *cons
             const Tail all = tail_split(ms[i], v, ms[i]->var_task[v], whole, sm, kStage32, kRagged32);
             if (all.S > 1) tail = {tail.full - std::min(whole - all.full, tail.full), all.S};
         }
-        add_items(gd, ms[i], v, ms[i]->var_W[v], ms[i]->var_task[v], ms[i]->var_rowmax[v], fhat[i], sizeof(float2),
-                  Qhat[i], sizeof(float2), n[i], tail);
+        const cudaError_t e = add_items(gd, ms[i], v, ms[i]->var_W[v], ms[i]->var_task[v], ms[i]->var_rowmax[v], fhat[i],
+                                        sizeof(float2), Qhat[i], sizeof(float2), n[i], tail);
+        if (e != cudaSuccess) return e;
     }
     if (gd.nitems == 0) return cudaSuccess;
     if (sm > 227 * 1024) return cudaErrorInvalidValue;

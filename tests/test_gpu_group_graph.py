@@ -94,3 +94,25 @@ def test_graph_step_equals_direct_launches(bz, precision):
     d2 = bz.imex_step(m, f, 1e-4, 5e-3, precision=precision)
     torch.cuda.synchronize()
     assert torch.equal(o2, d2)
+
+
+@pytest.mark.parametrize("N,variant", [(16, 0), (16, 10), (64, 0)])
+@pytest.mark.parametrize("count", [1, 7, 8, 9, 15, 16, 17, 33])
+def test_many_instances_on_one_variant(bz, monkeypatch, count, N, variant):
+    """Simulations on one grid, up to and beyond the sixteen of a launch, with the last wave shared by several CTAs
+    (the variant chosen by timing; 64^2) and without (a fixed variant): the bits of per-instance calls."""
+    import torch
+    if variant:
+        monkeypatch.setenv("BZ_MODESUM_VARIANT", str(variant))
+    m = bz.Modes(bz.Grid(2, N, 10.0), 1.0)
+    sizes = [1 + (37 * i) % 90 for i in range(count - 1)] + [7500 if N == 16 else 300]    # more than a wave of 16^2
+    f = [to_dev(workloads.bi_maxwellian(n, 2, N, 10.0, seed=100 + i), "fp32") for i, n in enumerate(sizes)]
+    refs = [bz.collide_batch(m, x, precision="fp32") for x in f]
+    entries = [(m, x, torch.full_like(x, float("nan"))) for x in f]
+    for order in (entries, entries[::-1]):               # the large instance last, then first
+        for _, _, Q in order:
+            Q.fill_(float("nan"))
+        bz.group_collide(order, precision="fp32")
+        bz.check()
+        for (_, _, Q), ref in zip(entries, refs):
+            assert torch.equal(Q, ref)
