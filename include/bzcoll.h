@@ -355,8 +355,9 @@ int fv_mesh_set_walls(bz_mesh *mesh, int64_t n_edges, const int64_t *edge_vertic
  *   f, L      : device arrays [n_cells][N^2] (n_cells of the mesh), double for
  *               BZ_FP64, float for BZ_FP32; must not overlap
  * Boundary faces are transmissive (the outer state equals the inner one)
- * unless fv_mesh_set_walls made them walls.
- * Scratch (orders 2 and 3: one value per face of the mesh and velocity,
+ * unless fv_mesh_set_walls made them walls; an edge that is its own reverse
+ * (of no length, or as long as a period) counts as one.
+ * Scratch (orders 2 and 3: one value per face of the mesh and velocity, about
  * (bz_mesh_info out[1] + out[2]) N^2, and in FP32 up to four more per face of
  * a thin cell; 3 n_cells N^2 values for order 2 in FP32 on triangle meshes)
  * comes from the stream-ordered pool.

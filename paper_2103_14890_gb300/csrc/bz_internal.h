@@ -158,6 +158,7 @@ struct bz_mesh {
     int device;
     int order;              // 1: piecewise constant, 2: CWENO of degree 1, 3: CWENO of degree 2
     int64_t n_cells, n_faces_interior, n_faces_boundary;
+    int64_t n_rows;         // faces as d_fid numbers them
     int max_faces;
     // index tables by position of the processing order (cells sorted along a
     // Morton curve of their barycentres), values are cell indices

@@ -292,15 +292,19 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         kx = Lx > 0 ? (int)llround(dx / Lx) : 0;
         ky = Ly > 0 ? (int)llround(dy / Ly) : 0;
     };
-    // directed edge (classes) -> owning cell and its copy of the edge's first vertex
-    std::unordered_map<uint64_t, std::pair<int64_t, int64_t>> owner;
+    // directed edge (classes) -> owning cell, its copy of the edge's first vertex, its face
+    struct Side {
+        int64_t cell, vertex;
+        int face;
+    };
+    std::unordered_map<uint64_t, Side> owner;
     owner.reserve((size_t)(n * 4));
     auto key = [](int64_t a, int64_t b) { return ((uint64_t)a << 32) | (uint64_t)b; };
     for (int64_t i = 0; i < n; ++i) {
         const auto &c = cells[i];
         for (size_t q = 0; q < c.size(); ++q) {
             const int64_t a = c[q], b = c[(q + 1) % c.size()];
-            if (!owner.emplace(key(vclass[a], vclass[b]), std::make_pair(i, a)).second)
+            if (!owner.emplace(key(vclass[a], vclass[b]), Side{i, a, (int)q}).second)
                 return fail(BZ_EINVAL, "build_fv_mesh: an edge is used twice in the same direction (overlapping or "
                                        "inconsistently oriented cells)");
         }
@@ -325,14 +329,13 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
             h.fn[2 * s + 1] = -dx;
             auto it = owner.find(key(vclass[b], vclass[a]));
             if (it != owner.end()) {
-                const int64_t j = it->second.first, wb = it->second.second;   // j's copy of b
+                const int64_t j = it->second.cell, wb = it->second.vertex;    // j's copy of b
                 int kx, ky;
                 lattice(xy[2 * b] - xy[2 * wb], xy[2 * b + 1] - xy[2 * wb + 1], kx, ky);
                 fsx[s] = kx * Lx;
                 fsy[s] = ky * Ly;
                 h.nb[s] = (int)j;
-                for (size_t t = 0; t < cells[j].size(); ++t)     // j's face starting at its copy of b
-                    if (cells[j][t] == wb) h.nbq[s] = (int)t;
+                h.nbq[s] = it->second.face;
                 ++interior;
             } else {
                 ++boundary;
@@ -589,9 +592,11 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
     }
     // faces in the processing order of their owners (the first cell of the two
     // in that order); the other side's normal is the owner's, negated, so both
-    // sides form the same normal velocities up to the sign
+    // sides form the same normal velocities up to the sign.  An edge that is its
+    // own reverse (both ends one point: of no length, or as long as a period) has
+    // no other side and is a transmissive boundary here.
     std::vector<int> meta((size_t)n, 0), fid((size_t)n * kFvMaxFaces, 0), two((size_t)n * kFvMaxFaces, 0);
-    int64_t n_two = 0;
+    int64_t n_two = 0, n_rows = 0;
     {
         for (int64_t i = 0; i < n; ++i) {
             double per = 0.0;
@@ -600,7 +605,6 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
             meta[i] = h.nface[i] | (per * sqrt(h.h2[i]) > kFvThin * area[i] ? kFvThinFlag : 0);
         }
         std::vector<char> done((size_t)n, 0);
-        int next = 0;
         for (int64_t p = 0; p < n; ++p) {
             const int64_t i = h.order[p];
             for (int q = 0; q < h.nface[i]; ++q) {
@@ -609,15 +613,15 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                 const bool thin = ((meta[i] | (j < 0 ? 0 : meta[j])) & kFvThinFlag) != 0;
                 if (thin) meta[i] |= (int)(1u << (24 + q));
                 const size_t o = j < 0 ? s : (size_t)j * kFvMaxFaces + h.nbq[s];
-                if (j < 0) meta[i] |= 1 << (16 + q);
-                if (j >= 0 && (done[j] || (j == i && h.nbq[s] < q))) {
+                if (o == s) meta[i] |= 1 << (16 + q);
+                if (o != s && (done[j] || (j == i && h.nbq[s] < q))) {
                     meta[i] |= 1 << (8 + q);
                     fid[s] = fid[o];
                     two[s] = two[o];
                     h.fn[2 * s] = -h.fn[2 * o];
                     h.fn[2 * s + 1] = -h.fn[2 * o + 1];
                 } else {
-                    fid[s] = next++;
+                    fid[s] = (int)n_rows++;
                     if (thin) two[s] = (int)n_two++;
                 }
             }
@@ -631,6 +635,7 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
     m->n_cells = n;
     m->n_faces_interior = interior / 2;
     m->n_faces_boundary = boundary;
+    m->n_rows = n_rows;
     m->max_faces = maxf;
     const std::vector<double> real = fill_real(h, true), plain = fill_real(h, false);
     const std::vector<float> real32(plain.begin(), plain.end());

@@ -1421,7 +1421,6 @@ FvIdx indices(const bz_mesh *m) {
     return FvIdx{m->d_order, m->d_meta, m->d_fid, m->d_two, m->d_ncen, m->d_cen, m->d_nsec, m->d_sec};
 }
 
-int64_t flux_rows(const bz_mesh *m) { return m->n_faces_interior + m->n_faces_boundary; }
 
 dim3 cell_grid(const bz_mesh *m, int nv, int vec) {
     return dim3((unsigned)m->n_cells, (unsigned)((nv / vec + kFvThreads - 1) / kFvThreads));
@@ -1447,10 +1446,10 @@ void faces_launch(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaSt
     const dim3 grid = cell_grid(m, nv, VEC);
     if (m->order == 3)
         fv_faces_kernel<T, VEC, MAXF, kFvCoef3, kFvCentral3><<<grid, kFvThreads, 0, st>>>(
-            f, FX, pick<T>(m), indices(m), flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+            f, FX, pick<T>(m), indices(m), m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
     else
         fv_faces_kernel<T, VEC, MAXF, 2, kFvCentral><<<grid, kFvThreads, 0, st>>>(
-            f, FX, pick<T>(m), indices(m), flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+            f, FX, pick<T>(m), indices(m), m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
 }
 
 // Threads of a block of the value passes, no more than a row needs as far as
@@ -1477,7 +1476,7 @@ template <int BT, bool TWO, int CPS>
 void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     const int nv = (int)g.nv;
     fv_faces3_persist_kernel<BT, TWO, CPS><<<values_grid(m, nv, CPS), BT, faces3_stage_bytes(BT), st>>>(
-        f, FX, m->t32, indices(m), TWO ? 0 : flux_rows(m), m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+        f, FX, m->t32, indices(m), TWO ? 0 : m->n_rows, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
 }
 // Blocks of 256 threads per SM: three where that saves rounds on a small mesh (a
 // round of three takes about 1.48 rounds of two, and a full one more).  Transport
@@ -1527,7 +1526,7 @@ cudaError_t faces(const bz_mesh *m, const GridView &g, const T *f, T *FX, cudaSt
                 faces3_launch<false>(m, g, f, FX, st);
             else
                 fv_faces_kernel<T, 4, 3, 2, kFvCentral><<<cell_grid(m, nv, 4), kFvThreads, 0, st>>>(
-                    f, FX, m->t32, indices(m), flux_rows(m), nv, g.N, (float)g.L, (float)g.dv);
+                    f, FX, m->t32, indices(m), m->n_rows, nv, g.N, (float)g.L, (float)g.dv);
         } else if (aligned(f, 8)) {
             if (tri) faces_launch<T, 2, 3>(m, g, f, FX, st);
             else faces_launch<T, 2, kFvMaxFaces>(m, g, f, FX, st);
@@ -1553,9 +1552,9 @@ cudaError_t sum_launch(const bz_mesh *m, const GridView &g, const T *FX, T *L, c
     const int *wall = m->n_walls > 0 ? m->d_wall : nullptr;
     if (m->order == 3)
         return launch_after(fv_sum_kernel<T, VEC, MAXF, kFvCoef3>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m),
-                            indices(m), wall, flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+                            indices(m), wall, m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
     return launch_after(fv_sum_kernel<T, VEC, MAXF, 2>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m), indices(m),
-                        wall, flux_rows(m), nv, g.N, (T)g.L, (T)g.dv);
+                        wall, m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
 }
 
 // 16-byte rows where L allows (N^2 is a multiple of 4)
@@ -1645,8 +1644,8 @@ bool fv_two_sided(const bz_mesh *m, bool f32) { return f32 && m->order == 3 && m
 
 int64_t fv_scratch_rows(const bz_mesh *m, bool f32, bool step) {
     if (m->order == 1) return 0;
-    if (step && fv_two_sided(m, f32)) return 4 * flux_rows(m);
-    const int64_t flux = flux_rows(m) + (f32 ? m->n_two * (m->order == 3 ? 4 : 2) : 0);
+    if (step && fv_two_sided(m, f32)) return 4 * m->n_rows;
+    const int64_t flux = m->n_rows + (f32 ? m->n_two * (m->order == 3 ? 4 : 2) : 0);
     return f32 && m->d_tripos ? std::max<int64_t>(flux, 3 * m->n_cells) : flux;
 }
 
