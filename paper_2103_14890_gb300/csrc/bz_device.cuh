@@ -76,7 +76,10 @@ template <int K> __device__ __forceinline__ void block_sum(double (&v)[K], doubl
 // every CTA of this grid has called it; griddep_wait: returns when the kernel
 // before has completed and its writes are visible (at once without the
 // attribute).  A kernel launched that way waits before it touches anything the
-// kernels before it read or write.
+// kernels before it read or write, and reads what they wrote by __ldcg or
+// cp.async: those memory changes while the kernel runs, so a pointer to it must
+// not be `const __restrict__` (the compiler would take it as read-only for the
+// kernel's lifetime and may read it by the non-coherent path, ahead of the wait).
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

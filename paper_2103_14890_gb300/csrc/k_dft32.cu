@@ -174,7 +174,7 @@ fft_fwd32_kernel(const TI *__restrict__ f, typename C2<T>::type *__restrict__ fh
 
 template <typename T, int N, int C>
 __global__ void __launch_bounds__(C * 16)
-fft_inv32_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ Q, T scale, Cinv cinv,
+fft_inv32_kernel(const typename C2<T>::type *Qhat, T *__restrict__ Q, T scale, Cinv cinv,
                  int conserve, const T *__restrict__ P_, T L, T dv, int64_t n) {
     using V2 = typename C2<T>::type;
     using S = T;
@@ -197,7 +197,7 @@ fft_inv32_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ 
 #pragma unroll
             for (int kk = 0; kk < M; ++kk) {
                 const int k2 = kk - (H - 1);
-                const V2 v = qt[(k1 * M + kk) * 32];
+                const V2 v = __ldcg(qt + (k1 * M + kk) * 32);
                 a[bitrev(k2 & (N - 1), LN)] = (k2 & 1) ? cmk<V2>(-v.x, -v.y) : v;
             }
             fft_dit<N, +1>(a);
@@ -403,7 +403,7 @@ __device__ __forceinline__ void invg_epilogue(T (&q)[N], int64_t cell, int j2, c
 
 template <typename T, int N, int C>
 __global__ void __launch_bounds__(C * threads_per_cell<N>())
-fftg_inv_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ Q, T scale, Cinv cinv,
+fftg_inv_kernel(const typename C2<T>::type *Qhat, T *__restrict__ Q, T scale, Cinv cinv,
                 int conserve, const T *__restrict__ P_, T L, T dv, int64_t n) {
     using V2 = typename C2<T>::type;
     using S = T;
@@ -425,7 +425,7 @@ fftg_inv_kernel(const typename C2<T>::type *__restrict__ Qhat, T *__restrict__ Q
 #pragma unroll
         for (int kk = 0; kk < M; ++kk) {
             const int k2 = kk - (H - 1);
-            const V2 v = qt[(k1 * M + kk) * 32];
+            const V2 v = __ldcg(qt + (k1 * M + kk) * 32);
             a[(k2 + N) % N] = (k2 & 1) ? cmk<V2>(-v.x, -v.y) : v;
         }
         fft_nat<N, +1>(a);

@@ -235,8 +235,9 @@ __device__ __forceinline__ void row_pass(const typename C2<T>::type *__restrict_
 // Copy this CTA's cells of the tile's half spectrum into shared memory
 // ([kPad + nhalf + kPad][CELLS], zero guards), or with every row's columns
 // reversed (rev: mode (row, c) <- (row, -c), the spectrum of f reflected in
-// the last velocity axis).
-template <typename V2, int CELLS>
+// the last velocity axis).  AFTER: in a kernel launched after the one that wrote
+// it programmatically.
+template <typename V2, int CELLS, bool AFTER = false>
 __device__ __forceinline__ void stage_spectrum(uint4 *smem16, const V2 *fhat, int64_t tile, int sub, int nhalf,
                                                int M, bool rev) {
     constexpr int VEC = 16 / (int)sizeof(V2);                    // cells per 16-byte vector
@@ -252,7 +253,9 @@ __device__ __forceinline__ void stage_spectrum(uint4 *smem16, const V2 *fhat, in
                 const int row = mode / M;
                 mode = row * M + (M - 1) - (mode - row * M);
             }
-            v = src[mode * ROW + (b % Q4)];
+            const uint4 *x = src + mode * ROW + (b % Q4);
+            if constexpr (AFTER) v = __ldcg(x);
+            else v = *x;
         }
         smem16[i] = v;
     }
@@ -687,7 +690,7 @@ __global__ void __launch_bounds__(WARPS * 32, RR == 2 ? 2 : WARPS <= 4 ? 3 : WAR
     int it = 0;
     while (it + 1 < gd.nitems && (int64_t)blockIdx.x >= gd.tile_start[it + 1]) ++it;
     const Mode32Item &ip = gd.item[it];
-    const float2 *__restrict__ fhat = static_cast<const float2 *>(ip.fhat);
+    const float2 *fhat = static_cast<const float2 *>(ip.fhat);
     float2 *__restrict__ Qhat = static_cast<float2 *>(ip.Qhat);
     const float *__restrict__ W = static_cast<const float *>(ip.W);
     const int *__restrict__ tasks = ip.tasks;
@@ -717,7 +720,7 @@ __global__ void __launch_bounds__(WARPS * 32, RR == 2 ? 2 : WARPS <= 4 ? 3 : WAR
         if (staged) stage_row(wbuf0, W + trec[t].woff, ROWS * trec[t].rowf * (int)sizeof(float), lane);
         griddep_wait();
     }
-    stage_spectrum<float2, CELLS>(smem16, fhat, tile, sub, nhalf, M, false);
+    stage_spectrum<float2, CELLS, RR == 2>(smem16, fhat, tile, sub, nhalf, M, false);
     __syncthreads();
     const float2 *F0 = Fs + (size_t)(kPad + h) * CELLS + cell;
     const bool valid = tile * 32 + sub * CELLS + cell < ip.n;

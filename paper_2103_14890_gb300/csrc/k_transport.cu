@@ -87,6 +87,23 @@ __device__ __forceinline__ Vec<T, VEC> ldv(const T *__restrict__ p) {
     }
     return r;
 }
+// The same for what the kernel before wrote, in a kernel launched after it
+// programmatically (see griddep_wait).
+template <typename T, int VEC>
+__device__ __forceinline__ Vec<T, VEC> ldv_after(const T *p) {
+    Vec<T, VEC> r;
+    if constexpr (VEC == 2) {
+        const typename C2<T>::type q = __ldcg(reinterpret_cast<const typename C2<T>::type *>(p));
+        r.v[0] = q.x; r.v[1] = q.y;
+    } else if constexpr (VEC == 4 && sizeof(T) == 4) {
+        const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
+        r.v[0] = q.x; r.v[1] = q.y; r.v[2] = q.z; r.v[3] = q.w;
+    } else {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) r.v[u] = __ldcg(p + u);
+    }
+    return r;
+}
 template <typename T, int VEC>
 __device__ __forceinline__ void stv(T *__restrict__ p, const Vec<T, VEC> &r) {
     if constexpr (VEC == 2) {
@@ -1057,7 +1074,7 @@ __device__ __forceinline__ RecF rec_f(const int4 *__restrict__ tripos, int64_t p
 
 template <int BT>
 __global__ void __launch_bounds__(BT, kFluxCtasPerSm * kFvThreads / BT)
-fv_flux_values_persist_kernel(const float *__restrict__ FV, float *__restrict__ L, FvTables<float> tb,
+fv_flux_values_persist_kernel(const float *FV, float *__restrict__ L, FvTables<float> tb,
                              const int4 *__restrict__ tripos, int64_t n, int nv, int N, float Lv, float dv) {
     extern __shared__ float4 stage[];            // [2][kFaceRows][BT], [2][warp][32]: 3 (nx, ny), 1 / area
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1191,7 +1208,7 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
 // written last still in L2.  DRAM-bound.
 template <typename T, int VEC, int MAXF, int B>
 __global__ void __launch_bounds__(kFvThreads)
-fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
+fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
               int64_t rows, int nv, int N, T Lv, T dv) {
     const int64_t p = gridDim.x - 1 - blockIdx.x;
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
@@ -1205,7 +1222,7 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
     Vec<T, VEC> x[MAXF];
 #pragma unroll
     for (int q = 0; q < MAXF; ++q)
-        if (q < nf) x[q] = ldv<T, VEC>(FX + (int64_t)row[q] * nv + k);
+        if (q < nf) x[q] = ldv_after<T, VEC>(FX + (int64_t)row[q] * nv + k);
     Vec<T, VEC> o;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] = (T)0;
@@ -1225,22 +1242,23 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
             if (!((two_sided >> q) & 1)) continue;
             const int64_t s = p * kFvMaxFaces + q;
             if (wall && __ldg(wall + s) >= 0) {          // the wall's flux row
-                const T *r = FX + (int64_t)__ldg(ix.fid + s) * nv + k;
-                for (int u = 0; u < VEC; ++u) o.v[u] += r[u];
+                const Vec<T, VEC> r = ldv_after<T, VEC>(FX + (int64_t)__ldg(ix.fid + s) * nv + k);
+                for (int u = 0; u < VEC; ++u) o.v[u] += r.v[u];
                 continue;
             }
             const int side = (meta >> (8 + q)) & 1, two = __ldg(ix.two + s);
             const bool boundary = (meta >> (16 + q)) & 1;
             const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
             for (int g = 0; g < GP; ++g) {
-                const T *a = FX + two_row<B>(rows, two, side, g) * nv + k;
+                const Vec<T, VEC> a = ldv_after<T, VEC>(FX + two_row<B>(rows, two, side, g) * nv + k);
                 // the other side's points run the other way
-                const T *b = boundary ? a : FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k;
+                const Vec<T, VEC> b =
+                    boundary ? a : ldv_after<T, VEC>(FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k);
                 for (int u = 0; u < VEC; ++u) {
                     const Velocity<T, 1> v(k + u, N, Lv, dv);
                     T vn[1];
                     normal_velocity<T, 1>(v.v1, v.v2, nx, ny, vn);
-                    const T h = half * vn[0], fl = a[u], fr = b[u];
+                    const T h = half * vn[0], fl = a.v[u], fr = b.v[u];
                     o.v[u] = fma(h, fl + fr, o.v[u]);
                     o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
                 }
@@ -1256,7 +1274,7 @@ fv_sum_kernel(const T *__restrict__ FX, T *__restrict__ L, FvTables<T> tb, FvIdx
 // both points of every face, term by term as in the two-sided faces above.
 template <int VEC, int MAXF>
 __global__ void __launch_bounds__(kFvThreads)
-fv_sum_two_kernel(const float *__restrict__ FX, float *__restrict__ L, FvTables<float> tb, FvIdx ix, int nv, int N,
+fv_sum_two_kernel(const float *FX, float *__restrict__ L, FvTables<float> tb, FvIdx ix, int nv, int N,
                   float Lv, float dv) {
     const int64_t p = gridDim.x - 1 - blockIdx.x;
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
@@ -1278,9 +1296,9 @@ fv_sum_two_kernel(const float *__restrict__ FX, float *__restrict__ L, FvTables<
         normal_velocity<float, VEC>(v.v1, v.v2, __ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
-            const Vec<float, VEC> a = ldv<float, VEC>(FX + two_row<kFvCoef3>(0, fid, side, g) * nv + k);
+            const Vec<float, VEC> a = ldv_after<float, VEC>(FX + two_row<kFvCoef3>(0, fid, side, g) * nv + k);
             const Vec<float, VEC> b =
-                boundary ? a : ldv<float, VEC>(FX + two_row<kFvCoef3>(0, fid, 1 - side, 1 - g) * nv + k);
+                boundary ? a : ldv_after<float, VEC>(FX + two_row<kFvCoef3>(0, fid, 1 - side, 1 - g) * nv + k);
 #pragma unroll
             for (int u = 0; u < VEC; ++u) {
                 const float h = 0.25f * vn[u];
