@@ -142,7 +142,9 @@ template <typename T> struct FvTables {
     const T *Rs;            // [p][face][4]  sector inverses (row-major 2 x 2)
     const T *quad;          // [p][4]  FP32: (mu20, mu11, mu02, h^2); FP64: the degree-2 smoothness form's
                             //         coefficients (4 mu20 + 4, mu20 + mu02 + 1, 4 mu02 + 4, 4 mu11)
-    const T *fn;            // [p][face][2]  |e| n_e outward (exactly opposite on the two sides of a face)
+    const T *fn;            // [p][face][2]  |e| n_e outward
+    const T *fs;            // [p][face][2]  the same, exactly opposite on the two sides of a face (fn may differ by
+                            //               rounding across a period): which side is upwind
     const T *phi;           // [p][face][B]  means of the basis over the face
     const T *phig;          // [p][face][2][B]  order 3: the basis at the face's two Gauss points
     const T *Rc;            // [p][B][K]  least-squares rows
@@ -321,8 +323,8 @@ cudaError_t launch_fill_zero(void *p, int64_t bytes, cudaStream_t st);
 
 // ---- transport residual (k_transport.cu) ----------------------------------
 // Order 1: L from f in one pass.  Orders 2 and 3: the reconstruction pass
-// writes the upwind flux of every face, FX [face][nv], each velocity by the
-// cell it leaves; then L [cell][nv] = the signed sum of a cell's face rows
+// writes the upwind mean over every face, FX [face][nv], each velocity by the
+// cell it leaves; then L [cell][nv] = the sum of v.n times a cell's face rows
 // over |P_i|.  FP32, order 2 on triangles without walls (N divisible by 4,
 // 16-byte aligned rows: fv_value_mode): the reconstruction writes each cell's
 // values at its three faces, FV [cell][3][nv], and the flux pass reads those

@@ -45,7 +45,7 @@ struct HostMesh {
     int64_t n = 0;
     int B = 0, K = 0;                  // coefficients and stencil cells of the order (0: order 1)
     std::vector<int> nface, nb, nbq, ncen, cen, nsec, sec, order;
-    std::vector<double> inv_area, h2, fn, Rc, Rs, phi, phig, mu;
+    std::vector<double> inv_area, h2, fn, fs, Rc, Rs, phi, phig, mu;
 };
 
 // Means over a polygon (vertices px, py in order, translated by (sx, sy)) of
@@ -113,6 +113,7 @@ FvTables<T> carve(void *base, const HostMesh &h) {
     t.Rs = p; p += n * (h.B ? kFvMaxFaces * 4 : 0);
     t.quad = p; p += n * (h.B ? 4 : 0);
     t.fn = p; p += n * kFvMaxFaces * 2;
+    t.fs = p; p += n * (h.B ? kFvMaxFaces * 2 : 0);
     t.phi = p; p += n * kFvMaxFaces * h.B;
     t.phig = p; p += n * kFvMaxFaces * (h.B == kFvCoef3 ? 2 * h.B : 0);
     t.Rc = p; p += n * h.B * h.K;
@@ -155,6 +156,7 @@ std::vector<double> fill_real(const HostMesh &h, bool folded) {
         put(quad, 4, one);
     }
     put(h.fn, kFvMaxFaces * 2, one);
+    put(h.fs, h.B ? kFvMaxFaces * 2 : 0, one);
     put(h.phi, kFvMaxFaces * h.B, ih);
     put(h.phig, h.B == kFvCoef3 ? kFvMaxFaces * 2 * h.B : 0, one);
     if (folded) {
@@ -591,8 +593,8 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
         for (int64_t i = 0; i < n; ++i) h.order[i] = key[i].second;
     }
     // faces in the processing order of their owners (the first cell of the two
-    // in that order); the other side's normal is the owner's, negated, so both
-    // sides form the same normal velocities up to the sign.  An edge that is its
+    // in that order); which side a velocity leaves is told by the owner's normal,
+    // negated on the other side, so both sides agree.  An edge that is its
     // own reverse (both ends one point: of no length, or as long as a period) has
     // no other side and is a transmissive boundary here.
     std::vector<int> meta((size_t)n, 0), fid((size_t)n * kFvMaxFaces, 0), two((size_t)n * kFvMaxFaces, 0);
@@ -605,6 +607,7 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
             meta[i] = h.nface[i] | (per * sqrt(h.h2[i]) > kFvThin * area[i] ? kFvThinFlag : 0);
         }
         std::vector<char> done((size_t)n, 0);
+        h.fs = h.fn;
         for (int64_t p = 0; p < n; ++p) {
             const int64_t i = h.order[p];
             for (int q = 0; q < h.nface[i]; ++q) {
@@ -618,8 +621,8 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                     meta[i] |= 1 << (8 + q);
                     fid[s] = fid[o];
                     two[s] = two[o];
-                    h.fn[2 * s] = -h.fn[2 * o];
-                    h.fn[2 * s + 1] = -h.fn[2 * o + 1];
+                    h.fs[2 * s] = -h.fs[2 * o];
+                    h.fs[2 * s + 1] = -h.fs[2 * o + 1];
                 } else {
                     fid[s] = (int)n_rows++;
                     if (thin) two[s] = (int)n_two++;
@@ -627,6 +630,7 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
             }
             done[i] = 1;
         }
+        if (!B) h.fs.clear();
     }
     bz_mesh *m = (bz_mesh *)calloc(1, sizeof(bz_mesh));
     if (!m) return fail(BZ_ENOMEM, "build_fv_mesh: host allocation");

@@ -16,12 +16,18 @@
 // the reconstruction per face (midpoint for degree 1, two Gauss points for
 // degree 2), on the upwind side only.
 //   Pass 1 reconstructs the polynomial of every (cell, velocity) in registers
-//   and writes the flux of the velocities that leave the cell through a face
-//   into that face's row, FX [face][nv]; the cell on the other side of the
-//   face writes the others.  Both sides form v.n from the same normal up to
-//   its sign, so every entry is written exactly once (v.n = 0: by the owner).
-//   Boundary faces are transmissive: their cell writes every velocity.
-//   Pass 2 sums a cell's face rows with their signs and divides by |P_i|.
+//   and writes its mean over a face, for the velocities that leave the cell
+//   there, into that face's row, FX [face][nv]; the cell on the other side of
+//   the face writes the others.  Both sides form v.n from the same normal up to
+//   its sign (table fs), so every entry is written exactly once (v.n = 0: by
+//   the owner).  Boundary faces are transmissive: their cell writes every
+//   velocity.
+//   Pass 2 sums v.n times a cell's face rows, the normals its own (table fn: they
+//   sum to zero over its faces, which the two sides' copies of a face in a
+//   periodic mesh, equal up to rounding only, would not), by FMA, and divides by
+//   |P_i|.  With rows of fluxes, rounded once more and formed with the owner's
+//   normal on both sides, FP64 errors were up to 3 times as large on Voronoi
+//   meshes (1200 cells x 16^2: 3.3e-15 of L's norm, @V16@ so) and 1.5 times on triangles.
 // FP32, thin cells (kFvThin; slivers of a Delaunay triangulation along the
 // boundary, half a percent of the cells): the fluxes cancel to L by a factor
 // of hundreds to thousands, which turns a rounding into a visible change of L.
@@ -61,6 +67,7 @@ namespace bz {
 namespace {
 
 constexpr int kFvThreads = 256;
+constexpr int kFvMaxNodes = 64;      // largest N of a 2-D grid
 
 // VEC consecutive velocities per thread, all in one row of the velocity grid
 // (N is even, and the host takes VEC = 4 only when 4 divides N): the cell's
@@ -164,28 +171,23 @@ __device__ __forceinline__ double scaled_rcp(double b, int scale) {
 // Signs and comparisons of finite FP64 values as integers, off the FP64 pipe.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.f; }
-__device__ __forceinline__ double negate_if(bool neg, double x) {
-    return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
-}
-__device__ __forceinline__ float negate_if(bool neg, float x) { return neg ? -x : x; }
 // Not negative (-0 included), for a velocity, never a NaN.
 template <typename T> __device__ __forceinline__ bool leaves(T vn) {
-    if constexpr (sizeof(T) == 8) return !positive(negate_if(true, vn));
+    if constexpr (sizeof(T) == 8) return !positive(__hiloint2double(__double2hiint(vn) ^ 0x80000000, __double2loint(vn)));
     else return vn >= (T)0;
 }
 
-// Write the flux of VEC velocities through a face: vn (outward normal velocity
-// times |e|) times the reconstructed mean `val`, in the owner's orientation,
-// where this cell is upwind (everywhere on a boundary face).
+// Write the reconstructed mean `val` of VEC velocities over a face, vn their
+// outward normal velocities, where this cell is upwind (everywhere on a boundary
+// face).
 template <typename T, int VEC>
-__device__ __forceinline__ void put_flux(T *__restrict__ row, const T (&vn)[VEC], const T (&val)[VEC], bool other,
-                                         bool boundary) {
+__device__ __forceinline__ void put_upwind(T *__restrict__ row, const T (&vn)[VEC], const T (&val)[VEC], bool other,
+                                           bool boundary) {
     Vec<T, VEC> o;
     bool on[VEC], all = true;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
-        const T fl = vn[u] * val[u];
-        o.v[u] = negate_if(other, fl);
+        o.v[u] = val[u];
         on[u] = boundary || (other ? positive(vn[u]) : leaves(vn[u]));
         all = all && on[u];
     }
@@ -556,15 +558,16 @@ template <int B> __device__ __forceinline__ int64_t two_row(int64_t rows, int tw
     return rows + ((int64_t)two * 2 + side) * GP + g;
 }
 
-// Face q of the cell at position p: the upwind flux, and on a two-sided face
-// (FP32) the values at its points.  fn, phi: the face's entries of these tables.
+// Face q of the cell at position p: its mean for the velocities it is upwind of,
+// and on a two-sided face (FP32) the values at its points.  fs, phi: the face's
+// entries of these tables.
 // TWO: only the values at its two points (every face taken as two-sided; the
 // rows number faces).
 template <typename T, int VEC, int B, bool SM, bool TWO = false>
 __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> &tb, const FvIdx &ix, int64_t rows,
                                           int64_t p, int q, int fid, int meta, int k, int nv, T v1,
                                           const T (&v2)[VEC], const Vec<T, VEC> &fi, const T (&c)[B][VEC],
-                                          const T *fn, const T *phi) {
+                                          const T *fs, const T *phi) {
     const int64_t s = p * kFvMaxFaces + q;
     T vn[VEC], val[VEC];
     const bool other = (meta >> (8 + q)) & 1, boundary = (meta >> (16 + q)) & 1;
@@ -580,13 +583,13 @@ __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> 
         }
     }
     if constexpr (TWO) return;
-    normal_velocity<T, VEC>(v1, v2, tab_load<SM>(fn), tab_load<SM>(fn + 1), vn);
+    normal_velocity<T, VEC>(v1, v2, tab_load<SM>(fs), tab_load<SM>(fs + 1), vn);
     bool any = boundary;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) any = any || leaves(vn[u]);
     if (!any) return;
     point_value<T, VEC, B, SM>(fi, c, phi, val);
-    put_flux<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
+    put_upwind<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
 }
 
 // Pass 1 of one cell, any polygon.
@@ -609,7 +612,7 @@ __device__ __forceinline__ void recon_faces(const T *__restrict__ f, T *__restri
     for (int q = 0; q < MAXF; ++q)
         if (q < nf)
             emit_face<T, VEC, B, false, TWO>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv, v1,
-                                             v2, fi, c, tb.fn + 2 * (p * kFvMaxFaces + q), tb.phi + (p * kFvMaxFaces + q) * B);
+                                             v2, fi, c, tb.fs + 2 * (p * kFvMaxFaces + q), tb.phi + (p * kFvMaxFaces + q) * B);
 }
 
 // Weights of one pair of velocities of a flagged triangle (kFvRegular: its
@@ -724,6 +727,28 @@ template <typename T, int VEC> struct Velocity {
     }
 };
 
+// The nodes of VEC consecutive velocities, the two of a pair (N is even) in one
+// row; node(j): the j-th node.
+template <typename T, int VEC> struct PairVelocity {
+    T v1[(VEC + 1) / 2], v2[VEC];
+    template <typename Node> __device__ __forceinline__ PairVelocity(int k, int N, Node node) {
+        int j1 = k / N, j2 = k - j1 * N;
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            if (u > 0 && u % 2 == 0 && j2 + u >= N) {
+                ++j1;
+                j2 -= N;
+            }
+            if (u % 2 == 0) v1[u / 2] = node(j1);
+            v2[u] = node(j2 + u);
+        }
+    }
+    __device__ __forceinline__ void normal(T nx, T ny, T (&vn)[VEC]) const {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) vn[u] = fma(v2[u], ny, v1[u / 2] * nx);
+    }
+};
+
 template <typename T, int VEC, int MAXF, int B, int K, bool TWO>
 __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restrict__ FX, const FvTables<T> &tb,
                                             const FvIdx &ix, int64_t rows, int nv, int N, T Lv, T dv) {
@@ -743,7 +768,7 @@ __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restri
 #pragma unroll
             for (int q = 0; q < 3; ++q)
                 emit_face<float, 4, B, false, TWO>(FX, tb, ix, rows, p, q, __ldg(ix.fid + p * kFvMaxFaces + q), meta, k, nv,
-                                              v.v1, v.v2, fi, c, tb.fn + 2 * (p * kFvMaxFaces + q),
+                                              v.v1, v.v2, fi, c, tb.fs + 2 * (p * kFvMaxFaces + q),
                                               tb.phi + (p * kFvMaxFaces + q) * B);
             return;
         }
@@ -805,7 +830,7 @@ constexpr size_t face_stage_bytes(int threads) {
 // (faces3_per_sm), and narrower blocks gain by the warps (24^2 on 19802 cells
 // 165 -> 158 us, on 472 cells 19.0 -> 16.5).
 constexpr int kRows3 = 1 + kFvCentral3;
-constexpr int kTab3Rs = 0, kTab3Quad = 12, kTab3Rc = 16, kTab3Phi = 71, kTab3Fn = 86, kTab3Values = 92;
+constexpr int kTab3Rs = 0, kTab3Quad = 12, kTab3Rc = 16, kTab3Phi = 71, kTab3Fs = 86, kTab3Values = 92;
 constexpr int kIdx3Cen = 0, kIdx3Fid = 11, kIdx3Order = 14, kIdx3Meta = 15, kIdx3Ncen = 16, kIdx3Values = 17;
 constexpr int kTab3Pitch = 96, kIdx3Pitch = 20;   // per warp and buffer
 constexpr size_t faces3_stage_bytes(int threads) {
@@ -839,9 +864,9 @@ fv_faces3_persist_kernel(const float *__restrict__ f, float *__restrict__ FX, Fv
     for (int u = 0; u < 3; ++u) {
         const int e = lane + 32 * u;
         ts[u] = e < kTab3Quad ? tb.Rs + e : e < kTab3Rc ? tb.quad + (e - kTab3Quad) : e < kTab3Phi ? tb.Rc + (e - kTab3Rc)
-              : e < kTab3Fn ? tb.phi + (e - kTab3Phi) : tb.fn + (e - kTab3Fn);
+              : e < kTab3Fs ? tb.phi + (e - kTab3Phi) : tb.fs + (e - kTab3Fs);
         td[u] = e < kTab3Quad ? kFvMaxFaces * 4 : e < kTab3Rc ? 4 : e < kTab3Phi ? B * K
-              : e < kTab3Fn ? kFvMaxFaces * B : kFvMaxFaces * 2;
+              : e < kTab3Fs ? kFvMaxFaces * B : kFvMaxFaces * 2;
     }
     auto issue_idx = [&](int64_t pr, int slot) {
         if (lane < kIdx3Values) cp_async4(idxs + slot * W * kIdx3Pitch + lane, is + pr * id);
@@ -890,7 +915,7 @@ fv_faces3_persist_kernel(const float *__restrict__ f, float *__restrict__ FX, Fv
 #pragma unroll
             for (int q = 0; act && q < 3; ++q)
                 emit_face<float, 4, B, true, TWO>(FX, tb, ix, rows, p, q, x[kIdx3Fid + q], meta, k, nv, v.v1, v.v2, fi, c,
-                                             tab + kTab3Fn + 2 * q, tab + kTab3Phi + B * q);
+                                             tab + kTab3Fs + 2 * q, tab + kTab3Phi + B * q);
         } else {
             ahead();
             if (act) recon_faces<float, 4, 3, B, K, TWO>(f, FX, tb, ix, rows, p, ncf, meta, k, nv, v.v1,
@@ -1150,10 +1175,10 @@ fv_flux_values_persist_kernel(const float *FV, float *__restrict__ L, FvTables<f
 
 // Incoming half of a wall face (full accommodation, eq. BOU with alpha = 1,
 // eq. MAXB, eq. MU): one block per wall holds all nv <= 1024 velocities, 4 per
-// thread.  mu, the ratio of the outgoing mass flux sum_{v.n > 0} f_L v.n (the
-// face row as pass 1 wrote it) to the incoming flux of the unit wall
+// thread.  mu, the ratio of the outgoing mass flux sum_{v.n > 0} f_L v.n (f_L
+// the face row as pass 1 wrote it) to the incoming flux of the unit wall
 // Maxwellian sum_{v.n < 0} M_w |v.n|, is a block reduction (FP64, fixed
-// order); velocities entering the domain get the flux (v.n) mu M_w(v).  For
+// order); velocities entering the domain get the value mu M_w(v).  For
 // degree 2 the balance at the face's two Gauss points is linear in the
 // outgoing flux, so the mean over the face is balanced once.
 template <typename T>
@@ -1178,7 +1203,7 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
     for (int u = 0; u < 4; ++u) {
         const T d1 = v.v1 - uw1, d2 = v.v2[u] - uw2;
         mw[u] = norm * exp(-(d1 * d1 + d2 * d2) * inv2th);
-        if (act && vn[u] > (T)0) num += (double)row[u];
+        if (act && vn[u] > (T)0) num += (double)(row[u] * vn[u]);
         if (act && vn[u] < (T)0) den += (double)(mw[u] * -vn[u]);
     }
 #pragma unroll
@@ -1200,19 +1225,30 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
     const T mu = (T)(num / den);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-        if (act && !(vn[u] > (T)0)) row[u] = vn[u] * (mu * mw[u]);
+        if (act && !(vn[u] > (T)0)) row[u] = mu * mw[u];
 }
 
-// Pass 2: L_i = (1/|P_i|) sum over the faces of the signed flux rows, the
-// cells in the reverse of pass 1's order, so that the first ones find the rows
-// written last still in L2.  DRAM-bound.
+// Pass 2: L_i = (1/|P_i|) sum over the faces of v.n times their rows, the cells
+// in the reverse of pass 1's order, so that the first ones find the rows written
+// last still in L2.  FP32: DRAM-bound.  FP64: as much by the FP64 pipe; the nodes
+// come from shared memory, formed once per block.
 template <typename T, int VEC, int MAXF, int B>
 __global__ void __launch_bounds__(kFvThreads)
 fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
               int64_t rows, int nv, int N, T Lv, T dv) {
+    constexpr bool F64 = sizeof(T) == 8;
+    __shared__ T nodes[F64 ? kFvMaxNodes : 1];
+    if constexpr (F64) {
+        if ((int)threadIdx.x < N) nodes[threadIdx.x] = -Lv + (T)threadIdx.x * dv;
+        __syncthreads();
+    }
     const int64_t p = gridDim.x - 1 - blockIdx.x;
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
     if (k >= nv) return;
+    const PairVelocity<T, VEC> v(k, N, [&](int j) {
+        if constexpr (F64) return nodes[j];
+        else return -Lv + (T)j * dv;
+    });
     const int meta = __ldg(ix.meta + p), nf = meta & 0xf;
     int row[MAXF];
 #pragma unroll
@@ -1230,9 +1266,10 @@ fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const in
 #pragma unroll
     for (int q = 0; q < MAXF; ++q)
         if (q < nf && !((two_sided >> q) & 1)) {
-            const bool other = (meta >> (8 + q)) & 1;
+            T vn[VEC];
+            v.normal(__ldg(tb.fn + 2 * (p * kFvMaxFaces + q)), __ldg(tb.fn + 2 * (p * kFvMaxFaces + q) + 1), vn);
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, x[q].v[u]);
+            for (int u = 0; u < VEC; ++u) o.v[u] = fma(vn[u], x[q].v[u], o.v[u]);
         }
     if (two_sided) {
         // faces of thin cells: (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2 at every face point
@@ -1241,24 +1278,24 @@ fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const in
         for (int q = 0; q < nf; ++q) {
             if (!((two_sided >> q) & 1)) continue;
             const int64_t s = p * kFvMaxFaces + q;
-            if (wall && __ldg(wall + s) >= 0) {          // the wall's flux row
+            T vn[VEC];
+            v.normal(__ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
+            if (wall && __ldg(wall + s) >= 0) {          // the wall's row
                 const Vec<T, VEC> r = ldv_after<T, VEC>(FX + (int64_t)__ldg(ix.fid + s) * nv + k);
-                for (int u = 0; u < VEC; ++u) o.v[u] += r.v[u];
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) o.v[u] = fma(vn[u], r.v[u], o.v[u]);
                 continue;
             }
             const int side = (meta >> (8 + q)) & 1, two = __ldg(ix.two + s);
             const bool boundary = (meta >> (16 + q)) & 1;
-            const T nx = __ldg(tb.fn + 2 * s), ny = __ldg(tb.fn + 2 * s + 1);
             for (int g = 0; g < GP; ++g) {
                 const Vec<T, VEC> a = ldv_after<T, VEC>(FX + two_row<B>(rows, two, side, g) * nv + k);
                 // the other side's points run the other way
                 const Vec<T, VEC> b =
                     boundary ? a : ldv_after<T, VEC>(FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k);
+#pragma unroll
                 for (int u = 0; u < VEC; ++u) {
-                    const Velocity<T, 1> v(k + u, N, Lv, dv);
-                    T vn[1];
-                    normal_velocity<T, 1>(v.v1, v.v2, nx, ny, vn);
-                    const T h = half * vn[0], fl = a.v[u], fr = b.v[u];
+                    const T h = half * vn[u], fl = a.v[u], fr = b.v[u];
                     o.v[u] = fma(h, fl + fr, o.v[u]);
                     o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
                 }
