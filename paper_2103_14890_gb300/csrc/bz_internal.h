@@ -154,6 +154,9 @@ template <typename T> struct FvTables {
 // equilateral triangle) cancels its face fluxes to L by that much.
 constexpr double kFvThin = 50.0;
 constexpr int kFvThinFlag = 0x10;     // in meta: a thin cell
+constexpr int kFvSplitFlag = 0x20;    // in meta: a cell with a split face
+constexpr int kFvSplit = 1 << 30;     // in d_two: a face whose two sides' normals are not exactly opposite (the two
+                                      // copies of a face across a period)
 }  // namespace bz
 
 struct bz_mesh {
@@ -165,12 +168,12 @@ struct bz_mesh {
     // index tables by position of the processing order (cells sorted along a
     // Morton curve of their barycentres), values are cell indices
     int *d_order;           // [p] cell
-    int *d_meta;            // [p] faces | kFvThinFlag | not-owner bits << 8 | boundary bits << 16 | two-sided
+    int *d_meta;            // [p] faces | kFvThinFlag | kFvSplitFlag | not-owner bits << 8 | boundary bits << 16 | two-sided
                             // bits << 24 (bit q: face q); the owner of a face is its first cell in the
                             // processing order; a two-sided face bounds a thin cell
     int *d_nb;              // [p][face] neighbour, -1 boundary
     int *d_fid;             // [p][face] face index, numbered in the processing order of the owners
-    int *d_two;             // [p][face] index of a two-sided face
+    int *d_two;             // [p][face] index of a two-sided face, | kFvSplit
     int64_t n_two;
     int *d_ncen;            // [p] central stencil size (<= K), | kFvRegular for a triangle whose stencil
                             // starts with its face neighbours, sector s on faces s, s+1
@@ -323,9 +326,9 @@ cudaError_t launch_fill_zero(void *p, int64_t bytes, cudaStream_t st);
 
 // ---- transport residual (k_transport.cu) ----------------------------------
 // Order 1: L from f in one pass.  Orders 2 and 3: the reconstruction pass
-// writes the upwind mean over every face, FX [face][nv], each velocity by the
-// cell it leaves; then L [cell][nv] = the sum of v.n times a cell's face rows
-// over |P_i|.  FP32, order 2 on triangles without walls (N divisible by 4,
+// writes the upwind mean over every face (FP64: the flux), FX [face][nv], each
+// velocity by the cell it leaves; then L [cell][nv] = the sum of v.n times a
+// cell's face rows over |P_i|.  FP32, order 2 on triangles without walls (N divisible by 4,
 // 16-byte aligned rows: fv_value_mode): the reconstruction writes each cell's
 // values at its three faces, FV [cell][3][nv], and the flux pass reads those
 // of the cell and its neighbours.  Scratch: fv_scratch_rows() rows of nv.

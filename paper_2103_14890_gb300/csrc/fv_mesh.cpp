@@ -623,6 +623,12 @@ int fv_mesh_create(int n_vertices, const double *xy, int64_t n_cells, const int6
                     two[s] = two[o];
                     h.fs[2 * s] = -h.fs[2 * o];
                     h.fs[2 * s + 1] = -h.fs[2 * o + 1];
+                    if (h.fs[2 * s] != h.fn[2 * s] || h.fs[2 * s + 1] != h.fn[2 * s + 1]) {
+                        two[s] |= kFvSplit;
+                        two[o] |= kFvSplit;
+                        meta[i] |= kFvSplitFlag;
+                        meta[j] |= kFvSplitFlag;
+                    }
                 } else {
                     fid[s] = (int)n_rows++;
                     if (thin) two[s] = (int)n_two++;

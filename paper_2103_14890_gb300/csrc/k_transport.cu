@@ -22,12 +22,15 @@
 //   its sign (table fs), so every entry is written exactly once (v.n = 0: by
 //   the owner).  Boundary faces are transmissive: their cell writes every
 //   velocity.
-//   Pass 2 sums v.n times a cell's face rows, the normals its own (table fn: they
-//   sum to zero over its faces, which the two sides' copies of a face in a
-//   periodic mesh, equal up to rounding only, would not), by FMA, and divides by
-//   |P_i|.  With rows of fluxes, rounded once more and formed with the owner's
-//   normal on both sides, FP64 errors were up to 3 times as large on Voronoi
-//   meshes (1200 cells x 16^2: 3.3e-15 of L's norm, @V16@ so) and 1.5 times on triangles.
+//   Pass 2 sums v.n times a cell's face rows by FMA, the normals its own (table
+//   fn), and divides by |P_i|.
+// FP64 rows hold the flux (v.n times the mean) instead, and pass 2 adds them up:
+// the product and the normal velocity would take as long again (0.106 ms for
+// 0.041 on 2603 cells x 30^2) and gain no accuracy.  The exception are faces whose
+// two copies, a period apart in a periodic mesh, differ by rounding (kFvSplit):
+// with one side's normal for both, a cell's normals no longer sum to zero (errors
+// on 300 and 1200 Voronoi cells 2.2e-15 and 3.3e-15 of L's norm, 1.1e-15 and
+// 1.2e-15 with its own).
 // FP32, thin cells (kFvThin; slivers of a Delaunay triangulation along the
 // boundary, half a percent of the cells): the fluxes cancel to L by a factor
 // of hundreds to thousands, which turns a rounding into a visible change of L.
@@ -67,7 +70,6 @@ namespace bz {
 namespace {
 
 constexpr int kFvThreads = 256;
-constexpr int kFvMaxNodes = 64;      // largest N of a 2-D grid
 
 // VEC consecutive velocities per thread, all in one row of the velocity grid
 // (N is even, and the host takes VEC = 4 only when 4 divides N): the cell's
@@ -171,23 +173,28 @@ __device__ __forceinline__ double scaled_rcp(double b, int scale) {
 // Signs and comparisons of finite FP64 values as integers, off the FP64 pipe.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+__device__ __forceinline__ double negate_if(bool neg, double x) {
+    return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
 // Not negative (-0 included), for a velocity, never a NaN.
 template <typename T> __device__ __forceinline__ bool leaves(T vn) {
-    if constexpr (sizeof(T) == 8) return !positive(__hiloint2double(__double2hiint(vn) ^ 0x80000000, __double2loint(vn)));
+    if constexpr (sizeof(T) == 8) return !positive(negate_if(true, vn));
     else return vn >= (T)0;
 }
 
-// Write the reconstructed mean `val` of VEC velocities over a face, vn their
-// outward normal velocities, where this cell is upwind (everywhere on a boundary
-// face).
+// Write a face's row where this cell is upwind (everywhere on a boundary face):
+// the reconstructed mean `val` of VEC velocities, vn their outward normal
+// velocities; flux (FP64): vn times it, in the owner's orientation.
 template <typename T, int VEC>
 __device__ __forceinline__ void put_upwind(T *__restrict__ row, const T (&vn)[VEC], const T (&val)[VEC], bool other,
-                                           bool boundary) {
+                                           bool boundary, bool flux) {
     Vec<T, VEC> o;
     bool on[VEC], all = true;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
         o.v[u] = val[u];
+        if constexpr (sizeof(T) == 8)
+            if (flux) o.v[u] = negate_if(other, vn[u] * val[u]);
         on[u] = boundary || (other ? positive(vn[u]) : leaves(vn[u]));
         all = all && on[u];
     }
@@ -572,7 +579,7 @@ __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> 
     T vn[VEC], val[VEC];
     const bool other = (meta >> (8 + q)) & 1, boundary = (meta >> (16 + q)) & 1;
     if (TWO || (sizeof(T) == 4 && ((meta >> (24 + q)) & 1))) {
-        const int two = TWO ? fid : __ldg(ix.two + s);
+        const int two = TWO ? fid : __ldg(ix.two + s) & (kFvSplit - 1);
 #pragma unroll
         for (int g = 0; g < (B == kFvCoef3 ? 2 : 1); ++g) {
             point_value<T, VEC, B>(fi, c, B == kFvCoef3 ? tb.phig + (s * 2 + g) * B : tb.phi + s * B, val);
@@ -589,7 +596,8 @@ __device__ __forceinline__ void emit_face(T *__restrict__ FX, const FvTables<T> 
     for (int u = 0; u < VEC; ++u) any = any || leaves(vn[u]);
     if (!any) return;
     point_value<T, VEC, B, SM>(fi, c, phi, val);
-    put_upwind<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary);
+    const bool flux = sizeof(T) == 8 && !((meta & kFvSplitFlag) && (__ldg(ix.two + s) & kFvSplit));
+    put_upwind<T, VEC>(FX + (int64_t)fid * nv + k, vn, val, other, boundary, flux);
 }
 
 // Pass 1 of one cell, any polygon.
@@ -728,24 +736,37 @@ template <typename T, int VEC> struct Velocity {
 };
 
 // The nodes of VEC consecutive velocities, the two of a pair (N is even) in one
-// row; node(j): the j-th node.
+// row.  k / N by a product: k < 2^12 and N <= 64, so (k + 1/2) / N lies further
+// from a whole number than FP32 rounds it.
 template <typename T, int VEC> struct PairVelocity {
     T v1[(VEC + 1) / 2], v2[VEC];
-    template <typename Node> __device__ __forceinline__ PairVelocity(int k, int N, Node node) {
-        int j1 = k / N, j2 = k - j1 * N;
+    __device__ __forceinline__ PairVelocity(int k, int N, float iN, T Lv, T dv) {
+        float j1 = floorf(((float)k + 0.5f) * iN), j2 = fmaf(-j1, (float)N, (float)k);
 #pragma unroll
         for (int u = 0; u < VEC; ++u) {
-            if (u > 0 && u % 2 == 0 && j2 + u >= N) {
-                ++j1;
-                j2 -= N;
+            if (u > 0 && u % 2 == 0 && j2 + u >= (float)N) {
+                j1 += 1.f;
+                j2 -= (float)N;
             }
-            if (u % 2 == 0) v1[u / 2] = node(j1);
-            v2[u] = node(j2 + u);
+            if (u % 2 == 0) v1[u / 2] = fma((T)j1, dv, -Lv);
+            v2[u] = fma((T)(j2 + u), dv, -Lv);
         }
     }
-    __device__ __forceinline__ void normal(T nx, T ny, T (&vn)[VEC]) const {
+    // acc += v.n x
+    __device__ __forceinline__ void add_flux(const typename C2<T>::type &n, const Vec<T, VEC> &x,
+                                             Vec<T, VEC> &acc) const {
+        if constexpr (sizeof(T) == 4 && VEC == 4) {
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) vn[u] = fma(v2[u], ny, v1[u / 2] * nx);
+            for (int u = 0; u < 4; u += 2) {
+                const float2 vn = fma2(make_float2(v2[u], v2[u + 1]), dup2(n.y), dup2(v1[u / 2] * n.x));
+                const float2 a = fma2(vn, make_float2(x.v[u], x.v[u + 1]), make_float2(acc.v[u], acc.v[u + 1]));
+                acc.v[u] = a.x;
+                acc.v[u + 1] = a.y;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) acc.v[u] = fma(fma(v2[u], n.y, v1[u / 2] * n.x), x.v[u], acc.v[u]);
+        }
     }
 };
 
@@ -1175,16 +1196,17 @@ fv_flux_values_persist_kernel(const float *FV, float *__restrict__ L, FvTables<f
 
 // Incoming half of a wall face (full accommodation, eq. BOU with alpha = 1,
 // eq. MAXB, eq. MU): one block per wall holds all nv <= 1024 velocities, 4 per
-// thread.  mu, the ratio of the outgoing mass flux sum_{v.n > 0} f_L v.n (f_L
-// the face row as pass 1 wrote it) to the incoming flux of the unit wall
-// Maxwellian sum_{v.n < 0} M_w |v.n|, is a block reduction (FP64, fixed
-// order); velocities entering the domain get the value mu M_w(v).  For
+// thread.  mu, the ratio of the outgoing mass flux sum_{v.n > 0} f_L v.n (the
+// face row as pass 1 wrote it; FP32: times v.n) to the incoming flux of the unit
+// wall Maxwellian sum_{v.n < 0} M_w |v.n|, is a block reduction (FP64, fixed
+// order); velocities entering the domain get mu M_w(v) (FP64: times v.n).  For
 // degree 2 the balance at the face's two Gauss points is linear in the
 // outgoing flux, so the mean over the face is balanced once.
 template <typename T>
 __global__ void __launch_bounds__(kFvThreads)
 fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__ fid, const int *__restrict__ wall,
                      const int64_t *__restrict__ wallslot, const T *__restrict__ wallp, int nv, int N, T Lv, T dv) {
+    constexpr bool FLUX = sizeof(T) == 8;
     __shared__ double red[2 * (kFvThreads / 32)];
     const int w = blockIdx.x;
     const int64_t s = wallslot[w];
@@ -1203,7 +1225,7 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
     for (int u = 0; u < 4; ++u) {
         const T d1 = v.v1 - uw1, d2 = v.v2[u] - uw2;
         mw[u] = norm * exp(-(d1 * d1 + d2 * d2) * inv2th);
-        if (act && vn[u] > (T)0) num += (double)(row[u] * vn[u]);
+        if (act && vn[u] > (T)0) num += (double)(FLUX ? row[u] : row[u] * vn[u]);
         if (act && vn[u] < (T)0) den += (double)(mw[u] * -vn[u]);
     }
 #pragma unroll
@@ -1225,35 +1247,37 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
     const T mu = (T)(num / den);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-        if (act && !(vn[u] > (T)0)) row[u] = mu * mw[u];
+        if (act && !(vn[u] > (T)0)) row[u] = FLUX ? vn[u] * (mu * mw[u]) : mu * mw[u];
 }
 
-// Pass 2: L_i = (1/|P_i|) sum over the faces of v.n times their rows, the cells
-// in the reverse of pass 1's order, so that the first ones find the rows written
-// last still in L2.  FP32: DRAM-bound.  FP64: as much by the FP64 pipe; the nodes
-// come from shared memory, formed once per block.
+// Pass 2: L_i = (1/|P_i|) sum over the faces of v.n times their rows (FP64: of the
+// signed rows), the cells in the reverse of pass 1's order, so that the first ones
+// find the rows written last still in L2.  DRAM-bound, and by latency: every
+// table value is asked for before the rows, and 32 registers keep the SMs full
+// (19802 triangles x 32^2, FP32: 51 us; 69 us with the normals loaded where they
+// are used, 56 with 40 registers).
 template <typename T, int VEC, int MAXF, int B>
-__global__ void __launch_bounds__(kFvThreads)
+__global__ void __launch_bounds__(kFvThreads, MAXF == 3 ? 8 : 4)
 fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
-              int64_t rows, int nv, int N, T Lv, T dv) {
+              int64_t rows, int nv, int N, float iN, T Lv, T dv) {
     constexpr bool F64 = sizeof(T) == 8;
-    __shared__ T nodes[F64 ? kFvMaxNodes : 1];
-    if constexpr (F64) {
-        if ((int)threadIdx.x < N) nodes[threadIdx.x] = -Lv + (T)threadIdx.x * dv;
-        __syncthreads();
-    }
     const int64_t p = gridDim.x - 1 - blockIdx.x;
     const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
     if (k >= nv) return;
-    const PairVelocity<T, VEC> v(k, N, [&](int j) {
-        if constexpr (F64) return nodes[j];
-        else return -Lv + (T)j * dv;
-    });
-    const int meta = __ldg(ix.meta + p), nf = meta & 0xf;
+    using V2 = typename C2<T>::type;
+    const V2 *fn = reinterpret_cast<const V2 *>(tb.fn) + p * kFvMaxFaces;
+    // every table value before the wait: they come from DRAM, one latency for all
+    const int meta = __ldg(ix.meta + p), nf = MAXF == 3 ? 3 : meta & 0xf;
     int row[MAXF];
+    V2 n[MAXF];
 #pragma unroll
-    for (int q = 0; q < MAXF; ++q) row[q] = q < nf ? __ldg(ix.fid + p * kFvMaxFaces + q) : 0;
+    for (int q = 0; q < MAXF; ++q) {
+        row[q] = __ldg(ix.fid + p * kFvMaxFaces + q);
+        if constexpr (!F64) n[q] = __ldg(fn + q);
+    }
     const T ia = __ldg(tb.inv_area + p);
+    const int64_t i = __ldg(ix.order + p);
+    auto velocity = [&] { return PairVelocity<T, VEC>(k, N, iN, Lv, dv); };
     griddep_wait();                      // launched while pass 1 ends: its rows from here on
     Vec<T, VEC> x[MAXF];
 #pragma unroll
@@ -1262,49 +1286,58 @@ fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const in
     Vec<T, VEC> o;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] = (T)0;
-    const unsigned two_sided = sizeof(T) == 4 ? (unsigned)meta >> 24 : 0u;
+    if constexpr (F64) {
+        const bool split = meta & kFvSplitFlag;
 #pragma unroll
-    for (int q = 0; q < MAXF; ++q)
-        if (q < nf && !((two_sided >> q) & 1)) {
-            T vn[VEC];
-            v.normal(__ldg(tb.fn + 2 * (p * kFvMaxFaces + q)), __ldg(tb.fn + 2 * (p * kFvMaxFaces + q) + 1), vn);
-#pragma unroll
-            for (int u = 0; u < VEC; ++u) o.v[u] = fma(vn[u], x[q].v[u], o.v[u]);
-        }
-    if (two_sided) {
-        // faces of thin cells: (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2 at every face point
-        constexpr int GP = B == kFvCoef3 ? 2 : 1;
-        constexpr T half = (T)(0.5 / GP);
-        for (int q = 0; q < nf; ++q) {
-            if (!((two_sided >> q) & 1)) continue;
-            const int64_t s = p * kFvMaxFaces + q;
-            T vn[VEC];
-            v.normal(__ldg(tb.fn + 2 * s), __ldg(tb.fn + 2 * s + 1), vn);
-            if (wall && __ldg(wall + s) >= 0) {          // the wall's row
-                const Vec<T, VEC> r = ldv_after<T, VEC>(FX + (int64_t)__ldg(ix.fid + s) * nv + k);
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) o.v[u] = fma(vn[u], r.v[u], o.v[u]);
+        for (int q = 0; q < MAXF; ++q) {
+            if (q >= nf) continue;
+            if (split && (__ldg(ix.two + p * kFvMaxFaces + q) & kFvSplit)) {
+                velocity().add_flux(__ldg(fn + q), x[q], o);
                 continue;
             }
-            const int side = (meta >> (8 + q)) & 1, two = __ldg(ix.two + s);
-            const bool boundary = (meta >> (16 + q)) & 1;
-            for (int g = 0; g < GP; ++g) {
-                const Vec<T, VEC> a = ldv_after<T, VEC>(FX + two_row<B>(rows, two, side, g) * nv + k);
-                // the other side's points run the other way
-                const Vec<T, VEC> b =
-                    boundary ? a : ldv_after<T, VEC>(FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k);
+            const bool other = (meta >> (8 + q)) & 1;
 #pragma unroll
-                for (int u = 0; u < VEC; ++u) {
-                    const T h = half * vn[u], fl = a.v[u], fr = b.v[u];
-                    o.v[u] = fma(h, fl + fr, o.v[u]);
-                    o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
+            for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, x[q].v[u]);
+        }
+    } else {
+        const unsigned two_sided = (unsigned)meta >> 24;
+        const PairVelocity<T, VEC> v = velocity();
+#pragma unroll
+        for (int q = 0; q < MAXF; ++q)
+            if (q < nf && !((two_sided >> q) & 1)) v.add_flux(n[q], x[q], o);
+        if (two_sided) {
+            // faces of thin cells: (v.n)(f_L + f_R)/2 - |v.n| (f_R - f_L)/2 at every face point
+            constexpr int GP = B == kFvCoef3 ? 2 : 1;
+            constexpr T half = (T)(0.5 / GP);
+#pragma unroll 1
+            for (int q = 0; q < nf; ++q) {
+                if (!((two_sided >> q) & 1)) continue;
+                const int64_t s = p * kFvMaxFaces + q;
+                const V2 nq = __ldg(fn + q);
+                if (wall && __ldg(wall + s) >= 0) {          // the wall's row
+                    v.add_flux(nq, ldv_after<T, VEC>(FX + (int64_t)__ldg(ix.fid + s) * nv + k), o);
+                    continue;
+                }
+                const int side = (meta >> (8 + q)) & 1, two = __ldg(ix.two + s) & (kFvSplit - 1);
+                const bool boundary = (meta >> (16 + q)) & 1;
+#pragma unroll 1
+                for (int g = 0; g < GP; ++g) {
+                    const T *a = FX + two_row<B>(rows, two, side, g) * nv + k;
+                    // the other side's points run the other way
+                    const T *b = boundary ? a : FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k;
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) {
+                        const T h = half * fma(v.v2[u], nq.y, v.v1[u / 2] * nq.x), fl = __ldcg(a + u), fr = __ldcg(b + u);
+                        o.v[u] = fma(h, fl + fr, o.v[u]);
+                        o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
+                    }
                 }
             }
         }
     }
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] *= ia;
-    stv<T, VEC>(L + (int64_t)__ldg(ix.order + p) * nv + k, o);
+    stv<T, VEC>(L + i * nv + k, o);
 }
 
 // Pass 2 where every face is two-sided (FP32, degree 2): the Rusanov form at
@@ -1607,9 +1640,9 @@ cudaError_t sum_launch(const bz_mesh *m, const GridView &g, const T *FX, T *L, c
     const int *wall = m->n_walls > 0 ? m->d_wall : nullptr;
     if (m->order == 3)
         return launch_after(fv_sum_kernel<T, VEC, MAXF, kFvCoef3>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m),
-                            indices(m), wall, m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
+                            indices(m), wall, m->n_rows, nv, g.N, 1.f / (float)g.N, (T)g.L, (T)g.dv);
     return launch_after(fv_sum_kernel<T, VEC, MAXF, 2>, grid, kFvThreads, 0, st, true, FX, L, pick<T>(m), indices(m),
-                        wall, m->n_rows, nv, g.N, (T)g.L, (T)g.dv);
+                        wall, m->n_rows, nv, g.N, 1.f / (float)g.N, (T)g.L, (T)g.dv);
 }
 
 // 16-byte rows where L allows (N^2 is a multiple of 4)
