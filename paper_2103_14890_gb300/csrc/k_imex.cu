@@ -128,7 +128,15 @@ __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageC
 //     FP32 full divisions were the larger part of the kernel's FP64 time);
 //   * the Maxwellian of a 2-D grid factorises, M(v1, v2) = pref e1(v1) e2(v2):
 //     each lane forms its row and column offsets v - u in FP64 and the rest of
-//     the exponent and the exponential in the state precision.
+//     the exponent and the exponential in the state precision;
+//   * any other N in FP32: dv is no FP32 number, and nodes rounded to FP32 would
+//     all lean one way (u_1 off by 3e-7 at N = 30, L = 10).  The sums along j1 are
+//     those of R, m R and m^2 R with m = j1 - N/2, whole numbers, each product's
+//     error kept by an FMA; dv enters once per cell in FP64.  The exponent of
+//     every point is the FP64 one rounded once, as an (hi, lo) sum, and M takes one
+//     exponential a point.  A five-stage BGK step, N = 30 on 2500 cells: 151 us
+//     (136 with rounded nodes and two factors, 2037 with the block form below and
+//     FP64 moments, whose errors these are).
 // Mean of a step's stages: FP32 N = 32 on 23160 cells 112 us with full divisions,
 // the error terms in FP64 and 8 cells a CTA, 95.5 us now; FP64 N = 30 on 2603
 // cells 139 -> 124 us (the row nodes from shared memory, not an FP64 fma per
@@ -145,6 +153,18 @@ __device__ __forceinline__ void acc2(T &s, T &e, T x) {
     }
 }
 
+// A number as hi + lo in FP32, and the sum of two such rounded to FP32 (the two
+// halves' sum is exact by TwoSum, so it is the rounded FP64 sum in all but rare
+// cases).
+__device__ __forceinline__ float2 split32(double x) {
+    const float h = (float)x;
+    return make_float2(h, (float)(x - (double)h));
+}
+__device__ __forceinline__ float sum32(float2 a, float2 b) {
+    const float s = a.x + b.x, bb = s - a.x;
+    return s + (((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y));
+}
+
 constexpr int kStageCells = 4;    // cells (warps) per CTA of the 2-D stage kernel
 
 // NMAX rows in registers; FIXED: N = NMAX at compile time, else any N <= NMAX.
@@ -155,6 +175,7 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
                                                                        const T *__restrict__ Lres, int64_t stride,
                                                                        int64_t n) {
     constexpr bool F32 = sizeof(T) == 4;
+    constexpr bool CENTRED = F32 && !FIXED;
     __shared__ double part[kStageCells][4][33];   // per-lane moment partials (pitch 33: no bank conflicts)
     __shared__ T perr[F32 ? kStageCells : 1][F32 ? 4 : 1][33];   // FP32: the partials' error terms
     __shared__ double par[kStageCells][3];        // u1, u2, inv2t
@@ -211,24 +232,29 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
                 v1 = vt[0][j];
                 q1 = vt[1][j];
             } else {
-                v1 = fma((T)j, dv, -L);
+                v1 = CENTRED ? (T)j - (T)(N / 2) : fma((T)j, dv, -L);
                 q1 = v1 * v1;
             }
             acc2(s0, e0, R[j]);
-            acc2(s1, e1, v1 * R[j]);
-            acc2(s3, e3, q1 * R[j]);
+            const T x1 = v1 * R[j], x3 = q1 * R[j];
+            if constexpr (CENTRED) {
+                e1 += fma(v1, R[j], -x1);
+                e3 += fma(q1, R[j], -x3);
+            }
+            acc2(s1, e1, x1);
+            acc2(s3, e3, x3);
         }
         const double vv = vd[lane], S0 = (double)s0;
         part[wib][0][lane] = S0;
         part[wib][1][lane] = (double)s1;
         part[wib][2][lane] = vv * S0;
-        part[wib][3][lane] = fma(vv * vv, S0, (double)s3);
+        part[wib][3][lane] = fma(vv * vv, S0, CENTRED ? g.dv * g.dv * (double)s3 : (double)s3);
         if constexpr (F32) {                 // of relative size 2^-24: their sums in FP32 lose nothing
             const T v = (T)vv;
             perr[wib][0][lane] = e0;
             perr[wib][1][lane] = e1;
             perr[wib][2][lane] = v * e0;
-            perr[wib][3][lane] = fma(v * v, e0, e3);
+            perr[wib][3][lane] = fma(v * v, e0, CENTRED ? dv * dv * e3 : e3);
         }
     }
     __syncthreads();
@@ -254,9 +280,16 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
     if (threadIdx.x < kStageCells) {
         const int cc = threadIdx.x;
         const double w = g.dv * g.dv, coef = c.coef;
-        const double rho = w * part[cc][0][32], yr = rcp64(rho);
-        const double u1 = div64(w * part[cc][1][32], rho, yr), u2 = div64(w * part[cc][2][32], rho, yr);
-        const double E = 0.5 * w * part[cc][3][32];
+        const double S0 = part[cc][0][32];
+        double S1 = part[cc][1][32], S3 = part[cc][3][32];
+        if constexpr (CENTRED) {             // v = c0 + m dv
+            const double c0 = fma((double)(N / 2), g.dv, -g.L), m1 = g.dv * S1;
+            S1 = fma(c0, S0, m1);
+            S3 = fma(c0, fma(c0, S0, 2.0 * m1), S3);
+        }
+        const double rho = w * S0, yr = rcp64(rho);
+        const double u1 = div64(w * S1, rho, yr), u2 = div64(w * part[cc][2][32], rho, yr);
+        const double E = 0.5 * w * S3;
         const double theta = (div64(2.0 * E, rho, yr) - (u1 * u1 + u2 * u2)) * 0.5, yt = rcp64(theta);
         const double cst = coef * rho, c1 = 1.0 + cst;
         par[cc][0] = u1;
@@ -272,28 +305,35 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
     if (!live) return;
     // separable Maxwellian: this lane's column factor and row factor j1 = lane;
     // offsets v - u in FP64, the rest of the exponent and the exp in T
-    // (any other N: the whole exponent in FP64)
+    // (any other N: the whole exponent in FP64; FP32: one exponential a point)
     const double vl = vd[lane];
     const double d2 = vl - par[wib][1], d1 = vl - par[wib][0];
-    T x1, x2;
+    T fcol = (T)0, frow_l = (T)0;
+    float2 xcol = make_float2(0.f, 0.f), xrow = xcol;
     if constexpr (FIXED) {
         const T i2t = parT[wib][1], t1 = (T)d1, t2 = (T)d2;
-        x1 = -t1 * t1 * i2t;
-        x2 = -t2 * t2 * i2t;
+        fcol = parT[wib][2] * exp(-t2 * t2 * i2t);
+        frow_l = exp(-t1 * t1 * i2t);
+    } else if constexpr (F32) {
+        xcol = split32(-d2 * d2 * par[wib][2]);
+        xrow = split32(-d1 * d1 * par[wib][2]);
     } else {
-        x1 = (T)(-d1 * d1 * par[wib][2]);
-        x2 = (T)(-d2 * d2 * par[wib][2]);
+        fcol = parT[wib][2] * exp(-d2 * d2 * par[wib][2]);
+        frow_l = exp(-d1 * d1 * par[wib][2]);
     }
-    const T fcol = parT[wib][2] * exp(x2);
-    const T frow_l = exp(x1);
     const T cT = parT[wib][3], denom = parT[wib][4], nuT = parT[wib][0];
     T *Fo = F + base;
     T *Po = P + (int64_t)c.stage * stride + base;
 #pragma unroll
     for (int j = 0; j < NMAX; ++j) {
         if (!FIXED && j >= N) break;
-        const T frow = __shfl_sync(0xffffffffu, frow_l, j);
-        const T Mx = fcol * frow;
+        T Mx;
+        if constexpr (CENTRED) {
+            const float2 xr = make_float2(__shfl_sync(0xffffffffu, xrow.x, j), __shfl_sync(0xffffffffu, xrow.y, j));
+            Mx = parT[wib][2] * exp(sum32(xcol, xr));
+        } else {
+            Mx = fcol * __shfl_sync(0xffffffffu, frow_l, j);
+        }
         const T Fi = (R[j] + cT * Mx) * denom;
         if (on) {
             if (c.store_F) Fo[j * N] = Fi;
