@@ -10,6 +10,8 @@
 //   factor for the Boltzmann model)
 // G_l = Q(F_l) - P_l is formed by the inverse-DFT epilogue of the collision
 // chain that follows this kernel.
+#include <type_traits>
+
 #include "bz_device.cuh"
 #include "bz_internal.h"
 
@@ -40,9 +42,27 @@ __device__ __forceinline__ T stage_rhs(const StageCoef &c, T r, const T *__restr
     return r;
 }
 
+// A number as hi + lo in FP32, and the sum of two such (the high parts' sum exact
+// by TwoSum).  round32: such a sum as one FP32 number, the rounded FP64 sum in
+// all but rare cases.
+__device__ __forceinline__ float2 split32(double x) {
+    const float h = (float)x;
+    return make_float2(h, (float)(x - (double)h));
+}
+__device__ __forceinline__ float2 add32(float2 a, float2 b) {
+    const float s = a.x + b.x, bb = s - a.x;
+    return make_float2(s, ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y));
+}
+__device__ __forceinline__ float round32(float2 a) { return a.x + a.y; }
+
 // Any grid (3-D, and 2-D with N > 32): one CTA per cell.  The Maxwellian is
-// the product of one factor per axis, each axis' N factors formed once per
-// cell (the exponent in FP64, the exponential in the state precision); 2-D, N = 40, FP64 on 2000 cells: 559 -> 347 us.
+// formed from one table entry per axis, each axis' N entries formed once per
+// cell.  FP64: its factors, pref on the first axis; 2-D, N = 40 on 2000 cells:
+// 559 -> 347 us.  FP32: their exponents as (hi, lo), so that a point's exponent is
+// the FP64 one rounded once and M takes one exponential (two or three factors
+// would round once more each, 0.87e-7 of F's norm for 0.74e-7 at N = 40, 1.03e-7
+// for 0.77e-7 in 3-D at N = 16).  A five-stage BGK step on 1406 cells of 40^2 takes
+// 953 us (943 with factors, 1428 with FP64 exponents point by point).
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageCoef c, const T *__restrict__ fn,
                                                               T *__restrict__ F, const T *__restrict__ G,
@@ -51,8 +71,9 @@ __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageC
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *red = reinterpret_cast<double *>(smem_raw);         // 32 * 5
     double *vt = red + 32 * 5;                                   // [N] nodes
-    T *fac = reinterpret_cast<T *>(vt + g.N);                    // [3][N] factors of the Maxwellian
-    T *R = fac + 3 * g.N;                                        // nv
+    using Entry = typename std::conditional<sizeof(T) == 8, double, float2>::type;
+    Entry *fac = reinterpret_cast<Entry *>(vt + g.N);            // [3][N] factors of the Maxwellian, or their exponents
+    T *R = reinterpret_cast<T *>(fac + 3 * g.N);                 // nv
     const unsigned N = g.N, nv = (unsigned)g.nv;
     const int64_t base = (int64_t)blockIdx.x * g.nv;
     const T dt = (T)c.dt, ieps = (T)(1.0 / c.eps);
@@ -94,19 +115,24 @@ __global__ void __launch_bounds__(kThreads) imex_stage_kernel(GridView g, StageC
     for (unsigned j = threadIdx.x; j < DIM * N; j += blockDim.x) {
         const int d = (int)(j / N);
         const double o = vt[j % N] - (d == 0 ? u[0] : d == 1 ? u[1] : u[2]);
-        fac[j] = (d == 0 ? (T)pref : (T)1) * exp((T)(-o * o * i2t));
+        if constexpr (sizeof(T) == 8) fac[j] = (d == 0 ? pref : 1.0) * exp(-o * o * i2t);
+        else fac[j] = split32(-o * o * i2t);
     }
     __syncthreads();
     T *Fo = F + base;
     T *Po = P + (int64_t)c.stage * stride + base;
     for (unsigned i = threadIdx.x; i < nv; i += blockDim.x) {
-        T Mx = (T)1;
         unsigned q = i;
+        Entry x = fac[(DIM - 1) * N + q % N];
 #pragma unroll
-        for (int d = DIM - 1; d >= 0; --d) {
-            Mx *= fac[d * N + q % N];
+        for (int d = DIM - 2; d >= 0; --d) {
             q /= N;
+            if constexpr (sizeof(T) == 8) x *= fac[d * N + q % N];
+            else x = add32(x, fac[d * N + q % N]);
         }
+        T Mx;
+        if constexpr (sizeof(T) == 8) Mx = x;
+        else Mx = (T)pref * exp(round32(x));
         const T Fi = (R[i] + cT * Mx) * denom;
         if (c.store_F) Fo[i] = Fi;
         if (c.store_P) Po[i] = nuT * (Mx - Fi);
@@ -151,18 +177,6 @@ __device__ __forceinline__ void acc2(T &s, T &e, T x) {
     } else {
         s += x;
     }
-}
-
-// A number as hi + lo in FP32, and the sum of two such rounded to FP32 (the two
-// halves' sum is exact by TwoSum, so it is the rounded FP64 sum in all but rare
-// cases).
-__device__ __forceinline__ float2 split32(double x) {
-    const float h = (float)x;
-    return make_float2(h, (float)(x - (double)h));
-}
-__device__ __forceinline__ float sum32(float2 a, float2 b) {
-    const float s = a.x + b.x, bb = s - a.x;
-    return s + (((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y));
 }
 
 constexpr int kStageCells = 4;    // cells (warps) per CTA of the 2-D stage kernel
@@ -330,7 +344,7 @@ __global__ void __launch_bounds__(kStageCells * 32) imex_stage2d_kernel(GridView
         T Mx;
         if constexpr (CENTRED) {
             const float2 xr = make_float2(__shfl_sync(0xffffffffu, xrow.x, j), __shfl_sync(0xffffffffu, xrow.y, j));
-            Mx = parT[wib][2] * exp(sum32(xcol, xr));
+            Mx = parT[wib][2] * exp(round32(add32(xcol, xr)));
         } else {
             Mx = fcol * __shfl_sync(0xffffffffu, frow_l, j);
         }
@@ -364,7 +378,7 @@ cudaError_t stage(const GridView &g, const StageCoef &c, const T *fn, T *F, cons
         else imex_stage2d_kernel<T, 32, false><<<blocks, thr, 0, st>>>(g, c, fn, F, G, P, Lres, stride, n);
         return cudaGetLastError();
     }
-    const size_t sm = sizeof(double) * (32 * 5 + g.N) + sizeof(T) * ((size_t)g.nv + 3 * g.N);
+    const size_t sm = sizeof(double) * (32 * 5 + 4 * g.N) + sizeof(T) * (size_t)g.nv;
     auto *kern = g.dim == 2 ? imex_stage_kernel<T, 2> : imex_stage_kernel<T, 3>;
     cudaError_t e = allow_dynamic_smem((const void *)kern, sm);
     if (e != cudaSuccess) return e;

@@ -21,7 +21,8 @@ def bz():
 
 
 @pytest.mark.parametrize("dim,N,L,n", [(2, 12, 5.0, 2000), (2, 20, 8.0, 2000), (2, 28, 10.0, 2000), (2, 30, 10.0, 2000),
-                                       (2, 30, 8.0, 2000)])
+                                       (2, 30, 8.0, 2000), (2, 40, 10.0, 500), (2, 34, 8.0, 500), (3, 10, 6.0, 500),
+                                       (3, 16, 8.0, 100)])
 def test_fluid_limit_stage_fp32(bz, dim, N, L, n):
     f = workloads.bi_maxwellian(n, dim, N, L, seed=N)
     fin = as_input(f, "fp32")
