@@ -28,9 +28,11 @@ template <typename V> __device__ __forceinline__ void cmac(V &acc, V a, V b) {
 // FP64 quotients that spare the FP64 pipe, on which a warp instruction takes 16
 // cycles of an SM.  rcp64: the hardware's approximate reciprocal y of b (relative
 // error e below 2^-17) and one step of the cubic iteration y (1 + e + e^2), e = 1 -
-// b y: three operations, error below 2^-51 plus a rounding.  div64: a / b from y =
-// rcp64(b) with the remainder's correction (Markstein), three more, within half
-// an ulp in all but rare cases.  The full division takes about three times as many.
+// b y (Householder's method of order 2): three operations, relative error below
+// 2^-51 plus a rounding, for 2^-1021 < |b| < 2^1021 (measured: 1 ulp).  div64: a / b from y =
+// rcp64(b) with the remainder's correction (Markstein 1990), three more, within
+// half an ulp in all but rare cases, one ulp in those (none in 2^20).  The full
+// division takes about three times as many.
 __device__ __forceinline__ double rcp64(double b) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
@@ -41,6 +43,13 @@ __device__ __forceinline__ double rcp64(double b) {
 __device__ __forceinline__ double div64(double a, double b, double y) {
     const double q = a * y;
     return fma(fma(-b, q, a), y, q);
+}
+
+// 2^e / b for a finite b >= 2^e, e given as scale = e << 20: rcp64 of b with the
+// power of two taken off its exponent, off the FP64 pipe (below 2^-1022: that).
+__device__ __forceinline__ double scaled_rcp(double b, int scale) {
+    const unsigned hi = min((unsigned)(__double2hiint(b) - scale), 0x7fd00000u);
+    return rcp64(__hiloint2double((int)hi, __double2loint(b)));
 }
 
 // Tiled half-spectrum layout: [cell / 32][mode][cell % 32].

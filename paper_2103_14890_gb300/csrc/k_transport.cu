@@ -158,18 +158,6 @@ struct FvIdx {
     const int *order, *meta, *fid, *two, *ncen, *cen, *nsec, *sec;
 };
 
-// 2^e / b for b > 0, e given as scale = e << 20: rcp64 with the power of two
-// added to the exponent of the first approximation, off the FP64 pipe.  The
-// result lies below 2^1022; below the normal range it is flushed to (nearly) 0.
-__device__ __forceinline__ double scaled_rcp(double b, int scale) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    double e = fma(-b, y, 1.0);
-    e = fma(e, e, e);
-    y = __hiloint2double(max(__double2hiint(y) + scale, 0), __double2loint(y));
-    return fma(y, e, y);
-}
-
 // Signs and comparisons of finite FP64 values as integers, off the FP64 pipe.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.f; }
