@@ -763,7 +763,7 @@ __device__ __forceinline__ void faces_block(const T *__restrict__ f, T *__restri
                                             const FvIdx &ix, int64_t rows, int nv, int N, T Lv, T dv) {
     griddep_launch();
     const int64_t p = blockIdx.x;
-    const int k = (blockIdx.y * kFvThreads + threadIdx.x) * VEC;
+    const int k = (blockIdx.y * blockDim.x + threadIdx.x) * VEC;
     if (k >= nv) return;
     const int ncf = __ldg(ix.ncen + p), meta = __ldg(ix.meta + p);
     const Vec<T, VEC> fi = ldv<T, VEC>(f + (int64_t)__ldg(ix.order + p) * nv + k);
@@ -790,6 +790,17 @@ __global__ void __launch_bounds__(kFvThreads)
 fv_faces_kernel(const T *__restrict__ f, T *__restrict__ FX, FvTables<T> tb, FvIdx ix, int64_t rows, int nv, int N, T Lv,
                 T dv) {
     faces_block<T, VEC, MAXF, B, K, TWO>(f, FX, tb, ix, rows, nv, N, Lv, dv);
+}
+
+// Degree 2 on FP32 triangles with 4 | N, a block per cell (see faces3_launch).
+// Bound by latency: four blocks of 256 threads per SM (64 registers, 36 bytes
+// spilled) before three without spills, 16.5 and 18.5 us of a transport call on
+// 409 cells x 32^2.
+template <int BT, bool TWO>
+__global__ void __launch_bounds__(BT, 4 * kFvThreads / BT)
+fv_faces3_cell_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix, int64_t rows,
+                      int nv, int N, float Lv, float dv) {
+    faces_block<float, 4, 3, kFvCoef3, kFvCentral3, TWO>(f, FX, tb, ix, rows, nv, N, Lv, dv);
 }
 
 // Degree 1 on FP32 triangles without walls: the same two passes with a cell's
@@ -829,15 +840,13 @@ constexpr size_t face_stage_bytes(int threads) {
     return 2 * kFaceRows * threads * sizeof(float4) + 2 * threads * sizeof(float);
 }
 
-// Degree 2 on FP32 triangles with 4 | N: pass 1 persistent in the same way, with
-// the 12 rows of a stencil, the cell's table values and its indices staged, the
-// indices one cell further ahead, per warp.  The rows have one buffer: the next
-// cell's are asked for as soon as the differences have been formed, and arrive
-// while this one's weights and faces are computed.  CPS: blocks per SM for 256
-// threads (58 KB each), as many threads with narrower ones.  Two have 128
-// registers a thread; three spill 36 bytes, but a small mesh takes fewer rounds
-// (faces3_per_sm), and narrower blocks gain by the warps (24^2 on 19802 cells
-// 165 -> 158 us, on 472 cells 19.0 -> 16.5).
+// Degree 2 on FP32 triangles, the staged form for large meshes (see
+// faces3_launch): pass 1 persistent in the same way, with the 12 rows of a
+// stencil, the cell's table values and its indices staged, the indices one cell
+// further ahead, per warp.  The rows have one buffer: the next cell's are asked
+// for as soon as the differences have been formed, and arrive while this one's
+// weights and faces are computed.  Blocks per SM: two of 256 threads (58 KB each,
+// 128 registers a thread), as many warps as three such with narrower ones.
 constexpr int kRows3 = 1 + kFvCentral3;
 constexpr int kTab3Rs = 0, kTab3Quad = 12, kTab3Rc = 16, kTab3Phi = 71, kTab3Fs = 86, kTab3Values = 92;
 constexpr int kIdx3Cen = 0, kIdx3Fid = 11, kIdx3Order = 14, kIdx3Meta = 15, kIdx3Ncen = 16, kIdx3Values = 17;
@@ -847,8 +856,9 @@ constexpr size_t faces3_stage_bytes(int threads) {
            threads / 32 * (2 * kTab3Pitch * sizeof(float) + 3 * kIdx3Pitch * sizeof(int));
 }
 
-template <int BT, bool TWO, int CPS>
-__global__ void __launch_bounds__(BT, CPS * kFvThreads / BT)
+constexpr int faces3_ctas_per_sm(int threads) { return threads < kFvThreads ? 3 : 2; }
+template <int BT, bool TWO>
+__global__ void __launch_bounds__(BT, faces3_ctas_per_sm(BT) * kFvThreads / BT)
 fv_faces3_persist_kernel(const float *__restrict__ f, float *__restrict__ FX, FvTables<float> tb, FvIdx ix,
                          int64_t rows, int64_t n, int nv, int N, float Lv, float dv) {
     constexpr int B = kFvCoef3, K = kFvCentral3, W = BT / 32;
@@ -1548,30 +1558,40 @@ void values_launch(const bz_mesh *m, const GridView &g, const float *f, float *F
     fv_values_persist_kernel<BT><<<values_grid(m, nv, kFacesCtasPerSm), BT, face_stage_bytes(BT), st>>>(
         f, FV, m->t32, indices(m), m->d_tripos, m->n_cells, nv);
 }
-template <int BT, bool TWO, int CPS>
+// Degree 2 on FP32 triangles: a block per cell, or the staged form.  Blocks per
+// cell are placed as SMs fall free and leave no lanes of a row idle beyond a block;
+// the staged form hides the latency of large meshes better where a row fills one
+// block.  Transport with blocks per cell and staged, us: 32^2 on 472, 2512, 7074,
+// 19802 cells 17.8 and 22.0, 38.3 and 40.8, 98.7 and 96.8, 253.7 and 242.7; 24^2
+// on 472, 5300, 12643, 19802 cells 15.1 and 16.5, 44.9 and 48.9, 107.7 and 106.1,
+// 163.5 and 160.3; on 19802 cells 16^2 74.2 and 76.8, 20^2 127.2 and 134.3, 28^2
+// 232.0 and 232.1; 36^2 on 12643 cells 228 and 293, 64^2 on 5300 cells 253 and 269.
+bool faces3_staged(const bz_mesh *m, int nv) {
+    const int bt = values_threads(nv);
+    return m->n_cells >= (int64_t)45 * fv_sm_count() && bt >= 160 && nv <= 4 * bt && 10 * nv >= 9 * 4 * bt;
+}
+template <int BT, bool TWO>
 void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     const int nv = (int)g.nv;
-    fv_faces3_persist_kernel<BT, TWO, CPS><<<values_grid(m, nv, CPS), BT, faces3_stage_bytes(BT), st>>>(
-        f, FX, m->t32, indices(m), TWO ? 0 : m->n_rows, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
-}
-// Blocks of 256 threads per SM: three where that saves rounds on a small mesh (a
-// round of three takes about 1.48 rounds of two, and a full one more).  Transport
-// of 32^2 with two and three: 312 cells 20.3 and 17.3 us, 472 cells 21.7 and
-// 22.9, 756 cells 22.9 and 21.4, 1105 cells 25.0 and 26.9, 19802 cells 237 and
-// 240.
-int faces3_per_sm(const bz_mesh *m) {
-    const int64_t n = m->n_cells, sms = fv_sm_count(), two = (n + 2 * sms - 1) / (2 * sms), three = (n + 3 * sms - 1) / (3 * sms);
-    return n <= 20 * sms && 1.48 * three < two && n <= 0.95 * (3 * sms * three) ? 3 : 2;
+    const int64_t rows = TWO ? 0 : m->n_rows;
+    if constexpr (BT >= 160) {
+        if (faces3_staged(m, nv)) {
+            fv_faces3_persist_kernel<BT, TWO><<<values_grid(m, nv, faces3_ctas_per_sm(BT)), BT, faces3_stage_bytes(BT), st>>>(
+                f, FX, m->t32, indices(m), rows, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+            return;
+        }
+    }
+    fv_faces3_cell_kernel<BT, TWO><<<dim3((unsigned)m->n_cells, (unsigned)((nv / 4 + BT - 1) / BT)), BT, 0, st>>>(
+        f, FX, m->t32, indices(m), rows, nv, g.N, (float)g.L, (float)g.dv);
 }
 template <bool TWO>
 void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     switch (values_threads((int)g.nv)) {
-        case 64: return faces3_launch<64, TWO, 3>(m, g, f, FX, st);
-        case 128: return faces3_launch<128, TWO, 3>(m, g, f, FX, st);
-        case 160: return faces3_launch<160, TWO, 3>(m, g, f, FX, st);
+        case 64: return faces3_launch<64, TWO>(m, g, f, FX, st);
+        case 128: return faces3_launch<128, TWO>(m, g, f, FX, st);
+        case 160: return faces3_launch<160, TWO>(m, g, f, FX, st);
     }
-    if (faces3_per_sm(m) == 3) return faces3_launch<kFvThreads, TWO, 3>(m, g, f, FX, st);
-    faces3_launch<kFvThreads, TWO, 2>(m, g, f, FX, st);
+    faces3_launch<kFvThreads, TWO>(m, g, f, FX, st);
 }
 // The flux pass starts while the reconstruction's last blocks end (on 760 to
 // 19802 triangles x 32^2 it saves 2 to 3 us), except on meshes so small that the
@@ -1702,10 +1722,8 @@ cudaError_t fv_values_setup() {
     const std::pair<const void *, size_t> big[] = {
         {(const void *)fv_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
         {(const void *)fv_flux_values_persist_kernel<kFvThreads>, face_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, false, 2>, faces3_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, false, 3>, faces3_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, true, 2>, faces3_stage_bytes(kFvThreads)},
-        {(const void *)fv_faces3_persist_kernel<kFvThreads, true, 3>, faces3_stage_bytes(kFvThreads)}};
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, false>, faces3_stage_bytes(kFvThreads)},
+        {(const void *)fv_faces3_persist_kernel<kFvThreads, true>, faces3_stage_bytes(kFvThreads)}};
     cudaError_t e = cudaSuccess;
     for (const auto &[kernel, bytes] : big)
         if (e == cudaSuccess) e = allow_dynamic_smem(kernel, bytes);
