@@ -1698,24 +1698,25 @@ cudaError_t first(const bz_mesh *m, const GridView &g, const T *f, T *L, cudaStr
 cudaError_t launch_fv_faces_two_f32(const bz_mesh *m, const GridView &g, const float *f, float *FX, cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
     const int nv = (int)g.nv;
-    if (m->max_faces <= 3 && g.N % 4 == 0 && aligned(f, 16))
-        faces3_launch<true>(m, g, f, FX, st);
-    else if (m->max_faces <= 3)
-        fv_faces_kernel<float, 1, 3, kFvCoef3, kFvCentral3, true><<<cell_grid(m, nv, 1), kFvThreads, 0, st>>>(
-            f, FX, m->t32, indices(m), 0, nv, g.N, (float)g.L, (float)g.dv);
-    else
-        fv_faces_kernel<float, 1, kFvMaxFaces, kFvCoef3, kFvCentral3, true><<<cell_grid(m, nv, 1), kFvThreads, 0, st>>>(
-            f, FX, m->t32, indices(m), 0, nv, g.N, (float)g.L, (float)g.dv);
+    auto launch = [&](auto kernel, int vec) {
+        kernel<<<cell_grid(m, nv, vec), kFvThreads, 0, st>>>(f, FX, m->t32, indices(m), 0, nv, g.N, (float)g.L, (float)g.dv);
+    };
+    const bool tri = m->max_faces <= 3;
+    if (tri && g.N % 4 == 0 && aligned(f, 16)) faces3_launch<true>(m, g, f, FX, st);
+    else if (tri) launch(fv_faces_kernel<float, 1, 3, kFvCoef3, kFvCentral3, true>, 1);
+    else if (aligned(f, 8)) launch(fv_faces_kernel<float, 2, kFvMaxFaces, kFvCoef3, kFvCentral3, true>, 2);
+    else launch(fv_faces_kernel<float, 1, kFvMaxFaces, kFvCoef3, kFvCentral3, true>, 1);
     return cudaGetLastError();
 }
 cudaError_t launch_fv_sum_two_f32(const bz_mesh *m, const GridView &g, const float *FX, float *L, cudaStream_t st) {
     if (m->n_cells <= 0) return cudaSuccess;
     const int nv = (int)g.nv;
-    if (m->max_faces <= 3 && g.N % 4 == 0 && aligned(L, 16))
-        return launch_after(fv_sum_two_kernel<4, 3>, cell_grid(m, nv, 4), kFvThreads, 0, st, true, FX, L, m->t32, indices(m),
-                            nv, g.N, (float)g.L, (float)g.dv);
-    return launch_after(fv_sum_two_kernel<1, kFvMaxFaces>, cell_grid(m, nv, 1), kFvThreads, 0, st, true, FX, L, m->t32,
-                        indices(m), nv, g.N, (float)g.L, (float)g.dv);
+    auto launch = [&](auto kernel, int vec) {
+        return launch_after(kernel, cell_grid(m, nv, vec), kFvThreads, 0, st, true, FX, L, m->t32, indices(m), nv, g.N,
+                            (float)g.L, (float)g.dv);
+    };
+    if (g.N % 4 || !aligned(L, 16)) return launch(fv_sum_two_kernel<1, kFvMaxFaces>, 1);
+    return m->max_faces <= 3 ? launch(fv_sum_two_kernel<4, 3>, 4) : launch(fv_sum_two_kernel<4, kFvMaxFaces>, 4);
 }
 
 cudaError_t fv_values_setup() {
