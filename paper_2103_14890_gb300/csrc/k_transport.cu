@@ -1594,15 +1594,16 @@ void faces3_launch(const bz_mesh *m, const GridView &g, const float *f, float *F
     faces3_launch<kFvThreads, TWO>(m, g, f, FX, st);
 }
 // The flux pass starts while the reconstruction's last blocks end (on 760 to
-// 19802 triangles x 32^2 it saves 2 to 3 us), except on meshes so small that the
-// host's part of a launch is the bound (the attribute takes it 1 us) and with
-// narrow blocks: beside those of the reconstruction they would be placed
-// unevenly (19802 triangles x 16^2: 45 us, 50 with it).
+// 19802 triangles x 32^2 it saves 2 to 3 us), except with narrow blocks on larger
+// meshes: beside those of the reconstruction they would be placed unevenly.  With
+// and without, us: 24^2 on 1105, 1298 cells 12.9 and 15.3, 14.5 and 16.3; 20^2 on
+// 1506, 2821, 3957, 7074 cells 14.3 and 15.8, 20.6 and 20.6, 25.1 and 22.7, 38.6 and
+// 33.6; 16^2 on 3957, 19802 cells 14.8 and 16.4, 50.3 and 45.3.
 template <int BT>
 cudaError_t flux_values_launch(const bz_mesh *m, const GridView &g, const float *FV, float *L, cudaStream_t st) {
     const int nv = (int)g.nv;
     return launch_after(fv_flux_values_persist_kernel<BT>, values_grid(m, nv, kFluxCtasPerSm), BT, face_stage_bytes(BT), st,
-                        BT == kFvThreads && m->n_cells * nv >= (1 << 19), FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
+                        BT == kFvThreads || m->n_cells * nv <= (5 << 18), FV, L, m->t32, m->d_tripos, m->n_cells, nv, g.N, (float)g.L, (float)g.dv);
 }
 
 // FP64 takes one velocity per thread (the FP64 pipe is the bound, so loads per
