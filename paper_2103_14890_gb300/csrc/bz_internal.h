@@ -175,8 +175,8 @@ struct bz_mesh {
     int *d_fid;             // [p][face] face index, numbered in the processing order of the owners
     int *d_two;             // [p][face] index of a two-sided face, | kFvSplit
     int64_t n_two;
-    int *d_ncen;            // [p] central stencil size (<= K), | kFvRegular for a triangle whose stencil
-                            // starts with its face neighbours, sector s on faces s, s+1
+    int *d_ncen;            // [p] central stencil size (<= K), | kFvRegular (any polygon): the stencil starts with
+                            // the face neighbours in face order, sector s on faces s, s + 1
     int *d_cen;             // [p][K]
     int *d_nsec;            // [p] sectors
     int *d_sec;             // [p][face][2] sector cells
@@ -259,7 +259,7 @@ struct Mode32Item {
 };
 struct Mode32Group {
     int nitems;
-    int64_t tile_start[kMaxGroup + 1];   // prefix sums of 32-cell tiles
+    int64_t tile_start[kMaxGroup + 1];   // prefix sums of CTAs (tiles of 8 to 32 cells, times the split)
     Mode32Item item[kMaxGroup];
 };
 bool modesum32_available(const bz_modes *m);
@@ -276,8 +276,6 @@ bool modesum32_tail_splits(const bz_modes *m);
 bool modesum32_small_batches_fast(const bz_modes *m);
 bool modesum64_available(const bz_modes *m);
 cudaError_t launch_modesum64(const bz_modes *m, const double2 *fhat, double2 *Qhat, int64_t n, cudaStream_t st);
-cudaError_t launch_modesum32_part(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
-                                  cudaStream_t st);
 // FP32X2 (double-float) mode sum on the FP64 tables: FP64 spectra in, Q-hat
 // rounded to FP32 out (k_modesum32.cu).
 bool modesum_x2_available(const bz_modes *m);

@@ -1567,12 +1567,12 @@ static cudaError_t add_items(Mode32Group &gd, const bz_modes *m, int v, const vo
 }
 
 static cudaError_t launch_variant(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
-                                  cudaStream_t st, int S = 1) {
+                                  cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     Mode32Group gd;
     memset(&gd, 0, sizeof gd);
     const cudaError_t e = add_items(gd, m, v, m->var_W[v], m->var_task[v], m->var_rowmax[v], fhat, sizeof(float2), Qhat,
-                                    sizeof(float2), n, {S > 1 ? 0 : ctas_for(v, n), S});
+                                    sizeof(float2), n, {ctas_for(v, n), 1});
     if (e != cudaSuccess) return e;
     return launch_group(gd, v, smem_bytes<float>(m->g->v, m->var_rowmax[v], v), st);
 }
@@ -1722,11 +1722,6 @@ cudaError_t launch_modesum32(const bz_modes *m, const float2 *fhat, float2 *Qhat
                   n, tail);
     if (e != cudaSuccess) return e;
     return launch_group(gd, sv, sm, st);
-}
-
-cudaError_t launch_modesum32_part(const bz_modes *m, int v, const float2 *fhat, float2 *Qhat, int64_t n,
-                                  cudaStream_t st) {
-    return launch_variant(m, v, fhat, Qhat, n, st);
 }
 
 // Heterogeneous instances in one launch; all items must use the same kernel
