@@ -361,6 +361,13 @@ int fv_mesh_set_walls(bz_mesh *mesh, int64_t n_edges, const int64_t *edge_vertic
  * (bz_mesh_info out[1] + out[2]) N^2, and in FP32 up to four more per face of
  * a thin cell; 3 n_cells N^2 values for order 2 in FP32 on triangle meshes)
  * comes from the stream-ordered pool.
+ * A NaN or infinity in f stays at its velocity: it makes L non-finite there in
+ * the cells whose reconstruction reads that value and in the cells downwind of
+ * those across a face.  Upwind ones may stay finite, as the flux takes the state
+ * that it leaves alone; order 1, FP32 order 2 on triangle meshes and the faces of
+ * thin cells in FP32 take both sides' states (steps of order 3 in FP32 on a mesh
+ * with thin cells: at every face) and spread it both ways.  At a wall it spreads
+ * over all velocities that enter there.
  * Errors: BZ_EINVAL, BZ_ENOTSUP (3-D grid; walls with N not divisible by 4 or
  * N^2 > 1024), BZ_ECUDA. */
 int transport_residual(const bz_mesh *mesh, const bz_grid *g, int precision, const void *f, void *L,

@@ -83,3 +83,26 @@ def test_linear_data_on_unusual_polygons(bz, kind, precision, N, order):
     bound = 64 * u * scale[:, None] * 1.25 * Lv * 2.0 * (1.0 + 2.0 * 16.0) * np.abs(f).max()
     err = np.abs(got - want)
     assert (err <= bound).all(), float((err / bound).max())
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("order", [1, 2, 3])
+@pytest.mark.parametrize("precision,N", [("fp32", 8), ("fp32", 6), ("fp64", 6)])
+def test_non_finite_values_stay_local(bz, precision, N, order, value):
+    """A NaN or infinity at one velocity of one cell: L is not finite there, other velocities and cells two stencils
+    away keep their bits."""
+    import torch
+    pts, quads = _lattice(12)
+    mesh, grid = bz.Mesh(pts, quads.tolist(), order=order), bz.Grid(2, N, 6.0)
+    f = to_dev(np.random.default_rng(6).uniform(1.0, 2.0, (len(quads), N * N)), precision)
+    want = bz.transport_residual(mesh, grid, f, precision=precision)
+    c, k = 6 * 12 + 6, N + 3
+    f[c, k] = value
+    got = bz.transport_residual(mesh, grid, f, precision=precision)
+    bz.check()
+    assert not torch.isfinite(got[c, k])
+    other = torch.arange(N * N, device="cuda") != k
+    assert torch.equal(got[:, other], want[:, other])
+    i = torch.arange(len(quads), device="cuda")
+    far = ((i // 12 - 6).abs() > 5) | ((i % 12 - 6).abs() > 5)
+    assert far.any() and torch.equal(got[far], want[far])
