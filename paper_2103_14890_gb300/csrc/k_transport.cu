@@ -1251,9 +1251,10 @@ fv_wall_faces_kernel(T *__restrict__ FX, FvTables<T> tb, const int *__restrict__
 // Pass 2: L_i = (1/|P_i|) sum over the faces of v.n times their rows (FP64: of the
 // signed rows), the cells in the reverse of pass 1's order, so that the first ones
 // find the rows written last still in L2.  DRAM-bound, and by latency: every
-// table value is asked for before the rows, and 32 registers keep the SMs full
-// (19802 triangles x 32^2, FP32: 51 us; 69 us with the normals loaded where they
-// are used, 56 with 40 registers).
+// table value is asked for before the rows, and 32 registers keep the SMs full, so
+// the thin cells' branch forms its velocities anew (19802 triangles x 32^2, FP32:
+// 49.5 us; 69 us with the normals loaded where they are used, 56 with 40
+// registers, 53 with the velocities kept, which spills).
 template <typename T, int VEC, int MAXF, int B>
 __global__ void __launch_bounds__(kFvThreads, MAXF == 3 ? 8 : 4)
 fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const int *__restrict__ wall,
@@ -1325,7 +1326,8 @@ fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const in
                     const T *b = boundary ? a : FX + two_row<B>(rows, two, 1 - side, GP - 1 - g) * nv + k;
 #pragma unroll
                     for (int u = 0; u < VEC; ++u) {
-                        const T h = half * fma(v.v2[u], nq.y, v.v1[u / 2] * nq.x), fl = __ldcg(a + u), fr = __ldcg(b + u);
+                        const PairVelocity<T, 1> w(k + u, N, iN, Lv, dv);
+                        const T h = half * fma(w.v2[0], nq.y, w.v1[0] * nq.x), fl = __ldcg(a + u), fr = __ldcg(b + u);
                         o.v[u] = fma(h, fl + fr, o.v[u]);
                         o.v[u] = fma(-fabs(h), fr - fl, o.v[u]);
                     }
