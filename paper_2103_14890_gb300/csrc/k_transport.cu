@@ -1286,17 +1286,28 @@ fv_sum_kernel(const T *FX, T *__restrict__ L, FvTables<T> tb, FvIdx ix, const in
 #pragma unroll
     for (int u = 0; u < VEC; ++u) o.v[u] = (T)0;
     if constexpr (F64) {
-        const bool split = meta & kFvSplitFlag;
+        if (!(meta & kFvSplitFlag)) {
 #pragma unroll
-        for (int q = 0; q < MAXF; ++q) {
-            if (q >= nf) continue;
-            if (split && (__ldg(ix.two + p * kFvMaxFaces + q) & kFvSplit)) {
-                velocity().add_flux(__ldg(fn + q), x[q], o);
-                continue;
+            for (int q = 0; q < MAXF; ++q) {
+                if (q >= nf) continue;
+                const bool other = (meta >> (8 + q)) & 1;
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, x[q].v[u]);
             }
-            const bool other = (meta >> (8 + q)) & 1;
+        } else {
+            const PairVelocity<T, VEC> v = velocity();
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, x[q].v[u]);
+            for (int q = 0; q < MAXF; ++q) {
+                if (q >= nf) continue;
+                const Vec<T, VEC> &y = x[q];
+                if (__ldg(ix.two + p * kFvMaxFaces + q) & kFvSplit) {
+                    v.add_flux(__ldg(fn + q), y, o);
+                } else {
+                    const bool other = (meta >> (8 + q)) & 1;
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) o.v[u] += negate_if(other, y.v[u]);
+                }
+            }
         }
     } else {
         const unsigned two_sided = (unsigned)meta >> 24;
