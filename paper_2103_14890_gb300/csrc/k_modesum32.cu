@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(WARPS * 32, RR == 2 ? 2 : WARPS <= 4 ? 3 : WAR
 // tables leave no padding (the earlier tables for blocks of 8 over the whole
 // row summed 1.24 pairs per useful one at 32^2, these 1.04), and two CTAs share
 // an SM at 32^2, so that the end of one tile overlaps the other.  4099 cells of
-// 32^2 in FP64: 8.76 -> 7.56 ms.
+// 32^2 in FP64: 8.76 -> 7.25 ms.
 //
 // One block of RR l_2 steps and one row pair, as block_pq and row_pass_pq; Term
 // supplies the value type (what a spectrum entry is) and the product sums.
@@ -899,7 +899,7 @@ struct Term64 {
 // accurate as if computed in twice the working precision; the real and
 // imaginary parts are the two lanes, and the _rn intrinsics pin the operations.
 // The FMA pipe bounds the kernel (70 % busy): 28 FP32x2 operations per pair.
-// 4096 cells of 32^2: 1.53 -> 1.27 ms by the tables and the split of the last tiles.
+// 4096 cells of 32^2: 1.53 -> 1.22 ms by the tables and the split of the last tiles.
 // Not kept: Dekker's three-operation sums on operands ordered by selects (22
 // operations, the same numbers) moved the bound to the ALU pipe, 1.55 ms; a
 // running sum biased so that it always exceeds the product needs 16 operations

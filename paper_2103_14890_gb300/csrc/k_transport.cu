@@ -26,7 +26,7 @@
 //   fn), and divides by |P_i|.
 // FP64 rows hold the flux (v.n times the mean) instead, and pass 2 adds them up:
 // the product and the normal velocity would take as long again (0.106 ms for
-// 0.041 on 2603 cells x 30^2) and gain no accuracy.  The exception are faces whose
+// 0.050 on 2603 cells x 30^2) and gain no accuracy.  The exception are faces whose
 // two copies, a period apart in a periodic mesh, differ by rounding (kFvSplit):
 // with one side's normal for both, a cell's normals no longer sum to zero (errors
 // on 300 and 1200 Voronoi cells 2.2e-15 and 3.3e-15 of L's norm, 1.1e-15 and
@@ -43,11 +43,11 @@
 // cell in place of 5 and 24 for degree 2) and cuts the arithmetic that bounds
 // FP64 (the GB300 does 2 FP64 operations per clock and SM): per hexagon face
 // and velocity 9 operations in place of 34.  19802 triangles x 32^2, FP32,
-// degree 2: 0.382 -> 0.253 ms; 2603 Voronoi cells x 30^2, FP64, degree 2: 2.13
+// degree 2: 0.382 -> 0.238 ms; 2603 Voronoi cells x 30^2, FP64, degree 2: 2.13
 // -> 1.34 ms, 1.20 with p_0's rows and one difference per neighbour in the
 // cells flagged kFvRegular (pass 1 1.27 -> 1.13 ms, the FP64 pipe nine tenths
 // busy), 1.03 with signs, comparisons and 1 / #sectors off that pipe (pass 1
-// 0.98 ms, sums 0.070 -> 0.041).
+// 0.98 ms, sums 0.070 -> 0.050).
 //
 // Reconstruction: the central (least-squares) coefficients and the sector
 // polynomials are linear in the averages (tables Rc, Rs of fv_mesh.cpp);
