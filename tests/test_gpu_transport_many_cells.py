@@ -42,7 +42,7 @@ def _check(got, want, per_area, L, fmax, extra=0.0):
 @pytest.mark.parametrize("order", [2, 3])
 @pytest.mark.parametrize("size,N", [(70, 12), (70, 16), (70, 20), (70, 24), (70, 28), (70, 32), (70, 36), (20, 24), (20, 32),
                                     (100, 32)])
-def test_many_rounds(bz, size, N, order):
+def test_many_cells_per_block(bz, size, N, order):
     import torch
     pts, tri, per_area = _mesh(size)
     L = 6.0
